@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libdsbcg.so")
-SOURCES = ["dslash.cu", "blas.cu", "blas_p64.cu", "blas_p32.cu", "blas_bf16.cu", "blas_f16.cu", "small.cu", "pack.cu", "force.cu", "solver.cu"]
+SOURCES = ["dslash.cu", "dslash_fx.cu", "blas.cu", "blas_p64.cu", "blas_p32.cu", "blas_bf16.cu", "blas_f16.cu", "small.cu", "pack.cu", "force.cu", "solver.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I" + INCLUDE, "-I" + CSRC]

@@ -1,0 +1,463 @@
+// The Wilson stencil of FP64 fields in block fixed point, on the integer
+// multiply-add pipe.
+//
+// GB300 retires 2 FP64 FMA per SM and clock but 64 32 x 32 -> 64 bit integer
+// multiply-adds (measured: 2.0 and 63.4), so the products of the stencil are
+// formed in integers: a real number is two limbs h 2^29 + l with |l| <= 2^28,
+// and a real multiply-add is three mad.wide (h h, h l, l h; the l l product
+// is below the last bit kept).  Limbs add without carries, so the spin
+// projections are 32-bit adds.
+//
+// Format of a field ("FX"): [32-site tile][spin-colour component 12][site of
+// the tile] int4 (re.h, re.l, im.h, im.l), so that a hop's loads are one
+// address and immediate offsets, and one exponent per site: component value =
+// (h 2^29 + l) 2^E with |h 2^29 + l| <= 2^57, the largest component of the
+// site above 2^56.  Links: the limbs of -k' u 2^58, where kappa = k' 2^-ks with
+// |k'| < 1, [mu][entry][site]; links in SU(3) only (|u| <= 1).  The factor
+// 2^-ks is an exponent offset of the hopping term.
+//
+// Error.  A hop's result is exact to about one unit 2^E of its neighbour site
+// (the dropped l l products, the rounding of the h l sums and of k' u), and
+// the sum over eight hops adds up to one unit of the largest exponent per
+// hop, a unit being at most 2^-57 of the largest component of the nine sites
+// and typically 2^-60: below the 2^-53 per operation of an FP64 chain.
+//
+// Overflow.  The limbs of a projected half spinor are at most 2^29 (sums of
+// two), those of a link at most 2^29 and 2^28.  A link row has norm <= 1, so
+// the h h sums of a component stay below 2^29 2^29 sqrt(6) < 2^60, the mixed
+// sums below 2^61, a hop's result below 2^59.3 and the sum over eight hops and
+// the diagonal term below 2^62.4.
+//
+// A site that is all zero has exponent FX_ZERO.  A site with a NaN, an
+// infinity or a largest exponent outside the range in which every result is
+// a normal FP64 number sets *flag and turns its neighbourhood into NaN
+// (FX_NAN) or, when tiny, counts as zero; dsbcg_apply then repeats the
+// application with the FP64 kernels.
+#include "kernels.h"
+
+namespace dsbcg {
+
+namespace {
+
+constexpr int FX_ZERO = -(1 << 20), FX_NAN = 1 << 20;
+// biased exponents of a site's largest component for which the FX path holds
+constexpr int FX_EB_MIN = 300, FX_EB_MAX = 1800;
+constexpr int FX_BASE = 29;                    // bits per limb
+constexpr int FX_BITS = 57;                    // magnitude bits of a field value
+constexpr int FX_TILE = 12 * 32;               // int4 per 32-site tile
+
+__device__ __forceinline__ int2 fx_split(long long x) {
+    const int h = (int)((x + (1ll << (FX_BASE - 1))) >> FX_BASE);
+    return make_int2(h, (int)((unsigned)x - ((unsigned)h << FX_BASE)));
+}
+__device__ __forceinline__ long long fx_join(int h, int l) { return (long long)h * (1 << FX_BASE) + l; }
+// x 2^-s rounded to nearest, s >= 0
+__device__ __forceinline__ long long fx_shift(long long x, int s) {
+    if (s > 62) return 0;
+    return s > 0 ? (x + (1ll << (s - 1))) >> s : x;
+}
+// FP64 v in units of 2^(eb - 1079), eb >= v's biased exponent
+__device__ __forceinline__ long long fx_of_double(double v, int eb) {
+    const int hi = __double2hiint(v);
+    const int e = (hi >> 20) & 0x7ff;
+    const long long mant =
+        ((long long)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 32) | (unsigned)__double2loint(v);
+    const long long x = fx_shift(mant << 4, eb - (e ? e : 1));
+    return hi < 0 ? -x : x;
+}
+// element of component 0 of site y
+__device__ __forceinline__ size_t fx_at(int y) { return (size_t)(y >> 5) * FX_TILE + (y & 31); }
+
+// FP64 field block (pair-chunk layout) -> FX fields and site exponents.  One
+// thread per (site, field).  Bound by HBM: 16 bytes per complex in and out.
+__global__ void __launch_bounds__(128) fx_convert_kernel(int4* __restrict__ out, int* __restrict__ eo,
+                                                         const double2* __restrict__ in, size_t ld, int V,
+                                                         const Ctl* __restrict__ ctl, int nf_static,
+                                                         int* __restrict__ flag) {
+    int nf = nf_static;
+    if (ctl) {
+        if (ctl->done) return;
+        nf = ctl->mk;
+    }
+    const int x = (int)(blockIdx.x * 128u + threadIdx.x), f = (int)blockIdx.y;
+    if (f >= nf || x >= V) return;
+    const double2* p = in + (size_t)f * ld;
+    double2 v[12];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const double2* q = p + ((size_t)c * V + x) * 2;
+        v[2 * c] = __ldg(q);
+        v[2 * c + 1] = __ldg(q + 1);
+    }
+    int mx = 0;
+    unsigned any = 0;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const int a = __double2hiint(v[c].x) & 0x7fffffff, b = __double2hiint(v[c].y) & 0x7fffffff;
+        mx = max(mx, max(a, b));
+        any |= (unsigned)(a | b) | (unsigned)__double2loint(v[c].x) | (unsigned)__double2loint(v[c].y);
+    }
+    const int eb = mx >> 20;
+    int E = eb - 1079;
+    if (!any) {
+        E = FX_ZERO;
+    } else if (eb > FX_EB_MAX) {
+        E = FX_NAN;
+        if (flag) atomicOr(flag, 1);
+    } else if (eb < FX_EB_MIN) {
+        E = FX_ZERO;
+        if (flag) atomicOr(flag, 1);
+    }
+    const bool live = E != FX_ZERO && E != FX_NAN;
+    eo[(size_t)f * V + x] = E;
+    int4* o = out + (size_t)f * ld + fx_at(x);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const int2 re = fx_split(live ? fx_of_double(v[c].x, eb) : 0ll);
+        const int2 im = fx_split(live ? fx_of_double(v[c].y, eb) : 0ll);
+        o[c * 32] = make_int4(re.x, re.y, im.x, im.y);
+    }
+}
+
+// canonical links -> FX links [mu][entry][site]; kfix = -k' 2^63.  The product
+// k' u is formed from u 2^62 (exact above 2^-9) in 128 bits.
+__global__ void fx_pack_links_kernel(int4* __restrict__ dst, const double2* __restrict__ src, size_t V,
+                                     long long kfix) {
+    const size_t total = V * 36;
+    auto limbs = [&](double u) {
+        const long long p = __mul64hi(__double2ll_rn(ldexp(u, 62)), kfix);      // -k' u 2^61
+        return fx_split((p + 4) >> 3);
+    };
+    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
+         t += (size_t)gridDim.x * blockDim.x) {
+        const size_t x = t % V;
+        const int r = (int)(t / V);                       // mu * 9 + entry
+        const double2 u = src[x * 36 + r];
+        const int2 re = limbs(u.x), im = limbs(u.y);
+        dst[t] = make_int4(re.x, re.y, im.x, im.y);
+    }
+}
+
+__device__ __forceinline__ int4 iadd(int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ int4 isub(int4 a, int4 b) { return make_int4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+// a + i b, a - i b
+__device__ __forceinline__ int4 iaddi(int4 a, int4 b) { return make_int4(a.x - b.z, a.y - b.w, a.z + b.x, a.w + b.y); }
+__device__ __forceinline__ int4 isubi(int4 a, int4 b) { return make_int4(a.x + b.z, a.y + b.w, a.z - b.x, a.w - b.y); }
+
+struct ll2 {
+    long long x, y;
+};
+// a += s q, s = +1 (PLUS) or -1, or s i q (ROT)
+template <bool PLUS, bool ROT>
+__device__ __forceinline__ void lacc(ll2& a, ll2 q) {
+    const long long x = ROT ? -q.y : q.x, y = ROT ? q.x : q.y;
+    if (PLUS) { a.x += x; a.y += y; }
+    else { a.x -= x; a.y -= y; }
+}
+
+// One hop, for the half-spinor component (spin) S of a site: p the
+// neighbour's components (stride 32), su the hop's link in shared memory
+// (entry stride 32; U^H already for a backward hop), sh the shift from the
+// hop's exponent to the accumulators'.  MINUS: projector 1 - gamma_MU, else
+// 1 + gamma_MU.  The result goes to spin S (up) and to the lower spin it
+// rebuilds (lo): the other thread's for mu = x, y, this thread's for z, t.
+template <int MU, bool MINUS, int S>
+__device__ __forceinline__ void fx_hop(const int4* __restrict__ p, const int4* su, int sh, ll2 up[3], ll2 lo[3]) {
+    constexpr int T = MU < 2 ? 1 - S : S;                 // lower spin of the projection
+    constexpr bool NEG = (MU == 1 || MU == 2) && S == 1 ? !MINUS : MINUS;
+    int4 h[3];
+    int2 ni[3];                                           // minus the imaginary parts
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int4 u = __ldg(p + (S * 3 + a) * 32), l = __ldg(p + ((2 + T) * 3 + a) * 32);
+        if (MU == 0 || MU == 2) h[a] = NEG ? isubi(u, l) : iaddi(u, l);
+        else h[a] = NEG ? isub(u, l) : iadd(u, l);
+        ni[a] = make_int2(-h[a].z, -h[a].w);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        long long hr = 0, hi = 0, mr = 0, mi = 0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int4 u = su[(a * 3 + b) * 32];
+            const int4 v = h[b];
+            hr += (long long)u.x * v.x;
+            hi += (long long)u.x * v.z;
+            mr += (long long)u.x * v.y;
+            mi += (long long)u.x * v.w;
+            hr += (long long)u.z * ni[b].x;
+            hi += (long long)u.z * v.x;
+            mr += (long long)u.y * v.x;
+            mi += (long long)u.y * v.z;
+            mr += (long long)u.z * ni[b].y;
+            mi += (long long)u.z * v.y;
+            mr += (long long)u.w * ni[b].x;
+            mi += (long long)u.w * v.x;
+        }
+        ll2 q;
+        q.x = (hr + (mr >> FX_BASE)) >> sh;
+        q.y = (hi + (mi >> FX_BASE)) >> sh;
+        lacc<true, false>(up[a], q);
+        // lower spins of 1 - gamma_mu: i q for x, (q1, -q0) for y, (i q0, -i q1)
+        // for z and -q for t; the opposite for 1 + gamma_mu
+        if (MU == 0) lacc<MINUS, true>(lo[a], q);
+        if (MU == 1) lacc<(S == 1) == MINUS, false>(lo[a], q);
+        if (MU == 2) lacc<(S == 0) == MINUS, true>(lo[a], q);
+        if (MU == 3) lacc<!MINUS, false>(lo[a], q);
+    }
+}
+
+// the four hops in x, y (HALFH = 0) or z, t (1); sy: their neighbour sites
+// (stride 32), sh: their shifts, six bits each
+template <bool DAG, int S, int HALFH>
+__device__ __forceinline__ void fx_hops(const int4* __restrict__ fin, const int* sy, const int4* sl, unsigned sh,
+                                        ll2 up[3], ll2 lo[3]) {
+    constexpr int HS = 9 * 32, M = 2 * HALFH;
+    sy += 4 * 32 * HALFH;
+    sl += 4 * HS * HALFH;
+    fx_hop<M, !DAG, S>(fin + fx_at(sy[0]), sl, (int)sh & 63, up, lo);
+    fx_hop<M, DAG, S>(fin + fx_at(sy[32]), sl + HS, (int)(sh >> 6) & 63, up, lo);
+    fx_hop<M + 1, !DAG, S>(fin + fx_at(sy[64]), sl + 2 * HS, (int)(sh >> 12) & 63, up, lo);
+    fx_hop<M + 1, DAG, S>(fin + fx_at(sy[96]), sl + 3 * HS, (int)(sh >> 18) & 63, up, lo);
+}
+
+// out = src - kappa H in (H the hopping term; DAG: gamma_5 H gamma_5), fields
+// in FX; out FP64 (pair-chunk layout, OUT64) or FX.  src = in gives D (D^H).
+// HALF: in on the other parity of the even-odd lattice, src and out on
+// `parity`.  src NULL and neg: out = kappa H in.
+//
+// A CTA covers 32 sites of FX_FIELDS fields, two warps per field (one per
+// spin of the half spinor: half the accumulators and operands per thread),
+// with the tile's eight links per site staged in shared memory once (36 KB;
+// backward links as U^H, the time-boundary sign folded in).  A thread first
+// takes the x and y hops, whose lower-spin sums belong to the other warp and
+// go to it through shared memory, then the z and t hops, so that only one set
+// of lower-spin sums is in registers.
+//
+// Bound: per site and field 1728 mad.wide at 64 per SM and clock, 27 clocks,
+// beside about as many adds, shifts and shared-memory loads; latency-bound at
+// 16 warps per SM (IPC 1.6).  Measured, 16^3 x 32, 12 fields, one D: 0.47 ms
+// against 2.51 ms of the FP64 kernel; 4^4, 4 fields: 12 against 36 us.  Other
+// shapes: one thread per site and field 0.60 ms; 80 registers and 24 warps
+// 0.50 (spills); 2 or 3 fields per CTA 0.57-0.60 (links staged more often).
+constexpr int FX_FIELDS = 4;
+static_assert(2 * FX_FIELDS <= 8, "the exchange of leading-zero counts reuses the 8 x 32 words of the sites");
+
+template <bool DAG, bool OUT64, bool HALF>
+__global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
+    void* __restrict__ outv, int* __restrict__ eo, const int4* __restrict__ in, const int* __restrict__ ei,
+    const int4* __restrict__ src, const int* __restrict__ es, size_t ld, const int4* __restrict__ links, Geom g,
+    int kshift, int neg, int parity, const Ctl* __restrict__ ctl, int nf_static, int ngrp) {
+    extern __shared__ __align__(16) unsigned char fx_smem[];
+    int4* sl = reinterpret_cast<int4*>(fx_smem);               // [hop][entry][lane]
+    ll2* ex = reinterpret_cast<ll2*>(sl + 8 * 9 * 32);         // [warp][colour][lane]
+    int* sy = reinterpret_cast<int*>(ex + 2 * FX_FIELDS * 3 * 32);     // [hop][lane]
+    int nf = nf_static;
+    if (ctl) {
+        if (ctl->done) return;
+        nf = ctl->mk;
+    }
+    const int nw = (int)(blockDim.x >> 5), nfc = nw >> 1;      // warps, fields of the CTA
+    const int grp = (int)(blockIdx.x % (unsigned)ngrp);
+    if (grp * nfc >= nf) return;                               // CTA-uniform
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const size_t V = (size_t)g.V;
+    const int Vf = HALF ? g.V / 2 : g.V;
+    const int k = (int)(blockIdx.x / (unsigned)ngrp) * 32 + lane;
+    const int ks = k < Vf ? k : Vf - 1;
+    int c[4], x;
+    if (HALF) {
+        const int hx = g.L[0] / 2;
+        const int row = ks / hx;
+        c[1] = row % g.L[1];
+        c[2] = (row / g.L[1]) % g.L[2];
+        c[3] = row / (g.L[1] * g.L[2]);
+        c[0] = 2 * (ks % hx) + ((parity + c[1] + c[2] + c[3]) & 1);
+        x = c[0] + g.L[0] * row;
+    } else {
+        x = ks;
+        c[0] = x % g.L[0];
+        int r = x / g.L[0];
+        c[1] = r % g.L[1];
+        r /= g.L[1];
+        c[2] = r % g.L[2];
+        c[3] = r / g.L[2];
+    }
+    // warp w stages the hops w, w + nw, ...: neighbour site and link
+    for (int h = w; h < 8; h += nw) {
+        const int mu = h >> 1;
+        const bool fwd = (h & 1) == 0;
+        int st = 1;
+        for (int d = 0; d < mu; ++d) st *= g.L[d];
+        const int cm = mu == 0 ? c[0] : mu == 1 ? c[1] : mu == 2 ? c[2] : c[3], L = g.L[mu];
+        const bool wrap = fwd ? cm == L - 1 : cm == 0;
+        const int y = x + (fwd ? st : -st) * (wrap ? 1 - L : 1);
+        const bool edge = mu == 3 && g.tap && wrap;
+        const int s = edge != (neg != 0) ? -1 : 1, sz = fwd ? s : -s;      // conjugate: the imaginary part's sign
+        const int4* u = links + (size_t)mu * 9 * V + (fwd ? x : y);
+        sy[h * 32 + lane] = HALF ? y >> 1 : y;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const int4 q = __ldg(u + (size_t)e * V);
+            sl[(h * 9 + (fwd ? e : (e % 3) * 3 + e / 3)) * 32 + lane] = make_int4(s * q.x, s * q.y, sz * q.z, sz * q.w);
+        }
+    }
+    __syncthreads();
+    const int S = w & 1;
+    const int f = grp * nfc + (w >> 1);
+    const bool on = f < nf;                                    // warp-uniform
+    ll2 up[3], lo[3];
+    int Em = FX_ZERO, e0 = FX_ZERO;
+    const int4* fin = in + (size_t)f * ld;
+    unsigned shl = 0, shh = 0;
+    // the diagonal term of spin s in the accumulators' unit (zero without src)
+    auto diag = [&](int s, ll2 d[3]) {
+        const int4* p = src + (size_t)f * ld + fx_at(ks) + s * 96;
+        const int sr = max(0, min(Em - e0, 63)), sf = max(0, e0 - Em);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            d[a] = ll2{0, 0};
+            if (src) {
+                const int4 u = __ldg(p + a * 32);
+                d[a] = ll2{fx_join(u.x, u.y) >> sr << sf, fx_join(u.z, u.w) >> sr << sf};
+            }
+        }
+    };
+    if (on) {
+        const int* fe = ei + (size_t)f * Vf;
+        if (src) e0 = __ldg(es + (size_t)f * Vf + ks);
+        int eh[8];
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+            eh[h] = __ldg(fe + sy[h * 32 + lane]) - kshift;
+            Em = max(Em, eh[h]);
+        }
+        // the diagonal term (at most 2^57) has bits to spare: its unit may be up to 2^4 of the accumulators'
+        Em = max(Em, e0 - 4);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            shl |= (unsigned)min(Em - eh[h], 63) << (6 * h);
+            shh |= (unsigned)min(Em - eh[4 + h], 63) << (6 * h);
+        }
+        diag(S, up);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) lo[a] = ll2{0, 0};
+        if (S == 0) fx_hops<DAG, 0, 0>(fin, sy + lane, sl + lane, shl, up, lo);
+        else fx_hops<DAG, 1, 0>(fin, sy + lane, sl + lane, shl, up, lo);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) ex[(w * 3 + a) * 32 + lane] = lo[a];
+        diag(2 + S, lo);
+        if (S == 0) fx_hops<DAG, 0, 1>(fin, sy + lane, sl + lane, shh, up, lo);
+        else fx_hops<DAG, 1, 1>(fin, sy + lane, sl + lane, shh, up, lo);
+    }
+    __syncthreads();
+    if (on) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const ll2 q = ex[((w ^ 1) * 3 + a) * 32 + lane];
+            lo[a].x += q.x;
+            lo[a].y += q.y;
+        }
+    }
+    const bool bad = Em > FX_NAN / 2;
+    const bool store = on && k < Vf;
+    if (OUT64) {
+        // v 2^Em: the conversion rounds to FP64, the exponent is added to its bits (the result is a normal
+        // number: FX_EB_MIN, FX_EB_MAX)
+        if (!store) return;
+        double2* o = reinterpret_cast<double2*>(outv) + (size_t)f * ld;
+        auto out = [&](long long v) -> double {
+            const double d = __ll2double_rn(v);
+            if (bad) return __longlong_as_double(0x7ff8000000000000ll);
+            return v ? __hiloint2double(__double2hiint(d) + Em * (1 << 20), __double2loint(d)) : 0.0;
+        };
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int i = S * 3 + a, j = (2 + S) * 3 + a;
+            o[((size_t)(i >> 1) * Vf + k) * 2 + (i & 1)] = make_double2(out(up[a].x), out(up[a].y));
+            o[((size_t)(j >> 1) * Vf + k) * 2 + (j & 1)] = make_double2(out(lo[a].x), out(lo[a].y));
+        }
+    } else {
+        unsigned long long mag = 0;
+        if (!on) up[0] = up[1] = up[2] = lo[0] = lo[1] = lo[2] = ll2{0, 0};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            mag |= (unsigned long long)(up[a].x ^ (up[a].x >> 63)) | (unsigned long long)(up[a].y ^ (up[a].y >> 63));
+            mag |= (unsigned long long)(lo[a].x ^ (lo[a].x >> 63)) | (unsigned long long)(lo[a].y ^ (lo[a].y >> 63));
+        }
+        // bits of the site's largest magnitude, over both warps -> FX_BITS
+        int* ez = sy;                                          // the neighbour sites are no longer needed
+        ez[w * 32 + lane] = __clzll((long long)mag);
+        __syncthreads();
+        if (!store) return;
+        const int lz = min(ez[w * 32 + lane], ez[(w ^ 1) * 32 + lane]);
+        const int sft = lz - (64 - FX_BITS);
+        int4* o = reinterpret_cast<int4*>(outv) + (size_t)f * ld + fx_at(k);
+        if (S == 0) eo[(size_t)f * Vf + k] = bad ? FX_NAN : (lz < 64 ? Em - sft : FX_ZERO);
+        auto limbs = [&](long long v) { return fx_split(sft >= 0 ? v << sft : fx_shift(v, -sft)); };
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int2 ur = limbs(up[a].x), ui = limbs(up[a].y), lr = limbs(lo[a].x), li = limbs(lo[a].y);
+            o[(S * 3 + a) * 32] = make_int4(ur.x, ur.y, ui.x, ui.y);
+            o[((2 + S) * 3 + a) * 32] = make_int4(lr.x, lr.y, li.x, li.y);
+        }
+    }
+}
+
+// kappa = k 2^-*shift with 1/2 <= |k| < 1 (0 for 0)
+double fx_mantissa(double kappa, int* shift) {
+    int e = 0;
+    const double k = frexp(kappa, &e);
+    *shift = kappa == 0.0 ? 0 : -e;
+    return k;
+}
+
+}  // namespace
+
+bool fx_kappa_fits(double kappa) { return kappa == 0.0 || (fabs(kappa) > 1e-9 && fabs(kappa) < 1e3); }
+
+void launch_fx_links(void* dst, const double2* src, size_t V, double kappa, cudaStream_t st) {
+    int ks;
+    const long long kfix = -(long long)ldexp(fx_mantissa(kappa, &ks), 63);
+    const size_t grid = (V * 36 + 255) / 256;
+    fx_pack_links_kernel<<<(unsigned)(grid < 65535 ? grid : 65535), 256, 0, st>>>((int4*)dst, src, V, kfix);
+}
+
+void launch_fx_convert(void* out, int* eo, const void* in, size_t ld, size_t Vf, const Ctl* ctl, int nf_static,
+                       int nf_max, int* flag, cudaStream_t st) {
+    const int nfg = ctl ? nf_max : nf_static;
+    const dim3 grid((unsigned)((Vf + 127) / 128), (unsigned)nfg);
+    fx_convert_kernel<<<grid, 128, 0, st>>>((int4*)out, eo, (const double2*)in, ld, (int)Vf, ctl, nf_static, flag);
+}
+
+void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const void* src, const int* es, size_t ld,
+                       const void* links, const Geom& g, double kappa, int dag, int half, int parity, int out64,
+                       const Ctl* ctl, int nf_static, int nf_max, cudaStream_t st) {
+    const int nfg = ctl ? nf_max : nf_static;
+    const int nfc = nfg < FX_FIELDS ? nfg : FX_FIELDS;
+    const int ngrp = (nfg + nfc - 1) / nfc;
+    const size_t Vf = half ? (size_t)g.V / 2 : (size_t)g.V;
+    const unsigned grid = (unsigned)((size_t)ngrp * ((Vf + 31) / 32));
+    int ks;
+    fx_mantissa(kappa, &ks);
+    const int neg = src ? 0 : 1;
+    constexpr int SMEM = 8 * 9 * 32 * sizeof(int4) + 2 * FX_FIELDS * 3 * 32 * sizeof(ll2) + 8 * 32 * sizeof(int);
+#define DSBCG_FX(DAG, O64, HALF)                                                                                    \
+    {                                                                                                              \
+        static std::atomic<unsigned long long> devs{0};                                                            \
+        max_dyn_smem_once(fx_stencil_kernel<DAG, O64, HALF>, SMEM, devs);                                          \
+        fx_stencil_kernel<DAG, O64, HALF><<<grid, 64 * nfc, SMEM, st>>>(out, eo, (const int4*)in, ei,               \
+                                                                        (const int4*)src, es, ld, (const int4*)links, \
+                                                                        g, ks, neg, parity, ctl, nf_static, ngrp);   \
+    }
+    if (half) {
+        if (out64) { if (dag) DSBCG_FX(true, true, true) else DSBCG_FX(false, true, true) }
+        else { if (dag) DSBCG_FX(true, false, true) else DSBCG_FX(false, false, true) }
+    } else {
+        if (out64) { if (dag) DSBCG_FX(true, true, false) else DSBCG_FX(false, true, false) }
+        else { if (dag) DSBCG_FX(true, false, false) else DSBCG_FX(false, false, false) }
+    }
+#undef DSBCG_FX
+}
+
+}  // namespace dsbcg

@@ -84,6 +84,22 @@ void launch_dslash_half(int prec, void* out, const void* in, const void* src, si
                         const Geom& g, double alpha, double beta, int parity, int g5in, int g5out, const Ctl* ctl,
                         int nf_static, int nf_max, float hscale, cudaStream_t st);
 
+// ---- dslash_fx.cu: FP64 fields in block fixed point (links in SU(3)) ----------
+// an FX field block takes the bytes of an FP64 one (stride ld complex, a
+// multiple of 384) plus one int exponent per site and field; FX links take
+// those of FP64 links
+bool fx_kappa_fits(double kappa);            // the hopping coefficient's exponent is in the range of the format
+void launch_fx_links(void* dst, const double2* src, size_t V, double kappa, cudaStream_t st);
+// FP64 fields (internal layout, Vf sites) -> FX; *flag |= 1 where the FX range does not hold (flag may be NULL)
+void launch_fx_convert(void* out, int* eo, const void* in, size_t ld, size_t Vf, const Ctl* ctl, int nf_static,
+                       int nf_max, int* flag, cudaStream_t st);
+// out = src - kappa H in (dag: gamma_5 H gamma_5), or kappa H in when src is
+// NULL.  Full lattice (half = 0) or half fields on `parity`; out64: FP64
+// output, else FX
+void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const void* src, const int* es, size_t ld,
+                       const void* links, const Geom& g, double kappa, int dag, int half, int parity, int out64,
+                       const Ctl* ctl, int nf_static, int nf_max, cudaStream_t st);
+
 // ---- blas.cu ----------------------------------------------------------------
 int gram_blocks(size_t n, int nf_max);
 // partial sums of X^H Y (nf x nf, FP64) per CTA; herm = 1 computes only the

@@ -70,6 +70,7 @@ struct Lane {
     cudaEvent_t ready = nullptr;                  // own lanes: main-stream work they wait for
     void *vring = nullptr, *zw = nullptr, *y = nullptr, *P = nullptr, *Xin = nullptr;
     void* eotmp = nullptr;                        // Schur operator: even-parity half fields
+    int* fxe = nullptr;                           // FP64 storage: site exponents of fixed-point fields
     double2* rhs = nullptr;                       // gathered right-hand sides (high precision)
     double* partials = nullptr;
     int nblk = 0;
@@ -110,6 +111,9 @@ struct dsbcg_ctx {
     // link of the field is in SU(3) to 1e-10 (su3); the stencil rebuilds row 2
     void* links12[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     bool su3 = false;
+    void* linksfx = nullptr;             // fixed-point copy for the FP64 stencil (SU(3) links only)
+    int* fx_flag = nullptr;              // device word: an application left the fixed-point range
+    int* h_fx_flag = nullptr;            // pinned
     float hscale = 1.f;
     bool gauge_ok = false;               // gauge64 holds a checked field and links[] were packed from it
     // refinement stream (true residuals, restarts' bookkeeping) beside the
@@ -137,6 +141,8 @@ struct dsbcg_ctx {
         void *vring = nullptr, *zw = nullptr, *y = nullptr;       // storage precision
         void* eotmp = nullptr;                                    // Schur: even-parity half fields
         double2* T64c = nullptr;                                  // Schur: high-precision half fields
+        int* fxe = nullptr;                                       // site exponents of the true residuals' fields
+        bool fx_resid = false;                                    // true residuals take the fixed-point stencil
         void *P = nullptr, *Xin = nullptr;                        // work precision
         double2 *B64 = nullptr, *X64 = nullptr, *R64 = nullptr, *T64a = nullptr, *T64b = nullptr, *rhs = nullptr;
         double2 *Xg = nullptr, *Bg = nullptr;
@@ -270,8 +276,39 @@ dsbcg_status ensure_links(dsbcg_ctx* c, int prec) {
         CK(cudaGetLastError());
         c->links12[prec] = q;
     }
+    if (c->su3 && prec == P64 && !c->linksfx) {
+        // the fixed-point links are an option: without memory for them the
+        // FP64 stencil runs on the FP64 pipe
+        void* q = nullptr;
+        if (cudaMalloc(&q, c->V * 36 * sizeof(double2)) == cudaSuccess) {
+            launch_fx_links(q, c->gauge64, c->V, c->kappa, c->st);
+            CK(cudaGetLastError());
+            c->linksfx = q;
+        } else {
+            cudaGetLastError();
+        }
+    }
     return DSBCG_OK;
 }
+
+// The fixed-point FP64 stencil serves this context's operator: links in
+// SU(3) and a kappa in the range of the format
+bool fx_usable(const dsbcg_ctx* c) {
+    return c->linksfx && fx_kappa_fits(c->kappa);
+}
+// True residuals of m columns in fixed point: always for FP64 storage, and for
+// the reduced storages from FX_RESID_MIN sites x columns of the full lattice.
+// Below it the FP64 residuals run beside latency-bound restarts and cost
+// little, and the solutions stay bitwise those of the FP64 chain, which an
+// FP32 link gradient that rounds them to 24 bits shows.  Solves (m of them,
+// s = 8, FP32 storage) on the FP64 pipe / in fixed point, ms: 8^3 x 16, 8:
+// 24.4 / 22.2; 8^3 x 16, 12: 35.5 / 32.3; 8^2 x 16^2, 8 (at the line): 34.7 /
+// 28.6; 12^3 x 24, 6: 53.6 / 44.2; 12^3 x 24, 12: 99.4 / 80.3.
+constexpr size_t FX_RESID_MIN = (size_t)1 << 17;
+bool fx_residuals(const dsbcg_ctx* c, int prec, int m) { return prec == P64 || c->V * m >= FX_RESID_MIN; }
+// site exponents of the fields of one fixed-point operator application of m
+// fields: input, middle and (Schur) even-parity fields
+size_t fx_exp_bytes(const dsbcg_ctx* c, int m) { return 3 * (size_t)m * c->Vf * sizeof(int); }
 
 // Block steps per shift-update chunk for a lane whose basis blocks take
 // block_bytes: cmax (a power of two, at most CTL_HIST), halved while the
@@ -316,6 +353,7 @@ dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
         CKS(dmalloc(c, &w.eotmp, m * fb));
         CKS(dmalloc(c, (void**)&w.T64c, m * db));
     }
+    if (c->linksfx) CKS(dmalloc(c, (void**)&w.fxe, fx_exp_bytes(c, m)));
     CKS(dmalloc(c, (void**)&w.P, (size_t)s * m * wb));
     CKS(dmalloc(c, (void**)&w.Xin, (size_t)s * m * wb));
     CKS(dmalloc(c, (void**)&w.B64, (size_t)nbb * m * db));
@@ -383,6 +421,7 @@ dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
     w.prec = prec;
     w.nbb = nbb;
     Lane L0;
+    if (c->linksfx && prec == P64) CKS(dmalloc(c, (void**)&L0.fxe, fx_exp_bytes(c, m)));
     L0.st = c->st;
     L0.vring = w.vring;
     L0.zw = w.zw;
@@ -428,7 +467,7 @@ int ensure_refine_lanes(dsbcg_ctx* c, int want) {
     const int chunk = chunk_steps((size_t)m * fb, 16, 64);
     const size_t lane_bytes = (c->schur ? 3 : 2) * m * fb + (size_t)(chunk + 1) * m * fb + 2 * m * wb + m * db +
                               gram_partial_doubles(M_MAX) * sizeof(double) + small_state_bytes(1) +
-                              (4 + 2 * (size_t)chunk) * tb;
+                              (4 + 2 * (size_t)chunk) * tb + (prec == P64 ? fx_exp_bytes(c, m) : 0);
     while ((int)w.lanes.size() < want) {
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
@@ -441,6 +480,7 @@ int ensure_refine_lanes(dsbcg_ctx* c, int want) {
         L.chunk = chunk;
         bool ok = dmalloc(c, &L.vring, (size_t)(chunk + 1) * m * fb) == DSBCG_OK && dmalloc(c, &L.zw, m * fb) == DSBCG_OK &&
                   (!c->schur || dmalloc(c, &L.eotmp, m * fb) == DSBCG_OK) &&
+                  (prec != P64 || !c->linksfx || dmalloc(c, (void**)&L.fxe, fx_exp_bytes(c, m)) == DSBCG_OK) &&
                   dmalloc(c, &L.y, m * fb) == DSBCG_OK && dmalloc(c, &L.P, m * wb) == DSBCG_OK &&
                   dmalloc(c, &L.Xin, m * wb) == DSBCG_OK && dmalloc(c, (void**)&L.rhs, m * db) == DSBCG_OK &&
                   dmalloc(c, (void**)&L.partials, gram_partial_doubles(M_MAX) * sizeof(double)) == DSBCG_OK &&
@@ -603,8 +643,42 @@ int residual_ctas(dsbcg_ctx* c) {
 // A = D^H D (two stencils; mid receives D in) or, on a context with the Schur
 // operator, Ahat = Dhat^H Dhat (four half-lattice passes; mid receives
 // Dhat in, tmp is scratch for even-parity half fields)
+//
+// FP64 fields with fxe (site exponents, see fx_exp_bytes) take the
+// fixed-point stencil where fx_usable: in is converted into out's memory, the
+// intermediate fields stay in fixed point and the last pass writes FP64.
+// flag: see launch_fx_convert.
 void apply_op(dsbcg_ctx* c, int p, void* out, void* mid, const void* in, void* tmp, size_t ld, const Ctl* ctl,
-              int nf_static, int nf_max, float hs, cudaStream_t st, int cls) {
+              int nf_static, int nf_max, float hs, cudaStream_t st, int cls, int* fxe = nullptr,
+              int* flag = nullptr) {
+    if (p == P64 && fxe && fx_usable(c)) {
+        int *e0 = fxe, *e1 = fxe + (size_t)(ctl ? nf_max : nf_static) * c->Vf;
+        int* e2 = e1 + (e1 - e0);
+        {
+            Prof q(c, cls == DSBCG_KCLASS_RESIDUAL ? cls : DSBCG_KCLASS_OTHER, 1, st);
+            launch_fx_convert(out, e0, in, ld, c->Vf, ctl, nf_static, nf_max, flag, st);
+        }
+        for (int dag = 0; dag < 2; ++dag) {
+            const void* x = dag ? mid : out;              // the pass's input, also its diagonal term
+            const int* ex = dag ? e1 : e0;
+            void* y = dag ? out : mid;
+            if (c->schur) {
+                {
+                    Prof q(c, cls, 1, st);
+                    launch_fx_stencil(tmp, e2, x, ex, nullptr, nullptr, ld, c->linksfx, c->g, c->kappa, dag, 1, 0, 0, ctl,
+                                      nf_static, nf_max, st);
+                }
+                Prof q(c, cls, 1, st);
+                launch_fx_stencil(y, e1, tmp, e2, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, dag,
+                                  ctl, nf_static, nf_max, st);
+            } else {
+                Prof q(c, cls, 1, st);
+                launch_fx_stencil(y, e1, x, ex, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, dag, ctl,
+                                  nf_static, nf_max, st);
+            }
+        }
+        return;
+    }
     if (c->schur) {
         apply_dhat(c, p, mid, in, tmp, ld, 0, ctl, nf_static, nf_max, hs, st, cls);
         apply_dhat(c, p, out, mid, tmp, ld, 1, ctl, nf_static, nf_max, hs, st, cls);
@@ -629,7 +703,8 @@ inline double link_passes(const dsbcg_ctx* c) { return c->schur ? 4.0 : 2.0; }
 
 // out = A in (or Ahat in) for nf high-precision fields (tmp receives D in), on stream st
 void apply_Ahp(dsbcg_ctx* c, int hp, void* out, const void* in, void* tmp, int nf, cudaStream_t st) {
-    apply_op(c, hp, out, tmp, in, c->ws.T64c, hp_ld(c, hp), nullptr, nf, nf, 1.f, st, DSBCG_KCLASS_RESIDUAL);
+    apply_op(c, hp, out, tmp, in, c->ws.T64c, hp_ld(c, hp), nullptr, nf, nf, 1.f, st, DSBCG_KCLASS_RESIDUAL,
+             c->ws.fx_resid ? c->ws.fxe : nullptr);
 }
 
 // r = b - sigma x - A x for m high-precision fields on stream st; squared
@@ -769,7 +844,7 @@ dsbcg_status lane_enqueue(dsbcg_ctx* c, Lane& L) {
         void* Vk = slot(step);
         void* Vo = slot(step - 1);     // V_{k-1} (unused at k = 1)
         const int hs = (step - 1) % C;                 // this step's coefficient and flag slot
-        apply_op(c, prec, L.y, L.zw, Vk, L.eotmp, ld, L.ctl, 0, m_in, c->hscale, st, DSBCG_KCLASS_DSLASH);
+        apply_op(c, prec, L.y, L.zw, Vk, L.eotmp, ld, L.ctl, 0, m_in, c->hscale, st, DSBCG_KCLASS_DSLASH, L.fxe);
         {
             Prof p(c, DSBCG_KCLASS_GRAM, 1, st);
             // alpha_k = V_k^H A V_k is hermitian: the upper 4 x 4 tiles of
@@ -942,6 +1017,7 @@ dsbcg_status solve_core(dsbcg_ctx* c, int m, const void* B, int nbb, int s, cons
     CKS(ensure_links(c, hp));
     CKS(ensure_ws(c, m, s, prec, nbb));
     auto& w = c->ws;
+    w.fx_resid = fx_residuals(c, prec, m);
     const size_t n = c->n, ld = c->ld;
     const size_t db = ld * sizeof(double2);
     for (int q = 0; q < 8; ++q) {
@@ -1471,7 +1547,7 @@ dsbcg_status dsbcg_create(dsbcg_ctx** out, const int dims[4], const void* gauge,
     c->V = V;
     c->Vf = V;
     c->n = 12 * V;
-    c->ld = (c->n + 127) / 128 * 128;
+    c->ld = (c->n + 383) / 384 * 384;
     c->kappa = kappa;
     c->st = (cudaStream_t)stream;
     // 16-bit scale: power of two near sqrt(n)
@@ -1502,6 +1578,8 @@ dsbcg_status dsbcg_update_gauge(dsbcg_ctx* c, const void* gauge) {
             c->links12[p] = nullptr;
         }
     }
+    if (c->linksfx) cudaFree(c->linksfx);
+    c->linksfx = nullptr;
     const size_t bytes = c->V * 36 * sizeof(double2);
     if (!c->gauge64) CK(cudaMalloc((void**)&c->gauge64, bytes));
     CK(cudaMemcpyAsync(c->gauge64, gauge, bytes, is_device_ptr(gauge) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
@@ -1548,6 +1626,9 @@ void dsbcg_destroy(dsbcg_ctx* c) {
         if (c->links[p]) cudaFree(c->links[p]);
         if (c->links12[p]) cudaFree(c->links12[p]);
     }
+    if (c->linksfx) cudaFree(c->linksfx);
+    if (c->fx_flag) cudaFree(c->fx_flag);
+    if (c->h_fx_flag) cudaFreeHost(c->h_fx_flag);
     if (c->gauge64) cudaFree(c->gauge64);
     if (c->rst) cudaStreamDestroy(c->rst);
     if (c->ev_joint) cudaEventDestroy(c->ev_joint);
@@ -1593,7 +1674,43 @@ dsbcg_status dsbcg_read_profile(dsbcg_ctx* c, double kernel_ms[8], long long ker
     return DSBCG_OK;
 }
 
-dsbcg_status dsbcg_apply(dsbcg_ctx* c, int op, int storage, int m, const void* in, void* out) {
+}  // extern "C"
+
+namespace {
+
+// D, D^H or A (Dhat, Dhat^H, Ahat) of m FP64 fields in fixed point: a -> b,
+// t and t2 (Schur) are scratch, a is kept; *c->fx_flag as launch_fx_convert
+void fx_apply(dsbcg_ctx* c, int op, void* b, void* t, void* t2, const void* a, int m, int* fxe) {
+    cudaMemsetAsync(c->fx_flag, 0, sizeof(int), c->st);
+    const size_t ld = c->ld;
+    if (op == DSBCG_OP_A) {
+        apply_op(c, P64, b, t, a, t2, ld, nullptr, m, m, 1.f, c->st, DSBCG_KCLASS_DSLASH, fxe, c->fx_flag);
+        return;
+    }
+    const int dag = op == DSBCG_OP_DDAG;
+    int *e0 = fxe, *e1 = fxe + (size_t)m * c->Vf;
+    {
+        Prof q(c, DSBCG_KCLASS_OTHER);
+        launch_fx_convert(t, e0, a, ld, c->Vf, nullptr, m, m, c->fx_flag, c->st);
+    }
+    if (c->schur) {
+        {
+            Prof q(c, DSBCG_KCLASS_DSLASH);
+            launch_fx_stencil(t2, e1, t, e0, nullptr, nullptr, ld, c->linksfx, c->g, c->kappa, dag, 1, 0, 0, nullptr, m, m,
+                              c->st);
+        }
+        Prof q(c, DSBCG_KCLASS_DSLASH);
+        launch_fx_stencil(b, nullptr, t2, e1, t, e0, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, 1, nullptr,
+                          m, m, c->st);
+    } else {
+        Prof q(c, DSBCG_KCLASS_DSLASH);
+        launch_fx_stencil(b, nullptr, t, e0, t, e0, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, 1, nullptr, m, m,
+                          c->st);
+    }
+}
+
+// dsbcg_apply; fixed: FP64 fields may take the fixed-point stencil
+dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* in, void* out, bool fixed) {
     if (!c || !in || !out || m < 1 || m > 4096 || op < 0 || op > 2 || storage < 0 || storage > PDD)
         return DSBCG_ERR_ARG;
     if (!c->gauge_ok) return DSBCG_ERR_ARG;
@@ -1601,9 +1718,19 @@ dsbcg_status dsbcg_apply(dsbcg_ctx* c, int op, int storage, int m, const void* i
     const size_t n = c->n, ld = hp_ld(c, storage);
     const size_t fb = prec_elem_bytes(storage) * c->ld;
     void *a = nullptr, *b = nullptr, *t = nullptr, *t2 = nullptr;
+    int* fxe = nullptr;
     double2 *din = nullptr, *dout = nullptr;
     const bool in_dev = is_device_ptr(in), out_dev = is_device_ptr(out);
     dsbcg_status rs = DSBCG_OK;
+    if (fixed && storage == P64 && fx_usable(c) &&
+        (!c->fx_flag && (cudaMalloc((void**)&c->fx_flag, sizeof(int)) != cudaSuccess ||
+                         cudaMallocHost((void**)&c->h_fx_flag, sizeof(int)) != cudaSuccess)))
+        cudaGetLastError();               // without the flag: the FP64 pipe
+    if (fixed && storage == P64 && fx_usable(c) && c->h_fx_flag &&
+        cudaMalloc((void**)&fxe, fx_exp_bytes(c, m)) != cudaSuccess) {
+        cudaGetLastError();
+        fxe = nullptr;
+    }
     auto fail = [&](dsbcg_status s) { rs = s; };
     if (cudaMalloc(&a, m * fb) != cudaSuccess || cudaMalloc(&b, m * fb) != cudaSuccess ||
         cudaMalloc(&t, m * fb) != cudaSuccess || (c->schur && cudaMalloc(&t2, m * fb) != cudaSuccess)) {
@@ -1620,7 +1747,9 @@ dsbcg_status dsbcg_apply(dsbcg_ctx* c, int op, int storage, int m, const void* i
         const double2* src = in_dev ? (const double2*)in : din;
         double2* dst = out_dev ? (double2*)out : dout;
         pack_any(c, storage, a, src, m);
-        if (op == DSBCG_OP_A) {
+        if (fxe) {
+            fx_apply(c, op, b, t, t2, a, m, fxe);
+        } else if (op == DSBCG_OP_A) {
             apply_op(c, storage, b, t, a, t2, ld, nullptr, m, m, c->hscale, c->st, DSBCG_KCLASS_DSLASH);
         } else if (c->schur) {
             apply_dhat(c, storage, b, a, t, ld, op == DSBCG_OP_DDAG, nullptr, m, m, c->hscale, c->st,
@@ -1632,17 +1761,30 @@ dsbcg_status dsbcg_apply(dsbcg_ctx* c, int op, int storage, int m, const void* i
         }
         unpack_any(c, storage, dst, b, m);
         if (!out_dev) cudaMemcpyAsync(out, dout, m * n * sizeof(double2), cudaMemcpyDeviceToHost, c->st);
+        if (fxe) cudaMemcpyAsync(c->h_fx_flag, c->fx_flag, sizeof(int), cudaMemcpyDeviceToHost, c->st);
         if (cudaGetLastError() != cudaSuccess) fail(DSBCG_ERR_CUDA);
         if (cudaStreamSynchronize(c->st) != cudaSuccess) fail(DSBCG_ERR_CUDA);
         prof_collect(c);
     }
+    // a site outside the fixed-point range (NaN, Inf, extreme magnitudes):
+    // the FP64 kernels' result replaces this one
+    const bool again = rs == DSBCG_OK && fxe && *c->h_fx_flag;
+    if (fxe) cudaFree(fxe);
     cudaFree(a);
     cudaFree(b);
     cudaFree(t);
     if (t2) cudaFree(t2);
     if (din) cudaFree(din);
     if (dout) cudaFree(dout);
-    return rs;
+    return again ? apply_fields(c, op, storage, m, in, out, false) : rs;
+}
+
+}  // namespace
+
+extern "C" {
+
+dsbcg_status dsbcg_apply(dsbcg_ctx* c, int op, int storage, int m, const void* in, void* out) {
+    return apply_fields(c, op, storage, m, in, out, true);
 }
 
 dsbcg_status dsbcg_set_operator(dsbcg_ctx* c, int op) {
@@ -1655,7 +1797,7 @@ dsbcg_status dsbcg_set_operator(dsbcg_ctx* c, int op) {
     c->schur = op == DSBCG_OPERATOR_SCHUR;
     c->Vf = c->schur ? c->V / 2 : c->V;
     c->n = 12 * c->Vf;
-    c->ld = (c->n + 127) / 128 * 128;
+    c->ld = (c->n + 383) / 384 * 384;
     c->hscale = (float)ldexp(1.0, (int)lround(0.5 * log2((double)c->n)));
     return DSBCG_OK;
 }
@@ -1903,8 +2045,9 @@ extern "C" dsbcg_status dsbcg_apply_static(dsbcg_ctx* c, int op, int storage, in
     if (!c->gauge_ok) return DSBCG_ERR_ARG;
     if (!is_device_ptr(in) || !is_device_ptr(out)) return DSBCG_ERR_ARG;
     if (!c->links[storage] || c->schur) return DSBCG_ERR_UNSUPPORTED;
-    const size_t ld = hp_ld(c, storage);
-    const size_t fb = prec_elem_bytes(storage) * c->ld;
+    // the documented scratch size: fields at multiples of 128 elements
+    const size_t ld0 = (c->n + 127) / 128 * 128, ld = storage == PDD ? 2 * ld0 : ld0;
+    const size_t fb = prec_elem_bytes(storage) * ld0;
     const size_t nbuf = op == DSBCG_OP_A ? 3 : 2;
     if ((size_t)m > (size_t)DSBCG_STATIC_SCRATCH_BYTES / (nbuf * fb)) return DSBCG_ERR_ARG;
     void* base = nullptr;
@@ -1914,7 +2057,10 @@ extern "C" dsbcg_status dsbcg_apply_static(dsbcg_ctx* c, int op, int storage, in
     char* t = b + (size_t)m * fb;
     const double2* src = (const double2*)in;
     double2* dst = (double2*)out;
-    pack_any(c, storage, a, src, m);
+    if (storage == PDD)
+        launch_pack_pairs((float2*)a, ld0, src, m, c->V, c->st);
+    else
+        launch_pack_fields(storage, a, ld0, src, m, c->V, c->hscale, c->st);
     if (op == DSBCG_OP_D) {
         launch_dslash(storage, b, a, ld, c->links[storage], c->g, c->kappa, 0, nullptr, m, m, c->hscale, c->st);
     } else if (op == DSBCG_OP_DDAG) {
@@ -1923,7 +2069,10 @@ extern "C" dsbcg_status dsbcg_apply_static(dsbcg_ctx* c, int op, int storage, in
         launch_dslash(storage, t, a, ld, c->links[storage], c->g, c->kappa, 0, nullptr, m, m, c->hscale, c->st);
         launch_dslash(storage, b, t, ld, c->links[storage], c->g, c->kappa, 1, nullptr, m, m, c->hscale, c->st);
     }
-    unpack_any(c, storage, dst, b, m);
+    if (storage == PDD)
+        launch_unpack_pairs(dst, (const float2*)b, ld0, m, c->V, c->st);
+    else
+        launch_unpack_fields(storage, dst, b, ld0, m, c->V, c->hscale, c->st);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->st));
     return DSBCG_OK;
