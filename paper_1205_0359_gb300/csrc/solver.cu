@@ -54,6 +54,14 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
+// One device block kept from call to call (scratch_get): grown on demand, and
+// given back when it is large, when the solver's workspace needs the memory,
+// and with the context.
+struct Scratch {
+    char* p = nullptr;
+    size_t bytes = 0, used = 0;
+};
+
 struct KEvent {
     int cls;
     cudaEvent_t a, b;
@@ -112,8 +120,14 @@ struct dsbcg_ctx {
     void* links12[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     bool su3 = false;
     void* linksfx = nullptr;             // fixed-point copy for the FP64 stencil (SU(3) links only)
-    int* fx_flag = nullptr;              // device word: an application left the fixed-point range
-    int* h_fx_flag = nullptr;            // pinned
+    // the buffers behind the pointers above: an update of the gauge field
+    // clears those (no copy of the old field stays in use) and fills these anew
+    void *links_mem[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    void *links12_mem[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    void* linksfx_mem = nullptr;
+    int* flags = nullptr;                // device words: [0] fixed-point range left, [1, 2] gauge checks
+    int* h_flags = nullptr;              // pinned copies
+    Scratch scr;                         // working fields of apply and force
     float hscale = 1.f;
     bool gauge_ok = false;               // gauge64 holds a checked field and links[] were packed from it
     // refinement stream (true residuals, restarts' bookkeeping) beside the
@@ -262,30 +276,81 @@ void free_ws(dsbcg_ctx* c) {
 
 size_t prec_elem_bytes(int p) { return (size_t)prec_bytes(p); }
 
+void scratch_free(dsbcg_ctx* c) {
+    if (c->scr.p) cudaFree(c->scr.p);
+    c->scr = Scratch();
+}
+// Make at least `bytes` of scratch available and start handing it out anew
+// (scratch_take).  The calls that use it run on the context's stream alone and
+// wait for it before they return, so a later call may write it.
+dsbcg_status scratch_get(Scratch& s, size_t bytes) {
+    s.used = 0;
+    if (s.bytes >= bytes) return DSBCG_OK;
+    if (s.p) cudaFree(s.p);
+    s = Scratch();
+    if (cudaMalloc((void**)&s.p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        s.p = nullptr;
+        return DSBCG_ERR_OOM;
+    }
+    s.bytes = bytes;
+    return DSBCG_OK;
+}
+constexpr size_t SCRATCH_ALIGN = 256;
+size_t scratch_round(size_t bytes) { return (bytes + SCRATCH_ALIGN - 1) / SCRATCH_ALIGN * SCRATCH_ALIGN; }
+void* scratch_take(Scratch& s, size_t bytes) {
+    void* p = s.p + s.used;
+    s.used += scratch_round(bytes);
+    return p;
+}
+// Kept blocks are at most 1/32 of the device memory; cudaMalloc and cudaFree
+// cost 0.65 ms of a 1.0 ms application of A to 12 FP32 fields of 16^3 x 32, and
+// 3.2 of 7.1 ms of a force call.
+void scratch_trim(Scratch& s) {
+    size_t fr = 0, tot = 0;
+    if (s.bytes <= (64u << 20)) return;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) cudaGetLastError();
+    if (s.bytes > tot / 32) {
+        cudaFree(s.p);
+        s = Scratch();
+    }
+}
+dsbcg_status ensure_flags(dsbcg_ctx* c) {
+    if (!c->flags) CK(cudaMalloc((void**)&c->flags, 4 * sizeof(int)));
+    if (!c->h_flags) CK(cudaMallocHost((void**)&c->h_flags, 4 * sizeof(int)));
+    return DSBCG_OK;
+}
+
+// a buffer of packed links, kept for the context's life
+dsbcg_status link_alloc(dsbcg_ctx* c, void** p, size_t bytes_per_site) {
+    if (*p || cudaMalloc(p, c->V * bytes_per_site) == cudaSuccess) return DSBCG_OK;
+    cudaGetLastError();
+    scratch_free(c);
+    if (cudaMalloc(p, c->V * bytes_per_site) == cudaSuccess) return DSBCG_OK;
+    cudaGetLastError();
+    *p = nullptr;
+    return DSBCG_ERR_OOM;
+}
+
 dsbcg_status ensure_links(dsbcg_ctx* c, int prec) {
     if (c->links[prec]) return DSBCG_OK;
-    void* p = nullptr;
-    CK(cudaMalloc(&p, c->V * 36 * prec_elem_bytes(prec)));
-    launch_pack_links(prec, p, c->gauge64, c->V, c->st);
+    CKS(link_alloc(c, &c->links_mem[prec], 36 * prec_elem_bytes(prec)));
+    launch_pack_links(prec, c->links_mem[prec], c->gauge64, c->V, c->st);
     CK(cudaGetLastError());
-    c->links[prec] = p;
+    c->links[prec] = c->links_mem[prec];
     if (c->su3 && (prec == P32 || prec == PBF16 || prec == PF16) && !c->links12[prec]) {
-        void* q = nullptr;
-        CK(cudaMalloc(&q, c->V * 24 * prec_elem_bytes(prec)));
-        launch_pack_links12(prec, q, c->gauge64, c->V, c->st);
+        CKS(link_alloc(c, &c->links12_mem[prec], 24 * prec_elem_bytes(prec)));
+        launch_pack_links12(prec, c->links12_mem[prec], c->gauge64, c->V, c->st);
         CK(cudaGetLastError());
-        c->links12[prec] = q;
+        c->links12[prec] = c->links12_mem[prec];
     }
     if (c->su3 && prec == P64 && !c->linksfx) {
         // the fixed-point links are an option: without memory for them the
         // FP64 stencil runs on the FP64 pipe
-        void* q = nullptr;
-        if (cudaMalloc(&q, c->V * 36 * sizeof(double2)) == cudaSuccess) {
-            launch_fx_links(q, c->gauge64, c->V, c->kappa, c->st);
+        if (link_alloc(c, &c->linksfx_mem, 36 * sizeof(double2)) == DSBCG_OK) {
+            launch_fx_links(c->linksfx_mem, c->gauge64, c->V, c->kappa, c->st);
             CK(cudaGetLastError());
-            c->linksfx = q;
-        } else {
-            cudaGetLastError();
+            c->linksfx = c->linksfx_mem;
         }
     }
     return DSBCG_OK;
@@ -342,6 +407,7 @@ dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
     auto& w = c->ws;
     if (w.prec == prec && w.m == m && w.s >= s && w.nbb >= nbb) return DSBCG_OK;
     free_ws(c);
+    scratch_free(c);                     // the workspace sizes itself by the memory that is free
     const size_t ld = c->ld, n = c->n;
     const size_t fb = prec_elem_bytes(prec) * ld;           // storage field bytes
     const size_t wb = prec_elem_bytes(work_prec(prec)) * ld; // work field bytes
@@ -468,6 +534,7 @@ int ensure_refine_lanes(dsbcg_ctx* c, int want) {
     const size_t lane_bytes = (c->schur ? 3 : 2) * m * fb + (size_t)(chunk + 1) * m * fb + 2 * m * wb + m * db +
                               gram_partial_doubles(M_MAX) * sizeof(double) + small_state_bytes(1) +
                               (4 + 2 * (size_t)chunk) * tb + (prec == P64 ? fx_exp_bytes(c, m) : 0);
+    if ((int)w.lanes.size() < want) scratch_free(c);
     while ((int)w.lanes.size() < want) {
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
@@ -1564,40 +1631,24 @@ dsbcg_status dsbcg_create(dsbcg_ctx** out, const int dims[4], const void* gauge,
 dsbcg_status dsbcg_update_gauge(dsbcg_ctx* c, const void* gauge) {
     if (!c || !gauge) return DSBCG_ERR_ARG;
     // From here until the new field has been checked and packed the context
-    // holds no usable field: the old packed links go first, so that no
-    // precision keeps links of the old field while gauge64 holds the new one.
+    // holds no usable field: the old packed links go out of use first, so that
+    // no precision keeps links of the old field while gauge64 holds the new one.
     c->gauge_ok = false;
     c->su3 = false;
-    for (int p = 0; p < 5; ++p) {
-        if (c->links[p]) {
-            cudaFree(c->links[p]);
-            c->links[p] = nullptr;
-        }
-        if (c->links12[p]) {
-            cudaFree(c->links12[p]);
-            c->links12[p] = nullptr;
-        }
-    }
-    if (c->linksfx) cudaFree(c->linksfx);
+    for (int p = 0; p < 5; ++p) c->links[p] = c->links12[p] = nullptr;
     c->linksfx = nullptr;
     const size_t bytes = c->V * 36 * sizeof(double2);
     if (!c->gauge64) CK(cudaMalloc((void**)&c->gauge64, bytes));
+    CKS(ensure_flags(c));
     CK(cudaMemcpyAsync(c->gauge64, gauge, bytes, is_device_ptr(gauge) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                        c->st));
-    int* flag = nullptr;
-    CK(cudaMalloc((void**)&flag, 2 * sizeof(int)));
-    cudaMemsetAsync(flag, 0, sizeof(int), c->st);
-    launch_check_finite(c->gauge64, c->V * 36, flag, c->st);
-    int h = 0;
-    cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+    CK(cudaMemsetAsync(c->flags + 1, 0, 2 * sizeof(int), c->st));
+    launch_check_finite(c->gauge64, c->V * 36, c->flags + 1, c->st);
     // a field in SU(3) to 1e-10 gets 12-real links for the reduced storages
-    int hs = 1;
-    cudaMemsetAsync(flag + 1, 0, sizeof(int), c->st);
-    launch_check_su3(c->gauge64, c->V * 4, 1e-10, flag + 1, c->st);
-    cudaMemcpyAsync(&hs, flag + 1, sizeof(int), cudaMemcpyDeviceToHost, c->st);
-    const cudaError_t e = cudaStreamSynchronize(c->st);
-    cudaFree(flag);
-    CK(e);
+    launch_check_su3(c->gauge64, c->V * 4, 1e-10, c->flags + 2, c->st);
+    CK(cudaMemcpyAsync(c->h_flags + 1, c->flags + 1, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    const int h = c->h_flags[1], hs = c->h_flags[2];
     if (h) return DSBCG_ERR_NONFINITE;
     c->su3 = (hs == 0);
     CKS(ensure_links(c, P64));
@@ -1622,13 +1673,14 @@ dsbcg_status dsbcg_solve_rational(dsbcg_ctx* c, int m, const void* B, int s, con
 void dsbcg_destroy(dsbcg_ctx* c) {
     if (!c) return;
     free_ws(c);
+    scratch_free(c);
     for (int p = 0; p < 5; ++p) {
-        if (c->links[p]) cudaFree(c->links[p]);
-        if (c->links12[p]) cudaFree(c->links12[p]);
+        if (c->links_mem[p]) cudaFree(c->links_mem[p]);
+        if (c->links12_mem[p]) cudaFree(c->links12_mem[p]);
     }
-    if (c->linksfx) cudaFree(c->linksfx);
-    if (c->fx_flag) cudaFree(c->fx_flag);
-    if (c->h_fx_flag) cudaFreeHost(c->h_fx_flag);
+    if (c->linksfx_mem) cudaFree(c->linksfx_mem);
+    if (c->flags) cudaFree(c->flags);
+    if (c->h_flags) cudaFreeHost(c->h_flags);
     if (c->gauge64) cudaFree(c->gauge64);
     if (c->rst) cudaStreamDestroy(c->rst);
     if (c->ev_joint) cudaEventDestroy(c->ev_joint);
@@ -1679,19 +1731,19 @@ dsbcg_status dsbcg_read_profile(dsbcg_ctx* c, double kernel_ms[8], long long ker
 namespace {
 
 // D, D^H or A (Dhat, Dhat^H, Ahat) of m FP64 fields in fixed point: a -> b,
-// t and t2 (Schur) are scratch, a is kept; *c->fx_flag as launch_fx_convert
+// t and t2 (Schur) are scratch, a is kept; *c->flags as launch_fx_convert
 void fx_apply(dsbcg_ctx* c, int op, void* b, void* t, void* t2, const void* a, int m, int* fxe) {
-    cudaMemsetAsync(c->fx_flag, 0, sizeof(int), c->st);
+    cudaMemsetAsync(c->flags, 0, sizeof(int), c->st);
     const size_t ld = c->ld;
     if (op == DSBCG_OP_A) {
-        apply_op(c, P64, b, t, a, t2, ld, nullptr, m, m, 1.f, c->st, DSBCG_KCLASS_DSLASH, fxe, c->fx_flag);
+        apply_op(c, P64, b, t, a, t2, ld, nullptr, m, m, 1.f, c->st, DSBCG_KCLASS_DSLASH, fxe, c->flags);
         return;
     }
     const int dag = op == DSBCG_OP_DDAG;
     int *e0 = fxe, *e1 = fxe + (size_t)m * c->Vf;
     {
         Prof q(c, DSBCG_KCLASS_OTHER);
-        launch_fx_convert(t, e0, a, ld, c->Vf, nullptr, m, m, c->fx_flag, c->st);
+        launch_fx_convert(t, e0, a, ld, c->Vf, nullptr, m, m, c->flags, c->st);
     }
     if (c->schur) {
         {
@@ -1717,33 +1769,26 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     CKS(ensure_links(c, storage));
     const size_t n = c->n, ld = hp_ld(c, storage);
     const size_t fb = prec_elem_bytes(storage) * c->ld;
-    void *a = nullptr, *b = nullptr, *t = nullptr, *t2 = nullptr;
-    int* fxe = nullptr;
-    double2 *din = nullptr, *dout = nullptr;
     const bool in_dev = is_device_ptr(in), out_dev = is_device_ptr(out);
+    bool fx = fixed && storage == P64 && fx_usable(c);
+    const size_t db = m * n * sizeof(double2);
+    Scratch& scr = c->scr;
+    const size_t need = (c->schur ? 4 : 3) * scratch_round(m * fb) + (in_dev ? 0 : scratch_round(db)) +
+                        (out_dev ? 0 : scratch_round(db));
+    // without room for the site exponents the FP64 kernels serve the call
+    if (fx && (ensure_flags(c) != DSBCG_OK ||
+               scratch_get(scr, need + scratch_round(fx_exp_bytes(c, m))) != DSBCG_OK))
+        fx = false;
+    if (!fx) CKS(scratch_get(scr, need));
+    void *a = scratch_take(scr, m * fb), *b = scratch_take(scr, m * fb), *t = scratch_take(scr, m * fb);
+    void* t2 = c->schur ? scratch_take(scr, m * fb) : nullptr;
+    int* fxe = fx ? (int*)scratch_take(scr, fx_exp_bytes(c, m)) : nullptr;
+    double2* din = in_dev ? nullptr : (double2*)scratch_take(scr, db);
+    double2* dout = out_dev ? nullptr : (double2*)scratch_take(scr, db);
     dsbcg_status rs = DSBCG_OK;
-    if (fixed && storage == P64 && fx_usable(c) &&
-        (!c->fx_flag && (cudaMalloc((void**)&c->fx_flag, sizeof(int)) != cudaSuccess ||
-                         cudaMallocHost((void**)&c->h_fx_flag, sizeof(int)) != cudaSuccess)))
-        cudaGetLastError();               // without the flag: the FP64 pipe
-    if (fixed && storage == P64 && fx_usable(c) && c->h_fx_flag &&
-        cudaMalloc((void**)&fxe, fx_exp_bytes(c, m)) != cudaSuccess) {
-        cudaGetLastError();
-        fxe = nullptr;
-    }
     auto fail = [&](dsbcg_status s) { rs = s; };
-    if (cudaMalloc(&a, m * fb) != cudaSuccess || cudaMalloc(&b, m * fb) != cudaSuccess ||
-        cudaMalloc(&t, m * fb) != cudaSuccess || (c->schur && cudaMalloc(&t2, m * fb) != cudaSuccess)) {
-        fail(DSBCG_ERR_OOM);
-    }
-    if (rs == DSBCG_OK && !in_dev) {
-        if (cudaMalloc((void**)&din, m * n * sizeof(double2)) != cudaSuccess) fail(DSBCG_ERR_OOM);
-        else cudaMemcpyAsync(din, in, m * n * sizeof(double2), cudaMemcpyHostToDevice, c->st);
-    }
-    if (rs == DSBCG_OK && !out_dev) {
-        if (cudaMalloc((void**)&dout, m * n * sizeof(double2)) != cudaSuccess) fail(DSBCG_ERR_OOM);
-    }
-    if (rs == DSBCG_OK) {
+    if (!in_dev) cudaMemcpyAsync(din, in, db, cudaMemcpyHostToDevice, c->st);
+    {
         const double2* src = in_dev ? (const double2*)in : din;
         double2* dst = out_dev ? (double2*)out : dout;
         pack_any(c, storage, a, src, m);
@@ -1761,21 +1806,15 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
         }
         unpack_any(c, storage, dst, b, m);
         if (!out_dev) cudaMemcpyAsync(out, dout, m * n * sizeof(double2), cudaMemcpyDeviceToHost, c->st);
-        if (fxe) cudaMemcpyAsync(c->h_fx_flag, c->fx_flag, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+        if (fxe) cudaMemcpyAsync(c->h_flags, c->flags, sizeof(int), cudaMemcpyDeviceToHost, c->st);
         if (cudaGetLastError() != cudaSuccess) fail(DSBCG_ERR_CUDA);
         if (cudaStreamSynchronize(c->st) != cudaSuccess) fail(DSBCG_ERR_CUDA);
         prof_collect(c);
     }
     // a site outside the fixed-point range (NaN, Inf, extreme magnitudes):
     // the FP64 kernels' result replaces this one
-    const bool again = rs == DSBCG_OK && fxe && *c->h_fx_flag;
-    if (fxe) cudaFree(fxe);
-    cudaFree(a);
-    cudaFree(b);
-    cudaFree(t);
-    if (t2) cudaFree(t2);
-    if (din) cudaFree(din);
-    if (dout) cudaFree(dout);
+    const bool again = rs == DSBCG_OK && fx && c->h_flags[0];
+    scratch_trim(scr);
     return again ? apply_fields(c, op, storage, m, in, out, false) : rs;
 }
 
@@ -1813,19 +1852,20 @@ dsbcg_status dsbcg_force(dsbcg_ctx* c, int m, int s, const void* X, const void* 
     const int nf = m * s;
     const size_t fb = prec_elem_bytes(storage) * ld;
     const size_t cb = (size_t)nf * n * sizeof(double2);
-    void *xf = nullptr, *lf = nullptr, *ex = nullptr, *el = nullptr;
-    double2 *stage = nullptr, *du = nullptr;
-    double* wf = nullptr;
+    const size_t ub = V * 36 * sizeof(double2);
     dsbcg_status rs = DSBCG_OK;
-    if (cudaMalloc(&xf, nf * fb) || cudaMalloc(&lf, nf * fb) || cudaMalloc(&ex, nf * fb) ||
-        cudaMalloc(&el, nf * fb) || cudaMalloc((void**)&du, V * 36 * sizeof(double2)) ||
-        cudaMalloc((void**)&wf, nf * sizeof(double)))
-        rs = DSBCG_ERR_OOM;
     const bool xd = is_device_ptr(X), ldv = is_device_ptr(Lambda), ud = is_device_ptr(dU);
-    if (rs == DSBCG_OK && (!xd || !ldv)) {
-        if (cudaMalloc((void**)&stage, cb)) rs = DSBCG_ERR_OOM;
-    }
-    if (rs == DSBCG_OK) {
+    // the kernel writes 16-byte elements: straight into the caller's device buffer when it is aligned to them
+    const bool direct = ud && (size_t)dU % sizeof(double2) == 0;
+    Scratch& scr = c->scr;
+    CKS(scratch_get(scr, 4 * scratch_round(nf * fb) + (direct ? 0 : scratch_round(ub)) + scratch_round(nf * sizeof(double)) +
+                                (xd && ldv ? 0 : scratch_round(cb))));
+    void *xf = scratch_take(scr, nf * fb), *lf = scratch_take(scr, nf * fb), *ex = scratch_take(scr, nf * fb),
+         *el = scratch_take(scr, nf * fb);
+    double2* du = direct ? (double2*)dU : (double2*)scratch_take(scr, ub);
+    double* wf = (double*)scratch_take(scr, nf * sizeof(double));
+    double2* stage = xd && ldv ? nullptr : (double2*)scratch_take(scr, cb);
+    {
         std::vector<double> wh(nf);
         for (int j = 0; j < s; ++j)
             for (int i = 0; i < m; ++i) wh[(size_t)j * m + i] = weights ? weights[j] : 1.0;
@@ -1850,21 +1890,12 @@ dsbcg_status dsbcg_force(dsbcg_ctx* c, int m, int s, const void* X, const void* 
             Prof p(c, DSBCG_KCLASS_OTHER);
             launch_force(storage, du, ex, lf, el, xf, ld, nf, wf, c->g, c->kappa, c->st);
         }
-        if (ud) {
-            cudaMemcpyAsync(dU, du, V * 36 * sizeof(double2), cudaMemcpyDeviceToDevice, c->st);
-        } else {
-            cudaMemcpyAsync(dU, du, V * 36 * sizeof(double2), cudaMemcpyDeviceToHost, c->st);
-        }
+        if (!direct)
+            cudaMemcpyAsync(dU, du, ub, ud ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->st);
         if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(c->st) != cudaSuccess) rs = DSBCG_ERR_CUDA;
         prof_collect(c);
     }
-    cudaFree(xf);
-    cudaFree(lf);
-    cudaFree(ex);
-    cudaFree(el);
-    cudaFree(du);
-    cudaFree(wf);
-    if (stage) cudaFree(stage);
+    scratch_trim(scr);
     return rs;
 }
 
