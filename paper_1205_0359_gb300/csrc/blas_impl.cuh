@@ -153,7 +153,22 @@ static __global__ void gram_reduce_kernel(const double* __restrict__ partials, i
     double s = 0.0;
     if (fp32) {
         const float* p = reinterpret_cast<const float*>(partials) + (size_t)tile * nblk * GSLOTS;
-        for (int b = 0; b < nblk; ++b) s += (double)p[(size_t)b * GSLOTS + q];
+        // one FP64 addition per partial, in order; loads sixteen ahead
+        constexpr int RC = 16;
+        float v[RC], w[RC];
+        auto fetch = [&](float* d, int b) {
+#pragma unroll
+            for (int r = 0; r < RC; ++r) d[r] = b + r < nblk ? p[(size_t)(b + r) * GSLOTS + q] : 0.f;
+        };
+        fetch(v, 0);
+        for (int b = 0; b < nblk; b += RC) {
+            fetch(w, b + RC);
+#pragma unroll
+            for (int r = 0; r < RC; ++r)
+                if (b + r < nblk) s += widen(v[r]);
+#pragma unroll
+            for (int r = 0; r < RC; ++r) v[r] = w[r];
+        }
     } else {
         const double* p = partials + (size_t)tile * nblk * GSLOTS;
         for (int b = 0; b < nblk; ++b) s += p[(size_t)b * GSLOTS + q];

@@ -123,6 +123,15 @@ template <class C> __device__ __forceinline__ C ctimesi(C a) { return mk(-a.y, a
 // -a (exact; a negation modifier of the consuming instruction in FP32/FP64)
 template <class C> __device__ __forceinline__ C cneg(C a) { return mk(-a.x, -a.y); }
 
+// FP32 -> FP64, exact: by its bits for zeros and normal numbers (the
+// conversion instruction runs at the FP64 rate, 1/64 of FP32's)
+__device__ __forceinline__ double widen(float v) {
+    const unsigned u = __float_as_uint(v), a = u & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(a << 29));
+    return a == 0 ? __hiloint2double((int)u, 0) : (double)v;
+}
+
 // ------------------------------------------------------------ double-float --
 // An unevaluated sum hi + lo of two FP32 numbers with |lo| <= ulp(hi) / 2:
 // 48 significand bits, the FP32 exponent range.  GB300 executes FP64 (and

@@ -158,12 +158,13 @@ void launch_small_init(SmallState* ss, Ctl* ctl, const double2* G0, const double
 // alpha_k from the Gram partials of V_k^H Y (+ coefficient tiles for the block update)
 void launch_small_alpha(SmallState* ss, const Ctl* ctl, const double* partials, int nblk, int nf_max,
                         int wprec, int sfp64, void* coef_a, void* coef_bh, cudaStream_t st);
-// W^H W from the Gram partials, pivoted QR with deflation, per-shift recurrences
-void launch_small_step(SmallState* ss, Ctl* ctl, const double* partials, int nblk, int s, int m,
-                       double dtol, const double* sigma_dev, const double* target_dev, int freeze,
-                       int wprec, int sfp64, void* coefS_w, void* coefU_w, void* coefL_w, int* active,
-                       int* conv_step, double* res_out, cudaStream_t st);
-void launch_small_finish(SmallState* ss, Ctl* ctl, int s, int m, const int* active, cudaStream_t st);
+// W^H W from the Gram partials, pivoted QR with deflation: S, beta_{k+1}, m_{k+1}
+void launch_small_qr(SmallState* ss, Ctl* ctl, const double* partials, int nblk, int m, double dtol, int wprec,
+                     int sfp64, void* coefS_w, cudaStream_t st);
+// per-shift recurrences (a CTA per shift) and the close of the block step
+void launch_small_recur(SmallState* ss, Ctl* ctl, int s, int m, const double* sigma_dev, const double* target_dev,
+                        int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* active, int* conv_step,
+                        double* res_out, cudaStream_t st);
 const double2* small_state_S(const SmallState* ss);
 
 // ---- force.cu ---------------------------------------------------------------

@@ -1,5 +1,6 @@
 // FP64 m x m kernels of the block Lanczos process and of the per-shift
-// recurrences (Sec. 3), run by one CTA (shared part) or one CTA per shift.
+// recurrences (Sec. 3): a few CTAs reduce the Gram partials and the last to
+// arrive does the shared m x m work; the recurrences take one CTA per shift.
 //
 // Block form.  The Lanczos blocks V_1, V_2, ... (widths m_k, shrinking on
 // deflation) satisfy
@@ -42,6 +43,10 @@
 
 namespace dsbcg {
 
+// group sums of one reduction: at most 1024 groups x slots, or 36 slots of
+// each of the 36 upper tiles of a 32 x 32 Gram matrix
+constexpr int RED_SLOTS = 36 * 36;
+
 template <class T>
 struct SmallSharedT {
     T alpha[M_MAX * M_MAX];          // alpha_k (hermitised)
@@ -49,6 +54,8 @@ struct SmallSharedT {
     T betan[M_MAX * M_MAX];          // beta_{k+1} (m_{k+1} x m_k)
     T S[M_MAX * M_MAX];              // V_{k+1} = W S (m_k x m_{k+1})
     T yy[M_MAX / 2];                 // ||A v_i||^2 (real scalars, two per entry)
+    double red[RED_SLOTS];           // group sums of the Gram partials (reduce_partials)
+    unsigned ticket[4];              // arrival counters of the multi-CTA kernels (zero between launches)
 };
 template <class T>
 struct SmallShiftT {
@@ -74,10 +81,12 @@ const double2* small_state_S(const SmallState* ss) { return ss->sh.S; }
 
 namespace {
 
-constexpr int WS = 32;             // the pivoted QR runs on one warp
-constexpr int NT = 1024;           // threads of the CTAs that also reduce partial sums
+constexpr int WS = 32;
+constexpr int QW = 4;              // warps of the pivoted QR: one per SM sub-partition
 constexpr int GSL = 36;            // slots per 4 x 4 tile in the Gram partials
-constexpr int RED_MAX = 1024;      // group sums held in shared memory by reduce_partials
+constexpr int RED_GROUPS = 1024;   // groups x slots of a reduction aim at this many chains
+constexpr int NRC = 8;             // CTAs of the kernels that reduce Gram partials
+constexpr int NT = 8 * GSL;        // threads per CTA: eight slot groups of a reduction, nine warps for the m x m work
 
 // ------------------------------------------------------------ scalars --
 // Sc<T>: real type R, complex T, and the operations the m x m algebra needs.
@@ -102,7 +111,7 @@ struct Sc<double2> {
     static __device__ __forceinline__ bool gt(R a, R b) { return a > b; }
     static __device__ __forceinline__ float2 f2(double2 a) { return make_float2((float)a.x, (float)a.y); }
     // sum of a Kahan-compensated FP32 sum (value s - c)
-    static __device__ __forceinline__ R kahan(float s, float c) { return (double)s - (double)c; }
+    static __device__ __forceinline__ R kahan(float s, float c) { return widen(s) - widen(c); }
 };
 
 // double-float reciprocal and square root: FP32 estimate refined by one
@@ -173,6 +182,24 @@ template <class T> __device__ __forceinline__ typename Sc<T>::R cnorm2(T a) {
 __device__ __forceinline__ void bsync() { __syncthreads(); }
 __device__ __forceinline__ void wsync() { __syncwarp(); }
 
+// True in the CTA of the grid that arrives last; every other CTA's earlier
+// writes are then visible to it (through ld_cg).  No CTA waits for another.
+// The counter wraps to zero for the next launch.
+__device__ __forceinline__ bool last_arrival(unsigned* ticket) {
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last != 0;
+}
+__device__ __forceinline__ double ld_cg(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ dd ld_cg(const dd* p) {
+    const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+    return dd(v.x, v.y);
+}
+
 // dst (r x c valid, R x Cc written, leading dim ld) <- src (M_MAX layout)
 template <class T>
 __device__ void ld_mat(T* dst, int ld, const T* src, int r, int c, int Rr, int Cc) {
@@ -187,32 +214,61 @@ template <class T>
 __device__ void st_mat_work(int wprec, void* dst, const T* src, int ld, int r, int c) {
     for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) {
         int i = t / M_MAX, j = t % M_MAX;
-        const T v = (i < r && j < c) ? src[i * ld + j] : cz<T>();
+        const bool in = i < r && j < c;
         if constexpr (is_fp64<T>()) {
             if (wprec == P64) {
-                reinterpret_cast<double2*>(dst)[t] = v;
+                reinterpret_cast<double2*>(dst)[t] = in ? src[i * ld + j] : cz<T>();
                 continue;
             }
         }
-        reinterpret_cast<float2*>(dst)[t] = Sc<T>::f2(v);
+        reinterpret_cast<float2*>(dst)[t] = in ? Sc<T>::f2(src[i * ld + j]) : make_float2(0.f, 0.f);
     }
 }
 
-// C (r x c) = op(A) op(B) (beta = 0) or C - op(A) op(B) (beta = 1), scaled
-// by sgn = +1 / -1 on the product; op: 0 plain, 1 conjugate transpose
+// real (0) or imaginary (1) part of an entry
+template <class T>
+__device__ __forceinline__ typename Sc<T>::R& part_of(T& a, int part) {
+    return reinterpret_cast<typename Sc<T>::R*>(&a)[part];
+}
+// x + a b and x - a b, one part of a complex entry (the expressions of cplus
+// and cminus with ctimes)
+template <class T>
+__device__ __forceinline__ typename Sc<T>::R plus_times(typename Sc<T>::R x, T a, T b, int part) {
+    using S = Sc<T>;
+    if (part == 0) return S::add(x, S::sub(S::mul(S::re(a), S::re(b)), S::mul(S::im(a), S::im(b))));
+    return S::add(x, S::add(S::mul(S::re(a), S::im(b)), S::mul(S::im(a), S::re(b))));
+}
+template <class T>
+__device__ __forceinline__ typename Sc<T>::R minus_times(typename Sc<T>::R x, T a, T b, int part) {
+    using S = Sc<T>;
+    if (part == 0) return S::sub(x, S::sub(S::mul(S::re(a), S::re(b)), S::mul(S::im(a), S::im(b))));
+    return S::sub(x, S::add(S::mul(S::re(a), S::im(b)), S::mul(S::im(a), S::re(b))));
+}
+// item t of 2 n: entry and part, the parts in different warps (up to one)
+__device__ __forceinline__ int item_of(int t, int n, int* part) {
+    *part = t >= n;
+    return t >= n ? t - n : t;
+}
+
+// C (r x c) = +-op(A) op(B), or C +- op(A) op(B) (accumulate); op: plain (0)
+// or conjugate transpose (1).  One thread per real number of the result, so
+// that the FP64 work spreads over the SM's sub-partitions.
 template <class T>
 __device__ void gemm(T* Cm, int ldc, const T* A, int lda, int ta, const T* B, int ldb, int tb, int r, int q, int c,
                      bool negate, bool accumulate) {
-    for (int t = threadIdx.x; t < r * c; t += blockDim.x) {
-        int i = t / c, j = t % c;
-        T s = cz<T>();
+    using S = Sc<T>;
+    for (int t = threadIdx.x; t < 2 * r * c; t += blockDim.x) {
+        int part;
+        const int e = item_of(t, r * c, &part), i = e / c, j = e % c;
+        typename S::R s = S::r(0.0);
         for (int l = 0; l < q; ++l) {
-            T a = ta ? cconj(A[l * lda + i]) : A[i * lda + l];
-            T b = tb ? cconj(B[j * ldb + l]) : B[l * ldb + j];
-            s = cplus(s, ctimes(a, b));
+            const T a = ta ? cconj(A[l * lda + i]) : A[i * lda + l];
+            const T b = tb ? cconj(B[j * ldb + l]) : B[l * ldb + j];
+            s = plus_times<T>(s, a, b, part);
         }
-        if (accumulate) Cm[i * ldc + j] = negate ? cminus(Cm[i * ldc + j], s) : cplus(Cm[i * ldc + j], s);
-        else Cm[i * ldc + j] = negate ? cminus(cz<T>(), s) : s;
+        typename S::R& o = part_of(Cm[i * ldc + j], part);
+        if (accumulate) o = negate ? S::sub(o, s) : S::add(o, s);
+        else o = negate ? S::sub(S::r(0.0), s) : s;
     }
     bsync();
 }
@@ -220,122 +276,163 @@ __device__ void gemm(T* Cm, int ldc, const T* A, int lda, int ta, const T* B, in
 // In-place inverse of a hermitian positive definite n x n matrix by
 // Gauss-Jordan elimination without pivoting (its pivots are the Schur
 // complement diagonals, positive for hpd).  Returns 0 if a pivot is <= 0.
+// The first warp alone forms each pivot's reciprocal and scales its row (an
+// FP64 division in all warps of the CTA cost 3 us per pivot); the elimination
+// takes one thread per real number.
 template <class T>
-__device__ int gj_inverse(T* A, int ld, int n, T* col) {
-    using S = Sc<T>;
-    int ok = 1;
-    for (int p = 0; p < n; ++p) {
-        typename S::R d = S::re(A[p * ld + p]);
-        if (!S::gt(d, S::r(0.0))) {
-            ok = 0;
-            d = S::r(1.0);
-        }
-        const typename S::R inv = S::rcp(d);
-        for (int r = threadIdx.x; r < n; r += blockDim.x) col[r] = A[r * ld + p];
-        bsync();
-        for (int c = threadIdx.x; c < n; c += blockDim.x)
-            A[p * ld + c] = (c == p) ? S::c(inv, S::r(0.0)) : cscal(A[p * ld + c], inv);
-        bsync();
-        for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-            int r = t / n, c = t % n;
-            if (r == p) continue;
-            const T f = col[r];
-            if (c == p) A[r * ld + p] = cscal(f, S::neg(inv));
-            else A[r * ld + c] = cminus(A[r * ld + c], ctimes(f, A[p * ld + c]));
-        }
-        bsync();
-    }
-    return ok;
-}
-
-// Pivoted Cholesky of the hermitian Gram matrix G (n x n, smem, ld) with the
-// deflation test: remaining squared norm <= dtol^2 * ref (the column's
-// squared norm when it was created).  Pivot: the largest remaining relative
-// squared norm, ties to the lowest index.  Produces the rank r, the r x n
-// factor R in permuted column order (Rm, ld n), S = Pi_r R11^{-1} (n x r)
-// and beta = R Pi^T (r x n), both in smem with leading dimension ld.
-// Runs on one warp.
-template <class T>
-__device__ int pivoted_qr(const T* G, int ld, int n, const typename Sc<T>::R* ref, typename Sc<T>::R dtol2, T* Rm,
-                          T* Sm, T* beta, int* perm, typename Sc<T>::R* dd_) {
+__device__ int gj_inverse(T* A, int ld, int n, T* col, typename Sc<T>::R* inv_s) {
     using S = Sc<T>;
     using R = typename S::R;
-    for (int i = threadIdx.x; i < n; i += WS) {
-        perm[i] = i;
-        dd_[i] = S::re(G[i * ld + i]);
+    __shared__ int ok_s;
+    if (threadIdx.x == 0) ok_s = 1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int p = 0; p < n; ++p) {
+        if (warp == 0) {
+            R d = S::re(A[p * ld + p]);
+            if (!S::gt(d, S::r(0.0))) {
+                if (lane == 0) ok_s = 0;
+                d = S::r(1.0);
+            }
+            const R inv = S::rcp(d);
+            wsync();
+            for (int t = lane; t < 2 * n; t += WS) {
+                const int c = t >> 1, part = t & 1;
+                R& o = part_of(A[p * ld + c], part);
+                o = c == p ? (part ? S::r(0.0) : inv) : S::mul(o, inv);
+            }
+            if (lane == 0) *inv_s = inv;
+        } else if (warp == 1) {
+            for (int r = lane; r < n; r += WS)
+                if (r != p) col[r] = A[r * ld + p];
+        }
+        bsync();
+        const R inv = *inv_s;
+        for (int t = threadIdx.x; t < 2 * n * n; t += blockDim.x) {
+            int part;
+            const int e = item_of(t, n * n, &part), r = e / n, c = e % n;
+            if (r == p) continue;
+            R& o = part_of(A[r * ld + c], part);
+            if (c == p) o = S::mul(part_of(col[r], part), S::neg(inv));
+            else o = minus_times<T>(o, col[r], A[p * ld + c], part);
+        }
+        bsync();
     }
-    for (int t = threadIdx.x; t < n * n; t += WS) Rm[t] = cz<T>();
-    wsync();
+    return ok_s;
+}
+
+// barrier of the QR's QW warps
+__device__ __forceinline__ void qsync() { asm volatile("bar.sync 1, %0;" ::"n"(QW * WS) : "memory"); }
+
+// Pivoted Cholesky of the hermitian Gram matrix G (n x n, smem, ld; its upper
+// and lower triangles are overwritten by the remainders) with the deflation
+// test: remaining squared norm <= dtol^2 * ref (the column's squared norm when
+// it was created).  Pivot: the largest remaining relative squared norm, ties
+// to the lowest position.  Produces the rank r, S = Pi_r R11^{-1} (n x r) and
+// beta = R Pi^T (r x n), both in smem with leading dimension ld (beta zeroed by
+// the caller).  R is kept in original column order.
+// Runs on QW warps (threads 0 .. QW * 32 - 1): a warp-wide FP64 instruction
+// occupies an SM sub-partition for 64 clocks, so the work is spread over the
+// four of them and over the lanes: the pairwise pivot comparisons (whose
+// outcomes every warp then scans as bits), the right-looking update of the
+// remainder (the subtractions per entry in the order of the pivots), and the
+// real and imaginary parts of the back substitution.
+template <class T>
+__device__ int pivoted_qr(T* G, int ld, int n, const typename Sc<T>::R* ref, typename Sc<T>::R dtol2, T* Rm, T* Sm,
+                          T* beta, int* perm, typename Sc<T>::R* dd_, typename Sc<T>::R* irp, unsigned* bits) {
+    using S = Sc<T>;
+    using R = typename S::R;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    unsigned* wb = bits + w * 16;              // this warp's comparison bits: pair (q, b < q) at q (q - 1) / 2 + b
+    if (tid < n) {
+        perm[tid] = tid;
+        dd_[tid] = S::re(G[tid * ld + tid]);
+    }
+    for (int t = tid; t < n * n; t += QW * WS) {
+        Rm[t] = cz<T>();
+        Sm[t / n * ld + t % n] = cz<T>();
+    }
+    const unsigned valid = __ballot_sync(0xffffffffu, lane < n && S::gt(ref[lane < n ? lane : 0], S::r(0.0)));
+    qsync();
     int rank = n;
     for (int p = 0; p < n; ++p) {
-        // pivot choice: every lane scans the same (short) candidate list;
-        // dd[q] / ref[q] > dd[b] / ref[b] is tested as dd[q] ref[b] >
-        // dd[b] ref[q] (both refs > 0), without divisions
-        int best = -1;
-        R bd = S::r(0.0), br = S::r(1.0);
-        for (int q = p; q < n; ++q) {
-            const R rq = ref[perm[q]];
-            if (!S::gt(rq, S::r(0.0))) continue;
-            if (best < 0 || S::gt(S::mul(dd_[q], br), S::mul(bd, rq))) {
-                bd = dd_[q];
-                br = rq;
-                best = q;
-            }
+        // dd[q] / ref[q] > dd[b] / ref[b] is tested as dd[q] ref[b] > dd[b] ref[q]
+        const int rem = n - p, np = rem * (rem - 1) / 2;
+        for (int base = 0; base < np; base += WS) {
+            const int idx = min(base + lane, np - 1);
+            int q = (int)((1.f + sqrtf(8.f * (float)idx + 1.f)) * 0.5f);
+            while (q * (q - 1) / 2 > idx) --q;
+            while (q * (q + 1) / 2 <= idx) ++q;
+            const int oq = perm[p + q], ob = perm[p + idx - q * (q - 1) / 2];
+            const unsigned m = __ballot_sync(0xffffffffu, S::gt(S::mul(dd_[oq], ref[ob]), S::mul(dd_[ob], ref[oq])));
+            if (lane == 0) wb[base / WS] = m;
         }
         wsync();
-        if (best < 0 || !S::gt(bd, S::mul(dtol2, br)) || !S::gt(dd_[best], S::r(0.0))) {
+        int best = -1;
+        for (int q = 0; q < rem; ++q) {
+            if (!(valid >> perm[p + q] & 1u)) continue;
+            const int at = q * (q - 1) / 2 + best;
+            if (best < 0 || (wb[at / WS] >> (at % WS) & 1u)) best = q;
+        }
+        bool stop = best < 0;
+        if (!stop) {
+            const R bd = dd_[perm[p + best]];
+            stop = !S::gt(bd, S::mul(dtol2, ref[perm[p + best]])) || !S::gt(bd, S::r(0.0));
+        }
+        if (stop) {
             rank = p;
             break;
         }
-        if (best != p) {
-            if (threadIdx.x == 0) {
-                int tp = perm[p];
-                perm[p] = perm[best];
-                perm[best] = tp;
-                R td = dd_[p];
-                dd_[p] = dd_[best];
-                dd_[best] = td;
-            }
-            for (int l = threadIdx.x; l < p; l += WS) {
-                T tr = Rm[l * n + p];
-                Rm[l * n + p] = Rm[l * n + best];
-                Rm[l * n + best] = tr;
-            }
-            wsync();
+        qsync();                               // every warp has chosen
+        if (tid == 0 && best != 0) {
+            const int tp = perm[p];
+            perm[p] = perm[p + best];
+            perm[p + best] = tp;
         }
-        const R rpp = S::sqrt_(dd_[p]);
-        const R irpp = S::rcp(rpp);
+        qsync();
         const int gp = perm[p];
-        if (threadIdx.x == 0) Rm[p * n + p] = S::c(rpp, S::r(0.0));
-        for (int r = p + 1 + threadIdx.x; r < n; r += WS) {
-            const int gr = perm[r];
-            T s = G[gp * ld + gr];
-            for (int l = 0; l < p; ++l) s = cminus(s, ctimes(cconj(Rm[l * n + p]), Rm[l * n + r]));
-            s = cscal(s, irpp);
-            Rm[p * n + r] = s;
-            dd_[r] = S::sub(dd_[r], cnorm2(s));
+        if (w == 0) {
+            const R rpp = S::sqrt_(dd_[gp]);
+            const R irpp = S::rcp(rpp);
+            if (lane == 0) {
+                Rm[p * n + gp] = S::c(rpp, S::r(0.0));
+                irp[p] = irpp;
+            }
+            if (p + 1 + lane < n) {
+                const int gr = perm[p + 1 + lane];
+                const T v = cscal(G[gp * ld + gr], irpp);
+                Rm[p * n + gr] = v;
+                dd_[gr] = S::sub(dd_[gr], cnorm2(v));
+            }
         }
-        wsync();
-    }
-    // beta = R Pi^T : beta[c'][perm[c]] = R[c'][c]
-    for (int t = threadIdx.x; t < n * n; t += WS) {
-        int cp = t / n, c = t % n;
-        if (cp < rank) beta[cp * ld + perm[c]] = (c >= cp) ? Rm[cp * n + c] : cz<T>();
-        Sm[t / n * ld + t % n] = cz<T>();
-    }
-    wsync();
-    // S = Pi_r R11^{-1}: lane c solves R11 y = e_c by back substitution
-    // (diagonal reciprocals formed once, in dd_[])
-    for (int i = threadIdx.x; i < rank; i += WS) dd_[i] = S::rcp(S::re(Rm[i * n + i]));
-    wsync();
-    for (int c = threadIdx.x; c < rank; c += WS) {
-        for (int i = c; i >= 0; --i) {
-            T s = (i == c) ? S::c(S::r(1.0), S::r(0.0)) : cz<T>();
-            for (int q = i + 1; q <= c; ++q) s = cminus(s, ctimes(Rm[i * n + q], Sm[perm[q] * ld + c]));
-            Sm[perm[i] * ld + c] = cscal(s, dd_[i]);
+        qsync();
+        const int m2 = n - 1 - p;
+        for (int e = tid; e < 2 * m2 * m2; e += QW * WS) {
+            int part;
+            const int t = item_of(e, m2 * m2, &part), a = t / m2, b = t % m2;
+            if (a == b) continue;
+            const int ga = perm[p + 1 + a], gb = perm[p + 1 + b];
+            R& o = part_of(G[ga * ld + gb], part);
+            o = minus_times<T>(o, cconj(Rm[p * n + ga]), Rm[p * n + gb], part);
         }
     }
-    wsync();
+    qsync();
+    // beta = R Pi^T
+    for (int t = tid; t < rank * n; t += QW * WS) {
+        const int cp = t / n, c = t % n;
+        if (c >= cp) beta[cp * ld + perm[c]] = Rm[cp * n + perm[c]];
+    }
+    // S = Pi_r R11^{-1}: column c solves R11 y = e_c by back substitution, a
+    // lane per column; even and odd columns and their real and imaginary
+    // parts in different warps
+    const int c = 2 * lane + (w & 1), part = w >> 1;
+    for (int i = rank - 1; i >= 0; --i) {
+        if (c < rank && i <= c) {
+            R s = S::r(i == c && part == 0 ? 1.0 : 0.0);
+            for (int q = i + 1; q <= c; ++q) s = minus_times<T>(s, Rm[i * n + perm[q]], Sm[perm[q] * ld + c], part);
+            part_of(Sm[perm[i] * ld + c], part) = S::mul(s, irp[i]);
+        }
+        qsync();
+    }
     return rank;
 }
 
@@ -379,31 +476,37 @@ __device__ __forceinline__ void reduce_store(T* G, int ld, typename Sc<T>::R* di
     }
 }
 
-// Sum the per-CTA Gram partials ([tile][blk][36], fixed order) into G (ld,
-// hermitian fill when herm) and the |y|^2 diagonal; all threads of the CTA.
-// FP64 partials (FP64 storage) are summed in FP64; FP32 partials (reduced
-// storage; they carry FP32 accuracy) with compensated (Kahan) FP32
-// additions, the chains combined in the state's scalar.  Consecutive threads take
-// consecutive slots (coalesced rows of 36); when the CTA has threads to spare,
-// ng groups split the CTAs' range and their sums are added in group order;
-// RC interleaved accumulators per thread keep several loads in flight (the
-// partials come from L2, so the sum is latency-bound).
+// Sum the per-CTA Gram partials ([tile][blk][36], fixed order).  FP64
+// partials (FP64 storage) are summed in FP64; FP32 partials (reduced storage;
+// they carry FP32 accuracy) with compensated (Kahan) FP32 additions, the
+// chains combined in the state's scalar.  The CTAs' range is split into
+// red_groups groups per tile, whose sums are added in group order by
+// reduce_combine; RC interleaved accumulators per thread keep several loads in
+// flight (the partials come from L2, so the sum is latency-bound).
+// The NRC CTAs of the launch share the (tile, group) units: the scalar
+// additions that close the chains are FP64, 64 clocks per warp and
+// sub-partition, which on one SM cost 8 us for three tiles.  Returns true in the CTA that
+// arrives last, with every group sum in red[group * slots + slot].
 // Fixed order: bitwise reproducible.
+__host__ __device__ inline int red_groups(int ntiles) {
+    const int items = ntiles * GSL, g = RED_GROUPS / items;
+    return g < 1 ? 1 : g;
+}
+
 template <class T>
-__device__ void reduce_partials(const double* __restrict__ part, int nblk, int nf_max, int herm, T* G, int ld,
-                                typename Sc<T>::R* diag, bool fp64_part) {
+__device__ bool reduce_partials(const double* __restrict__ part, int nblk, int nf_max, typename Sc<T>::R* red,
+                                unsigned* ticket, bool fp64_part) {
     using S = Sc<T>;
     using R = typename S::R;
     const int Tt = (nf_max + 3) / 4;
-    const int ntiles = herm ? Tt * (Tt + 1) / 2 : Tt * Tt;
+    const int ntiles = Tt * (Tt + 1) / 2;
     const int items = ntiles * GSL;
-    __shared__ R red[RED_MAX];
-    const int ng = max(1, min((int)blockDim.x / items, RED_MAX / items));
+    const int ng = red_groups(ntiles);
     const int chunk = (nblk + ng - 1) / ng;
-    for (int u = threadIdx.x; u < items * ng; u += blockDim.x) {
-        const int it = u % items, grp = u / items;
+    const int q = threadIdx.x % GSL;
+    for (int u = blockIdx.x + NRC * (threadIdx.x / GSL); u < ntiles * ng; u += NRC * (NT / GSL)) {
+        const int tile = u % ntiles, grp = u / ntiles;
         const int b0 = grp * chunk, b1 = min(nblk, b0 + chunk);
-        const int tile = it / GSL, q = it % GSL;
         const size_t off = (size_t)tile * nblk * GSL + q;
         constexpr int RC = 8;
         R s;
@@ -449,16 +552,21 @@ __device__ void reduce_partials(const double* __restrict__ part, int nblk, int n
 #pragma unroll
             for (int r = 1; r < RC; ++r) s = S::add(s, S::kahan(sum[r], comp[r]));
         }
-        if (ng > 1) red[grp * items + it] = s;
-        else reduce_store<T>(G, ld, diag, Tt, herm, nf_max, it, s);
+        red[grp * items + tile * GSL + q] = s;
     }
-    if (ng > 1) {
-        __syncthreads();
-        for (int it = threadIdx.x; it < items; it += blockDim.x) {
-            R s = red[it];
-            for (int g = 1; g < ng; ++g) s = S::add(s, red[g * items + it]);
-            reduce_store<T>(G, ld, diag, Tt, herm, nf_max, it, s);
-        }
+    return last_arrival(ticket);
+}
+// G (ld, hermitian fill) and the |y|^2 diagonal from the group sums
+template <class T>
+__device__ void reduce_combine(const typename Sc<T>::R* red, int nf_max, T* G, int ld, typename Sc<T>::R* diag) {
+    using S = Sc<T>;
+    using R = typename S::R;
+    const int Tt = (nf_max + 3) / 4;
+    const int ntiles = Tt * (Tt + 1) / 2, items = ntiles * GSL, ng = red_groups(ntiles);
+    for (int it = threadIdx.x; it < items; it += blockDim.x) {
+        R s = ld_cg(red + it);
+        for (int g = 1; g < ng; ++g) s = S::add(s, ld_cg(red + g * items + it));
+        reduce_store<T>(G, ld, diag, Tt, 1, nf_max, it, s);
     }
 }
 
@@ -470,6 +578,7 @@ __global__ void small_init_kernel(SmallStateT<T>* ss, Ctl* ctl, const double2* _
     using S = Sc<T>;
     using R = typename S::R;
     extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ unsigned bits[QW * 16];
     T* G = (T*)sm;
     T* Rm = G + m * m;
     T* Sm = Rm + m * m;
@@ -477,15 +586,16 @@ __global__ void small_init_kernel(SmallStateT<T>* ss, Ctl* ctl, const double2* _
     int* perm = (int*)(rho + m * m);
     R* dd_ = (R*)(perm + M_MAX);
     R* rf = dd_ + M_MAX;
-    for (int t = threadIdx.x; t < m * m; t += WS) {
+    R* irp = rf + M_MAX;
+    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
         const double2 g = G0[(t / m) * M_MAX + t % m];
         G[t] = S::c(S::r(g.x), S::r(g.y));
         rho[t] = cz<T>();
     }
-    for (int i = threadIdx.x; i < m; i += WS) rf[i] = S::r(ref[i]);
-    wsync();
-    const int r = pivoted_qr<T>(G, m, m, rf, S::r(dtol * dtol), Rm, Sm, rho, perm, dd_);
-    for (int t = threadIdx.x; t < M_MAX * M_MAX; t += WS) {
+    for (int i = threadIdx.x; i < m; i += blockDim.x) rf[i] = S::r(ref[i]);
+    bsync();
+    const int r = pivoted_qr<T>(G, m, m, rf, S::r(dtol * dtol), Rm, Sm, rho, perm, dd_, irp, bits);
+    for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) {
         const int i = t / M_MAX, j = t % M_MAX;
         ss->sh.S[t] = (i < m && j < m) ? Sm[i * m + j] : cz<T>();
         const T v = (i < r && j < m) ? rho[i * m + j] : cz<T>();
@@ -494,10 +604,9 @@ __global__ void small_init_kernel(SmallStateT<T>* ss, Ctl* ctl, const double2* _
             ss->sf[q].Lam[t] = cz<T>();
         }
     }
-    for (int q = 0; q < s; ++q) {
-        for (int t = threadIdx.x; t < M_MAX; t += WS) ss->sf[q].conv[t] = 0;
-        if (threadIdx.x == 0) ss->sf[q].alive = 1;
-    }
+    for (int t = threadIdx.x; t < s * M_MAX; t += blockDim.x) ss->sf[t / M_MAX].conv[t % M_MAX] = 0;
+    for (int q = threadIdx.x; q < s; q += blockDim.x) ss->sf[q].alive = 1;
+    if (threadIdx.x < 4) ss->sh.ticket[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         ctl->k = 1;
         ctl->mk = r;
@@ -516,25 +625,30 @@ __global__ void small_init_kernel(SmallStateT<T>* ss, Ctl* ctl, const double2* _
 // alpha_k from the Gram partials of the upper tiles of V_k^H Y (alpha_k =
 // V_k^H A V_k is hermitian; the lower tiles are the conjugates of the upper
 // ones, the diagonal tiles are hermitised); coef_a = alpha and
-// coef_bh = beta_k^H in the work precision (M_MAX tiles); ||y_i||^2
+// coef_bh = beta_k^H in the work precision (M_MAX tiles); ||y_i||^2.  NRC
+// CTAs reduce, the last one to arrive forms the result.
 template <class T>
-__global__ void small_alpha_kernel(SmallStateT<T>* ss, const Ctl* __restrict__ ctl, const double* __restrict__ part,
-                                   int nblk, int nf_max, int wprec, void* coef_a, void* coef_bh) {
+__global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, const Ctl* __restrict__ ctl,
+                                                         const double* __restrict__ part, int nblk, int nf_max,
+                                                         int wprec, void* coef_a, void* coef_bh) {
     using S = Sc<T>;
     using R = typename S::R;
     if (ctl->done) return;
+    R* red = reinterpret_cast<R*>(ss->sh.red);
+    if (!reduce_partials<T>(part, nblk, nf_max, red, &ss->sh.ticket[0], wprec == P64)) return;
     __shared__ T A[M_MAX * M_MAX];
     __shared__ R yy[M_MAX];
-    reduce_partials<T>(part, nblk, nf_max, 1, A, M_MAX, yy, wprec == P64);
+    reduce_combine<T>(red, nf_max, A, M_MAX, yy);
     __syncthreads();
     const int mk_ = ctl->mk, mp = ctl->k > 1 ? ctl->mprev : 0;
     const R half = S::r(0.5);
     for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) {
         int i = t / M_MAX, j = t % M_MAX;
-        T v = cz<T>();
-        if (i < mk_ && j < mk_) v = cscal(cplus(A[i * M_MAX + j], cconj(A[j * M_MAX + i])), half);
+        const bool ina = i < mk_ && j < mk_, inb = i < mp && j < mk_;
+        T v = cz<T>(), bh = cz<T>();
+        if (ina) v = cscal(cplus(A[i * M_MAX + j], cconj(A[j * M_MAX + i])), half);
+        if (inb) bh = cconj(ss->sh.betak[j * M_MAX + i]);
         ss->sh.alpha[t] = v;
-        const T bh = (i < mp && j < mk_) ? cconj(ss->sh.betak[j * M_MAX + i]) : cz<T>();
         if constexpr (is_fp64<T>()) {
             if (wprec == P64) {
                 ((double2*)coef_a)[t] = v;
@@ -542,86 +656,97 @@ __global__ void small_alpha_kernel(SmallStateT<T>* ss, const Ctl* __restrict__ c
                 continue;
             }
         }
-        ((float2*)coef_a)[t] = S::f2(v);
-        ((float2*)coef_bh)[t] = S::f2(bh);
+        ((float2*)coef_a)[t] = ina ? S::f2(v) : make_float2(0.f, 0.f);
+        ((float2*)coef_bh)[t] = inb ? S::f2(bh) : make_float2(0.f, 0.f);
     }
     R* yys = reinterpret_cast<R*>(ss->sh.yy);
     for (int t = threadIdx.x; t < M_MAX; t += blockDim.x) yys[t] = t < mk_ ? yy[t] : S::r(0.0);
 }
 
-// One block step's m x m work, one CTA per shift: reduce G = W^H W from the
-// partials, pivoted QR (every CTA computes the same deterministic result;
-// CTA 0 publishes S, beta_{k+1}, m_{k+1}), then this shift's recurrences.
+// The block step's QR: G = W^H W from the partials (NRC CTAs), pivoted QR with
+// deflation in the CTA that arrives last, which publishes S, beta_{k+1} and
+// m_{k+1}.
 template <class T>
-__global__ void small_step_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* __restrict__ part, int nblk, int m,
-                                  double dtol, const double* __restrict__ sigma, const double* __restrict__ target,
-                                  int freeze, int wprec, void* coefS_w, void* coefU_w, void* coefL_w, int* active,
-                                  int* conv_step, double* res_out, int MM) {
+__global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* __restrict__ part,
+                                                      int nblk, int m, double dtol, int wprec, void* coefS_w, int MM) {
     using S = Sc<T>;
     using R = typename S::R;
     if (ctl->done) return;
+    R* red = reinterpret_cast<R*>(ss->sh.red);
+    if (!reduce_partials<T>(part, nblk, m, red, &ss->sh.ticket[1], wprec == P64)) return;
     extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ unsigned bits[QW * 16];
+    __shared__ int mn_s;
     T* G = (T*)sm;
     T* Rm = G + MM * MM;
     T* Bn = Rm + MM * MM;       // beta_{k+1} (mn x mk)
     T* Sm = Bn + MM * MM;       // mk x mn
-    T* Dl = Sm + MM * MM;       // Delta -> Delta^{-1}
-    T* T1 = Dl + MM * MM;
-    T* Ut = T1 + MM * MM;
-    T* LH = Ut + MM * MM;
-    T* Cc = LH + MM * MM;
-    T* col = Cc + MM * MM;
-    R* res = (R*)(col + MM);
-    R* dd_ = res + MM;
+    R* dd_ = (R*)(Sm + MM * MM);
     R* rf = dd_ + MM;
-    int* perm = (int*)(rf + MM);
-    const int j = blockIdx.x;
-    const int k = ctl->k, mk_ = ctl->mk, mp = k > 1 ? ctl->mprev : 0;
-    reduce_partials<T>(part, nblk, m, 1, G, MM, nullptr, wprec == P64);
+    R* irp = rf + MM;
+    int* perm = (int*)(irp + MM);
+    const int mk_ = ctl->mk;
+    reduce_combine<T>(red, m, G, MM, nullptr);
     const R* yys = reinterpret_cast<const R*>(ss->sh.yy);
     for (int i = threadIdx.x; i < mk_; i += blockDim.x) rf[i] = yys[i];
     for (int t = threadIdx.x; t < MM * MM; t += blockDim.x) Bn[t] = cz<T>();
-    __shared__ int mn_s;
     bsync();
-    if (threadIdx.x < WS) {
-        const int r = pivoted_qr<T>(G, MM, mk_, rf, S::r(dtol * dtol), Rm, Sm, Bn, perm, dd_);
+    if (threadIdx.x < QW * WS) {
+        const int r = pivoted_qr<T>(G, MM, mk_, rf, S::r(dtol * dtol), Rm, Sm, Bn, perm, dd_, irp, bits);
         if (threadIdx.x == 0) mn_s = r;
     }
     bsync();
     const int mn = mn_s;
-    if (j == 0) {
-        for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) {
-            const int a = t / M_MAX, b = t % M_MAX;
-            const T sv = (a < mk_ && b < mn) ? Sm[a * MM + b] : cz<T>();
-            ss->sh.S[t] = sv;
-            ss->sh.betan[t] = (a < mn && b < mk_) ? Bn[a * MM + b] : cz<T>();
-            if constexpr (is_fp64<T>()) {
-                if (wprec == P64) {
-                    ((double2*)coefS_w)[t] = sv;
-                    continue;
-                }
-            }
-            ((float2*)coefS_w)[t] = S::f2(sv);
-        }
-        if (threadIdx.x == 0) {
-            ctl->mnext = mn;
-            ctl->deflations += mk_ - mn;
-        }
+    for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) {
+        const int a = t / M_MAX, b = t % M_MAX;
+        ss->sh.S[t] = (a < mk_ && b < mn) ? Sm[a * MM + b] : cz<T>();
+        ss->sh.betan[t] = (a < mn && b < mk_) ? Bn[a * MM + b] : cz<T>();
     }
+    st_mat_work<T>(wprec, coefS_w, Sm, MM, mk_, mn);
+    if (threadIdx.x == 0) {
+        ctl->mnext = mn;
+        ctl->deflations += mk_ - mn;
+    }
+}
+
+// One shift's recurrences of block step k (a CTA per shift).
+template <class T>
+__device__ void shift_recurrence(SmallStateT<T>* ss, Ctl* ctl, int j, int m, const double* __restrict__ sigma,
+                                 const double* __restrict__ target, int freeze, int wprec, void* coefU_w,
+                                 void* coefL_w, int* active, int* conv_step, double* res_out, int MM,
+                                 unsigned char* sm) {
+    using S = Sc<T>;
+    using R = typename S::R;
     SmallShiftT<T>& sf = ss->sf[j];
     if (!sf.alive) {
         if (threadIdx.x == 0) active[j] = 0;
         return;
     }
+    T* Bn = (T*)sm;             // beta_{k+1} (mn x mk)
+    T* Dl = Bn + MM * MM;       // Delta -> Delta^{-1}
+    T* T1 = Dl + MM * MM;
+    T* Ut = T1 + MM * MM;
+    T* LH = Ut + MM * MM;
+    T* Cc = LH + MM * MM;
+    T* Bk = Cc + MM * MM;       // beta_k (mk x mp)
+    T* col = Bk + MM * MM;
+    R* res = (R*)(col + MM);
+    R* inv = res + MM;
+    const int k = ctl->k, mk_ = ctl->mk, mp = k > 1 ? ctl->mprev : 0, mn = ctl->mnext;
     const size_t tile = (size_t)M_MAX * M_MAX;
     const size_t cb = wprec == P64 ? 16 : 8;
     // Delta_k = alpha_k + sigma I - Lambda_k beta_k^H
     ld_mat<T>(Dl, MM, ss->sh.alpha, mk_, mk_, mk_, mk_);
-    if (k > 1 && mp > 0) ld_mat<T>(T1, MM, sf.Lam, mk_, mp, mk_, mp);
+    ld_mat<T>(Bn, MM, ss->sh.betan, mn, mk_, mn, mk_);
+    if (k > 1 && mp > 0) {
+        ld_mat<T>(T1, MM, sf.Lam, mk_, mp, mk_, mp);
+        ld_mat<T>(Bk, MM, ss->sh.betak, mk_, mp, mk_, mp);
+    }
     bsync();
-    if (k > 1 && mp > 0) gemm<T>(Dl, MM, T1, MM, 0, ss->sh.betak, M_MAX, 1, mk_, mp, mk_, true, true);
+    if (k > 1 && mp > 0) gemm<T>(Dl, MM, T1, MM, 0, Bk, MM, 1, mk_, mp, mk_, true, true);
     const R sj = S::r(sigma[j]);
     for (int i = threadIdx.x; i < mk_; i += blockDim.x) Dl[i * MM + i].x = S::add(Dl[i * MM + i].x, sj);
+    ld_mat<T>(T1, MM, sf.U, mk_, m, mk_, m);
     bsync();
     const R half = S::r(0.5);
     for (int t = threadIdx.x; t < mk_ * mk_; t += blockDim.x) {      // exact hermitian symmetry
@@ -633,7 +758,7 @@ __global__ void small_step_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* __
         }
     }
     bsync();
-    if (!gj_inverse<T>(Dl, MM, mk_, col)) {
+    if (!gj_inverse<T>(Dl, MM, mk_, col, inv)) {
         if (threadIdx.x == 0) {
             atomicCAS(&ctl->status, 0, ST_NOT_HPD);
             active[j] = 0;
@@ -642,8 +767,6 @@ __global__ void small_step_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* __
         return;
     }
     // Ut = Delta^{-1} U_k (mk x m); Lambda_{k+1}^H = Delta^{-1} beta_{k+1}^H (mk x mn)
-    ld_mat<T>(T1, MM, sf.U, mk_, m, mk_, m);
-    bsync();
     gemm<T>(Ut, MM, Dl, MM, 0, T1, MM, 0, mk_, mk_, m, false, false);
     gemm<T>(LH, MM, Dl, MM, 0, Bn, MM, 1, mk_, mk_, mn, false, false);
     // C = -beta_{k+1} Ut (mn x m) gives the residual estimates, and it is also
@@ -654,7 +777,6 @@ __global__ void small_step_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* __
         for (int c = 0; c < mn; ++c) s2 = S::add(s2, cnorm2(Cc[c * MM + i]));
         res[i] = S::sqrt_(s2);
     }
-    bsync();
     // shift-update coefficients: Ut with the columns frozen before this step zeroed
     for (int t = threadIdx.x; t < mk_ * m; t += blockDim.x) {
         int a = t / m, i = t % m;
@@ -668,32 +790,43 @@ __global__ void small_step_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* __
         sf.Lam[t] = (c < mn && a < mk_) ? cconj(LH[a * MM + c]) : cz<T>();
         sf.U[t] = (c < mn && a < m) ? Cc[c * MM + a] : cz<T>();
     }
-    bsync();
-    if (threadIdx.x == 0) {
-        int any_before = 0, any_after = 0;
-        for (int i = 0; i < m; ++i) {
-            if (!sf.conv[i]) any_before = 1;
+    if (threadIdx.x < WS) {
+        const int i = threadIdx.x;
+        int was = 1, now = 1;
+        if (i < m) {
+            was = sf.conv[i];
             const double ri = S::d(res[i]);
             res_out[(size_t)j * m + i] = ri;
-            if (!sf.conv[i] && ri <= target[(size_t)j * m + i]) {
+            now = was || ri <= target[(size_t)j * m + i];
+            if (now && !was) {
                 sf.conv[i] = 1;
                 if (conv_step) conv_step[(size_t)j * m + i] = k;
             }
-            if (!sf.conv[i]) any_after = 1;
         }
-        active[j] = freeze ? any_before : 1;
-        sf.alive = any_after;
+        const int any_before = __any_sync(0xffffffffu, !was), any_after = __any_sync(0xffffffffu, !now);
+        if (i == 0) {
+            active[j] = freeze ? any_before : 1;
+            sf.alive = any_after;
+        }
     }
 }
 
-// scalar-independent: counters, beta_k <- beta_{k+1} (16-byte entries), k++
-__global__ void small_finish_kernel(SmallState* ss, Ctl* ctl, int s, int m, const int* __restrict__ active) {
+// The recurrences of every shift; the CTA that arrives last closes the block
+// step: counters, beta_k <- beta_{k+1}, k++.
+template <class T>
+__global__ void __launch_bounds__(NT) small_recur_kernel(SmallStateT<T>* ss, Ctl* ctl, int s, int m,
+                                                         const double* __restrict__ sigma,
+                                                         const double* __restrict__ target, int freeze, int wprec,
+                                                         void* coefU_w, void* coefL_w, int* active, int* conv_step,
+                                                         double* res_out, int MM) {
     if (ctl->done) return;
-    int nalive = 0, nkd = 0;
-    for (int j = 0; j < s; ++j) {
-        nalive += ss->sf[j].alive;
-        nkd += active[j];
-    }
+    extern __shared__ __align__(16) unsigned char sm[];
+    shift_recurrence<T>(ss, ctl, (int)blockIdx.x, m, sigma, target, freeze, wprec, coefU_w, coefL_w, active,
+                        conv_step, res_out, MM, sm);
+    if (!last_arrival(&ss->sh.ticket[2])) return;
+    const int j = threadIdx.x;                     // s <= S_MAX shifts
+    const int nalive = __syncthreads_count(j < s && __ldcg(&ss->sf[j < s ? j : 0].alive));
+    const int nkd = __syncthreads_count(j < s && __ldcg(&active[j < s ? j : 0]));
     const int mk_ = ctl->mk, mn = ctl->mnext, mp = ctl->k > 1 ? ctl->mprev : 0;
     for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) ss->sh.betak[t] = ss->sh.betan[t];
     __syncthreads();
@@ -711,13 +844,12 @@ __global__ void small_finish_kernel(SmallState* ss, Ctl* ctl, int s, int m, cons
         ctl->k += 1;
         ctl->mprev = mk_;
         ctl->mk = mn;
-        if (mn == 0 || nalive == 0 || ctl->status != 0) ctl->done = 1;
+        if (mn == 0 || nalive == 0 || __ldcg(&ctl->status) != 0) ctl->done = 1;
     }
 }
 
-size_t step_smem(int MM) {
-    return 9 * (size_t)MM * MM * sizeof(double2) + MM * sizeof(double2) + 3 * MM * sizeof(double) + M_MAX * sizeof(int);
-}
+size_t qr_smem(int MM) { return 4 * (size_t)MM * MM * sizeof(double2) + 3 * MM * sizeof(double) + M_MAX * sizeof(int); }
+size_t recur_smem(int MM) { return 7 * (size_t)MM * MM * sizeof(double2) + MM * sizeof(double2) + (MM + 2) * sizeof(double); }
 
 template <class T>
 SmallStateT<T>* as_state(SmallState* ss) { return reinterpret_cast<SmallStateT<T>*>(ss); }
@@ -729,48 +861,57 @@ SmallStateT<T>* as_state(SmallState* ss) { return reinterpret_cast<SmallStateT<T
 // FP64 storage, else FP32) and of the coefficient copies
 void launch_small_init(SmallState* ss, Ctl* ctl, const double2* G0, const double* ref, int m, int s, double dtol,
                        int sfp64, cudaStream_t st) {
-    size_t sm = 4 * (size_t)m * m * sizeof(double2) + M_MAX * sizeof(int) + 2 * M_MAX * sizeof(double);
+    auto bytes = [](int w) {
+        return 4 * (size_t)w * w * sizeof(double2) + M_MAX * sizeof(int) + 3 * M_MAX * sizeof(double);
+    };
     // above 48 KB from m = 28 on
-    const int sm_max = (int)(4 * (size_t)M_MAX * M_MAX * sizeof(double2) + M_MAX * sizeof(int) + 2 * M_MAX * sizeof(double));
     static std::atomic<unsigned long long> devs64{0}, devsdd{0};
-    max_dyn_smem_once(small_init_kernel<double2>, sm_max, devs64);
-    max_dyn_smem_once(small_init_kernel<ddc>, sm_max, devsdd);
+    max_dyn_smem_once(small_init_kernel<double2>, (int)bytes(M_MAX), devs64);
+    max_dyn_smem_once(small_init_kernel<ddc>, (int)bytes(M_MAX), devsdd);
     if (sfp64)
-        small_init_kernel<double2><<<1, WS, sm, st>>>(as_state<double2>(ss), ctl, G0, ref, m, s, dtol);
+        small_init_kernel<double2><<<1, QW * WS, bytes(m), st>>>(as_state<double2>(ss), ctl, G0, ref, m, s, dtol);
     else
-        small_init_kernel<ddc><<<1, WS, sm, st>>>(as_state<ddc>(ss), ctl, G0, ref, m, s, dtol);
+        small_init_kernel<ddc><<<1, QW * WS, bytes(m), st>>>(as_state<ddc>(ss), ctl, G0, ref, m, s, dtol);
 }
 
 void launch_small_alpha(SmallState* ss, const Ctl* ctl, const double* partials, int nblk, int nf_max, int wprec,
                         int sfp64, void* coef_a, void* coef_bh, cudaStream_t st) {
     if (sfp64)
-        small_alpha_kernel<double2><<<1, NT, 0, st>>>(as_state<double2>(ss), ctl, partials, nblk, nf_max, wprec,
-                                                      coef_a, coef_bh);
+        small_alpha_kernel<double2><<<NRC, NT, 0, st>>>(as_state<double2>(ss), ctl, partials, nblk, nf_max, wprec,
+                                                        coef_a, coef_bh);
     else
-        small_alpha_kernel<ddc><<<1, NT, 0, st>>>(as_state<ddc>(ss), ctl, partials, nblk, nf_max, wprec, coef_a,
-                                                  coef_bh);
+        small_alpha_kernel<ddc><<<NRC, NT, 0, st>>>(as_state<ddc>(ss), ctl, partials, nblk, nf_max, wprec, coef_a,
+                                                    coef_bh);
 }
 
-void launch_small_step(SmallState* ss, Ctl* ctl, const double* partials, int nblk, int s, int m, double dtol,
-                       const double* sigma_dev, const double* target_dev, int freeze, int wprec, int sfp64,
-                       void* coefS_w, void* coefU_w, void* coefL_w, int* active, int* conv_step, double* res_out,
-                       cudaStream_t st) {
-    const int MM = m;                  // block widths never exceed the initial width m
+void launch_small_qr(SmallState* ss, Ctl* ctl, const double* partials, int nblk, int m, double dtol, int wprec,
+                     int sfp64, void* coefS_w, cudaStream_t st) {
     static std::atomic<unsigned long long> devs64{0}, devsdd{0};
-    max_dyn_smem_once(small_step_kernel<double2>, (int)step_smem(M_MAX), devs64);
-    max_dyn_smem_once(small_step_kernel<ddc>, (int)step_smem(M_MAX), devsdd);
+    max_dyn_smem_once(small_qr_kernel<double2>, (int)qr_smem(M_MAX), devs64);
+    max_dyn_smem_once(small_qr_kernel<ddc>, (int)qr_smem(M_MAX), devsdd);
+    // matrices at the initial width m, which block widths never exceed
     if (sfp64)
-        small_step_kernel<double2><<<s, NT, step_smem(MM), st>>>(as_state<double2>(ss), ctl, partials, nblk, m, dtol,
-                                                                 sigma_dev, target_dev, freeze, wprec, coefS_w,
-                                                                 coefU_w, coefL_w, active, conv_step, res_out, MM);
+        small_qr_kernel<double2><<<NRC, NT, qr_smem(m), st>>>(as_state<double2>(ss), ctl, partials, nblk, m, dtol,
+                                                              wprec, coefS_w, m);
     else
-        small_step_kernel<ddc><<<s, NT, step_smem(MM), st>>>(as_state<ddc>(ss), ctl, partials, nblk, m, dtol,
-                                                             sigma_dev, target_dev, freeze, wprec, coefS_w, coefU_w,
-                                                             coefL_w, active, conv_step, res_out, MM);
+        small_qr_kernel<ddc><<<NRC, NT, qr_smem(m), st>>>(as_state<ddc>(ss), ctl, partials, nblk, m, dtol, wprec,
+                                                          coefS_w, m);
 }
 
-void launch_small_finish(SmallState* ss, Ctl* ctl, int s, int m, const int* active, cudaStream_t st) {
-    small_finish_kernel<<<1, 128, 0, st>>>(ss, ctl, s, m, active);
+void launch_small_recur(SmallState* ss, Ctl* ctl, int s, int m, const double* sigma_dev, const double* target_dev,
+                        int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* active, int* conv_step,
+                        double* res_out, cudaStream_t st) {
+    static std::atomic<unsigned long long> devs64{0}, devsdd{0};
+    max_dyn_smem_once(small_recur_kernel<double2>, (int)recur_smem(M_MAX), devs64);
+    max_dyn_smem_once(small_recur_kernel<ddc>, (int)recur_smem(M_MAX), devsdd);
+    if (sfp64)
+        small_recur_kernel<double2><<<s, NT, recur_smem(m), st>>>(as_state<double2>(ss), ctl, s, m, sigma_dev,
+                                                                  target_dev, freeze, wprec, coefU_w, coefL_w, active,
+                                                                  conv_step, res_out, m);
+    else
+        small_recur_kernel<ddc><<<s, NT, recur_smem(m), st>>>(as_state<ddc>(ss), ctl, s, m, sigma_dev, target_dev,
+                                                              freeze, wprec, coefU_w, coefL_w, active, conv_step,
+                                                              res_out, m);
 }
 
 }  // namespace dsbcg

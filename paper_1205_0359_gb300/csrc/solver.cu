@@ -126,7 +126,6 @@ struct dsbcg_ctx {
     void *links12_mem[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     void* linksfx_mem = nullptr;
     int* flags = nullptr;                // device words: [0] fixed-point range left, [1, 2] gauge checks
-    int* h_flags = nullptr;              // pinned copies
     Scratch scr;                         // working fields of apply and force
     float hscale = 1.f;
     bool gauge_ok = false;               // gauge64 holds a checked field and links[] were packed from it
@@ -156,6 +155,7 @@ struct dsbcg_ctx {
         void* eotmp = nullptr;                                    // Schur: even-parity half fields
         double2* T64c = nullptr;                                  // Schur: high-precision half fields
         int* fxe = nullptr;                                       // site exponents of the true residuals' fields
+        bool fx = false;                                          // sized with the exponents (where there was room)
         bool fx_resid = false;                                    // true residuals take the fixed-point stencil
         void *P = nullptr, *Xin = nullptr;                        // work precision
         double2 *B64 = nullptr, *X64 = nullptr, *R64 = nullptr, *T64a = nullptr, *T64b = nullptr, *rhs = nullptr;
@@ -315,11 +315,6 @@ void scratch_trim(Scratch& s) {
         s = Scratch();
     }
 }
-dsbcg_status ensure_flags(dsbcg_ctx* c) {
-    if (!c->flags) CK(cudaMalloc((void**)&c->flags, 4 * sizeof(int)));
-    if (!c->h_flags) CK(cudaMallocHost((void**)&c->h_flags, 4 * sizeof(int)));
-    return DSBCG_OK;
-}
 
 // a buffer of packed links, kept for the context's life
 dsbcg_status link_alloc(dsbcg_ctx* c, void** p, size_t bytes_per_site) {
@@ -344,23 +339,20 @@ dsbcg_status ensure_links(dsbcg_ctx* c, int prec) {
         CK(cudaGetLastError());
         c->links12[prec] = c->links12_mem[prec];
     }
-    if (c->su3 && prec == P64 && !c->linksfx) {
-        // the fixed-point links are an option: without memory for them the
-        // FP64 stencil runs on the FP64 pipe
-        if (link_alloc(c, &c->linksfx_mem, 36 * sizeof(double2)) == DSBCG_OK) {
-            launch_fx_links(c->linksfx_mem, c->gauge64, c->V, c->kappa, c->st);
-            CK(cudaGetLastError());
-            c->linksfx = c->linksfx_mem;
-        }
-    }
     return DSBCG_OK;
 }
 
-// The fixed-point FP64 stencil serves this context's operator: links in
-// SU(3) and a kappa in the range of the format
-bool fx_usable(const dsbcg_ctx* c) {
-    return c->linksfx && fx_kappa_fits(c->kappa);
+// The links of the fixed-point stencil, on first use.  They are an option:
+// without memory for them the FP64 stencil runs on the FP64 pipe.
+dsbcg_status ensure_fx_links(dsbcg_ctx* c) {
+    if (!c->su3 || c->linksfx || !fx_kappa_fits(c->kappa)) return DSBCG_OK;
+    if (link_alloc(c, &c->linksfx_mem, 36 * sizeof(double2)) != DSBCG_OK) return DSBCG_OK;
+    launch_fx_links(c->linksfx_mem, c->gauge64, c->V, c->kappa, c->st);
+    CK(cudaGetLastError());
+    c->linksfx = c->linksfx_mem;
+    return DSBCG_OK;
 }
+
 // True residuals of m columns in fixed point: always for FP64 storage, and for
 // the reduced storages from FX_RESID_MIN sites x columns of the full lattice.
 // Below it the FP64 residuals run beside latency-bound restarts and cost
@@ -405,7 +397,8 @@ int stream_prio(bool refinement) {
 
 dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
     auto& w = c->ws;
-    if (w.prec == prec && w.m == m && w.s >= s && w.nbb >= nbb) return DSBCG_OK;
+    const bool fx = c->linksfx && fx_residuals(c, prec, m);
+    if (w.prec == prec && w.m == m && w.s >= s && w.nbb >= nbb && (!fx || w.fx)) return DSBCG_OK;
     free_ws(c);
     scratch_free(c);                     // the workspace sizes itself by the memory that is free
     const size_t ld = c->ld, n = c->n;
@@ -419,7 +412,9 @@ dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
         CKS(dmalloc(c, &w.eotmp, m * fb));
         CKS(dmalloc(c, (void**)&w.T64c, m * db));
     }
-    if (c->linksfx) CKS(dmalloc(c, (void**)&w.fxe, fx_exp_bytes(c, m)));
+    // the exponents are an option: without memory for them the FP64 pipe serves
+    w.fx = fx;
+    if (fx && dmalloc(c, (void**)&w.fxe, fx_exp_bytes(c, m)) != DSBCG_OK) w.fxe = nullptr;
     CKS(dmalloc(c, (void**)&w.P, (size_t)s * m * wb));
     CKS(dmalloc(c, (void**)&w.Xin, (size_t)s * m * wb));
     CKS(dmalloc(c, (void**)&w.B64, (size_t)nbb * m * db));
@@ -487,7 +482,7 @@ dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
     w.prec = prec;
     w.nbb = nbb;
     Lane L0;
-    if (c->linksfx && prec == P64) CKS(dmalloc(c, (void**)&L0.fxe, fx_exp_bytes(c, m)));
+    if (fx && prec == P64 && dmalloc(c, (void**)&L0.fxe, fx_exp_bytes(c, m)) != DSBCG_OK) L0.fxe = nullptr;
     L0.st = c->st;
     L0.vring = w.vring;
     L0.zw = w.zw;
@@ -712,13 +707,13 @@ int residual_ctas(dsbcg_ctx* c) {
 // Dhat in, tmp is scratch for even-parity half fields)
 //
 // FP64 fields with fxe (site exponents, see fx_exp_bytes) take the
-// fixed-point stencil where fx_usable: in is converted into out's memory, the
+// fixed-point stencil when its links exist: in is converted into out's memory, the
 // intermediate fields stay in fixed point and the last pass writes FP64.
 // flag: see launch_fx_convert.
 void apply_op(dsbcg_ctx* c, int p, void* out, void* mid, const void* in, void* tmp, size_t ld, const Ctl* ctl,
               int nf_static, int nf_max, float hs, cudaStream_t st, int cls, int* fxe = nullptr,
               int* flag = nullptr) {
-    if (p == P64 && fxe && fx_usable(c)) {
+    if (p == P64 && fxe && c->linksfx) {
         int *e0 = fxe, *e1 = fxe + (size_t)(ctl ? nf_max : nf_static) * c->Vf;
         int* e2 = e1 + (e1 - e0);
         {
@@ -941,10 +936,7 @@ dsbcg_status lane_enqueue(dsbcg_ctx* c, Lane& L) {
         }
         {
             Prof p(c, DSBCG_KCLASS_SMALL, 1, st);
-            launch_small_step(L.ss, L.ctl, L.partials, L.nblk, s_in, m_in, L.dtol, L.sigma, L.target, L.freeze, wp,
-                              L.sfp64, L.coefS, (char*)L.coefU + (size_t)hs * s_in * cb,
-                              (char*)L.coefL + (size_t)hs * s_in * cb, L.active + (size_t)hs * s_in, L.conv_step,
-                              L.res, st);
+            launch_small_qr(L.ss, L.ctl, L.partials, L.nblk, m_in, L.dtol, wp, L.sfp64, L.coefS, st);
         }
         {
             Prof p(c, DSBCG_KCLASS_UPDATE, 1, st);
@@ -952,7 +944,9 @@ dsbcg_status lane_enqueue(dsbcg_ctx* c, Lane& L) {
         }
         {
             Prof p(c, DSBCG_KCLASS_SMALL, 1, st);
-            launch_small_finish(L.ss, L.ctl, s_in, m_in, L.active + (size_t)hs * s_in, st);
+            launch_small_recur(L.ss, L.ctl, s_in, m_in, L.sigma, L.target, L.freeze, wp, L.sfp64,
+                               (char*)L.coefU + (size_t)hs * s_in * cb, (char*)L.coefL + (size_t)hs * s_in * cb,
+                               L.active + (size_t)hs * s_in, L.conv_step, L.res, st);
         }
         if (L.step - L.k0 == C) flush();
     }
@@ -1082,6 +1076,7 @@ dsbcg_status solve_core(dsbcg_ctx* c, int m, const void* B, int nbb, int s, cons
     const int hp = sfp64 ? P64 : PDD;
     CKS(ensure_links(c, prec));
     CKS(ensure_links(c, hp));
+    if (hp == P64 && fx_residuals(c, prec, m)) CKS(ensure_fx_links(c));
     CKS(ensure_ws(c, m, s, prec, nbb));
     auto& w = c->ws;
     w.fx_resid = fx_residuals(c, prec, m);
@@ -1639,16 +1634,17 @@ dsbcg_status dsbcg_update_gauge(dsbcg_ctx* c, const void* gauge) {
     c->linksfx = nullptr;
     const size_t bytes = c->V * 36 * sizeof(double2);
     if (!c->gauge64) CK(cudaMalloc((void**)&c->gauge64, bytes));
-    CKS(ensure_flags(c));
+    if (!c->flags) CK(cudaMalloc((void**)&c->flags, 4 * sizeof(int)));
     CK(cudaMemcpyAsync(c->gauge64, gauge, bytes, is_device_ptr(gauge) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                        c->st));
     CK(cudaMemsetAsync(c->flags + 1, 0, 2 * sizeof(int), c->st));
     launch_check_finite(c->gauge64, c->V * 36, c->flags + 1, c->st);
     // a field in SU(3) to 1e-10 gets 12-real links for the reduced storages
     launch_check_su3(c->gauge64, c->V * 4, 1e-10, c->flags + 2, c->st);
-    CK(cudaMemcpyAsync(c->h_flags + 1, c->flags + 1, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
+    int hf[2] = {1, 1};
+    CK(cudaMemcpyAsync(hf, c->flags + 1, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    const int h = c->h_flags[1], hs = c->h_flags[2];
+    const int h = hf[0], hs = hf[1];
     if (h) return DSBCG_ERR_NONFINITE;
     c->su3 = (hs == 0);
     CKS(ensure_links(c, P64));
@@ -1680,7 +1676,6 @@ void dsbcg_destroy(dsbcg_ctx* c) {
     }
     if (c->linksfx_mem) cudaFree(c->linksfx_mem);
     if (c->flags) cudaFree(c->flags);
-    if (c->h_flags) cudaFreeHost(c->h_flags);
     if (c->gauge64) cudaFree(c->gauge64);
     if (c->rst) cudaStreamDestroy(c->rst);
     if (c->ev_joint) cudaEventDestroy(c->ev_joint);
@@ -1770,15 +1765,14 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     const size_t n = c->n, ld = hp_ld(c, storage);
     const size_t fb = prec_elem_bytes(storage) * c->ld;
     const bool in_dev = is_device_ptr(in), out_dev = is_device_ptr(out);
-    bool fx = fixed && storage == P64 && fx_usable(c);
+    if (fixed && storage == P64) CKS(ensure_fx_links(c));
+    bool fx = fixed && storage == P64 && c->linksfx;
     const size_t db = m * n * sizeof(double2);
     Scratch& scr = c->scr;
     const size_t need = (c->schur ? 4 : 3) * scratch_round(m * fb) + (in_dev ? 0 : scratch_round(db)) +
                         (out_dev ? 0 : scratch_round(db));
     // without room for the site exponents the FP64 kernels serve the call
-    if (fx && (ensure_flags(c) != DSBCG_OK ||
-               scratch_get(scr, need + scratch_round(fx_exp_bytes(c, m))) != DSBCG_OK))
-        fx = false;
+    if (fx && scratch_get(scr, need + scratch_round(fx_exp_bytes(c, m))) != DSBCG_OK) fx = false;
     if (!fx) CKS(scratch_get(scr, need));
     void *a = scratch_take(scr, m * fb), *b = scratch_take(scr, m * fb), *t = scratch_take(scr, m * fb);
     void* t2 = c->schur ? scratch_take(scr, m * fb) : nullptr;
@@ -1786,6 +1780,7 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     double2* din = in_dev ? nullptr : (double2*)scratch_take(scr, db);
     double2* dout = out_dev ? nullptr : (double2*)scratch_take(scr, db);
     dsbcg_status rs = DSBCG_OK;
+    int left = 0;                        // a site was outside the fixed-point range
     auto fail = [&](dsbcg_status s) { rs = s; };
     if (!in_dev) cudaMemcpyAsync(din, in, db, cudaMemcpyHostToDevice, c->st);
     {
@@ -1806,14 +1801,14 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
         }
         unpack_any(c, storage, dst, b, m);
         if (!out_dev) cudaMemcpyAsync(out, dout, m * n * sizeof(double2), cudaMemcpyDeviceToHost, c->st);
-        if (fxe) cudaMemcpyAsync(c->h_flags, c->flags, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+        if (fxe) cudaMemcpyAsync(&left, c->flags, sizeof(int), cudaMemcpyDeviceToHost, c->st);
         if (cudaGetLastError() != cudaSuccess) fail(DSBCG_ERR_CUDA);
         if (cudaStreamSynchronize(c->st) != cudaSuccess) fail(DSBCG_ERR_CUDA);
         prof_collect(c);
     }
     // a site outside the fixed-point range (NaN, Inf, extreme magnitudes):
     // the FP64 kernels' result replaces this one
-    const bool again = rs == DSBCG_OK && fx && c->h_flags[0];
+    const bool again = rs == DSBCG_OK && left;
     scratch_trim(scr);
     return again ? apply_fields(c, op, storage, m, in, out, false) : rs;
 }
