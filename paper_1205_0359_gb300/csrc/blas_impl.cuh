@@ -496,6 +496,28 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// FP64 fields: consumer warps per 4 x 4 tile, dealt rows in turn.  A tile's
+// warp-wide FP64 instruction holds one SM sub-partition for 64 clocks, so a
+// narrow block with one warp per tile leaves the other sub-partitions idle
+// (two CTAs per SM: widths up to 4 ran 2 of 4, 0.23 ms per launch at 16^4).
+__host__ __device__ inline int gram_split(int prec, int ntiles) {
+    if (prec != P64) return 1;
+    return ntiles <= 4 ? 4 : ntiles <= 8 ? 2 : 1;
+}
+// sum over the warp of 32 values per lane: lane q receives value q's sum
+__device__ __forceinline__ double warp_transpose_sum(double v[32], int lane) {
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+            const double mine = up ? v[i + o] : v[i], other = up ? v[i] : v[i + o];
+            v[i] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+        }
+    }
+    return v[0];
+}
+
 template <int P>
 __global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2* __restrict__ X,
                                                         const typename Tr<P>::S2* __restrict__ Y, size_t ld,
@@ -518,7 +540,8 @@ __global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2
     uint64_t* full = reinterpret_cast<uint64_t*>(g_smem + GNST * stage * sizeof(SE));
     uint64_t* empty = full + GNST;
     const int T = (nf_max + 3) / 4;
-    const int ncons = ntiles_of(nf_max, herm);        // consumer warps; warp ncons produces
+    const int ntl = ntiles_of(nf_max, herm), split = P == P64 ? gram_split(P, ntl) : 1;
+    const int ncons = ntl * split;                    // consumer warps; warp ncons produces
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const size_t ntr = (n + GR - 1) / GR;
     const size_t G = gridDim.x;
@@ -526,6 +549,7 @@ __global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2
     // set by a consumer warp whose wait gave up: the producer stops waiting
     // for buffers that will not be released and drains its copies
     __shared__ int aborted;
+    __shared__ double sred[P == P64 ? 16 : 1][GSLOTS];     // FP64: the consumer warps' sums
     if (threadIdx.x == 0) {
         for (int b = 0; b < GNST; ++b) {
             mbar_init(&full[b], 1);
@@ -565,10 +589,12 @@ __global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2
     } else {
         // consumers
         int ti, tj;
-        tile_coords(warp, T, herm, &ti, &tj);
+        const int tile = P == P64 ? warp % ntl : warp, part = P == P64 ? warp / ntl : 0;   // part of the tile's rows
+        tile_coords(tile, T, herm, &ti, &tj);
         const int i0 = ti * 4, j0 = tj * 4;
         const int ni = max(0, min(4, nf - i0)), nj = max(0, min(4, nf - j0));
         const bool dodiag = diag_yy && ti == tj;
+        const bool tri = P == P64 && herm && same && ti == tj;    // X^H X: the tile's upper triangle
         const R inv = (P == PBF16 || P == PF16) ? R(1) / R(hscale) : R(1);
         C acc[4][4];
         R yy[4];
@@ -599,17 +625,27 @@ __global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2
             const SE* sx = buf0 + (size_t)b * stage;
             const SE* sy = same ? sx : sx + (size_t)nf_max * GR;
             if (ni > 0 && nj > 0) {
-                for (int r = lane; r < rows; r += 32) {
+                for (int r = lane + 32 * part; r < rows; r += 32 * split) {
                     C x[4], y[4];
 #pragma unroll
                     for (int a = 0; a < 4; ++a) {
                         x[a] = a < ni ? Elem<P>::ld(sx, (size_t)(i0 + a) * GR + r, inv) : mk(R(0), R(0));
                         y[a] = a < nj ? Elem<P>::ld(sy, (size_t)(j0 + a) * GR + r, inv) : mk(R(0), R(0));
                     }
+                    if (P == P64 && tri) {
 #pragma unroll
-                    for (int a = 0; a < 4; ++a)
+                        for (int a = 0; a < 4; ++a) {
+                            acc[a][a].x = fma(x[a].x, x[a].x, acc[a][a].x);
+                            acc[a][a].x = fma(x[a].y, x[a].y, acc[a][a].x);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) cfmac(acc[a][c], x[a], y[c]);
+                            for (int c = a + 1; c < 4; ++c) cfmac(acc[a][c], x[a], x[c]);
+                        }
+                    } else {
+#pragma unroll
+                        for (int a = 0; a < 4; ++a)
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) cfmac(acc[a][c], x[a], y[c]);
+                    }
                     if (dodiag) {
 #pragma unroll
                         for (int c = 0; c < 4; ++c) yy[c] = fma(y[c].x, y[c].x, fma(y[c].y, y[c].y, yy[c]));
@@ -619,36 +655,71 @@ __global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[b]);
         }
-        // fixed-order warp reduction of the 36 slots, then one write per slot
-        R v[GSLOTS];
+        if constexpr (P == P64) {
+            // the 32 accumulators by a transposing sum (31 FP64 additions per
+            // lane instead of 160), the norms by a plain one; the parts of a
+            // tile are added below
+            double v[32];
+            if (tri) {
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+                for (int a = 1; a < 4; ++a)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                v[2 * (a * 4 + c)] = acc[a][c].x;
-                v[2 * (a * 4 + c) + 1] = acc[a][c].y;
+                    for (int c = 0; c < a; ++c) acc[a][c] = mk(acc[c][a].x, -acc[c][a].y);
             }
 #pragma unroll
-        for (int c = 0; c < 4; ++c) v[32 + c] = yy[c];
+            for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
+                for (int c = 0; c < 4; ++c) {
+                    v[2 * (a * 4 + c)] = acc[a][c].x;
+                    v[2 * (a * 4 + c) + 1] = acc[a][c].y;
+                }
+            sred[warp][lane] = warp_transpose_sum(v, lane);
+            if (dodiag) {
 #pragma unroll
-            for (int qq = 0; qq < GSLOTS; ++qq) v[qq] += __shfl_down_sync(0xffffffffu, v[qq], o);
-        if (lane == 0) {
-            const size_t base = ((size_t)warp * G + blockIdx.x) * GSLOTS;
+                for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-            for (int qq = 0; qq < GSLOTS; ++qq) {
-                if constexpr (P == P64)
-                    partials[base + qq] = (double)v[qq];
-                else
-                    reinterpret_cast<float*>(partials)[base + qq] = (float)v[qq];
+                    for (int c = 0; c < 4; ++c) yy[c] += __shfl_down_sync(0xffffffffu, yy[c], o);
             }
+            if (lane == 0) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) sred[warp][32 + c] = yy[c];
+            }
+        } else {
+            // fixed-order warp reduction of the 36 slots, then one write per slot
+            R v[GSLOTS];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    v[2 * (a * 4 + c)] = acc[a][c].x;
+                    v[2 * (a * 4 + c) + 1] = acc[a][c].y;
+                }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) v[32 + c] = yy[c];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int qq = 0; qq < GSLOTS; ++qq) v[qq] += __shfl_down_sync(0xffffffffu, v[qq], o);
+            if (lane == 0) {
+                const size_t base = ((size_t)warp * G + blockIdx.x) * GSLOTS;
+#pragma unroll
+                for (int qq = 0; qq < GSLOTS; ++qq) reinterpret_cast<float*>(partials)[base + qq] = (float)v[qq];
+            }
+        }
+    }
+    if constexpr (P == P64) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < ntl * GSLOTS; t += blockDim.x) {
+            const int tile = t / GSLOTS, q = t % GSLOTS;
+            double sum = sred[tile][q];
+            for (int h = 1; h < split; ++h) sum += sred[h * ntl + tile][q];
+            partials[((size_t)tile * G + blockIdx.x) * GSLOTS + q] = sum;
         }
     }
     if (__syncthreads_or(!ok)) {
         // a wait gave up: poison every partial of this CTA
         if (threadIdx.x == 0 && ctl) atomicCAS(&ctl->status, 0, ST_WAIT_TIMEOUT);
-        for (int t = threadIdx.x; t < ncons * GSLOTS; t += blockDim.x) {
+        for (int t = threadIdx.x; t < ntl * GSLOTS; t += blockDim.x) {
             const size_t at = ((size_t)(t / GSLOTS) * G + blockIdx.x) * GSLOTS + t % GSLOTS;
             if constexpr (P == P64)
                 partials[at] = __longlong_as_double(0x7ff8000000000000LL);
@@ -664,7 +735,7 @@ void launch_gram_tile_t(const void* X, const void* Y, size_t ld, size_t n, Ctl* 
                         int first_wait) {
     using SE = typename Tr<P>::S2;
     constexpr int GNST = gram_stages<P>();
-    const int npb = ntiles_of(nf_max, herm);
+    const int npb = ntiles_of(nf_max, herm) * gram_split(P, ntiles_of(nf_max, herm));
     const int nbuf_fields = (X == Y) ? nf_max : 2 * nf_max;
     const size_t smem = GNST * (size_t)nbuf_fields * GR * sizeof(SE) + 2 * GNST * sizeof(uint64_t);
     static std::atomic<unsigned long long> devs{0};
