@@ -58,16 +58,16 @@ void launch_gram_reduce(const double* partials, int nblk, int nf_max, int herm, 
 
 #define EXTERN_P(P)                                                                                      \
     extern template void launch_bu_t<P>(void*, const void*, const void*, const void*, size_t, size_t, const Ctl*, \
-                                        int, const void*, const void*, float, cudaStream_t);                 \
+                                        int, const void*, const void*, const int*, float, cudaStream_t);     \
     extern template void launch_ug_t<P>(void*, const void*, const void*, const void*, size_t, size_t, const Ctl*, \
                                         int, const void*, const void*, double*, int, float, cudaStream_t);   \
     extern template void launch_ib_t<P>(void*, size_t, const void*, int, size_t, size_t, const double2*, int, \
                                         const Ctl*, int, float, cudaStream_t);                               \
     extern template void launch_vu_t<P>(void*, const void*, size_t, size_t, const Ctl*, int, const void*,     \
-                                        float, cudaStream_t);                                                 \
+                                        const int*, float, cudaStream_t);                                     \
     extern template void launch_sc_t<P>(const void*, size_t, int, size_t, void*, void*, size_t, size_t, int,  \
                                         int, Ctl*, int, int, int, const void*, const void*, const int*,       \
-                                        float, cudaStream_t);
+                                        const int*, float, cudaStream_t);
 namespace blas_impl {
 EXTERN_P(P64)
 EXTERN_P(P32)
@@ -77,13 +77,13 @@ EXTERN_P(PF16)
 #undef EXTERN_P
 
 void launch_block_update(int prec, void* W, const void* Y, const void* Vk, const void* Vp, size_t ld, size_t n,
-                         const Ctl* ctl, int nf_max, const void* coef_a, const void* coef_bh, float hscale,
+                         const Ctl* ctl, int nf_max, const void* coef_a, const void* coef_bh, const int* ce, float hscale,
                          cudaStream_t st) {
     switch (prec) {
-        case P64: launch_bu_t<P64>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, hscale, st); break;
-        case P32: launch_bu_t<P32>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, hscale, st); break;
-        case PBF16: launch_bu_t<PBF16>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, hscale, st); break;
-        case PF16: launch_bu_t<PF16>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, hscale, st); break;
+        case P64: launch_bu_t<P64>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, ce, hscale, st); break;
+        case P32: launch_bu_t<P32>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, ce, hscale, st); break;
+        case PBF16: launch_bu_t<PBF16>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, ce, hscale, st); break;
+        case PF16: launch_bu_t<PF16>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, ce, hscale, st); break;
     }
 }
 
@@ -113,19 +113,19 @@ void launch_init_basis(int prec, void* V1, size_t ldv, const void* B, int bprec,
 }
 
 void launch_v_update(int prec, void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl, int nf_max,
-                     const void* coefS, float hscale, cudaStream_t st) {
+                     const void* coefS, const int* ce, float hscale, cudaStream_t st) {
     switch (prec) {
-        case P64: launch_vu_t<P64>(Vnext, W, ld, n, ctl, nf_max, coefS, hscale, st); break;
-        case P32: launch_vu_t<P32>(Vnext, W, ld, n, ctl, nf_max, coefS, hscale, st); break;
-        case PBF16: launch_vu_t<PBF16>(Vnext, W, ld, n, ctl, nf_max, coefS, hscale, st); break;
-        case PF16: launch_vu_t<PF16>(Vnext, W, ld, n, ctl, nf_max, coefS, hscale, st); break;
+        case P64: launch_vu_t<P64>(Vnext, W, ld, n, ctl, nf_max, coefS, ce, hscale, st); break;
+        case P32: launch_vu_t<P32>(Vnext, W, ld, n, ctl, nf_max, coefS, ce, hscale, st); break;
+        case PBF16: launch_vu_t<PBF16>(Vnext, W, ld, n, ctl, nf_max, coefS, ce, hscale, st); break;
+        case PF16: launch_vu_t<PF16>(Vnext, W, ld, n, ctl, nf_max, coefS, ce, hscale, st); break;
     }
 }
 
 void launch_shift_chunk(int prec, const void* ring, size_t slot_elems, int R, size_t ld, void* P, void* X,
                         size_t ldw, size_t n, int s, int m, Ctl* ctl, int nf_max, int k0, int C, const void* coefU,
-                        const void* coefL, const int* active, float hscale, cudaStream_t st) {
-#define SC_ARGS ring, slot_elems, R, ld, P, X, ldw, n, s, m, ctl, nf_max, k0, C, coefU, coefL, active, hscale, st
+                        const void* coefL, const int* ce, const int* active, float hscale, cudaStream_t st) {
+#define SC_ARGS ring, slot_elems, R, ld, P, X, ldw, n, s, m, ctl, nf_max, k0, C, coefU, coefL, ce, active, hscale, st
     switch (prec) {
         case P64: launch_sc_t<P64>(SC_ARGS); break;
         case P32: launch_sc_t<P32>(SC_ARGS); break;

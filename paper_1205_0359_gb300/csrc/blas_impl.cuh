@@ -13,6 +13,7 @@
 // FP32/BF16/FP16 fields), reduced across threads in that precision and
 // across CTAs in FP64 in a fixed order (bitwise reproducible).
 #pragma once
+#include "fx.cuh"
 #include "kernels.h"
 
 namespace dsbcg {
@@ -913,6 +914,243 @@ __global__ void __launch_bounds__(ROWS, (NF <= 12 && PW == P32) ? 4 : 1) shift_c
     }
 }
 
+// The same chunk for FP64 fields in block fixed point (fx.cuh), block widths up
+// to SHIFT_FX_NF_MAX.  P_j's row is held as limbs with one exponent per row, X_j's
+// in FP64; the coefficient tiles arrive as limbs with one exponent per column
+// (written by the m x m kernel), so right-hand sides of any scale keep their
+// own.  Per step
+//     X_j += P_j Ut_j:  limb sums, one conversion and one FP64 addition per
+//                       real number;
+//     P_j <- V_{k+1} - P_j Lh_j:  V's row and the limb sums aligned in 64 bits,
+//                       rounded to FP64 (what a chunk's end stores, so the
+//                       result does not depend on the chunk length) and split.
+// Limbs of P_j hold 56 bits and those of the coefficients 57, so the middle
+// sums stay below 2^62 at width 12.  A product sum is exact to about one unit of
+// 2^-56 of the row's largest entry times the column's, below the 2^-53 of every
+// step of an FP64 chain.  Bound: 24 NF^2 mad.wide per row and step at 64 per SM
+// and clock beside 6 NF conversions and additions on the FP64 pipe, where the
+// FP64 form takes 8 NF^2 FMA at 2 per SM and clock.
+// A row with a NaN or an infinity, or a bad coefficient column, ends as NaN.
+constexpr int SCFX_BITS = 56;
+
+template <int NF>
+__host__ __device__ constexpr size_t scfx_smem_bytes() {
+    return 4 * (size_t)NF * NF * sizeof(int4) + 4 * NF * sizeof(int);
+}
+
+// largest biased exponent of a row of NF FP64 values (at least 1)
+template <int NF>
+__device__ __forceinline__ int scfx_exp(const double2 v[NF]) {
+    int mx = 0;
+#pragma unroll
+    for (int a = 0; a < NF; ++a)
+        mx = max(mx, max(__double2hiint(v[a].x) & 0x7fffffff, __double2hiint(v[a].y) & 0x7fffffff));
+    return max(mx >> 20, 1);
+}
+// its limbs (SCFX_BITS bits); returns their exponent
+template <int NF>
+__device__ __forceinline__ int scfx_row(const double2 v[NF], int4 t[NF], bool& bad) {
+    const int eb = scfx_exp<NF>(v) + (FX_BITS - SCFX_BITS);
+    bad |= eb >= 0x7ff;
+#pragma unroll
+    for (int a = 0; a < NF; ++a) {
+        const int2 re = fx_split(fx_of_double(v[a].x, eb)), im = fx_split(fx_of_double(v[a].y, eb));
+        t[a] = make_int4(re.x, re.y, im.x, im.y);
+    }
+    return eb - 1079;
+}
+
+// Block update and basis update of FP64 fields in the same form, one thread per
+// row: W = Y - V_k a - V_{k-1} b^H and V_{k+1} = W S, coefficient tiles as limbs
+// with column exponents (ce: a, bh or S).  12 NF^2 mad.wide per product and row
+// and 2 NF conversions, against 4 NF^2 FP64 FMA.
+constexpr int UFX_ROWS = 128;
+
+// tile (NF x NF of M_MAX-strided entries) and its column exponents to shared memory
+template <int NF>
+__device__ __forceinline__ void ufx_stage(int4* st, int* se, const int4* __restrict__ c, const int* __restrict__ ce) {
+    for (int u = threadIdx.x; u < NF * NF; u += blockDim.x) st[u] = c[(u / NF) * M_MAX + u % NF];
+    if (threadIdx.x < NF) se[threadIdx.x] = ce[threadIdx.x];
+}
+
+template <int NF>
+__global__ void __launch_bounds__(UFX_ROWS) block_update_fx_kernel(
+    double2* __restrict__ W, const double2* __restrict__ Y, const double2* __restrict__ Vk,
+    const double2* __restrict__ Vp, size_t ld, size_t n, const Ctl* __restrict__ ctl, const int4* __restrict__ ca,
+    const int4* __restrict__ cb, const int* __restrict__ ce) {
+    if (ctl->done) return;
+    const int mk_ = ctl->mk, mp = (ctl->k > 1) ? ctl->mprev : 0;
+    __shared__ int4 sa[NF * NF], sb[NF * NF];
+    __shared__ int ea[NF], eb[NF];
+    ufx_stage<NF>(sa, ea, ca, ce);
+    ufx_stage<NF>(sb, eb, cb, ce + M_MAX);
+    const size_t e = (size_t)blockIdx.x * UFX_ROWS + threadIdx.x, er = e < n ? e : n - 1;
+    double2 v[NF], vp[NF], y[NF];
+#pragma unroll
+    for (int a = 0; a < NF; ++a) {
+        v[a] = a < mk_ ? Vk[(size_t)a * ld + er] : make_double2(0.0, 0.0);
+        vp[a] = a < mp ? Vp[(size_t)a * ld + er] : make_double2(0.0, 0.0);
+        y[a] = a < mk_ ? Y[(size_t)a * ld + er] : make_double2(0.0, 0.0);
+    }
+    int4 t[NF], tp[NF];
+    bool bad = false;
+    const int et = scfx_row<NF>(v, t, bad), ep = scfx_row<NF>(vp, tp, bad);
+    __syncthreads();
+    if (e >= n) return;
+#pragma unroll
+    for (int b = 0; b < NF; ++b) {
+        if (b < mk_) {
+            long long hr = 0, mr = 0, hi = 0, mi = 0, gr = 0, nr = 0, gi = 0, ni = 0;
+#pragma unroll
+            for (int a = 0; a < NF; ++a) {
+                fx_mac(t[a], sa[a * NF + b], hr, mr, hi, mi);
+                fx_mac(tp[a], sb[a * NF + b], gr, nr, gi, ni);
+            }
+            const int yb = scfx_exp<1>(&y[b]), ey = yb - 1079;
+            const bool nan = bad || yb == 0x7ff || ea[b] == FX_NAN || eb[b] == FX_NAN;
+            const int e1 = et + ea[b] + 2 * FX_BASE, e2 = ep + eb[b] + 2 * FX_BASE;
+            const int ec = max(ey - 3, max(e1, e2));       // y, at most 2^57 in its unit, may use 60 bits
+            const long long r = fx_align(fx_of_double(y[b].x, yb), ey - ec) - fx_align(hr + (mr >> FX_BASE), e1 - ec) -
+                                fx_align(gr + (nr >> FX_BASE), e2 - ec);
+            const long long i = fx_align(fx_of_double(y[b].y, yb), ey - ec) - fx_align(hi + (mi >> FX_BASE), e1 - ec) -
+                                fx_align(gi + (ni >> FX_BASE), e2 - ec);
+            const double q = __longlong_as_double(0x7ff8000000000000ll);
+            W[(size_t)b * ld + e] = nan ? make_double2(q, q) : make_double2(fx_to_double(r, ec), fx_to_double(i, ec));
+        }
+    }
+}
+
+template <int NF>
+__global__ void __launch_bounds__(UFX_ROWS) v_update_fx_kernel(double2* __restrict__ Vn, const double2* __restrict__ W,
+                                                               size_t ld, size_t n, const Ctl* __restrict__ ctl,
+                                                               const int4* __restrict__ cS, const int* __restrict__ ce) {
+    if (ctl->done) return;
+    const int mk_ = ctl->mk, mn = ctl->mnext;
+    __shared__ int4 sS[NF * NF];
+    __shared__ int eS[NF];
+    ufx_stage<NF>(sS, eS, cS, ce);
+    const size_t e = (size_t)blockIdx.x * UFX_ROWS + threadIdx.x, er = e < n ? e : n - 1;
+    double2 w[NF];
+#pragma unroll
+    for (int a = 0; a < NF; ++a) w[a] = a < mk_ ? W[(size_t)a * ld + er] : make_double2(0.0, 0.0);
+    int4 t[NF];
+    bool bad = false;
+    const int et = scfx_row<NF>(w, t, bad);
+    __syncthreads();
+    if (e >= n) return;
+#pragma unroll
+    for (int c = 0; c < NF; ++c) {
+        if (c < mn) {
+            long long hr = 0, mr = 0, hi = 0, mi = 0;
+#pragma unroll
+            for (int a = 0; a < NF; ++a) fx_mac(t[a], sS[a * NF + c], hr, mr, hi, mi);
+            const int ec = et + eS[c] + 2 * FX_BASE;
+            const double q = __longlong_as_double(0x7ff8000000000000ll);
+            Vn[(size_t)c * ld + e] = (bad || eS[c] == FX_NAN)
+                                         ? make_double2(q, q)
+                                         : make_double2(fx_to_double(hr + (mr >> FX_BASE), ec),
+                                                        fx_to_double(hi + (mi >> FX_BASE), ec));
+        }
+    }
+}
+
+template <int NF, int ROWS>
+__global__ void __launch_bounds__(ROWS, NF <= 4 ? 4 : NF <= 8 ? 2 : 1) shift_chunk_fx_kernel(
+    const double2* __restrict__ ring, size_t slot_elems, int R, size_t ld, double2* __restrict__ Pb,
+    double2* __restrict__ Xb, size_t ldw, size_t n, int s, int m, Ctl* __restrict__ ctl, int k0, int C,
+    const int4* __restrict__ cU, const int4* __restrict__ cL, const int* __restrict__ cE, const int* __restrict__ act) {
+    const int j = (int)(blockIdx.x % (unsigned)s);
+    const int kend = min(k0 + C, ctl->last_step);
+    if (kend <= k0 || !act[(size_t)(k0 % C) * s + j]) return;
+    extern __shared__ __align__(16) unsigned char sc_smem[];
+    int4* sT = reinterpret_cast<int4*>(sc_smem);                 // [2 buffers][U, L][NF * NF]
+    int* sE = reinterpret_cast<int*>(sT + 4 * NF * NF);          // [2 buffers][U, L][NF]
+    const int tid = threadIdx.x;
+    const size_t e0 = (size_t)(blockIdx.x / (unsigned)s) * ROWS;
+    const bool ok = e0 + tid < n;
+    const size_t e = e0 + (ok ? tid : 0);
+    const size_t tile = (size_t)M_MAX * M_MAX;
+    double2* Pj = Pb + (size_t)j * m * ldw;
+    double2* Xj = Xb + (size_t)j * m * ldw;
+    const int mk_ = ctl->hmk[k0 & (CTL_HIST - 1)];
+    bool bad = false;
+    int4 t[NF];
+    int et;
+    double2 p[NF], x[NF];
+#pragma unroll
+    for (int a = 0; a < NF; ++a) {
+        p[a] = make_double2(0.0, 0.0);
+        if (a < mk_) p[a] = (k0 == 0) ? ring[(size_t)(1 % R) * slot_elems + (size_t)a * ld + e] : Pj[(size_t)a * ldw + e];
+        x[a] = a < m ? Xj[(size_t)a * ldw + e] : make_double2(0.0, 0.0);
+    }
+    et = scfx_row<NF>(p, t, bad);
+    int mn = mk_;
+    for (int k = k0 + 1; k <= kend; ++k) {
+        const int q = (k - 1) % C;
+        if (!act[(size_t)q * s + j]) break;
+        mn = ctl->hmn[(k - 1) & (CTL_HIST - 1)];
+        // this step's tiles into buffer b (its previous readers, step k - 2, are
+        // past the barrier of step k - 1)
+        const int b = (k - k0) & 1;
+        int4 *bU = sT + 2 * b * NF * NF, *bL = bU + NF * NF;
+        int *eU = sE + 2 * b * NF, *eL = eU + NF;
+        const int4* gU = cU + ((size_t)q * s + j) * tile;
+        const int4* gL = cL + ((size_t)q * s + j) * tile;
+        const int* gE = cE + ((size_t)q * s + j) * 2 * M_MAX;
+        for (int u = tid; u < NF * NF; u += ROWS) {
+            bU[u] = gU[(u / NF) * M_MAX + u % NF];
+            bL[u] = gL[(u / NF) * M_MAX + u % NF];
+        }
+        if (tid < NF) {
+            eU[tid] = gE[tid];
+            eL[tid] = gE[M_MAX + tid];
+        }
+#pragma unroll
+        for (int c = 0; c < NF; ++c)
+            p[c] = c < mn ? ring[(size_t)((k + 1) % R) * slot_elems + (size_t)c * ld + e] : make_double2(0.0, 0.0);
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+            long long hr = 0, mr = 0, hi = 0, mi = 0;
+#pragma unroll
+            for (int a = 0; a < NF; ++a) fx_mac(t[a], bU[a * NF + i], hr, mr, hi, mi);
+            const int ex = eU[i];
+            bad |= ex == FX_NAN;
+            x[i].x += fx_to_double(hr + (mr >> FX_BASE), et + ex + 2 * FX_BASE);
+            x[i].y += fx_to_double(hi + (mi >> FX_BASE), et + ex + 2 * FX_BASE);
+        }
+        const int eb = scfx_exp<NF>(p), ev = eb - 1079;
+        bad |= eb == 0x7ff;
+        // unit of column c's sum: V, at most 2^57 in its own, may use 61 bits
+#pragma unroll
+        for (int c = 0; c < NF; ++c) {
+            if (c < mn) {
+                long long hr = 0, mr = 0, hi = 0, mi = 0;
+#pragma unroll
+                for (int a = 0; a < NF; ++a) fx_mac(t[a], bL[a * NF + c], hr, mr, hi, mi);
+                bad |= eL[c] == FX_NAN;
+                const int es = et + eL[c] + 2 * FX_BASE, ec = max(ev - 4, es);
+                const long long r = fx_align(hr + (mr >> FX_BASE), es - ec), i = fx_align(hi + (mi >> FX_BASE), es - ec);
+                p[c].x = fx_to_double(fx_align(fx_of_double(p[c].x, eb), ev - ec) - r, ec);
+                p[c].y = fx_to_double(fx_align(fx_of_double(p[c].y, eb), ev - ec) - i, ec);
+            }
+        }
+        et = scfx_row<NF>(p, t, bad);
+    }
+    if (ok) {
+        const double nan1 = __longlong_as_double(0x7ff8000000000000ll);
+        const double2 nan2 = make_double2(nan1, nan1);
+#pragma unroll
+        for (int i = 0; i < NF; ++i)
+            if (i < m) Xj[(size_t)i * ldw + e] = bad ? nan2 : x[i];
+#pragma unroll
+        for (int c = 0; c < NF; ++c)
+            if (c < mn) Pj[(size_t)c * ldw + e] = bad ? nan2 : p[c];
+    }
+    if (blockIdx.x < (unsigned)s && tid == 0)
+        atomicAdd(reinterpret_cast<unsigned long long*>(&ctl->f_shift_w), (unsigned long long)(mk_ + 2 * m + mn));
+}
+
 inline int nf_bucket(int nf) { return nf <= 4 ? 4 : nf <= 8 ? 8 : nf <= 12 ? 12 : nf <= 16 ? 16 : nf <= 24 ? 24 : 32; }
 
 
@@ -927,9 +1165,28 @@ inline int nf_bucket(int nf) { return nf <= 4 ? 4 : nf <= 8 ? 8 : nf <= 12 ? 12 
         default: MACRO(32); break;    \
     }
 
+// widths the fixed-point kernels serve (coef_fx)
+#define BI_DISPATCH_FX(nf, MACRO) \
+    switch (nf_bucket(nf)) {       \
+        case 4: MACRO(4); break;   \
+        case 8: MACRO(8); break;   \
+        default: MACRO(12); break; \
+    }
+
 template <int P>
 void launch_bu_t(void* W, const void* Y, const void* Vk, const void* Vp, size_t ld, size_t n, const Ctl* ctl,
-                 int nf_max, const void* coef_a, const void* coef_bh, float hscale, cudaStream_t st) {
+                 int nf_max, const void* coef_a, const void* coef_bh, const int* ce, float hscale, cudaStream_t st) {
+    if constexpr (P == P64) {
+        if (ce) {
+#define BI_BUFX(NF)                                                                                            \
+    block_update_fx_kernel<NF><<<(unsigned)((n + UFX_ROWS - 1) / UFX_ROWS), UFX_ROWS, 0, st>>>(                 \
+        (double2*)W, (const double2*)Y, (const double2*)Vk, (const double2*)Vp, ld, n, ctl, (const int4*)coef_a, \
+        (const int4*)coef_bh, ce)
+            BI_DISPATCH_FX(nf_max, BI_BUFX)
+#undef BI_BUFX
+            return;
+        }
+    }
     using S2 = typename Tr<P>::S2;
     using C = typename Tr<P>::C;
     int g = (int)((n + 255) / 256);
@@ -1161,7 +1418,17 @@ __global__ void __launch_bounds__(ROWS, NF <= 12 ? 4 : 1) shift_chunk32_kernel(
 
 template <int P>
 void launch_vu_t(void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl, int nf_max, const void* coefS,
-                 float hscale, cudaStream_t st) {
+                 const int* ce, float hscale, cudaStream_t st) {
+    if constexpr (P == P64) {
+        if (ce) {
+#define BI_VUFX(NF)                                                                                       \
+    v_update_fx_kernel<NF><<<(unsigned)((n + UFX_ROWS - 1) / UFX_ROWS), UFX_ROWS, 0, st>>>(                \
+        (double2*)Vnext, (const double2*)W, ld, n, ctl, (const int4*)coefS, ce)
+            BI_DISPATCH_FX(nf_max, BI_VUFX)
+#undef BI_VUFX
+            return;
+        }
+    }
     constexpr int PW = (P == P64) ? P64 : P32;
     using S2 = typename Tr<P>::S2;
     using CW = typename Tr<PW>::C;
@@ -1175,7 +1442,22 @@ void launch_vu_t(void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl
 template <int P>
 void launch_sc_t(const void* ring, size_t slot_elems, int R, size_t ld, void* Pp, void* X, size_t ldw, size_t n,
                  int s, int m, Ctl* ctl, int nf_max, int k0, int C, const void* coefU, const void* coefL,
-                 const int* active, float hscale, cudaStream_t st) {
+                 const int* ce, const int* active, float hscale, cudaStream_t st) {
+    if constexpr (P == P64) {
+        if (ce) {
+#define BI_SCFX(NF)                                                                                          \
+    {                                                                                                        \
+        constexpr int ROWS = 128;                                                                            \
+        constexpr size_t SMEM = scfx_smem_bytes<NF>();                                                       \
+        shift_chunk_fx_kernel<NF, ROWS><<<(unsigned)(((n + ROWS - 1) / ROWS) * (size_t)s), ROWS, SMEM, st>>>( \
+            (const double2*)ring, slot_elems, R, ld, (double2*)Pp, (double2*)X, ldw, n, s, m, ctl, k0, C,     \
+            (const int4*)coefU, (const int4*)coefL, ce, active);                                             \
+    }
+            BI_DISPATCH_FX(nf_max, BI_SCFX)
+#undef BI_SCFX
+            return;
+        }
+    }
     constexpr int PW = (P == P64) ? P64 : P32;
     using S2 = typename Tr<P>::S2;
     using W2 = typename Tr<PW>::S2;
@@ -1206,15 +1488,16 @@ void launch_sc_t(const void* ring, size_t slot_elems, int R, size_t ld, void* Pp
 
 #define BI_INSTANTIATE(P)                                                                                  \
     template void launch_bu_t<P>(void*, const void*, const void*, const void*, size_t, size_t, const Ctl*, int, \
-                                 const void*, const void*, float, cudaStream_t);                          \
+                                 const void*, const void*, const int*, float, cudaStream_t);              \
     template void launch_ug_t<P>(void*, const void*, const void*, const void*, size_t, size_t, const Ctl*, int, \
                                  const void*, const void*, double*, int, float, cudaStream_t);            \
     template void launch_ib_t<P>(void*, size_t, const void*, int, size_t, size_t, const double2*, int,       \
                                  const Ctl*, int, float, cudaStream_t);                                    \
-    template void launch_vu_t<P>(void*, const void*, size_t, size_t, const Ctl*, int, const void*, float,    \
-                                 cudaStream_t);                                                            \
+    template void launch_vu_t<P>(void*, const void*, size_t, size_t, const Ctl*, int, const void*, const int*, \
+                                 float, cudaStream_t);                                                     \
     template void launch_sc_t<P>(const void*, size_t, int, size_t, void*, void*, size_t, size_t, int, int,   \
-                                 Ctl*, int, int, int, const void*, const void*, const int*, float, cudaStream_t);
+                                 Ctl*, int, int, int, const void*, const void*, const int*, const int*, float, \
+                                 cudaStream_t);
 
 }  // namespace blas_impl
 }  // namespace dsbcg

@@ -33,38 +33,17 @@
 // a normal FP64 number sets *flag and turns its neighbourhood into NaN
 // (FX_NAN) or, when tiny, counts as zero; dsbcg_apply then repeats the
 // application with the FP64 kernels.
+#include "fx.cuh"
 #include "kernels.h"
 
 namespace dsbcg {
 
 namespace {
 
-constexpr int FX_ZERO = -(1 << 20), FX_NAN = 1 << 20;
 // biased exponents of a site's largest component for which the FX path holds
 constexpr int FX_EB_MIN = 300, FX_EB_MAX = 1800;
-constexpr int FX_BASE = 29;                    // bits per limb
-constexpr int FX_BITS = 57;                    // magnitude bits of a field value
 constexpr int FX_TILE = 12 * 32;               // int4 per 32-site tile
 
-__device__ __forceinline__ int2 fx_split(long long x) {
-    const int h = (int)((x + (1ll << (FX_BASE - 1))) >> FX_BASE);
-    return make_int2(h, (int)((unsigned)x - ((unsigned)h << FX_BASE)));
-}
-__device__ __forceinline__ long long fx_join(int h, int l) { return (long long)h * (1 << FX_BASE) + l; }
-// x 2^-s rounded to nearest, s >= 0
-__device__ __forceinline__ long long fx_shift(long long x, int s) {
-    if (s > 62) return 0;
-    return s > 0 ? (x + (1ll << (s - 1))) >> s : x;
-}
-// FP64 v in units of 2^(eb - 1079), eb >= v's biased exponent
-__device__ __forceinline__ long long fx_of_double(double v, int eb) {
-    const int hi = __double2hiint(v);
-    const int e = (hi >> 20) & 0x7ff;
-    const long long mant =
-        ((long long)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 32) | (unsigned)__double2loint(v);
-    const long long x = fx_shift(mant << 4, eb - (e ? e : 1));
-    return hi < 0 ? -x : x;
-}
 // element of component 0 of site y
 __device__ __forceinline__ size_t fx_at(int y) { return (size_t)(y >> 5) * FX_TILE + (y & 31); }
 

@@ -116,10 +116,15 @@ size_t gram_partial_doubles(int nf_max);
 void launch_gram_reduce(const double* partials, int nblk, int nf_max, int herm, int diag_yy,
                         double2* G, double* diag, const Ctl* ctl, int nf_static, int fp32,
                         cudaStream_t st);
-// W = Y - V a - Vp b^H, coefficients from the device (work precision copies)
+// FP64 blocks of widths up to 12 run their products with the m x m coefficients
+// in block fixed point (fx.cuh): the coefficient tiles then hold limbs, and ce
+// (else NULL) their column exponents, M_MAX words per tile
+inline bool coef_fx(int prec, int m) { return prec == P64 && m <= 12; }
+// W = Y - V a - Vp b^H, coefficients from the device (work precision copies;
+// ce: exponents of a, then of b^H)
 void launch_block_update(int prec, void* W, const void* Y, const void* Vk, const void* Vp,
                          size_t ld, size_t n, const Ctl* ctl, int nf_max,
-                         const void* coef_a, const void* coef_bh, float hscale, cudaStream_t st);
+                         const void* coef_a, const void* coef_bh, const int* ce, float hscale, cudaStream_t st);
 // Block update fused with the Gram of its result: W as launch_block_update,
 // and W^H W (hermitian, upper 4 x 4 tiles, no diagonal norms) as partials of
 // nblk blocks in the Gram kernel's layout.  Reduced storages and block widths
@@ -135,18 +140,20 @@ void launch_init_basis(int prec, void* V1, size_t ldv, const void* B, int bprec,
                        const double2* S, int s_dd, const Ctl* ctl, int nf_in, float hscale, cudaStream_t st);
 // V_{k+1} = W S (S from the step's QR, M_MAX-strided work-precision tile)
 void launch_v_update(int prec, void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl, int nf_max,
-                     const void* coefS, float hscale, cudaStream_t st);
+                     const void* coefS, const int* ce, float hscale, cudaStream_t st);
 // shift update (the per-shift short recurrences, Sec. 3) over the block
 // steps k0+1 .. min(k0 + C, last executed step): for every step in which
 // shift j is active, X_j += P_j Ut_j and P_j <- V_{k+1} - P_j LhT_j, with P_j
 // and X_j kept on chip across the steps.  ring: R slots of slot_elems
 // storage-precision elements, slot k mod R holding V_k (V_1 is the search
 // block of step 1).  coefU / coefL: per step slot (k - 1) mod C, s tiles of
-// M_MAX x M_MAX work-precision entries; active: per step slot, s flags.  P
+// M_MAX x M_MAX work-precision entries (ce: per step and shift the exponents of
+// both); active: per step slot, s flags.  P
 // and X hold s blocks of m fields of ldw elements (field-major).
 void launch_shift_chunk(int prec, const void* ring, size_t slot_elems, int R, size_t ld, void* P, void* X,
                         size_t ldw, size_t n, int s, int m, Ctl* ctl, int nf_max, int k0, int C, const void* coefU,
-                        const void* coefL, const int* active, float hscale, cudaStream_t st);
+                        const void* coefL, const int* ce, const int* active, float hscale,
+                        cudaStream_t st);
 
 // ---- small.cu ---------------------------------------------------------------
 struct SmallState;     // device m x m state (FP64 or double-float), defined in small.cu
@@ -157,14 +164,14 @@ void launch_small_init(SmallState* ss, Ctl* ctl, const double2* G0, const double
                        int sfp64, cudaStream_t st);
 // alpha_k from the Gram partials of V_k^H Y (+ coefficient tiles for the block update)
 void launch_small_alpha(SmallState* ss, const Ctl* ctl, const double* partials, int nblk, int nf_max,
-                        int wprec, int sfp64, void* coef_a, void* coef_bh, cudaStream_t st);
+                        int wprec, int sfp64, void* coef_a, void* coef_bh, int* ce, cudaStream_t st);
 // W^H W from the Gram partials, pivoted QR with deflation: S, beta_{k+1}, m_{k+1}
 void launch_small_qr(SmallState* ss, Ctl* ctl, const double* partials, int nblk, int m, double dtol, int wprec,
-                     int sfp64, void* coefS_w, cudaStream_t st);
+                     int sfp64, void* coefS_w, int* ce, cudaStream_t st);
 // per-shift recurrences (a CTA per shift) and the close of the block step
 void launch_small_recur(SmallState* ss, Ctl* ctl, int s, int m, const double* sigma_dev, const double* target_dev,
-                        int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* active, int* conv_step,
-                        double* res_out, cudaStream_t st);
+                        int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* ce, int* active,
+                        int* conv_step, double* res_out, cudaStream_t st);
 const double2* small_state_S(const SmallState* ss);
 
 // ---- force.cu ---------------------------------------------------------------

@@ -39,6 +39,7 @@
 // so the device state has one layout.
 #include <math.h>
 
+#include "fx.cuh"
 #include "kernels.h"
 
 namespace dsbcg {
@@ -223,6 +224,40 @@ __device__ void st_mat_work(int wprec, void* dst, const T* src, int ld, int r, i
         }
         reinterpret_cast<float2*>(dst)[t] = in ? Sc<T>::f2(src[i * ld + j]) : make_float2(0.f, 0.f);
     }
+}
+
+// The M_MAX x M_MAX tile get(i, j) (zero outside r x c) as limbs with one
+// exponent per column (fx.cuh): the coefficient form of the fixed-point
+// kernels.  All threads of the CTA.
+template <class F>
+__device__ void st_mat_fx(int4* dst, int* ce, int r, int c, F get) {
+    __shared__ int es[M_MAX];
+    const int lane = threadIdx.x & 31;
+    for (int j = threadIdx.x >> 5; j < M_MAX; j += blockDim.x >> 5) {
+        int mx = 0;
+        if (lane < r && j < c) {
+            const double2 v = get(lane, j);
+            mx = max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+        }
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) {
+            const int eb = max(mx >> 20, 1);
+            es[j] = eb;
+            ce[j] = mx == 0 ? FX_ZERO : eb == 0x7ff ? FX_NAN : eb - 1079;
+        }
+    }
+    bsync();
+    for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) {
+        const int i = t / M_MAX, j = t % M_MAX;
+        int4 q = make_int4(0, 0, 0, 0);
+        if (i < r && j < c) {
+            const double2 v = get(i, j);
+            const int2 re = fx_split(fx_of_double(v.x, es[j])), im = fx_split(fx_of_double(v.y, es[j]));
+            q = make_int4(re.x, re.y, im.x, im.y);
+        }
+        dst[t] = q;
+    }
+    bsync();
 }
 
 // real (0) or imaginary (1) part of an entry
@@ -630,7 +665,7 @@ __global__ void small_init_kernel(SmallStateT<T>* ss, Ctl* ctl, const double2* _
 template <class T>
 __global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, const Ctl* __restrict__ ctl,
                                                          const double* __restrict__ part, int nblk, int nf_max,
-                                                         int wprec, void* coef_a, void* coef_bh) {
+                                                         int wprec, void* coef_a, void* coef_bh, int* ce) {
     using S = Sc<T>;
     using R = typename S::R;
     if (ctl->done) return;
@@ -651,6 +686,7 @@ __global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, con
         ss->sh.alpha[t] = v;
         if constexpr (is_fp64<T>()) {
             if (wprec == P64) {
+                if (ce) continue;
                 ((double2*)coef_a)[t] = v;
                 ((double2*)coef_bh)[t] = bh;
                 continue;
@@ -661,6 +697,14 @@ __global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, con
     }
     R* yys = reinterpret_cast<R*>(ss->sh.yy);
     for (int t = threadIdx.x; t < M_MAX; t += blockDim.x) yys[t] = t < mk_ ? yy[t] : S::r(0.0);
+    if constexpr (is_fp64<T>()) {
+        if (ce) {
+            st_mat_fx((int4*)coef_a, ce, mk_, mk_, [&](int i, int j) {
+                return cscal(cplus(A[i * M_MAX + j], cconj(A[j * M_MAX + i])), half);
+            });
+            st_mat_fx((int4*)coef_bh, ce + M_MAX, mp, mk_, [&](int i, int j) { return cconj(ss->sh.betak[j * M_MAX + i]); });
+        }
+    }
 }
 
 // The block step's QR: G = W^H W from the partials (NRC CTAs), pivoted QR with
@@ -668,7 +712,7 @@ __global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, con
 // m_{k+1}.
 template <class T>
 __global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* __restrict__ part,
-                                                      int nblk, int m, double dtol, int wprec, void* coefS_w, int MM) {
+                                                      int nblk, int m, double dtol, int wprec, void* coefS_w, int* ce, int MM) {
     using S = Sc<T>;
     using R = typename S::R;
     if (ctl->done) return;
@@ -702,7 +746,12 @@ __global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* c
         ss->sh.S[t] = (a < mk_ && b < mn) ? Sm[a * MM + b] : cz<T>();
         ss->sh.betan[t] = (a < mn && b < mk_) ? Bn[a * MM + b] : cz<T>();
     }
-    st_mat_work<T>(wprec, coefS_w, Sm, MM, mk_, mn);
+    bool fx = false;
+    if constexpr (is_fp64<T>()) {
+        fx = ce != nullptr;
+        if (fx) st_mat_fx((int4*)coefS_w, ce + 2 * M_MAX, mk_, mn, [&](int i, int j) { return Sm[i * MM + j]; });
+    }
+    if (!fx) st_mat_work<T>(wprec, coefS_w, Sm, MM, mk_, mn);
     if (threadIdx.x == 0) {
         ctl->mnext = mn;
         ctl->deflations += mk_ - mn;
@@ -713,7 +762,7 @@ __global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* c
 template <class T>
 __device__ void shift_recurrence(SmallStateT<T>* ss, Ctl* ctl, int j, int m, const double* __restrict__ sigma,
                                  const double* __restrict__ target, int freeze, int wprec, void* coefU_w,
-                                 void* coefL_w, int* active, int* conv_step, double* res_out, int MM,
+                                 void* coefL_w, int* ce, int* active, int* conv_step, double* res_out, int MM,
                                  unsigned char* sm) {
     using S = Sc<T>;
     using R = typename S::R;
@@ -783,8 +832,19 @@ __device__ void shift_recurrence(SmallStateT<T>* ss, Ctl* ctl, int j, int m, con
         if (freeze && sf.conv[i]) Ut[a * MM + i] = cz<T>();
     }
     bsync();
-    st_mat_work<T>(wprec, (char*)coefU_w + (size_t)j * tile * cb, Ut, MM, mk_, m);
-    st_mat_work<T>(wprec, (char*)coefL_w + (size_t)j * tile * cb, LH, MM, mk_, mn);
+    bool fx = false;
+    if constexpr (is_fp64<T>()) {
+        fx = ce != nullptr;
+        if (fx) {
+            int* e = ce + (size_t)j * 2 * M_MAX;
+            st_mat_fx((int4*)coefU_w + (size_t)j * tile, e, mk_, m, [&](int a, int b) { return Ut[a * MM + b]; });
+            st_mat_fx((int4*)coefL_w + (size_t)j * tile, e + M_MAX, mk_, mn, [&](int a, int b) { return LH[a * MM + b]; });
+        }
+    }
+    if (!fx) {
+        st_mat_work<T>(wprec, (char*)coefU_w + (size_t)j * tile * cb, Ut, MM, mk_, m);
+        st_mat_work<T>(wprec, (char*)coefL_w + (size_t)j * tile * cb, LH, MM, mk_, mn);
+    }
     for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) {
         int c = t / M_MAX, a = t % M_MAX;
         sf.Lam[t] = (c < mn && a < mk_) ? cconj(LH[a * MM + c]) : cz<T>();
@@ -817,11 +877,11 @@ template <class T>
 __global__ void __launch_bounds__(NT) small_recur_kernel(SmallStateT<T>* ss, Ctl* ctl, int s, int m,
                                                          const double* __restrict__ sigma,
                                                          const double* __restrict__ target, int freeze, int wprec,
-                                                         void* coefU_w, void* coefL_w, int* active, int* conv_step,
-                                                         double* res_out, int MM) {
+                                                         void* coefU_w, void* coefL_w, int* ce, int* active,
+                                                         int* conv_step, double* res_out, int MM) {
     if (ctl->done) return;
     extern __shared__ __align__(16) unsigned char sm[];
-    shift_recurrence<T>(ss, ctl, (int)blockIdx.x, m, sigma, target, freeze, wprec, coefU_w, coefL_w, active,
+    shift_recurrence<T>(ss, ctl, (int)blockIdx.x, m, sigma, target, freeze, wprec, coefU_w, coefL_w, ce, active,
                         conv_step, res_out, MM, sm);
     if (!last_arrival(&ss->sh.ticket[2])) return;
     const int j = threadIdx.x;                     // s <= S_MAX shifts
@@ -875,42 +935,42 @@ void launch_small_init(SmallState* ss, Ctl* ctl, const double2* G0, const double
 }
 
 void launch_small_alpha(SmallState* ss, const Ctl* ctl, const double* partials, int nblk, int nf_max, int wprec,
-                        int sfp64, void* coef_a, void* coef_bh, cudaStream_t st) {
+                        int sfp64, void* coef_a, void* coef_bh, int* ce, cudaStream_t st) {
     if (sfp64)
         small_alpha_kernel<double2><<<NRC, NT, 0, st>>>(as_state<double2>(ss), ctl, partials, nblk, nf_max, wprec,
-                                                        coef_a, coef_bh);
+                                                        coef_a, coef_bh, ce);
     else
         small_alpha_kernel<ddc><<<NRC, NT, 0, st>>>(as_state<ddc>(ss), ctl, partials, nblk, nf_max, wprec, coef_a,
-                                                    coef_bh);
+                                                    coef_bh, ce);
 }
 
 void launch_small_qr(SmallState* ss, Ctl* ctl, const double* partials, int nblk, int m, double dtol, int wprec,
-                     int sfp64, void* coefS_w, cudaStream_t st) {
+                     int sfp64, void* coefS_w, int* ce, cudaStream_t st) {
     static std::atomic<unsigned long long> devs64{0}, devsdd{0};
     max_dyn_smem_once(small_qr_kernel<double2>, (int)qr_smem(M_MAX), devs64);
     max_dyn_smem_once(small_qr_kernel<ddc>, (int)qr_smem(M_MAX), devsdd);
     // matrices at the initial width m, which block widths never exceed
     if (sfp64)
         small_qr_kernel<double2><<<NRC, NT, qr_smem(m), st>>>(as_state<double2>(ss), ctl, partials, nblk, m, dtol,
-                                                              wprec, coefS_w, m);
+                                                              wprec, coefS_w, ce, m);
     else
         small_qr_kernel<ddc><<<NRC, NT, qr_smem(m), st>>>(as_state<ddc>(ss), ctl, partials, nblk, m, dtol, wprec,
-                                                          coefS_w, m);
+                                                          coefS_w, ce, m);
 }
 
 void launch_small_recur(SmallState* ss, Ctl* ctl, int s, int m, const double* sigma_dev, const double* target_dev,
-                        int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* active, int* conv_step,
-                        double* res_out, cudaStream_t st) {
+                        int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* ce, int* active,
+                        int* conv_step, double* res_out, cudaStream_t st) {
     static std::atomic<unsigned long long> devs64{0}, devsdd{0};
     max_dyn_smem_once(small_recur_kernel<double2>, (int)recur_smem(M_MAX), devs64);
     max_dyn_smem_once(small_recur_kernel<ddc>, (int)recur_smem(M_MAX), devsdd);
     if (sfp64)
         small_recur_kernel<double2><<<s, NT, recur_smem(m), st>>>(as_state<double2>(ss), ctl, s, m, sigma_dev,
-                                                                  target_dev, freeze, wprec, coefU_w, coefL_w, active,
+                                                                  target_dev, freeze, wprec, coefU_w, coefL_w, ce, active,
                                                                   conv_step, res_out, m);
     else
         small_recur_kernel<ddc><<<s, NT, recur_smem(m), st>>>(as_state<ddc>(ss), ctl, s, m, sigma_dev, target_dev,
-                                                              freeze, wprec, coefU_w, coefL_w, active, conv_step,
+                                                              freeze, wprec, coefU_w, coefL_w, ce, active, conv_step,
                                                               res_out, m);
 }
 

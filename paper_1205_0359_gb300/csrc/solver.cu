@@ -87,6 +87,8 @@ struct Lane {
     double2* G = nullptr;
     double* diag = nullptr;
     void *coef_a = nullptr, *coef_bh = nullptr, *coefS = nullptr, *coefU = nullptr, *coefL = nullptr;
+    int* ce = nullptr;                            // column exponents of fixed-point coefficients (coef_fx): a, bh, S,
+                                                  // then U and L of every chunk slot and shift
     int *active = nullptr, *conv_step = nullptr;
     double *res = nullptr, *sigma = nullptr, *target = nullptr;
     dsbcg::Ctl* h_ctl = nullptr;                  // pinned
@@ -395,6 +397,9 @@ int stream_prio(bool refinement) {
     return refinement ? greatest : least;
 }
 
+// exponents of a lane's coefficient tiles: a, bh, S, and U, L per chunk slot and shift
+size_t ce_bytes(int chunk, int s) { return (3 + 2 * (size_t)chunk * s) * M_MAX * sizeof(int); }
+
 dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
     auto& w = c->ws;
     const bool fx = c->linksfx && fx_residuals(c, prec, m);
@@ -511,6 +516,7 @@ dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
     L0.h_conv = w.h_conv;
     L0.h_active = w.h_active;
     L0.chunk = chunk0;
+    if (coef_fx(prec, m)) CKS(dmalloc(c, (void**)&L0.ce, ce_bytes(chunk0, s)));
     w.lanes.assign(1, L0);
     return DSBCG_OK;
 }
@@ -553,6 +559,7 @@ int ensure_refine_lanes(dsbcg_ctx* c, int want) {
                   dmalloc(c, &L.coef_a, tb) == DSBCG_OK && dmalloc(c, &L.coef_bh, tb) == DSBCG_OK &&
                   dmalloc(c, &L.coefS, tb) == DSBCG_OK && dmalloc(c, &L.coefU, (size_t)chunk * tb) == DSBCG_OK &&
                   dmalloc(c, &L.coefL, (size_t)chunk * tb) == DSBCG_OK &&
+                  (!coef_fx(prec, m) || dmalloc(c, (void**)&L.ce, ce_bytes(chunk, 1)) == DSBCG_OK) &&
                   dmalloc(c, (void**)&L.active, (size_t)chunk * sizeof(int)) == DSBCG_OK &&
                   dmalloc(c, (void**)&L.conv_step, m * sizeof(int)) == DSBCG_OK &&
                   dmalloc(c, (void**)&L.res, m * sizeof(double)) == DSBCG_OK &&
@@ -892,13 +899,15 @@ dsbcg_status lane_enqueue(dsbcg_ctx* c, Lane& L) {
     cudaStream_t st = L.st;
     char* ring = (char*)L.vring;
     const int C = L.chunk_used, R = C + 1;
+    int* const ce = coef_fx(prec, m_in) ? L.ce : nullptr;
+    int* const ceUL = ce ? ce + 3 * M_MAX : nullptr;
     auto slot = [&](int k) { return ring + (size_t)(k % R) * m_in * fb; };     // V_k
     // P_j and X_j take the steps L.k0 + 1 .. L.step (the chunk's executed ones)
     auto flush = [&]() {
         if (L.step == L.k0) return;
         Prof p(c, DSBCG_KCLASS_SHIFT, 1, st);
         launch_shift_chunk(prec, ring, (size_t)m_in * ld, R, ld, L.P, L.Xin, ld, n, s_in, m_in, L.ctl, m_in, L.k0,
-                           C, L.coefU, L.coefL, L.active, c->hscale, st);
+                           C, L.coefU, L.coefL, ceUL, L.active, c->hscale, st);
         L.k0 = L.step;
     };
     for (int q = 0; q < L.poll_every && L.step < L.max_steps; ++q) {
@@ -916,7 +925,7 @@ dsbcg_status lane_enqueue(dsbcg_ctx* c, Lane& L) {
         }
         {
             Prof p(c, DSBCG_KCLASS_SMALL, 1, st);
-            launch_small_alpha(L.ss, L.ctl, L.partials, L.nblk, m_in, wp, L.sfp64, L.coef_a, L.coef_bh, st);
+            launch_small_alpha(L.ss, L.ctl, L.partials, L.nblk, m_in, wp, L.sfp64, L.coef_a, L.coef_bh, ce, st);
         }
         if (update_gram_fits(prec, m_in)) {
             // W and its Gram W^H W in one pass over the rows
@@ -926,7 +935,7 @@ dsbcg_status lane_enqueue(dsbcg_ctx* c, Lane& L) {
         } else {
             {
                 Prof p(c, DSBCG_KCLASS_UPDATE, 1, st);
-                launch_block_update(prec, L.zw, L.y, Vk, Vo, ld, n, L.ctl, m_in, L.coef_a, L.coef_bh, c->hscale,
+                launch_block_update(prec, L.zw, L.y, Vk, Vo, ld, n, L.ctl, m_in, L.coef_a, L.coef_bh, ce, c->hscale,
                                     st);
             }
             {
@@ -936,17 +945,18 @@ dsbcg_status lane_enqueue(dsbcg_ctx* c, Lane& L) {
         }
         {
             Prof p(c, DSBCG_KCLASS_SMALL, 1, st);
-            launch_small_qr(L.ss, L.ctl, L.partials, L.nblk, m_in, L.dtol, wp, L.sfp64, L.coefS, st);
+            launch_small_qr(L.ss, L.ctl, L.partials, L.nblk, m_in, L.dtol, wp, L.sfp64, L.coefS, ce, st);
         }
         {
             Prof p(c, DSBCG_KCLASS_UPDATE, 1, st);
-            launch_v_update(prec, slot(step + 1), L.zw, ld, n, L.ctl, m_in, L.coefS, c->hscale, st);
+            launch_v_update(prec, slot(step + 1), L.zw, ld, n, L.ctl, m_in, L.coefS, ce ? ce + 2 * M_MAX : nullptr, c->hscale,
+                            st);
         }
         {
             Prof p(c, DSBCG_KCLASS_SMALL, 1, st);
             launch_small_recur(L.ss, L.ctl, s_in, m_in, L.sigma, L.target, L.freeze, wp, L.sfp64,
                                (char*)L.coefU + (size_t)hs * s_in * cb, (char*)L.coefL + (size_t)hs * s_in * cb,
-                               L.active + (size_t)hs * s_in, L.conv_step, L.res, st);
+                               ceUL ? ceUL + (size_t)hs * s_in * 2 * M_MAX : nullptr, L.active + (size_t)hs * s_in, L.conv_step, L.res, st);
         }
         if (L.step - L.k0 == C) flush();
     }
