@@ -3,15 +3,13 @@
 //   (D psi)(x) = psi(x) - kappa * sum_mu [ (1 - gamma_mu) U_mu(x) psi(x+mu)
 //                                        + (1 + gamma_mu) U_mu(x-mu)^H psi(x-mu) ]
 //
-// One CTA of 32 threads covers 32 consecutive sites of one field; the grid
-// is (fields, site tiles) with the field index fastest, so the CTAs of all
-// fields of a site tile are issued together and the SU(3) links they share
-// are fetched from HBM once and then served from L1/L2 (read-only path).
-// Each thread owns one (site, field) pair; every pair-chunk load of a
-// neighbour spinor is one contiguous 512-byte warp access.  Staging the links
-// in shared memory per CTA was measured slower on GB300 (1.3 vs 3.3 TB/s at
-// 16^3 x 32 with 12 FP32 fields): the staging barrier serialises each CTA's
-// link and spinor loads.
+// FP32 and 16-bit fields run in dslash_cta_kernel (links staged in shared
+// memory), FP64 and double-float ones in dslash_kernel: one CTA of 32 threads
+// covers 32 consecutive sites of one field, field index fastest, so the links
+// that all fields of a site tile share are fetched from HBM once and then
+// served from L1/L2.  (FP64 fields with SU(3) links: dslash_fx.cu.)  A thread
+// owns one (site, field) pair; every pair-chunk load of a neighbour spinor is
+// one contiguous warp access.
 // Spin projection in the chiral basis (gamma_k = [[0, i s_k], [-i s_k, 0]],
 // gamma_4 = [[0, 1], [1, 0]]): with upper/lower spin pairs u = (p0, p1),
 // l = (p2, p3),
@@ -333,26 +331,32 @@ __global__ void __launch_bounds__(32, (P == PDD || P == P64) ? 12 : 24) dslash_k
     }
 }
 
+// coordinates of the half index k on `parity` of an all-even lattice
+__device__ __forceinline__ Site half_coords(const Geom& g, int k, int parity) {
+    const int hx = g.L[0] / 2;
+    const int row = k / hx;
+    Site s;
+    s.c[1] = row % g.L[1];
+    s.c[2] = (row / g.L[1]) % g.L[2];
+    s.c[3] = row / (g.L[1] * g.L[2]);
+    s.c[0] = 2 * (k % hx) + ((parity + s.c[1] + s.c[2] + s.c[3]) & 1);
+    return s;
+}
+
 // Projection of the hop (mu, dir) of spinor p: the half spinor h of
-// (1 - gamma_mu) p (dir 0) or (1 + gamma_mu) p (dir 1), with the upper spins
-// scaled by su and the lower by sl (gamma_5 and time-boundary signs).
-template <class C, class R>
-__device__ __forceinline__ void hop_project(int mu, int dir, const C p[12], R su, R sl_, C h[2][3]) {
+// (1 - gamma_mu) p (dir 0) or (1 + gamma_mu) p (dir 1); DAG: D^H = gamma_5 D
+// gamma_5, whose hops have the other projector (the signs of gamma_5 on input
+// and output cancel exactly).
+template <bool DAG, class C>
+__device__ __forceinline__ void hop_project_signed(int mu, int dir, const C p[12], C h[2][3]) {
+    const bool minus = (dir == 0) != DAG;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        C u0 = cscale(p[0 * 3 + a], su), u1 = cscale(p[1 * 3 + a], su);
-        C l0 = cscale(p[2 * 3 + a], sl_), l1 = cscale(p[3 * 3 + a], sl_);
-        if (dir == 0) {
-            if (mu == 0) { h[0][a] = csub(u0, ctimesi(l1)); h[1][a] = csub(u1, ctimesi(l0)); }
-            if (mu == 1) { h[0][a] = csub(u0, l1); h[1][a] = cadd(u1, l0); }
-            if (mu == 2) { h[0][a] = csub(u0, ctimesi(l0)); h[1][a] = cadd(u1, ctimesi(l1)); }
-            if (mu == 3) { h[0][a] = csub(u0, l0); h[1][a] = csub(u1, l1); }
-        } else {
-            if (mu == 0) { h[0][a] = cadd(u0, ctimesi(l1)); h[1][a] = cadd(u1, ctimesi(l0)); }
-            if (mu == 1) { h[0][a] = cadd(u0, l1); h[1][a] = csub(u1, l0); }
-            if (mu == 2) { h[0][a] = cadd(u0, ctimesi(l0)); h[1][a] = csub(u1, ctimesi(l1)); }
-            if (mu == 3) { h[0][a] = cadd(u0, l0); h[1][a] = cadd(u1, l1); }
-        }
+        const C u0 = p[a], u1 = p[3 + a], l0 = p[6 + a], l1 = p[9 + a];
+        if (mu == 0) { h[0][a] = minus ? csub(u0, ctimesi(l1)) : cadd(u0, ctimesi(l1)); h[1][a] = minus ? csub(u1, ctimesi(l0)) : cadd(u1, ctimesi(l0)); }
+        if (mu == 1) { h[0][a] = minus ? csub(u0, l1) : cadd(u0, l1); h[1][a] = minus ? cadd(u1, l0) : csub(u1, l0); }
+        if (mu == 2) { h[0][a] = minus ? csub(u0, ctimesi(l0)) : cadd(u0, ctimesi(l0)); h[1][a] = minus ? cadd(u1, ctimesi(l1)) : csub(u1, ctimesi(l1)); }
+        if (mu == 3) { h[0][a] = minus ? csub(u0, l0) : cadd(u0, l0); h[1][a] = minus ? csub(u1, l1) : cadd(u1, l1); }
     }
 }
 
@@ -387,18 +391,27 @@ __device__ __forceinline__ void hop_reconstruct(int mu, int dir, const C uh[2][3
 // use), then each warp applies the stencil to its field with the links read
 // from shared memory and the neighbour spinors from L1/L2.  Against one field
 // per 32-thread CTA with links from L1 this reads each link from L2 once per
-// 4 fields and removes 72 of the 126 global loads per site and field:
-// 9-13% faster on GB300 at 16^3 x 32, 24^3 x 48 and 32^3 x 64 (12, 8 and
-// 16 FP32 fields); larger field groups measured slower (fewer resident CTAs).
+// 4 fields and removes 72 of the 126 global loads per site and field; larger
+// field groups measured slower (fewer resident CTAs).
+//
+// 16-bit fields are taken as stored: their scale is a power of two and the
+// operator is linear, so scaling the loads back and the store again cancels
+// exactly.  The signs of gamma_5 are compile-time and the time-boundary sign
+// touches the t hops alone; 72 registers, 7 CTAs per SM.  Bound by the latency
+// and L1 traffic of the neighbour loads (issue slots half used).  ms per
+// launch, run-time signs and scaled loads at 80 registers / this: 16^3 x 32,
+// 12 FP32 fields 0.109 / 0.103; 24^3 x 48, 8 fields, FP32 0.361 / 0.334, BF16
+// 0.411 / 0.356.  8 CTAs (64 registers) spill: 0.108, 0.355, 0.363.
+//
+// HALF: the hopping term of the even-odd operator (see dslash_half_kernel),
+// out = alpha src + beta H in on `parity`, or beta H in without src.
 constexpr int CTA_FIELDS = 4;
 
-template <int P, bool L12>
-__global__ void __launch_bounds__(32 * CTA_FIELDS, P == P32 ? 6 : 5) dslash_cta_kernel(typename Tr<P>::S2* __restrict__ out,
-                                                       const typename Tr<P>::S2* __restrict__ in, size_t ld,
-                                                       const typename Tr<P>::S2* __restrict__ links,
-                                                       const typename Tr<P>::S2* __restrict__ links12, Geom g,
-                                                       float kappa, int g5in, int g5out, const Ctl* __restrict__ ctl,
-                                                       int nf_static, float hscale, int ngrp) {
+template <int P, bool L12, bool DAG, bool HALF>
+__global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kernel(
+    typename Tr<P>::S2* __restrict__ out, const typename Tr<P>::S2* __restrict__ in,
+    const typename Tr<P>::S2* __restrict__ src, size_t ld, const typename Tr<P>::S2* __restrict__ links, Geom g,
+    float alpha, float beta, int parity, const Ctl* __restrict__ ctl, int nf_static, int ngrp) {
     // [hop][entry][site of the tile]: rows 0 and 1 of SU(3) links (L12), with
     // row 2 rebuilt at each use, else all nine entries
     __shared__ float2 sl[8][L12 ? 6 : 9][32];
@@ -412,65 +425,51 @@ __global__ void __launch_bounds__(32 * CTA_FIELDS, P == P32 ? 6 : 5) dslash_cta_
     const int tile = (int)(blockIdx.x / (unsigned)ngrp);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const size_t V = (size_t)g.V;
-    const int x = tile * 32 + lane;
-    const bool valid = x < g.V;
-    const int xs = valid ? x : g.V - 1;
-    const Site s = coords(g, xs);
+    const int Vf = HALF ? g.V / 2 : g.V;
+    const int k = tile * 32 + lane;          // site of the field
+    const bool valid = k < Vf;
+    const int ks = valid ? k : Vf - 1;
+    Site s;
+    int xs = ks;                             // site of the lattice
+    if constexpr (HALF) {
+        s = half_coords(g, ks, parity);
+        xs = s.c[0] + g.L[0] * (ks / (g.L[0] / 2));
+    } else {
+        s = coords(g, xs);
+    }
     for (int h = w; h < 8; h += CTA_FIELDS) {
         const int mu = h >> 1, dir = h & 1;
         float sgn;
         const int y = neighbour(g, xs, s, mu, dir == 0 ? 1 : -1, &sgn);
         const size_t site = dir == 0 ? (size_t)xs : (size_t)y;
-        if (links12) {
-            // 12-real links: rows 0 and 1; row 2 = conj(row 0 x row 1) (SU(3))
-            const typename Tr<P>::S2* u = links12 + (size_t)mu * 6 * V + site;
-            float2 r[6];
+        constexpr int NE = L12 ? 6 : 9;
+        const typename Tr<P>::S2* u = links + (size_t)mu * NE * V + site;
 #pragma unroll
-            for (int e = 0; e < 6; ++e) {
-                r[e] = ld_link<P>(u + (size_t)e * V, 0);
-                sl[h][e][lane] = r[e];
-            }
-            if constexpr (!L12) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const int i = (k + 1) % 3, j = (k + 2) % 3;
-                    float2 t = cmul(r[i], r[3 + j]);
-                    cfms(t, r[j], r[3 + i]);
-                    sl[h][6 + k][lane] = make_float2(t.x, -t.y);
-                }
-            }
-        } else if constexpr (!L12) {
-            const typename Tr<P>::S2* u = links + (size_t)mu * 9 * V + site;
-#pragma unroll
-            for (int e = 0; e < 9; ++e) sl[h][e][lane] = ld_link<P>(u + (size_t)e * V, 0);
-        }
+        for (int e = 0; e < NE; ++e) sl[h][e][lane] = ld_link<P>(u + (size_t)e * V, 0);
     }
     __syncthreads();
     const int f = grp * CTA_FIELDS + w;
     if (!valid || f >= nf) return;
-    float inv = 1.f, scl = 1.f;
-    if constexpr (P == PBF16 || P == PF16) {
-        inv = 1.f / hscale;
-        scl = hscale;
-    }
-    const float g5i = g5in ? -1.f : 1.f;
     const typename Tr<P>::S2* fin = in + (size_t)f * ld;
     float2 acc[4][3];
-#pragma unroll
-    for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) acc[sp][a] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
 #pragma unroll
         for (int dir = 0; dir < 2; ++dir) {
             const int h = 2 * mu + dir;
             float sgn;
-            const int y = neighbour(g, x, s, mu, dir == 0 ? 1 : -1, &sgn);
+            const int y = neighbour(g, xs, s, mu, dir == 0 ? 1 : -1, &sgn);
             float2 p[12];
-            SpinorIO<P>::load(fin, V, (size_t)y, p, inv, 0);
+            SpinorIO<P>::load(fin, (size_t)Vf, (size_t)(HALF ? y >> 1 : y), p, 1.f, 0);
             float2 hh[2][3];
-            hop_project(mu, dir, p, sgn * g5i, sgn, hh);
+            hop_project_signed<DAG>(mu, dir, p, hh);
+            if (mu == 3) {                       // the time-boundary sign
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    hh[0][a] = cscale(hh[0][a], sgn);
+                    hh[1][a] = cscale(hh[1][a], sgn);
+                }
+            }
             // the hop's link: 9 entries from shared memory, or rows 0 and 1
             // with row 2 = conj(row 0 x row 1) rebuilt here
             float2 lk[L12 ? 9 : 1];
@@ -509,24 +508,30 @@ __global__ void __launch_bounds__(32 * CTA_FIELDS, P == P32 ? 6 : 5) dslash_cta_
                         cfmac(uh[1][a], uba, hh[1][b]);
                     }
                 }
-            hop_reconstruct(mu, dir, uh, acc);
+            if (h == 0) {
+#pragma unroll
+                for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) acc[sp][a] = make_float2(0.f, 0.f);
+            }
+            hop_reconstruct(mu, DAG ? 1 - dir : dir, uh, acc);
         }
     }
     float2 p[12];
-    SpinorIO<P>::load(fin, V, (size_t)x, p, inv, 0);
-    const float go = g5out ? -1.f : 1.f;
+    const typename Tr<P>::S2* diag = HALF ? src : in;
+    if (diag) {
+        SpinorIO<P>::load(diag + (size_t)f * ld, (size_t)Vf, (size_t)k, p, 1.f, 0);
 #pragma unroll
-    for (int sp = 0; sp < 4; ++sp) {
-        const float sgi = (sp < 2) ? g5i : 1.f, sgo = (sp < 2) ? go : 1.f;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            float2 v = cscale(p[sp * 3 + a], sgi);
-            v.x = fmaf(-kappa, acc[sp][a].x, v.x);
-            v.y = fmaf(-kappa, acc[sp][a].y, v.y);
-            p[sp * 3 + a] = cscale(v, sgo);
+        for (int i = 0; i < 12; ++i) {
+            const float2 a = acc[i / 3][i % 3];
+            const float2 d = HALF ? cscale(p[i], alpha) : p[i];
+            p[i] = make_float2(fmaf(beta, a.x, d.x), fmaf(beta, a.y, d.y));
         }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 12; ++i) p[i] = cscale(acc[i / 3][i % 3], beta);
     }
-    SpinorIO<P>::store(out + (size_t)f * ld, V, (size_t)x, p, scl, 0);
+    SpinorIO<P>::store(out + (size_t)f * ld, (size_t)Vf, (size_t)k, p, 1.f, 0);
 }
 
 // Half-lattice hopping term for the even-odd (Schur) operator.  With every
@@ -565,14 +570,8 @@ __global__ void __launch_bounds__(32, (P == PDD || P == P64) ? 12 : 24) dslash_h
     const size_t loff = (P == PDD) ? 36 * (size_t)g.V : 0;
     const size_t V = (size_t)g.V;
     // full-lattice site of half index k
-    const int hx = g.L[0] / 2;
-    const int row = k / hx;
-    Site s;
-    s.c[1] = row % g.L[1];
-    s.c[2] = (row / g.L[1]) % g.L[2];
-    s.c[3] = row / (g.L[1] * g.L[2]);
-    s.c[0] = 2 * (k % hx) + ((parity + s.c[1] + s.c[2] + s.c[3]) & 1);
-    const int x = s.c[0] + g.L[0] * row;
+    const Site s = half_coords(g, k, parity);
+    const int x = s.c[0] + g.L[0] * (k / (g.L[0] / 2));
     const R g5i = g5in ? R(-1) : R(1);
     const typename Tr<P>::S2* fin = in + (size_t)f * ld;
     C acc[4][3];
@@ -676,22 +675,24 @@ void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* l
     // kernels of other streams
     if (max_ctas > 0 && grid.x > (unsigned)max_ctas) grid.x = (unsigned)max_ctas;
     const size_t sm = 0;
-    // (SU(3) links: rows 0 and 1 staged, row 2 rebuilt at each use; 12 KB of
-    // shared memory per CTA instead of 18, and 3.5% faster at 16^3 x 32)
-#define DSBCG_CTA_LAUNCH(PP, S2T)                                                                               \
-    if (links12)                                                                                                \
-        dslash_cta_kernel<PP, true><<<cgrid, cblock, 0, st>>>((S2T*)out, (const S2T*)in, ld, (const S2T*)links,   \
-                                                              (const S2T*)links12, g, (float)kappa, g5in, g5out,  \
-                                                              ctl, nf_static, hscale, ngrp);                      \
-    else                                                                                                        \
-        dslash_cta_kernel<PP, false><<<cgrid, cblock, 0, st>>>((S2T*)out, (const S2T*)in, ld, (const S2T*)links,  \
-                                                               nullptr, g, (float)kappa, g5in, g5out, ctl,        \
-                                                               nf_static, hscale, ngrp)
     // FP32 and 16-bit fields: CTAs of 32 sites x CTA_FIELDS fields with the
-    // tile's links staged in shared memory
+    // tile's links staged in shared memory (SU(3) links: rows 0 and 1, row 2
+    // rebuilt at each use; 12 KB of shared memory per CTA instead of 18)
     const int ngrp = (nf_grid + CTA_FIELDS - 1) / CTA_FIELDS;
     dim3 cgrid((unsigned)(ngrp * ((g.V + 31) / 32)));
     dim3 cblock(32 * CTA_FIELDS);
+#define DSBCG_CTA_LAUNCH2(PP, S2T, L12, DAG)                                                                    \
+    dslash_cta_kernel<PP, L12, DAG, false><<<cgrid, cblock, 0, st>>>(                                            \
+        (S2T*)out, (const S2T*)in, nullptr, ld, (const S2T*)(L12 ? links12 : links), g, 1.f, -(float)kappa, 0,    \
+        ctl, nf_static, ngrp)
+#define DSBCG_CTA_LAUNCH(PP, S2T)                                                                               \
+    if (links12) {                                                                                              \
+        if (dag) DSBCG_CTA_LAUNCH2(PP, S2T, true, true);                                                        \
+        else DSBCG_CTA_LAUNCH2(PP, S2T, true, false);                                                           \
+    } else {                                                                                                    \
+        if (dag) DSBCG_CTA_LAUNCH2(PP, S2T, false, true);                                                       \
+        else DSBCG_CTA_LAUNCH2(PP, S2T, false, false);                                                          \
+    }
     switch (prec) {
         case P64:
             dslash_kernel<P64><<<grid, block, sm, st>>>((double2*)out, (const double2*)in, ld,
@@ -709,6 +710,7 @@ void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* l
             break;
     }
 #undef DSBCG_CTA_LAUNCH
+#undef DSBCG_CTA_LAUNCH2
 }
 
 void launch_dslash_half(int prec, void* out, const void* in, const void* src, size_t ld, const void* links,
@@ -718,18 +720,33 @@ void launch_dslash_half(int prec, void* out, const void* in, const void* src, si
     const int nf_grid = nfg < 1 ? 1 : nfg;
     dim3 block(32);
     dim3 grid((unsigned)(nf_grid * ((g.V / 2 + 31) / 32)));
+    const int ngrp = (nf_grid + CTA_FIELDS - 1) / CTA_FIELDS;
+    dim3 cgrid((unsigned)(ngrp * ((g.V / 2 + 31) / 32)));
+    dim3 cblock(32 * CTA_FIELDS);
+    const int dag = g5in || g5out;
+    // FP32 and 16-bit fields: gamma_5 on the input of the first pass and on the
+    // output of the second (dag) is gamma_5 H gamma_5 in both
+#define DSBCG_HALF_CTA2(PP, S2T, DAG)                                                                          \
+    dslash_cta_kernel<PP, false, DAG, true><<<cgrid, cblock, 0, st>>>((S2T*)out, (const S2T*)in, (const S2T*)src, ld, \
+                                                                      (const S2T*)links, g, (float)alpha,        \
+                                                                      (float)beta, parity, ctl, nf_static, ngrp)
+#define DSBCG_HALF_CTA(PP, S2T)                                                                                \
+    if (dag) DSBCG_HALF_CTA2(PP, S2T, true);                                                                   \
+    else DSBCG_HALF_CTA2(PP, S2T, false)
 #define DSBCG_HALF_LAUNCH(PP, S2T, RA, RB)                                                                     \
     dslash_half_kernel<PP><<<grid, block, 0, st>>>((S2T*)out, (const S2T*)in, (const S2T*)src, ld,            \
                                                    (const S2T*)links, g, RA, RB, parity, g5in, g5out, ctl,    \
                                                    nf_static, hscale, nf_grid)
     switch (prec) {
         case P64: DSBCG_HALF_LAUNCH(P64, double2, alpha, beta); break;
-        case P32: DSBCG_HALF_LAUNCH(P32, float2, (float)alpha, (float)beta); break;
-        case PBF16: DSBCG_HALF_LAUNCH(PBF16, __nv_bfloat162, (float)alpha, (float)beta); break;
-        case PF16: DSBCG_HALF_LAUNCH(PF16, __half2, (float)alpha, (float)beta); break;
+        case P32: DSBCG_HALF_CTA(P32, float2); break;
+        case PBF16: DSBCG_HALF_CTA(PBF16, __nv_bfloat162); break;
+        case PF16: DSBCG_HALF_CTA(PF16, __half2); break;
         case PDD: DSBCG_HALF_LAUNCH(PDD, float2, dd::from_double(alpha), dd::from_double(beta)); break;
     }
 #undef DSBCG_HALF_LAUNCH
+#undef DSBCG_HALF_CTA
+#undef DSBCG_HALF_CTA2
 }
 
 }  // namespace dsbcg

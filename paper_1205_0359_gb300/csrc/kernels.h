@@ -79,7 +79,9 @@ void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* l
 // fields of V / 2 sites, half index = canonical site / 2):
 // out_f = alpha src_f + beta G5o H G5i in_f, out and src on `parity`, in on
 // the other parity; src may be NULL (alpha ignored); G5i/G5o: gamma_5 on the
-// input / on the hopping term's output when g5in / g5out.
+// input / on the hopping term's output when g5in / g5out.  FP32 and 16-bit
+// fields take gamma_5 on both sides when either is asked for: the two passes of
+// D^H (g5in, then g5out) compose to the same.
 void launch_dslash_half(int prec, void* out, const void* in, const void* src, size_t ld, const void* links,
                         const Geom& g, double alpha, double beta, int parity, int g5in, int g5out, const Ctl* ctl,
                         int nf_static, int nf_max, float hscale, cudaStream_t st);
