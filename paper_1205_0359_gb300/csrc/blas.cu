@@ -27,7 +27,7 @@ int gram_blocks(size_t n, int nf_max) {
 }
 
 void launch_gram(int prec, const void* X, const void* Y, size_t ld, size_t n, const Ctl* ctl, int nf_static,
-                 int nf_max, int herm, int diag_yy, double* partials, int nblk, float hscale, cudaStream_t st,
+                 int nf_max, int herm, int diag_yy, double* partials, int nblk, float hscale, Stream st,
                  int first_wait) {
     if (nf_max <= 16) {
         // shared-memory tiled kernel: one CTA per partial slot, nblk CTAs
@@ -58,16 +58,16 @@ void launch_gram_reduce(const double* partials, int nblk, int nf_max, int herm, 
 
 #define EXTERN_P(P)                                                                                      \
     extern template void launch_bu_t<P>(void*, const void*, const void*, const void*, size_t, size_t, const Ctl*, \
-                                        int, const void*, const void*, const int*, float, cudaStream_t);     \
+                                        int, const void*, const void*, const int*, float, Stream);     \
     extern template void launch_ug_t<P>(void*, const void*, const void*, const void*, size_t, size_t, const Ctl*, \
-                                        int, const void*, const void*, double*, int, float, cudaStream_t);   \
+                                        int, const void*, const void*, double*, int, float, Stream);   \
     extern template void launch_ib_t<P>(void*, size_t, const void*, int, size_t, size_t, const double2*, int, \
                                         const Ctl*, int, float, cudaStream_t);                               \
     extern template void launch_vu_t<P>(void*, const void*, size_t, size_t, const Ctl*, int, const void*,     \
-                                        const int*, float, cudaStream_t);                                     \
+                                        const int*, float, Stream);                                     \
     extern template void launch_sc_t<P>(const void*, size_t, int, size_t, void*, void*, size_t, size_t, int,  \
                                         int, Ctl*, int, int, int, const void*, const void*, const int*,       \
-                                        const int*, float, cudaStream_t);
+                                        const int*, float, Stream);
 namespace blas_impl {
 EXTERN_P(P64)
 EXTERN_P(P32)
@@ -78,7 +78,7 @@ EXTERN_P(PF16)
 
 void launch_block_update(int prec, void* W, const void* Y, const void* Vk, const void* Vp, size_t ld, size_t n,
                          const Ctl* ctl, int nf_max, const void* coef_a, const void* coef_bh, const int* ce, float hscale,
-                         cudaStream_t st) {
+                         Stream st) {
     switch (prec) {
         case P64: launch_bu_t<P64>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, ce, hscale, st); break;
         case P32: launch_bu_t<P32>(W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, ce, hscale, st); break;
@@ -91,7 +91,7 @@ bool update_gram_fits(int prec, int nf_max) { return prec != P64 && nf_max <= UG
 
 void launch_update_gram(int prec, void* W, const void* Y, const void* Vk, const void* Vp, size_t ld, size_t n,
                         const Ctl* ctl, int nf_max, const void* coef_a, const void* coef_bh, double* partials,
-                        int nblk, float hscale, cudaStream_t st) {
+                        int nblk, float hscale, Stream st) {
 #define UG_ARGS W, Y, Vk, Vp, ld, n, ctl, nf_max, coef_a, coef_bh, partials, nblk, hscale, st
     switch (prec) {
         case P64: launch_ug_t<P64>(UG_ARGS); break;
@@ -113,7 +113,7 @@ void launch_init_basis(int prec, void* V1, size_t ldv, const void* B, int bprec,
 }
 
 void launch_v_update(int prec, void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl, int nf_max,
-                     const void* coefS, const int* ce, float hscale, cudaStream_t st) {
+                     const void* coefS, const int* ce, float hscale, Stream st) {
     switch (prec) {
         case P64: launch_vu_t<P64>(Vnext, W, ld, n, ctl, nf_max, coefS, ce, hscale, st); break;
         case P32: launch_vu_t<P32>(Vnext, W, ld, n, ctl, nf_max, coefS, ce, hscale, st); break;
@@ -124,7 +124,7 @@ void launch_v_update(int prec, void* Vnext, const void* W, size_t ld, size_t n, 
 
 void launch_shift_chunk(int prec, const void* ring, size_t slot_elems, int R, size_t ld, void* P, void* X,
                         size_t ldw, size_t n, int s, int m, Ctl* ctl, int nf_max, int k0, int C, const void* coefU,
-                        const void* coefL, const int* ce, const int* active, float hscale, cudaStream_t st) {
+                        const void* coefL, const int* ce, const int* active, float hscale, Stream st) {
 #define SC_ARGS ring, slot_elems, R, ld, P, X, ldw, n, s, m, ctl, nf_max, k0, C, coefU, coefL, ce, active, hscale, st
     switch (prec) {
         case P64: launch_sc_t<P64>(SC_ARGS); break;

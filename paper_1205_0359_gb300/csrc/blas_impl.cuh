@@ -44,7 +44,7 @@ __device__ inline void tile_coords(int t, int T, int herm, int* ti, int* tj) {
 template <int P>
 __global__ void __launch_bounds__(GT) gram_kernel(const typename Tr<P>::S2* __restrict__ X,
                                                   const typename Tr<P>::S2* __restrict__ Y, size_t ld,
-                                                  size_t n, const Ctl* __restrict__ ctl, int nf_static,
+                                                  size_t n, const Ctl* ctl, int nf_static,
                                                   int nf_max, int herm, int diag_yy,
                                                   double* __restrict__ partials, float hscale) {
     using C = typename Tr<P>::C;
@@ -55,8 +55,8 @@ __global__ void __launch_bounds__(GT) gram_kernel(const typename Tr<P>::S2* __re
     double* out = partials + ((size_t)tile * nblk + blockIdx.y) * GSLOTS;
     int nf = nf_static;
     if (ctl) {
-        if (ctl->done) return;
-        nf = ctl->mk;
+        if (cget(ctl->done)) return;
+        nf = cget(ctl->mk);
     }
     int ti, tj;
     tile_coords(tile, T, herm, &ti, &tj);
@@ -143,8 +143,8 @@ __global__ void __launch_bounds__(GT) gram_kernel(const typename Tr<P>::S2* __re
 // as written by the reduced-precision Gram kernels); one CTA per tile
 static __global__ void gram_reduce_kernel(const double* __restrict__ partials, int nblk, int nf_max, int herm,
                                    int diag_yy, double2* __restrict__ G, double* __restrict__ diag,
-                                   const Ctl* __restrict__ ctl, int fp32) {
-    if (ctl && ctl->done) return;
+                                   const Ctl* ctl, int fp32) {
+    if (ctl && cget(ctl->done)) return;
     const int T = (nf_max + 3) / 4;
     const int tile = blockIdx.x;
     int ti, tj;
@@ -198,14 +198,15 @@ __global__ void __launch_bounds__(256) block_update_kernel(typename Tr<P>::S2* _
                                                            const typename Tr<P>::S2* __restrict__ Y,
                                                            const typename Tr<P>::S2* __restrict__ Vk,
                                                            const typename Tr<P>::S2* __restrict__ Vp,
-                                                           size_t ld, size_t n, const Ctl* __restrict__ ctl,
+                                                           size_t ld, size_t n, const Ctl* ctl,
                                                            const typename Tr<P>::C* __restrict__ ca,
                                                            const typename Tr<P>::C* __restrict__ cbh,
                                                            float hscale) {
+    step_begin();
     using C = typename Tr<P>::C;
     using R = typename Tr<P>::R;
-    if (ctl->done) return;
-    const int mk_ = ctl->mk, mp = (ctl->k > 1) ? ctl->mprev : 0;
+    if (cget(ctl->done)) return;
+    const int mk_ = cget(ctl->mk), mp = (cget(ctl->k) > 1) ? cget(ctl->mprev) : 0;
     __shared__ C sa[NF * NF], sb[NF * NF];
     for (int t = threadIdx.x; t < NF * NF; t += blockDim.x) {
         int a = t / NF, b = t % NF;
@@ -257,14 +258,15 @@ template <int P, int NF>
 __global__ void __launch_bounds__(UG_ROWS, 2) update_gram_kernel(
     typename Tr<P>::S2* __restrict__ W, const typename Tr<P>::S2* __restrict__ Y,
     const typename Tr<P>::S2* __restrict__ Vk, const typename Tr<P>::S2* __restrict__ Vp, size_t ld, size_t n,
-    const Ctl* __restrict__ ctl, int nf_max, const typename Tr<P>::C* __restrict__ ca,
+    const Ctl* ctl, int nf_max, const typename Tr<P>::C* __restrict__ ca,
     const typename Tr<P>::C* __restrict__ cbh, double* __restrict__ partials, float hscale) {
+    step_begin();
     static_assert(NF <= UG_NF_MAX, "fused update and Gram: widths up to 12");
     using C = typename Tr<P>::C;
     using R = typename Tr<P>::R;
     using SE = typename Tr<P>::S2;
-    if (ctl->done) return;
-    const int mk_ = ctl->mk, mp = (ctl->k > 1) ? ctl->mprev : 0;
+    if (cget(ctl->done)) return;
+    const int mk_ = cget(ctl->mk), mp = (cget(ctl->k) > 1) ? cget(ctl->mprev) : 0;
     __shared__ C sa[NF * NF], sb[NF * NF];
     extern __shared__ __align__(16) unsigned char ug_smem[];
     SE* sW = reinterpret_cast<SE*>(ug_smem);                // [NF][UG_ROWS]
@@ -366,13 +368,13 @@ template <int P, int NF, int PIN>
 __global__ void __launch_bounds__(256) init_basis_kernel(typename Tr<P>::S2* __restrict__ V1, size_t ldv,
                                                          const typename Tr<PIN>::S2* __restrict__ B, size_t ldb,
                                                          size_t n, const double2* __restrict__ S, int s_dd,
-                                                         const Ctl* __restrict__ ctl, int nf_in, float hscale) {
+                                                         const Ctl* ctl, int nf_in, float hscale) {
     // the product is formed in the arithmetic precision of the storage: FP64
     // for FP64 fields, FP32 otherwise (the result is stored in FP32 or less);
     // S is read once per CTA
     using R = typename Tr<P>::R;
     using C = typename Tr<P>::C;
-    const int m1 = ctl->mk;
+    const int m1 = cget(ctl->mk);
     __shared__ C ss[NF * NF];
     for (int t = threadIdx.x; t < NF * NF; t += blockDim.x) {
         if (!s_dd) {
@@ -522,17 +524,18 @@ __device__ __forceinline__ double warp_transpose_sum(double v[32], int lane) {
 template <int P>
 __global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2* __restrict__ X,
                                                         const typename Tr<P>::S2* __restrict__ Y, size_t ld,
-                                                        size_t n, Ctl* __restrict__ ctl, int nf_static, int nf_max,
+                                                        size_t n, Ctl* ctl, int nf_static, int nf_max,
                                                         int herm, int diag_yy, double* __restrict__ partials,
                                                         float hscale, int first_wait) {
+    step_begin();
     using C = typename Tr<P>::C;
     using R = typename Tr<P>::R;
     using SE = typename Tr<P>::S2;
     constexpr int GNST = gram_stages<P>();
     int nf = nf_static;
     if (ctl) {
-        if (ctl->done) return;
-        nf = ctl->mk;
+        if (cget(ctl->done)) return;
+        nf = cget(ctl->mk);
     }
     extern __shared__ __align__(128) unsigned char g_smem[];
     const bool same = (X == Y);
@@ -732,7 +735,7 @@ __global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2
 
 template <int P>
 void launch_gram_tile_t(const void* X, const void* Y, size_t ld, size_t n, Ctl* ctl, int nf_static, int nf_max,
-                        int herm, int diag_yy, double* partials, int nblk, float hscale, cudaStream_t st,
+                        int herm, int diag_yy, double* partials, int nblk, float hscale, Stream st,
                         int first_wait) {
     using SE = typename Tr<P>::S2;
     constexpr int GNST = gram_stages<P>();
@@ -741,7 +744,7 @@ void launch_gram_tile_t(const void* X, const void* Y, size_t ld, size_t n, Ctl* 
     const size_t smem = GNST * (size_t)nbuf_fields * GR * sizeof(SE) + 2 * GNST * sizeof(uint64_t);
     static std::atomic<unsigned long long> devs{0};
     max_dyn_smem_once(gram_tile_kernel<P>, (int)(GNST * 2 * 16 * GR * sizeof(SE) + 2 * GNST * sizeof(uint64_t)), devs);
-    gram_tile_kernel<P><<<nblk, (npb + 1) * 32, smem, st>>>((const SE*)X, (const SE*)Y, ld, n, ctl, nf_static, nf_max, herm,
+    launch_step(gram_tile_kernel<P>, nblk, (npb + 1) * 32, smem, st, (const SE*)X, (const SE*)Y, ld, n, ctl, nf_static, nf_max, herm,
                                                       diag_yy, partials, hscale, first_wait);
 }
 
@@ -749,14 +752,15 @@ void launch_gram_tile_t(const void* X, const void* Y, size_t ld, size_t n, Ctl* 
 template <int P, int NF>
 __global__ void __launch_bounds__(256) v_update_kernel(typename Tr<P>::S2* __restrict__ Vn,
                                                        const typename Tr<P>::S2* __restrict__ W, size_t ld,
-                                                       size_t n, const Ctl* __restrict__ ctl,
+                                                       size_t n, const Ctl* ctl,
                                                        const typename Tr<(P == P64 ? P64 : P32)>::C* __restrict__ cS,
                                                        float hscale) {
+    step_begin();
     constexpr int PW = (P == P64) ? P64 : P32;
     using C = typename Tr<PW>::C;
     using R = typename Tr<PW>::R;
-    if (ctl->done) return;
-    const int mk_ = ctl->mk, mn = ctl->mnext;
+    if (cget(ctl->done)) return;
+    const int mk_ = cget(ctl->mk), mn = cget(ctl->mnext);
     __shared__ C sS[NF * NF];
     for (int t = threadIdx.x; t < NF * NF; t += blockDim.x) sS[t] = cS[(t / NF) * M_MAX + (t % NF)];
     __syncthreads();
@@ -808,13 +812,14 @@ template <int P, int PW, int NF, int ROWS>
 __global__ void __launch_bounds__(ROWS, (NF <= 12 && PW == P32) ? 4 : 1) shift_chunk_kernel(
     const typename Tr<P>::S2* __restrict__ ring, size_t slot_elems, int R, size_t ld,
     typename Tr<PW>::S2* __restrict__ Pb, typename Tr<PW>::S2* __restrict__ Xb, size_t ldw, size_t n, int s, int m,
-    Ctl* __restrict__ ctl, int k0, int C, const typename Tr<PW>::C* __restrict__ cU,
+    Ctl* ctl, int k0, int C, const typename Tr<PW>::C* __restrict__ cU,
     const typename Tr<PW>::C* __restrict__ cL, const int* __restrict__ act, float hscale) {
+    step_begin();
     using C2 = typename Tr<PW>::C;
     using R2 = typename Tr<PW>::R;
     using SE = typename Tr<P>::S2;
     const int j = (int)(blockIdx.x % (unsigned)s);
-    const int kend = min(k0 + C, ctl->last_step);
+    const int kend = min(k0 + C, cget(ctl->last_step));
     if (kend <= k0 || !act[(size_t)(k0 % C) * s + j]) return;
     extern __shared__ __align__(16) unsigned char sc_smem[];
     C2* sU = reinterpret_cast<C2*>(sc_smem);            // [2][NF * NF]
@@ -831,7 +836,7 @@ __global__ void __launch_bounds__(ROWS, (NF <= 12 && PW == P32) ? 4 : 1) shift_c
     const size_t tile = (size_t)M_MAX * M_MAX;
     typename Tr<PW>::S2* Pj = Pb + (size_t)j * m * ldw;
     typename Tr<PW>::S2* Xj = Xb + (size_t)j * m * ldw;
-    int mk_ = ctl->hmk[k0 & (CTL_HIST - 1)];
+    int mk_ = cget(ctl->hmk[k0 & (CTL_HIST - 1)]);
     C2 t[NF], x[NF];
 #pragma unroll
     for (int a = 0; a < NF; ++a) {
@@ -844,7 +849,7 @@ __global__ void __launch_bounds__(ROWS, (NF <= 12 && PW == P32) ? 4 : 1) shift_c
     for (; k <= kend; ++k) {
         const int q = (k - 1) % C;
         if (!act[(size_t)q * s + j]) break;
-        mn = ctl->hmn[(k - 1) & (CTL_HIST - 1)];
+        mn = cget(ctl->hmn[(k - 1) & (CTL_HIST - 1)]);
         // this step's tiles into buffer b; the sync also orders the reads of
         // step k - 2 (same buffer) before the writes
         const int b = (k - k0) & 1;
@@ -976,10 +981,11 @@ __device__ __forceinline__ void ufx_stage(int4* st, int* se, const int4* __restr
 template <int NF>
 __global__ void __launch_bounds__(UFX_ROWS) block_update_fx_kernel(
     double2* __restrict__ W, const double2* __restrict__ Y, const double2* __restrict__ Vk,
-    const double2* __restrict__ Vp, size_t ld, size_t n, const Ctl* __restrict__ ctl, const int4* __restrict__ ca,
+    const double2* __restrict__ Vp, size_t ld, size_t n, const Ctl* ctl, const int4* __restrict__ ca,
     const int4* __restrict__ cb, const int* __restrict__ ce) {
-    if (ctl->done) return;
-    const int mk_ = ctl->mk, mp = (ctl->k > 1) ? ctl->mprev : 0;
+    step_begin();
+    if (cget(ctl->done)) return;
+    const int mk_ = cget(ctl->mk), mp = (cget(ctl->k) > 1) ? cget(ctl->mprev) : 0;
     __shared__ int4 sa[NF * NF], sb[NF * NF];
     __shared__ int ea[NF], eb[NF];
     ufx_stage<NF>(sa, ea, ca, ce);
@@ -1022,10 +1028,11 @@ __global__ void __launch_bounds__(UFX_ROWS) block_update_fx_kernel(
 
 template <int NF>
 __global__ void __launch_bounds__(UFX_ROWS) v_update_fx_kernel(double2* __restrict__ Vn, const double2* __restrict__ W,
-                                                               size_t ld, size_t n, const Ctl* __restrict__ ctl,
+                                                               size_t ld, size_t n, const Ctl* ctl,
                                                                const int4* __restrict__ cS, const int* __restrict__ ce) {
-    if (ctl->done) return;
-    const int mk_ = ctl->mk, mn = ctl->mnext;
+    step_begin();
+    if (cget(ctl->done)) return;
+    const int mk_ = cget(ctl->mk), mn = cget(ctl->mnext);
     __shared__ int4 sS[NF * NF];
     __shared__ int eS[NF];
     ufx_stage<NF>(sS, eS, cS, ce);
@@ -1057,10 +1064,11 @@ __global__ void __launch_bounds__(UFX_ROWS) v_update_fx_kernel(double2* __restri
 template <int NF, int ROWS>
 __global__ void __launch_bounds__(ROWS, NF <= 4 ? 4 : NF <= 8 ? 2 : 1) shift_chunk_fx_kernel(
     const double2* __restrict__ ring, size_t slot_elems, int R, size_t ld, double2* __restrict__ Pb,
-    double2* __restrict__ Xb, size_t ldw, size_t n, int s, int m, Ctl* __restrict__ ctl, int k0, int C,
+    double2* __restrict__ Xb, size_t ldw, size_t n, int s, int m, Ctl* ctl, int k0, int C,
     const int4* __restrict__ cU, const int4* __restrict__ cL, const int* __restrict__ cE, const int* __restrict__ act) {
+    step_begin();
     const int j = (int)(blockIdx.x % (unsigned)s);
-    const int kend = min(k0 + C, ctl->last_step);
+    const int kend = min(k0 + C, cget(ctl->last_step));
     if (kend <= k0 || !act[(size_t)(k0 % C) * s + j]) return;
     extern __shared__ __align__(16) unsigned char sc_smem[];
     int4* sT = reinterpret_cast<int4*>(sc_smem);                 // [2 buffers][U, L][NF * NF]
@@ -1072,7 +1080,7 @@ __global__ void __launch_bounds__(ROWS, NF <= 4 ? 4 : NF <= 8 ? 2 : 1) shift_chu
     const size_t tile = (size_t)M_MAX * M_MAX;
     double2* Pj = Pb + (size_t)j * m * ldw;
     double2* Xj = Xb + (size_t)j * m * ldw;
-    const int mk_ = ctl->hmk[k0 & (CTL_HIST - 1)];
+    const int mk_ = cget(ctl->hmk[k0 & (CTL_HIST - 1)]);
     bool bad = false;
     int4 t[NF];
     int et;
@@ -1088,7 +1096,7 @@ __global__ void __launch_bounds__(ROWS, NF <= 4 ? 4 : NF <= 8 ? 2 : 1) shift_chu
     for (int k = k0 + 1; k <= kend; ++k) {
         const int q = (k - 1) % C;
         if (!act[(size_t)q * s + j]) break;
-        mn = ctl->hmn[(k - 1) & (CTL_HIST - 1)];
+        mn = cget(ctl->hmn[(k - 1) & (CTL_HIST - 1)]);
         // this step's tiles into buffer b (its previous readers, step k - 2, are
         // past the barrier of step k - 1)
         const int b = (k - k0) & 1;
@@ -1175,11 +1183,11 @@ inline int nf_bucket(int nf) { return nf <= 4 ? 4 : nf <= 8 ? 8 : nf <= 12 ? 12 
 
 template <int P>
 void launch_bu_t(void* W, const void* Y, const void* Vk, const void* Vp, size_t ld, size_t n, const Ctl* ctl,
-                 int nf_max, const void* coef_a, const void* coef_bh, const int* ce, float hscale, cudaStream_t st) {
+                 int nf_max, const void* coef_a, const void* coef_bh, const int* ce, float hscale, Stream st) {
     if constexpr (P == P64) {
         if (ce) {
 #define BI_BUFX(NF)                                                                                            \
-    block_update_fx_kernel<NF><<<(unsigned)((n + UFX_ROWS - 1) / UFX_ROWS), UFX_ROWS, 0, st>>>(                 \
+    launch_step(block_update_fx_kernel<NF>, (unsigned)((n + UFX_ROWS - 1) / UFX_ROWS), UFX_ROWS, 0, st, \
         (double2*)W, (const double2*)Y, (const double2*)Vk, (const double2*)Vp, ld, n, ctl, (const int4*)coef_a, \
         (const int4*)coef_bh, ce)
             BI_DISPATCH_FX(nf_max, BI_BUFX)
@@ -1191,7 +1199,7 @@ void launch_bu_t(void* W, const void* Y, const void* Vk, const void* Vp, size_t 
     using C = typename Tr<P>::C;
     int g = (int)((n + 255) / 256);
 #define BI_BU(NF)                                                                                       \
-    block_update_kernel<P, NF><<<g, 256, 0, st>>>((S2*)W, (const S2*)Y, (const S2*)Vk, (const S2*)Vp, ld, n, ctl, \
+    launch_step(block_update_kernel<P, NF>, g, 256, 0, st, (S2*)W, (const S2*)Y, (const S2*)Vk, (const S2*)Vp, ld, n, ctl, \
                                                   (const C*)coef_a, (const C*)coef_bh, hscale)
     BI_DISPATCH_NF(nf_max, BI_BU)
 #undef BI_BU
@@ -1200,7 +1208,7 @@ void launch_bu_t(void* W, const void* Y, const void* Vk, const void* Vp, size_t 
 template <int P>
 void launch_ug_t(void* W, const void* Y, const void* Vk, const void* Vp, size_t ld, size_t n, const Ctl* ctl,
                  int nf_max, const void* coef_a, const void* coef_bh, double* partials, int nblk, float hscale,
-                 cudaStream_t st) {
+                 Stream st) {
     using S2 = typename Tr<P>::S2;
     using C = typename Tr<P>::C;
 #define BI_UG(NF)                                                                                            \
@@ -1208,7 +1216,7 @@ void launch_ug_t(void* W, const void* Y, const void* Vk, const void* Vp, size_t 
         constexpr int SMEM = NF * UG_ROWS * (int)sizeof(S2);                                                 \
         static std::atomic<unsigned long long> devs{0};                                                      \
         max_dyn_smem_once(update_gram_kernel<P, NF>, SMEM, devs);                                            \
-        update_gram_kernel<P, NF><<<nblk, UG_ROWS, SMEM, st>>>((S2*)W, (const S2*)Y, (const S2*)Vk,            \
+        launch_step(update_gram_kernel<P, NF>, nblk, UG_ROWS, SMEM, st, (S2*)W, (const S2*)Y, (const S2*)Vk,            \
                                                                (const S2*)Vp, ld, n, ctl, nf_max, (const C*)coef_a, \
                                                                (const C*)coef_bh, partials, hscale);          \
     }
@@ -1267,13 +1275,14 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <int P, int NF, int ROWS>
 __global__ void __launch_bounds__(ROWS, NF <= 12 ? 4 : 1) shift_chunk32_kernel(
     const typename Tr<P>::S2* __restrict__ ring, size_t slot_elems, int R, size_t ld, float2* __restrict__ Pb,
-    float2* __restrict__ Xb, size_t ldw, size_t n, int s, int m, Ctl* __restrict__ ctl, int k0, int C,
+    float2* __restrict__ Xb, size_t ldw, size_t n, int s, int m, Ctl* ctl, int k0, int C,
     const float2* __restrict__ cU, const float2* __restrict__ cL, const int* __restrict__ act, float hscale) {
+    step_begin();
     static_assert(NF % 2 == 0, "column pairs");
     constexpr int NP = NF / 2;
     using SE = typename Tr<P>::S2;
     const int j = (int)(blockIdx.x % (unsigned)s);
-    const int kend = min(k0 + C, ctl->last_step);
+    const int kend = min(k0 + C, cget(ctl->last_step));
     if (kend <= k0 || !act[(size_t)(k0 % C) * s + j]) return;
     extern __shared__ __align__(16) unsigned char sc_smem[];
     float* sCo = reinterpret_cast<float*>(sc_smem);                           // [2 buffers][U, L][NP][NF][4]
@@ -1295,7 +1304,7 @@ __global__ void __launch_bounds__(ROWS, NF <= 12 ? 4 : 1) shift_chunk32_kernel(
             if (c < m) cp_async_elem<sizeof(SE)>(d + c * ROWS, g + (size_t)c * ld);
         cp_async_commit();
     };
-    int mk_ = ctl->hmk[k0 & (CTL_HIST - 1)];
+    int mk_ = cget(ctl->hmk[k0 & (CTL_HIST - 1)]);
     float2 t[NF];
     float2 xr[NP], xi[NP];
 #pragma unroll
@@ -1324,7 +1333,7 @@ __global__ void __launch_bounds__(ROWS, NF <= 12 ? 4 : 1) shift_chunk32_kernel(
     int mn = mk_;
     for (int k = k0 + 1; k <= kend; ++k) {
         if (!act[(size_t)q * s + j]) break;
-        mn = ctl->hmn[(k - 1) & (CTL_HIST - 1)];
+        mn = cget(ctl->hmn[(k - 1) & (CTL_HIST - 1)]);
         const int b = (k - k0 - 1) & 1;
         const int vs_next = vs + 1 == R ? 0 : vs + 1;
         const bool ahead = k < kend;
@@ -1418,11 +1427,11 @@ __global__ void __launch_bounds__(ROWS, NF <= 12 ? 4 : 1) shift_chunk32_kernel(
 
 template <int P>
 void launch_vu_t(void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl, int nf_max, const void* coefS,
-                 const int* ce, float hscale, cudaStream_t st) {
+                 const int* ce, float hscale, Stream st) {
     if constexpr (P == P64) {
         if (ce) {
 #define BI_VUFX(NF)                                                                                       \
-    v_update_fx_kernel<NF><<<(unsigned)((n + UFX_ROWS - 1) / UFX_ROWS), UFX_ROWS, 0, st>>>(                \
+    launch_step(v_update_fx_kernel<NF>, (unsigned)((n + UFX_ROWS - 1) / UFX_ROWS), UFX_ROWS, 0, st, \
         (double2*)Vnext, (const double2*)W, ld, n, ctl, (const int4*)coefS, ce)
             BI_DISPATCH_FX(nf_max, BI_VUFX)
 #undef BI_VUFX
@@ -1433,7 +1442,7 @@ void launch_vu_t(void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl
     using S2 = typename Tr<P>::S2;
     using CW = typename Tr<PW>::C;
 #define BI_VU(NF)                                                                                           \
-    v_update_kernel<P, NF><<<(unsigned)((n + 255) / 256), 256, 0, st>>>((S2*)Vnext, (const S2*)W, ld, n, ctl, \
+    launch_step(v_update_kernel<P, NF>, (unsigned)((n + 255) / 256), 256, 0, st, (S2*)Vnext, (const S2*)W, ld, n, ctl, \
                                                                        (const CW*)coefS, hscale)
     BI_DISPATCH_NF(nf_max, BI_VU)
 #undef BI_VU
@@ -1442,14 +1451,14 @@ void launch_vu_t(void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl
 template <int P>
 void launch_sc_t(const void* ring, size_t slot_elems, int R, size_t ld, void* Pp, void* X, size_t ldw, size_t n,
                  int s, int m, Ctl* ctl, int nf_max, int k0, int C, const void* coefU, const void* coefL,
-                 const int* ce, const int* active, float hscale, cudaStream_t st) {
+                 const int* ce, const int* active, float hscale, Stream st) {
     if constexpr (P == P64) {
         if (ce) {
 #define BI_SCFX(NF)                                                                                          \
     {                                                                                                        \
         constexpr int ROWS = 128;                                                                            \
         constexpr size_t SMEM = scfx_smem_bytes<NF>();                                                       \
-        shift_chunk_fx_kernel<NF, ROWS><<<(unsigned)(((n + ROWS - 1) / ROWS) * (size_t)s), ROWS, SMEM, st>>>( \
+        launch_step(shift_chunk_fx_kernel<NF, ROWS>, (unsigned)(((n + ROWS - 1) / ROWS) * (size_t)s), ROWS, SMEM, st, \
             (const double2*)ring, slot_elems, R, ld, (double2*)Pp, (double2*)X, ldw, n, s, m, ctl, k0, C,     \
             (const int4*)coefU, (const int4*)coefL, ce, active);                                             \
     }
@@ -1470,14 +1479,14 @@ void launch_sc_t(const void* ring, size_t slot_elems, int R, size_t ld, void* Pp
             constexpr size_t SMEM = sc_smem_bytes<NF, PW>();                                                \
             static std::atomic<unsigned long long> devs{0};                                                 \
             max_dyn_smem_once(shift_chunk_kernel<P, PW, NF, ROWS>, (int)SMEM, devs);                        \
-            shift_chunk_kernel<P, PW, NF, ROWS><<<g, ROWS, SMEM, st>>>(                                      \
+            launch_step(shift_chunk_kernel<P, PW, NF, ROWS>, g, ROWS, SMEM, st, \
                 (const S2*)ring, slot_elems, R, ld, (W2*)Pp, (W2*)X, ldw, n, s, m, ctl, k0, C,              \
                 (const CW*)coefU, (const CW*)coefL, active, hscale);                                        \
         } else {                                                                                            \
             constexpr size_t SMEM = sc32_smem_bytes<NF, P>(ROWS);                                           \
             static std::atomic<unsigned long long> devs{0};                                                 \
             max_dyn_smem_once(shift_chunk32_kernel<P, NF, ROWS>, (int)SMEM, devs);                          \
-            shift_chunk32_kernel<P, NF, ROWS><<<g, ROWS, SMEM, st>>>(                                        \
+            launch_step(shift_chunk32_kernel<P, NF, ROWS>, g, ROWS, SMEM, st, \
                 (const S2*)ring, slot_elems, R, ld, (float2*)Pp, (float2*)X, ldw, n, s, m, ctl, k0, C,      \
                 (const float2*)coefU, (const float2*)coefL, active, hscale);                                \
         }                                                                                                   \
@@ -1488,16 +1497,16 @@ void launch_sc_t(const void* ring, size_t slot_elems, int R, size_t ld, void* Pp
 
 #define BI_INSTANTIATE(P)                                                                                  \
     template void launch_bu_t<P>(void*, const void*, const void*, const void*, size_t, size_t, const Ctl*, int, \
-                                 const void*, const void*, const int*, float, cudaStream_t);              \
+                                 const void*, const void*, const int*, float, Stream);              \
     template void launch_ug_t<P>(void*, const void*, const void*, const void*, size_t, size_t, const Ctl*, int, \
-                                 const void*, const void*, double*, int, float, cudaStream_t);            \
+                                 const void*, const void*, double*, int, float, Stream);            \
     template void launch_ib_t<P>(void*, size_t, const void*, int, size_t, size_t, const double2*, int,       \
                                  const Ctl*, int, float, cudaStream_t);                                    \
     template void launch_vu_t<P>(void*, const void*, size_t, size_t, const Ctl*, int, const void*, const int*, \
-                                 float, cudaStream_t);                                                     \
+                                 float, Stream);                                                     \
     template void launch_sc_t<P>(const void*, size_t, int, size_t, void*, void*, size_t, size_t, int, int,   \
                                  Ctl*, int, int, int, const void*, const void*, const int*, const int*, float, \
-                                 cudaStream_t);
+                                 Stream);
 
 }  // namespace blas_impl
 }  // namespace dsbcg

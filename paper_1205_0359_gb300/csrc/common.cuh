@@ -51,6 +51,43 @@ inline void max_dyn_smem_once(F* func, int bytes, std::atomic<unsigned long long
     devs.fetch_or(bit);
 }
 
+// A stream and how the kernels of a block step follow one another on it.
+// ahead: the next kernel is launched programmatically, so that its CTAs start
+// (launch latency, block scheduling) while the last CTAs of the one before
+// still run; every such kernel begins with step_begin(), which waits until all
+// earlier work of the stream is complete and visible, and lets the next kernel
+// in only after that wait, so at most one kernel per stream is ahead.
+struct Stream {
+    cudaStream_t st;
+    bool ahead;
+    Stream(cudaStream_t s, bool a = false) : st(s), ahead(a) {}
+    operator cudaStream_t() const { return st; }
+};
+template <class... KA, class... A>
+inline void launch_step(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, Stream st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st.st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = st.ahead ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
+}
+__device__ __forceinline__ void step_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// A word of the control block, from L2: the kernel before may have read the
+// block on this SM before its last CTA wrote it.
+template <class T>
+__device__ __forceinline__ T cget(const T& v) {
+    return __ldcg(&v);
+}
+
 constexpr int M_MAX = 32;      // largest block width (right-hand sides in a block)
 constexpr int CTL_HIST = 16;   // block widths kept per step (the longest shift-update chunk)
 constexpr int S_MAX = 64;      // largest number of shifts

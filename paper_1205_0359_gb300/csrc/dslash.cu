@@ -217,14 +217,14 @@ __global__ void __launch_bounds__(32, (P == PDD || P == P64) ? 12 : 24) dslash_k
                                                    const typename Tr<P>::S2* __restrict__ in,
                                                    size_t ld, const typename Tr<P>::S2* __restrict__ links,
                                                    Geom g, typename Tr<P>::R kappa, int g5in, int g5out,
-                                                   const Ctl* __restrict__ ctl, int nf_static, float hscale,
+                                                   const Ctl* ctl, int nf_static, float hscale,
                                                    int nfg) {
     using C = typename Tr<P>::C;
     using R = typename Tr<P>::R;
     int nf = nf_static;
     if (ctl) {
-        if (ctl->done) return;
-        nf = ctl->mk;
+        if (cget(ctl->done)) return;
+        nf = cget(ctl->mk);
     }
     // 1D work index: block b covers field b % nfg of site tile b / nfg
     // (fields fastest); a grid smaller than the work strides over it
@@ -411,14 +411,15 @@ template <int P, bool L12, bool DAG, bool HALF>
 __global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kernel(
     typename Tr<P>::S2* __restrict__ out, const typename Tr<P>::S2* __restrict__ in,
     const typename Tr<P>::S2* __restrict__ src, size_t ld, const typename Tr<P>::S2* __restrict__ links, Geom g,
-    float alpha, float beta, int parity, const Ctl* __restrict__ ctl, int nf_static, int ngrp) {
+    float alpha, float beta, int parity, const Ctl* ctl, int nf_static, int ngrp) {
+    step_begin();
     // [hop][entry][site of the tile]: rows 0 and 1 of SU(3) links (L12), with
     // row 2 rebuilt at each use, else all nine entries
     __shared__ float2 sl[8][L12 ? 6 : 9][32];
     int nf = nf_static;
     if (ctl) {
-        if (ctl->done) return;
-        nf = ctl->mk;
+        if (cget(ctl->done)) return;
+        nf = cget(ctl->mk);
     }
     const int grp = (int)(blockIdx.x % (unsigned)ngrp);
     if (grp * CTA_FIELDS >= nf) return;      // CTA-uniform
@@ -547,14 +548,14 @@ template <int P>
 __global__ void __launch_bounds__(32, (P == PDD || P == P64) ? 12 : 24) dslash_half_kernel(
     typename Tr<P>::S2* __restrict__ out, const typename Tr<P>::S2* __restrict__ in,
     const typename Tr<P>::S2* __restrict__ src, size_t ld, const typename Tr<P>::S2* __restrict__ links, Geom g,
-    typename Tr<P>::R alpha, typename Tr<P>::R beta, int parity, int g5in, int g5out, const Ctl* __restrict__ ctl,
+    typename Tr<P>::R alpha, typename Tr<P>::R beta, int parity, int g5in, int g5out, const Ctl* ctl,
     int nf_static, float hscale, int nfg) {
     using C = typename Tr<P>::C;
     using R = typename Tr<P>::R;
     int nf = nf_static;
     if (ctl) {
-        if (ctl->done) return;
-        nf = ctl->mk;
+        if (cget(ctl->done)) return;
+        nf = cget(ctl->mk);
     }
     const int f = (int)(blockIdx.x % (unsigned)nfg);
     if (f >= nf) return;
@@ -661,7 +662,7 @@ __global__ void __launch_bounds__(32, (P == PDD || P == P64) ? 12 : 24) dslash_h
 
 void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* links, const Geom& g,
                    double kappa, int dag, const Ctl* ctl, int nf_static, int nf_max, float hscale,
-                   cudaStream_t st, const void* links12, int max_ctas) {
+                   Stream st, const void* links12, int max_ctas) {
     // D^H = gamma_5 D gamma_5: gamma_5 on the input and on the output
     const int g5in = dag, g5out = dag;
     // one CTA per (field, 32-site tile); with a control block the width is
@@ -682,7 +683,7 @@ void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* l
     dim3 cgrid((unsigned)(ngrp * ((g.V + 31) / 32)));
     dim3 cblock(32 * CTA_FIELDS);
 #define DSBCG_CTA_LAUNCH2(PP, S2T, L12, DAG)                                                                    \
-    dslash_cta_kernel<PP, L12, DAG, false><<<cgrid, cblock, 0, st>>>(                                            \
+    launch_step(dslash_cta_kernel<PP, L12, DAG, false>, cgrid, cblock, 0, st,                                             \
         (S2T*)out, (const S2T*)in, nullptr, ld, (const S2T*)(L12 ? links12 : links), g, 1.f, -(float)kappa, 0,    \
         ctl, nf_static, ngrp)
 #define DSBCG_CTA_LAUNCH(PP, S2T)                                                                               \
@@ -715,7 +716,7 @@ void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* l
 
 void launch_dslash_half(int prec, void* out, const void* in, const void* src, size_t ld, const void* links,
                         const Geom& g, double alpha, double beta, int parity, int g5in, int g5out, const Ctl* ctl,
-                        int nf_static, int nf_max, float hscale, cudaStream_t st) {
+                        int nf_static, int nf_max, float hscale, Stream st) {
     const int nfg = ctl ? nf_max : nf_static;
     const int nf_grid = nfg < 1 ? 1 : nfg;
     dim3 block(32);
@@ -727,7 +728,7 @@ void launch_dslash_half(int prec, void* out, const void* in, const void* src, si
     // FP32 and 16-bit fields: gamma_5 on the input of the first pass and on the
     // output of the second (dag) is gamma_5 H gamma_5 in both
 #define DSBCG_HALF_CTA2(PP, S2T, DAG)                                                                          \
-    dslash_cta_kernel<PP, false, DAG, true><<<cgrid, cblock, 0, st>>>((S2T*)out, (const S2T*)in, (const S2T*)src, ld, \
+    launch_step(dslash_cta_kernel<PP, false, DAG, true>, cgrid, cblock, 0, st, (S2T*)out, (const S2T*)in, (const S2T*)src, ld, \
                                                                       (const S2T*)links, g, (float)alpha,        \
                                                                       (float)beta, parity, ctl, nf_static, ngrp)
 #define DSBCG_HALF_CTA(PP, S2T)                                                                                \

@@ -51,12 +51,13 @@ __device__ __forceinline__ size_t fx_at(int y) { return (size_t)(y >> 5) * FX_TI
 // thread per (site, field).  Bound by HBM: 16 bytes per complex in and out.
 __global__ void __launch_bounds__(128) fx_convert_kernel(int4* __restrict__ out, int* __restrict__ eo,
                                                          const double2* __restrict__ in, size_t ld, int V,
-                                                         const Ctl* __restrict__ ctl, int nf_static,
+                                                         const Ctl* ctl, int nf_static,
                                                          int* __restrict__ flag) {
+    step_begin();
     int nf = nf_static;
     if (ctl) {
-        if (ctl->done) return;
-        nf = ctl->mk;
+        if (cget(ctl->done)) return;
+        nf = cget(ctl->mk);
     }
     const int x = (int)(blockIdx.x * 128u + threadIdx.x), f = (int)blockIdx.y;
     if (f >= nf || x >= V) return;
@@ -226,15 +227,16 @@ template <bool DAG, bool OUT64, bool HALF>
 __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
     void* __restrict__ outv, int* __restrict__ eo, const int4* __restrict__ in, const int* __restrict__ ei,
     const int4* __restrict__ src, const int* __restrict__ es, size_t ld, const int4* __restrict__ links, Geom g,
-    int kshift, int neg, int parity, const Ctl* __restrict__ ctl, int nf_static, int ngrp) {
+    int kshift, int neg, int parity, const Ctl* ctl, int nf_static, int ngrp) {
+    step_begin();
     extern __shared__ __align__(16) unsigned char fx_smem[];
     int4* sl = reinterpret_cast<int4*>(fx_smem);               // [hop][entry][lane]
     ll2* ex = reinterpret_cast<ll2*>(sl + 8 * 9 * 32);         // [warp][colour][lane]
     int* sy = reinterpret_cast<int*>(ex + 2 * FX_FIELDS * 3 * 32);     // [hop][lane]
     int nf = nf_static;
     if (ctl) {
-        if (ctl->done) return;
-        nf = ctl->mk;
+        if (cget(ctl->done)) return;
+        nf = cget(ctl->mk);
     }
     const int nw = (int)(blockDim.x >> 5), nfc = nw >> 1;      // warps, fields of the CTA
     const int grp = (int)(blockIdx.x % (unsigned)ngrp);
@@ -403,15 +405,15 @@ void launch_fx_links(void* dst, const double2* src, size_t V, double kappa, cuda
 }
 
 void launch_fx_convert(void* out, int* eo, const void* in, size_t ld, size_t Vf, const Ctl* ctl, int nf_static,
-                       int nf_max, int* flag, cudaStream_t st) {
+                       int nf_max, int* flag, Stream st) {
     const int nfg = ctl ? nf_max : nf_static;
     const dim3 grid((unsigned)((Vf + 127) / 128), (unsigned)nfg);
-    fx_convert_kernel<<<grid, 128, 0, st>>>((int4*)out, eo, (const double2*)in, ld, (int)Vf, ctl, nf_static, flag);
+    launch_step(fx_convert_kernel, grid, 128, 0, st, (int4*)out, eo, (const double2*)in, ld, (int)Vf, ctl, nf_static, flag);
 }
 
 void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const void* src, const int* es, size_t ld,
                        const void* links, const Geom& g, double kappa, int dag, int half, int parity, int out64,
-                       const Ctl* ctl, int nf_static, int nf_max, cudaStream_t st) {
+                       const Ctl* ctl, int nf_static, int nf_max, Stream st) {
     const int nfg = ctl ? nf_max : nf_static;
     const int nfc = nfg < FX_FIELDS ? nfg : FX_FIELDS;
     const int ngrp = (nfg + nfc - 1) / nfc;
@@ -425,7 +427,7 @@ void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const 
     {                                                                                                              \
         static std::atomic<unsigned long long> devs{0};                                                            \
         max_dyn_smem_once(fx_stencil_kernel<DAG, O64, HALF>, SMEM, devs);                                          \
-        fx_stencil_kernel<DAG, O64, HALF><<<grid, 64 * nfc, SMEM, st>>>(out, eo, (const int4*)in, ei,               \
+        launch_step(fx_stencil_kernel<DAG, O64, HALF>, grid, 64 * nfc, SMEM, st, out, eo, (const int4*)in, ei,               \
                                                                         (const int4*)src, es, ld, (const int4*)links, \
                                                                         g, ks, neg, parity, ctl, nf_static, ngrp);   \
     }

@@ -72,7 +72,7 @@ void launch_dot_re_blocks(const double2* a, const double2* b, int s, size_t cnt,
 // layout of launch_pack_links12, used instead of `links` when given
 void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* links,
                    const Geom& g, double kappa, int dag, const Ctl* ctl,
-                   int nf_static, int nf_max, float hscale, cudaStream_t st,
+                   int nf_static, int nf_max, float hscale, Stream st,
                    const void* links12 = nullptr, int max_ctas = 0);
 
 // Half-lattice hopping term of the even-odd operator (every extent even; half
@@ -84,7 +84,7 @@ void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* l
 // D^H (g5in, then g5out) compose to the same.
 void launch_dslash_half(int prec, void* out, const void* in, const void* src, size_t ld, const void* links,
                         const Geom& g, double alpha, double beta, int parity, int g5in, int g5out, const Ctl* ctl,
-                        int nf_static, int nf_max, float hscale, cudaStream_t st);
+                        int nf_static, int nf_max, float hscale, Stream st);
 
 // ---- dslash_fx.cu: FP64 fields in block fixed point (links in SU(3)) ----------
 // an FX field block takes the bytes of an FP64 one (stride ld complex, a
@@ -94,13 +94,13 @@ bool fx_kappa_fits(double kappa);            // the hopping coefficient's expone
 void launch_fx_links(void* dst, const double2* src, size_t V, double kappa, cudaStream_t st);
 // FP64 fields (internal layout, Vf sites) -> FX; *flag |= 1 where the FX range does not hold (flag may be NULL)
 void launch_fx_convert(void* out, int* eo, const void* in, size_t ld, size_t Vf, const Ctl* ctl, int nf_static,
-                       int nf_max, int* flag, cudaStream_t st);
+                       int nf_max, int* flag, Stream st);
 // out = src - kappa H in (dag: gamma_5 H gamma_5), or kappa H in when src is
 // NULL.  Full lattice (half = 0) or half fields on `parity`; out64: FP64
 // output, else FX
 void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const void* src, const int* es, size_t ld,
                        const void* links, const Geom& g, double kappa, int dag, int half, int parity, int out64,
-                       const Ctl* ctl, int nf_static, int nf_max, cudaStream_t st);
+                       const Ctl* ctl, int nf_static, int nf_max, Stream st);
 
 // ---- blas.cu ----------------------------------------------------------------
 int gram_blocks(size_t n, int nf_max);
@@ -112,7 +112,7 @@ int gram_blocks(size_t n, int nf_max);
 // (copies drained, ST_WAIT_TIMEOUT in ctl->status, NaN partials)
 void launch_gram(int prec, const void* X, const void* Y, size_t ld, size_t n, const Ctl* ctl,
                  int nf_static, int nf_max, int herm, int diag_yy, double* partials, int nblk,
-                 float hscale, cudaStream_t st, int first_wait = -1);
+                 float hscale, Stream st, int first_wait = -1);
 size_t gram_partial_doubles(int nf_max);
 // reduce partials -> G (FP64, M_MAX x M_MAX, complex), diag (M_MAX)
 void launch_gram_reduce(const double* partials, int nblk, int nf_max, int herm, int diag_yy,
@@ -126,7 +126,7 @@ inline bool coef_fx(int prec, int m) { return prec == P64 && m <= 12; }
 // ce: exponents of a, then of b^H)
 void launch_block_update(int prec, void* W, const void* Y, const void* Vk, const void* Vp,
                          size_t ld, size_t n, const Ctl* ctl, int nf_max,
-                         const void* coef_a, const void* coef_bh, const int* ce, float hscale, cudaStream_t st);
+                         const void* coef_a, const void* coef_bh, const int* ce, float hscale, Stream st);
 // Block update fused with the Gram of its result: W as launch_block_update,
 // and W^H W (hermitian, upper 4 x 4 tiles, no diagonal norms) as partials of
 // nblk blocks in the Gram kernel's layout.  Reduced storages and block widths
@@ -134,7 +134,7 @@ void launch_block_update(int prec, void* W, const void* Y, const void* Vk, const
 bool update_gram_fits(int prec, int nf_max);
 void launch_update_gram(int prec, void* W, const void* Y, const void* Vk, const void* Vp, size_t ld, size_t n,
                         const Ctl* ctl, int nf_max, const void* coef_a, const void* coef_bh, double* partials,
-                        int nblk, float hscale, cudaStream_t st);
+                        int nblk, float hscale, Stream st);
 // V1 = B S (B in precision bprec: FP64, or FP32 for reduced storage;
 // storage-precision V1), S from the device m x m state (M_MAX x M_MAX, FP64,
 // or double-float when s_dd)
@@ -142,7 +142,7 @@ void launch_init_basis(int prec, void* V1, size_t ldv, const void* B, int bprec,
                        const double2* S, int s_dd, const Ctl* ctl, int nf_in, float hscale, cudaStream_t st);
 // V_{k+1} = W S (S from the step's QR, M_MAX-strided work-precision tile)
 void launch_v_update(int prec, void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl, int nf_max,
-                     const void* coefS, const int* ce, float hscale, cudaStream_t st);
+                     const void* coefS, const int* ce, float hscale, Stream st);
 // shift update (the per-shift short recurrences, Sec. 3) over the block
 // steps k0+1 .. min(k0 + C, last executed step): for every step in which
 // shift j is active, X_j += P_j Ut_j and P_j <- V_{k+1} - P_j LhT_j, with P_j
@@ -155,7 +155,7 @@ void launch_v_update(int prec, void* Vnext, const void* W, size_t ld, size_t n, 
 void launch_shift_chunk(int prec, const void* ring, size_t slot_elems, int R, size_t ld, void* P, void* X,
                         size_t ldw, size_t n, int s, int m, Ctl* ctl, int nf_max, int k0, int C, const void* coefU,
                         const void* coefL, const int* ce, const int* active, float hscale,
-                        cudaStream_t st);
+                        Stream st);
 
 // ---- small.cu ---------------------------------------------------------------
 struct SmallState;     // device m x m state (FP64 or double-float), defined in small.cu
@@ -166,14 +166,14 @@ void launch_small_init(SmallState* ss, Ctl* ctl, const double2* G0, const double
                        int sfp64, cudaStream_t st);
 // alpha_k from the Gram partials of V_k^H Y (+ coefficient tiles for the block update)
 void launch_small_alpha(SmallState* ss, const Ctl* ctl, const double* partials, int nblk, int nf_max,
-                        int wprec, int sfp64, void* coef_a, void* coef_bh, int* ce, cudaStream_t st);
+                        int wprec, int sfp64, void* coef_a, void* coef_bh, int* ce, Stream st);
 // W^H W from the Gram partials, pivoted QR with deflation: S, beta_{k+1}, m_{k+1}
 void launch_small_qr(SmallState* ss, Ctl* ctl, const double* partials, int nblk, int m, double dtol, int wprec,
-                     int sfp64, void* coefS_w, int* ce, cudaStream_t st);
+                     int sfp64, void* coefS_w, int* ce, Stream st);
 // per-shift recurrences (a CTA per shift) and the close of the block step
 void launch_small_recur(SmallState* ss, Ctl* ctl, int s, int m, const double* sigma_dev, const double* target_dev,
                         int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* ce, int* active,
-                        int* conv_step, double* res_out, cudaStream_t st);
+                        int* conv_step, double* res_out, Stream st);
 const double2* small_state_S(const SmallState* ss);
 
 // ---- force.cu ---------------------------------------------------------------

@@ -663,19 +663,20 @@ __global__ void small_init_kernel(SmallStateT<T>* ss, Ctl* ctl, const double2* _
 // coef_bh = beta_k^H in the work precision (M_MAX tiles); ||y_i||^2.  NRC
 // CTAs reduce, the last one to arrive forms the result.
 template <class T>
-__global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, const Ctl* __restrict__ ctl,
+__global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, const Ctl* ctl,
                                                          const double* __restrict__ part, int nblk, int nf_max,
                                                          int wprec, void* coef_a, void* coef_bh, int* ce) {
+    step_begin();
     using S = Sc<T>;
     using R = typename S::R;
-    if (ctl->done) return;
+    if (cget(ctl->done)) return;
     R* red = reinterpret_cast<R*>(ss->sh.red);
     if (!reduce_partials<T>(part, nblk, nf_max, red, &ss->sh.ticket[0], wprec == P64)) return;
     __shared__ T A[M_MAX * M_MAX];
     __shared__ R yy[M_MAX];
     reduce_combine<T>(red, nf_max, A, M_MAX, yy);
     __syncthreads();
-    const int mk_ = ctl->mk, mp = ctl->k > 1 ? ctl->mprev : 0;
+    const int mk_ = cget(ctl->mk), mp = cget(ctl->k) > 1 ? cget(ctl->mprev) : 0;
     const R half = S::r(0.5);
     for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) {
         int i = t / M_MAX, j = t % M_MAX;
@@ -713,9 +714,10 @@ __global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, con
 template <class T>
 __global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* __restrict__ part,
                                                       int nblk, int m, double dtol, int wprec, void* coefS_w, int* ce, int MM) {
+    step_begin();
     using S = Sc<T>;
     using R = typename S::R;
-    if (ctl->done) return;
+    if (cget(ctl->done)) return;
     R* red = reinterpret_cast<R*>(ss->sh.red);
     if (!reduce_partials<T>(part, nblk, m, red, &ss->sh.ticket[1], wprec == P64)) return;
     extern __shared__ __align__(16) unsigned char sm[];
@@ -729,7 +731,7 @@ __global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* c
     R* rf = dd_ + MM;
     R* irp = rf + MM;
     int* perm = (int*)(irp + MM);
-    const int mk_ = ctl->mk;
+    const int mk_ = cget(ctl->mk);
     reduce_combine<T>(red, m, G, MM, nullptr);
     const R* yys = reinterpret_cast<const R*>(ss->sh.yy);
     for (int i = threadIdx.x; i < mk_; i += blockDim.x) rf[i] = yys[i];
@@ -754,7 +756,7 @@ __global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* c
     if (!fx) st_mat_work<T>(wprec, coefS_w, Sm, MM, mk_, mn);
     if (threadIdx.x == 0) {
         ctl->mnext = mn;
-        ctl->deflations += mk_ - mn;
+        ctl->deflations = cget(ctl->deflations) + mk_ - mn;
     }
 }
 
@@ -781,7 +783,7 @@ __device__ void shift_recurrence(SmallStateT<T>* ss, Ctl* ctl, int j, int m, con
     T* col = Bk + MM * MM;
     R* res = (R*)(col + MM);
     R* inv = res + MM;
-    const int k = ctl->k, mk_ = ctl->mk, mp = k > 1 ? ctl->mprev : 0, mn = ctl->mnext;
+    const int k = cget(ctl->k), mk_ = cget(ctl->mk), mp = k > 1 ? cget(ctl->mprev) : 0, mn = cget(ctl->mnext);
     const size_t tile = (size_t)M_MAX * M_MAX;
     const size_t cb = wprec == P64 ? 16 : 8;
     // Delta_k = alpha_k + sigma I - Lambda_k beta_k^H
@@ -879,7 +881,8 @@ __global__ void __launch_bounds__(NT) small_recur_kernel(SmallStateT<T>* ss, Ctl
                                                          const double* __restrict__ target, int freeze, int wprec,
                                                          void* coefU_w, void* coefL_w, int* ce, int* active,
                                                          int* conv_step, double* res_out, int MM) {
-    if (ctl->done) return;
+    step_begin();
+    if (cget(ctl->done)) return;
     extern __shared__ __align__(16) unsigned char sm[];
     shift_recurrence<T>(ss, ctl, (int)blockIdx.x, m, sigma, target, freeze, wprec, coefU_w, coefL_w, ce, active,
                         conv_step, res_out, MM, sm);
@@ -887,21 +890,24 @@ __global__ void __launch_bounds__(NT) small_recur_kernel(SmallStateT<T>* ss, Ctl
     const int j = threadIdx.x;                     // s <= S_MAX shifts
     const int nalive = __syncthreads_count(j < s && __ldcg(&ss->sf[j < s ? j : 0].alive));
     const int nkd = __syncthreads_count(j < s && __ldcg(&active[j < s ? j : 0]));
-    const int mk_ = ctl->mk, mn = ctl->mnext, mp = ctl->k > 1 ? ctl->mprev : 0;
+    const int mk_ = cget(ctl->mk), mn = cget(ctl->mnext), mp = cget(ctl->k) > 1 ? cget(ctl->mprev) : 0;
     for (int t = threadIdx.x; t < M_MAX * M_MAX; t += blockDim.x) ss->sh.betak[t] = ss->sh.betan[t];
     __syncthreads();
     if (threadIdx.x == 0) {
-        ctl->mvms += mk_;
-        ctl->f_dslash += 4LL * mk_;                 // D: V in, Z out; D^H: Z in, Y out
-        ctl->f_gram += 3LL * mk_;                   // V, Y for alpha; W for W^H W
-        ctl->f_update += 3LL * mk_ + mp + mk_ + mn; // Y, V_k, V_{k-1} in, W out; V_{k+1} = W S
-        if (nkd > 0) ctl->f_shift_s += mn;          // V_{k+1} rows, read once per row tile
-        ctl->f_shift_cmac += (long long)nkd * mk_ * (m + mn);   // X_j += P_j Ut_j, P_j <- V - P_j Lh_j
-        ctl->hmk[(ctl->k - 1) & (CTL_HIST - 1)] = mk_;
-        ctl->hmn[(ctl->k - 1) & (CTL_HIST - 1)] = mn;
-        ctl->last_step = ctl->k;
+        const int k = cget(ctl->k);
+        ctl->mvms = cget(ctl->mvms) + mk_;
+        ctl->f_dslash = cget(ctl->f_dslash) + 4LL * mk_;                 // D: V in, Z out; D^H: Z in, Y out
+        ctl->f_gram = cget(ctl->f_gram) + 3LL * mk_;                     // V, Y for alpha; W for W^H W
+        // Y, V_k, V_{k-1} in, W out; V_{k+1} = W S
+        ctl->f_update = cget(ctl->f_update) + 3LL * mk_ + mp + mk_ + mn;
+        if (nkd > 0) ctl->f_shift_s = cget(ctl->f_shift_s) + mn;         // V_{k+1} rows, read once per row tile
+        // X_j += P_j Ut_j, P_j <- V - P_j Lh_j
+        ctl->f_shift_cmac = cget(ctl->f_shift_cmac) + (long long)nkd * mk_ * (m + mn);
+        ctl->hmk[(k - 1) & (CTL_HIST - 1)] = mk_;
+        ctl->hmn[(k - 1) & (CTL_HIST - 1)] = mn;
+        ctl->last_step = k;
         ctl->nact = nalive;
-        ctl->k += 1;
+        ctl->k = k + 1;
         ctl->mprev = mk_;
         ctl->mk = mn;
         if (mn == 0 || nalive == 0 || __ldcg(&ctl->status) != 0) ctl->done = 1;
@@ -935,41 +941,41 @@ void launch_small_init(SmallState* ss, Ctl* ctl, const double2* G0, const double
 }
 
 void launch_small_alpha(SmallState* ss, const Ctl* ctl, const double* partials, int nblk, int nf_max, int wprec,
-                        int sfp64, void* coef_a, void* coef_bh, int* ce, cudaStream_t st) {
+                        int sfp64, void* coef_a, void* coef_bh, int* ce, Stream st) {
     if (sfp64)
-        small_alpha_kernel<double2><<<NRC, NT, 0, st>>>(as_state<double2>(ss), ctl, partials, nblk, nf_max, wprec,
+        launch_step(small_alpha_kernel<double2>, NRC, NT, 0, st, as_state<double2>(ss), ctl, partials, nblk, nf_max, wprec,
                                                         coef_a, coef_bh, ce);
     else
-        small_alpha_kernel<ddc><<<NRC, NT, 0, st>>>(as_state<ddc>(ss), ctl, partials, nblk, nf_max, wprec, coef_a,
+        launch_step(small_alpha_kernel<ddc>, NRC, NT, 0, st, as_state<ddc>(ss), ctl, partials, nblk, nf_max, wprec, coef_a,
                                                     coef_bh, ce);
 }
 
 void launch_small_qr(SmallState* ss, Ctl* ctl, const double* partials, int nblk, int m, double dtol, int wprec,
-                     int sfp64, void* coefS_w, int* ce, cudaStream_t st) {
+                     int sfp64, void* coefS_w, int* ce, Stream st) {
     static std::atomic<unsigned long long> devs64{0}, devsdd{0};
     max_dyn_smem_once(small_qr_kernel<double2>, (int)qr_smem(M_MAX), devs64);
     max_dyn_smem_once(small_qr_kernel<ddc>, (int)qr_smem(M_MAX), devsdd);
     // matrices at the initial width m, which block widths never exceed
     if (sfp64)
-        small_qr_kernel<double2><<<NRC, NT, qr_smem(m), st>>>(as_state<double2>(ss), ctl, partials, nblk, m, dtol,
+        launch_step(small_qr_kernel<double2>, NRC, NT, qr_smem(m), st, as_state<double2>(ss), ctl, partials, nblk, m, dtol,
                                                               wprec, coefS_w, ce, m);
     else
-        small_qr_kernel<ddc><<<NRC, NT, qr_smem(m), st>>>(as_state<ddc>(ss), ctl, partials, nblk, m, dtol, wprec,
+        launch_step(small_qr_kernel<ddc>, NRC, NT, qr_smem(m), st, as_state<ddc>(ss), ctl, partials, nblk, m, dtol, wprec,
                                                           coefS_w, ce, m);
 }
 
 void launch_small_recur(SmallState* ss, Ctl* ctl, int s, int m, const double* sigma_dev, const double* target_dev,
                         int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* ce, int* active,
-                        int* conv_step, double* res_out, cudaStream_t st) {
+                        int* conv_step, double* res_out, Stream st) {
     static std::atomic<unsigned long long> devs64{0}, devsdd{0};
     max_dyn_smem_once(small_recur_kernel<double2>, (int)recur_smem(M_MAX), devs64);
     max_dyn_smem_once(small_recur_kernel<ddc>, (int)recur_smem(M_MAX), devsdd);
     if (sfp64)
-        small_recur_kernel<double2><<<s, NT, recur_smem(m), st>>>(as_state<double2>(ss), ctl, s, m, sigma_dev,
+        launch_step(small_recur_kernel<double2>, s, NT, recur_smem(m), st, as_state<double2>(ss), ctl, s, m, sigma_dev,
                                                                   target_dev, freeze, wprec, coefU_w, coefL_w, ce, active,
                                                                   conv_step, res_out, m);
     else
-        small_recur_kernel<ddc><<<s, NT, recur_smem(m), st>>>(as_state<ddc>(ss), ctl, s, m, sigma_dev, target_dev,
+        launch_step(small_recur_kernel<ddc>, s, NT, recur_smem(m), st, as_state<ddc>(ss), ctl, s, m, sigma_dev, target_dev,
                                                               freeze, wprec, coefU_w, coefL_w, ce, active, conv_step,
                                                               res_out, m);
 }

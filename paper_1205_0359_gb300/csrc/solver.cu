@@ -673,7 +673,7 @@ void unpack_any(dsbcg_ctx* c, int p, double2* dst, const void* src, int m, cudaS
 // Dhat = 1 - kappa^2 H_oe H_eo, Dhat^H = gamma_5 Dhat gamma_5; tmp receives
 // the even-parity H_eo (gamma_5) in.  Two half-lattice passes.
 void apply_dhat(dsbcg_ctx* c, int p, void* out, const void* in, void* tmp, size_t ld, int dag, const Ctl* ctl,
-                int nf_static, int nf_max, float hs, cudaStream_t st, int cls) {
+                int nf_static, int nf_max, float hs, Stream st, int cls) {
     {
         Prof q(c, cls, 1, st);
         launch_dslash_half(p, tmp, in, nullptr, ld, c->links[p], c->g, 0.0, 1.0, 0, dag, 0, ctl, nf_static, nf_max,
@@ -718,7 +718,7 @@ int residual_ctas(dsbcg_ctx* c) {
 // intermediate fields stay in fixed point and the last pass writes FP64.
 // flag: see launch_fx_convert.
 void apply_op(dsbcg_ctx* c, int p, void* out, void* mid, const void* in, void* tmp, size_t ld, const Ctl* ctl,
-              int nf_static, int nf_max, float hs, cudaStream_t st, int cls, int* fxe = nullptr,
+              int nf_static, int nf_max, float hs, Stream st, int cls, int* fxe = nullptr,
               int* flag = nullptr) {
     if (p == P64 && fxe && c->linksfx) {
         int *e0 = fxe, *e1 = fxe + (size_t)(ctl ? nf_max : nf_static) * c->Vf;
@@ -891,12 +891,22 @@ dsbcg_status lane_start(dsbcg_ctx* c, Lane& L, const void* rhs, int rhs_prec, si
     return DSBCG_OK;
 }
 
+// Block steps of fewer than AHEAD_MAX sites x columns (of the full lattice) are
+// bound by launch and m x m latency: their kernels are launched ahead (Stream).
+// Above it the waiting CTAs hold slots that the running kernels of this and the
+// other lanes would use.  ms per solve, plain / ahead: fp64 4^4 m=4 (1 k) 9.1 /
+// 7.5, rational step 8^3 x 16 m=2 (16 k) 26.3 / 23.1, gradient 7x9x10x13 m=5
+// (41 k) 25.4 / 22.4; Schur 12^3 x 24 m=6 (249 k) 19.6 / 20.2, fp64 16^4 m=4 (262
+// k) 119 / 133, fp32 16^3 x 32 m=12 (1.6 M) 244 / 250.
+constexpr size_t AHEAD_MAX = (size_t)1 << 17;
+bool steps_ahead(const dsbcg_ctx* c, int m) { return !c->profiling && c->V * m < AHEAD_MAX; }
+
 dsbcg_status lane_enqueue(dsbcg_ctx* c, Lane& L) {
     const int prec = L.prec, wp = work_prec(prec), m_in = L.m_in, s_in = L.s_in;
     const size_t ld = c->ld, n = c->n;
     const size_t fb = prec_elem_bytes(prec) * ld;
     const size_t cb = (wp == P64 ? 16 : 8) * (size_t)M_MAX * M_MAX;    // one coefficient tile
-    cudaStream_t st = L.st;
+    const Stream st(L.st, steps_ahead(c, m_in));
     char* ring = (char*)L.vring;
     const int C = L.chunk_used, R = C + 1;
     int* const ce = coef_fx(prec, m_in) ? L.ce : nullptr;
