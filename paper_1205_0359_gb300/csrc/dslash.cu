@@ -411,18 +411,23 @@ template <int P, bool L12, bool DAG, bool HALF>
 __global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kernel(
     typename Tr<P>::S2* __restrict__ out, const typename Tr<P>::S2* __restrict__ in,
     const typename Tr<P>::S2* __restrict__ src, size_t ld, const typename Tr<P>::S2* __restrict__ links, Geom g,
-    float alpha, float beta, int parity, const Ctl* ctl, int nf_static, int ngrp) {
-    step_begin();
+    float alpha, float beta, int parity, const Ctl* ctl, int nf_static, int ngrp, int ahead) {
+    // launched ahead: the links, which no kernel of a solve writes, are staged
+    // before the wait for the kernel that writes the fields
+    if (!ahead) step_begin();
     // [hop][entry][site of the tile]: rows 0 and 1 of SU(3) links (L12), with
     // row 2 rebuilt at each use, else all nine entries
     __shared__ float2 sl[8][L12 ? 6 : 9][32];
     int nf = nf_static;
-    if (ctl) {
-        if (cget(ctl->done)) return;
-        nf = cget(ctl->mk);
-    }
     const int grp = (int)(blockIdx.x % (unsigned)ngrp);
-    if (grp * CTA_FIELDS >= nf) return;      // CTA-uniform
+    auto idle = [&]() {                      // CTA-uniform
+        if (ctl) {
+            if (cget(ctl->done)) return true;
+            nf = cget(ctl->mk);
+        }
+        return grp * CTA_FIELDS >= nf;
+    };
+    if (!ahead && idle()) return;
     const int tile = (int)(blockIdx.x / (unsigned)ngrp);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const size_t V = (size_t)g.V;
@@ -447,6 +452,10 @@ __global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kern
         const typename Tr<P>::S2* u = links + (size_t)mu * NE * V + site;
 #pragma unroll
         for (int e = 0; e < NE; ++e) sl[h][e][lane] = ld_link<P>(u + (size_t)e * V, 0);
+    }
+    if (ahead) {
+        step_begin();
+        if (idle()) return;
     }
     __syncthreads();
     const int f = grp * CTA_FIELDS + w;
@@ -685,7 +694,7 @@ void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* l
 #define DSBCG_CTA_LAUNCH2(PP, S2T, L12, DAG)                                                                    \
     launch_step(dslash_cta_kernel<PP, L12, DAG, false>, cgrid, cblock, 0, st,                                             \
         (S2T*)out, (const S2T*)in, nullptr, ld, (const S2T*)(L12 ? links12 : links), g, 1.f, -(float)kappa, 0,    \
-        ctl, nf_static, ngrp)
+        ctl, nf_static, ngrp, st.ahead)
 #define DSBCG_CTA_LAUNCH(PP, S2T)                                                                               \
     if (links12) {                                                                                              \
         if (dag) DSBCG_CTA_LAUNCH2(PP, S2T, true, true);                                                        \
@@ -730,7 +739,7 @@ void launch_dslash_half(int prec, void* out, const void* in, const void* src, si
 #define DSBCG_HALF_CTA2(PP, S2T, DAG)                                                                          \
     launch_step(dslash_cta_kernel<PP, false, DAG, true>, cgrid, cblock, 0, st, (S2T*)out, (const S2T*)in, (const S2T*)src, ld, \
                                                                       (const S2T*)links, g, (float)alpha,        \
-                                                                      (float)beta, parity, ctl, nf_static, ngrp)
+                                                                      (float)beta, parity, ctl, nf_static, ngrp, st.ahead)
 #define DSBCG_HALF_CTA(PP, S2T)                                                                                \
     if (dag) DSBCG_HALF_CTA2(PP, S2T, true);                                                                   \
     else DSBCG_HALF_CTA2(PP, S2T, false)

@@ -227,20 +227,23 @@ template <bool DAG, bool OUT64, bool HALF>
 __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
     void* __restrict__ outv, int* __restrict__ eo, const int4* __restrict__ in, const int* __restrict__ ei,
     const int4* __restrict__ src, const int* __restrict__ es, size_t ld, const int4* __restrict__ links, Geom g,
-    int kshift, int neg, int parity, const Ctl* ctl, int nf_static, int ngrp) {
-    step_begin();
+    int kshift, int neg, int parity, const Ctl* ctl, int nf_static, int ngrp, int ahead) {
+    if (!ahead) step_begin();                                  // else after staging the links (as dslash_cta_kernel)
     extern __shared__ __align__(16) unsigned char fx_smem[];
     int4* sl = reinterpret_cast<int4*>(fx_smem);               // [hop][entry][lane]
     ll2* ex = reinterpret_cast<ll2*>(sl + 8 * 9 * 32);         // [warp][colour][lane]
     int* sy = reinterpret_cast<int*>(ex + 2 * FX_FIELDS * 3 * 32);     // [hop][lane]
     int nf = nf_static;
-    if (ctl) {
-        if (cget(ctl->done)) return;
-        nf = cget(ctl->mk);
-    }
     const int nw = (int)(blockDim.x >> 5), nfc = nw >> 1;      // warps, fields of the CTA
     const int grp = (int)(blockIdx.x % (unsigned)ngrp);
-    if (grp * nfc >= nf) return;                               // CTA-uniform
+    auto idle = [&]() {                                        // CTA-uniform
+        if (ctl) {
+            if (cget(ctl->done)) return true;
+            nf = cget(ctl->mk);
+        }
+        return grp * nfc >= nf;
+    };
+    if (!ahead && idle()) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const size_t V = (size_t)g.V;
     const int Vf = HALF ? g.V / 2 : g.V;
@@ -282,6 +285,10 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
             const int4 q = __ldg(u + (size_t)e * V);
             sl[(h * 9 + (fwd ? e : (e % 3) * 3 + e / 3)) * 32 + lane] = make_int4(s * q.x, s * q.y, sz * q.z, sz * q.w);
         }
+    }
+    if (ahead) {
+        step_begin();
+        if (idle()) return;
     }
     __syncthreads();
     const int S = w & 1;
@@ -429,7 +436,7 @@ void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const 
         max_dyn_smem_once(fx_stencil_kernel<DAG, O64, HALF>, SMEM, devs);                                          \
         launch_step(fx_stencil_kernel<DAG, O64, HALF>, grid, 64 * nfc, SMEM, st, out, eo, (const int4*)in, ei,               \
                                                                         (const int4*)src, es, ld, (const int4*)links, \
-                                                                        g, ks, neg, parity, ctl, nf_static, ngrp);   \
+                                                                        g, ks, neg, parity, ctl, nf_static, ngrp, st.ahead);   \
     }
     if (half) {
         if (out64) { if (dag) DSBCG_FX(true, true, true) else DSBCG_FX(false, true, true) }

@@ -880,13 +880,18 @@ __global__ void __launch_bounds__(NT) small_recur_kernel(SmallStateT<T>* ss, Ctl
                                                          const double* __restrict__ sigma,
                                                          const double* __restrict__ target, int freeze, int wprec,
                                                          void* coefU_w, void* coefL_w, int* ce, int* active,
-                                                         int* conv_step, double* res_out, int MM) {
-    step_begin();
+                                                         int* conv_step, double* res_out, int MM, int ahead) {
+    // Launched ahead of v_update's end: the recurrences read nothing that
+    // v_update writes, and it let this kernel in after its own wait, that is
+    // with the QR complete; the last CTA waits for v_update before it closes
+    // the step (whose widths v_update reads), so this kernel ends after it.
+    if (!ahead) step_begin();
     if (cget(ctl->done)) return;
     extern __shared__ __align__(16) unsigned char sm[];
     shift_recurrence<T>(ss, ctl, (int)blockIdx.x, m, sigma, target, freeze, wprec, coefU_w, coefL_w, ce, active,
                         conv_step, res_out, MM, sm);
     if (!last_arrival(&ss->sh.ticket[2])) return;
+    if (ahead) step_begin();
     const int j = threadIdx.x;                     // s <= S_MAX shifts
     const int nalive = __syncthreads_count(j < s && __ldcg(&ss->sf[j < s ? j : 0].alive));
     const int nkd = __syncthreads_count(j < s && __ldcg(&active[j < s ? j : 0]));
@@ -973,11 +978,11 @@ void launch_small_recur(SmallState* ss, Ctl* ctl, int s, int m, const double* si
     if (sfp64)
         launch_step(small_recur_kernel<double2>, s, NT, recur_smem(m), st, as_state<double2>(ss), ctl, s, m, sigma_dev,
                                                                   target_dev, freeze, wprec, coefU_w, coefL_w, ce, active,
-                                                                  conv_step, res_out, m);
+                                                                  conv_step, res_out, m, st.ahead);
     else
         launch_step(small_recur_kernel<ddc>, s, NT, recur_smem(m), st, as_state<ddc>(ss), ctl, s, m, sigma_dev, target_dev,
                                                               freeze, wprec, coefU_w, coefL_w, ce, active, conv_step,
-                                                              res_out, m);
+                                                              res_out, m, st.ahead);
 }
 
 }  // namespace dsbcg

@@ -894,9 +894,9 @@ dsbcg_status lane_start(dsbcg_ctx* c, Lane& L, const void* rhs, int rhs_prec, si
 // Block steps of fewer than AHEAD_MAX sites x columns (of the full lattice) are
 // bound by launch and m x m latency: their kernels are launched ahead (Stream).
 // Above it the waiting CTAs hold slots that the running kernels of this and the
-// other lanes would use.  ms per solve, plain / ahead: fp64 4^4 m=4 (1 k) 9.1 /
-// 7.5, rational step 8^3 x 16 m=2 (16 k) 26.3 / 23.1, gradient 7x9x10x13 m=5
-// (41 k) 25.4 / 22.4; Schur 12^3 x 24 m=6 (249 k) 19.6 / 20.2, fp64 16^4 m=4 (262
+// other lanes would use.  ms per call, plain / ahead: fp64 4^4 m=4 (1 k) 9.1 /
+// 7.2, rational step 8^3 x 16 m=2 (16 k) 26.6 / 23.8, gradient 7x9x10x13 m=5
+// (41 k) 25.4 / 22.7; Schur 12^3 x 24 m=6 (249 k) 19.6 / 20.2, fp64 16^4 m=4 (262
 // k) 119 / 133, fp32 16^3 x 32 m=12 (1.6 M) 244 / 250.
 constexpr size_t AHEAD_MAX = (size_t)1 << 17;
 bool steps_ahead(const dsbcg_ctx* c, int m) { return !c->profiling && c->V * m < AHEAD_MAX; }
