@@ -201,12 +201,12 @@ __global__ void __launch_bounds__(256) block_update_kernel(typename Tr<P>::S2* _
                                                            size_t ld, size_t n, const Ctl* ctl,
                                                            const typename Tr<P>::C* __restrict__ ca,
                                                            const typename Tr<P>::C* __restrict__ cbh,
-                                                           float hscale) {
+                                                           float hscale, int ahead) {
     step_begin();
     using C = typename Tr<P>::C;
     using R = typename Tr<P>::R;
-    if (cget(ctl->done)) return;
-    const int mk_ = cget(ctl->mk), mp = (cget(ctl->k) > 1) ? cget(ctl->mprev) : 0;
+    if (cget(ctl->done, ahead)) return;
+    const int mk_ = cget(ctl->mk, ahead), mp = (cget(ctl->k, ahead) > 1) ? cget(ctl->mprev, ahead) : 0;
     __shared__ C sa[NF * NF], sb[NF * NF];
     for (int t = threadIdx.x; t < NF * NF; t += blockDim.x) {
         int a = t / NF, b = t % NF;
@@ -754,13 +754,13 @@ __global__ void __launch_bounds__(256) v_update_kernel(typename Tr<P>::S2* __res
                                                        const typename Tr<P>::S2* __restrict__ W, size_t ld,
                                                        size_t n, const Ctl* ctl,
                                                        const typename Tr<(P == P64 ? P64 : P32)>::C* __restrict__ cS,
-                                                       float hscale) {
+                                                       float hscale, int ahead) {
     step_begin();
     constexpr int PW = (P == P64) ? P64 : P32;
     using C = typename Tr<PW>::C;
     using R = typename Tr<PW>::R;
-    if (cget(ctl->done)) return;
-    const int mk_ = cget(ctl->mk), mn = cget(ctl->mnext);
+    if (cget(ctl->done, ahead)) return;
+    const int mk_ = cget(ctl->mk, ahead), mn = cget(ctl->mnext, ahead);
     __shared__ C sS[NF * NF];
     for (int t = threadIdx.x; t < NF * NF; t += blockDim.x) sS[t] = cS[(t / NF) * M_MAX + (t % NF)];
     __syncthreads();
@@ -982,10 +982,10 @@ template <int NF>
 __global__ void __launch_bounds__(UFX_ROWS) block_update_fx_kernel(
     double2* __restrict__ W, const double2* __restrict__ Y, const double2* __restrict__ Vk,
     const double2* __restrict__ Vp, size_t ld, size_t n, const Ctl* ctl, const int4* __restrict__ ca,
-    const int4* __restrict__ cb, const int* __restrict__ ce) {
+    const int4* __restrict__ cb, const int* __restrict__ ce, int ahead) {
     step_begin();
-    if (cget(ctl->done)) return;
-    const int mk_ = cget(ctl->mk), mp = (cget(ctl->k) > 1) ? cget(ctl->mprev) : 0;
+    if (cget(ctl->done, ahead)) return;
+    const int mk_ = cget(ctl->mk, ahead), mp = (cget(ctl->k, ahead) > 1) ? cget(ctl->mprev, ahead) : 0;
     __shared__ int4 sa[NF * NF], sb[NF * NF];
     __shared__ int ea[NF], eb[NF];
     ufx_stage<NF>(sa, ea, ca, ce);
@@ -1029,10 +1029,10 @@ __global__ void __launch_bounds__(UFX_ROWS) block_update_fx_kernel(
 template <int NF>
 __global__ void __launch_bounds__(UFX_ROWS) v_update_fx_kernel(double2* __restrict__ Vn, const double2* __restrict__ W,
                                                                size_t ld, size_t n, const Ctl* ctl,
-                                                               const int4* __restrict__ cS, const int* __restrict__ ce) {
+                                                               const int4* __restrict__ cS, const int* __restrict__ ce, int ahead) {
     step_begin();
-    if (cget(ctl->done)) return;
-    const int mk_ = cget(ctl->mk), mn = cget(ctl->mnext);
+    if (cget(ctl->done, ahead)) return;
+    const int mk_ = cget(ctl->mk, ahead), mn = cget(ctl->mnext, ahead);
     __shared__ int4 sS[NF * NF];
     __shared__ int eS[NF];
     ufx_stage<NF>(sS, eS, cS, ce);
@@ -1189,7 +1189,7 @@ void launch_bu_t(void* W, const void* Y, const void* Vk, const void* Vp, size_t 
 #define BI_BUFX(NF)                                                                                            \
     launch_step(block_update_fx_kernel<NF>, (unsigned)((n + UFX_ROWS - 1) / UFX_ROWS), UFX_ROWS, 0, st, \
         (double2*)W, (const double2*)Y, (const double2*)Vk, (const double2*)Vp, ld, n, ctl, (const int4*)coef_a, \
-        (const int4*)coef_bh, ce)
+        (const int4*)coef_bh, ce, st.ahead)
             BI_DISPATCH_FX(nf_max, BI_BUFX)
 #undef BI_BUFX
             return;
@@ -1200,7 +1200,7 @@ void launch_bu_t(void* W, const void* Y, const void* Vk, const void* Vp, size_t 
     int g = (int)((n + 255) / 256);
 #define BI_BU(NF)                                                                                       \
     launch_step(block_update_kernel<P, NF>, g, 256, 0, st, (S2*)W, (const S2*)Y, (const S2*)Vk, (const S2*)Vp, ld, n, ctl, \
-                                                  (const C*)coef_a, (const C*)coef_bh, hscale)
+                                                  (const C*)coef_a, (const C*)coef_bh, hscale, st.ahead)
     BI_DISPATCH_NF(nf_max, BI_BU)
 #undef BI_BU
 }
@@ -1432,7 +1432,7 @@ void launch_vu_t(void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl
         if (ce) {
 #define BI_VUFX(NF)                                                                                       \
     launch_step(v_update_fx_kernel<NF>, (unsigned)((n + UFX_ROWS - 1) / UFX_ROWS), UFX_ROWS, 0, st, \
-        (double2*)Vnext, (const double2*)W, ld, n, ctl, (const int4*)coefS, ce)
+        (double2*)Vnext, (const double2*)W, ld, n, ctl, (const int4*)coefS, ce, st.ahead)
             BI_DISPATCH_FX(nf_max, BI_VUFX)
 #undef BI_VUFX
             return;
@@ -1443,7 +1443,7 @@ void launch_vu_t(void* Vnext, const void* W, size_t ld, size_t n, const Ctl* ctl
     using CW = typename Tr<PW>::C;
 #define BI_VU(NF)                                                                                           \
     launch_step(v_update_kernel<P, NF>, (unsigned)((n + 255) / 256), 256, 0, st, (S2*)Vnext, (const S2*)W, ld, n, ctl, \
-                                                                       (const CW*)coefS, hscale)
+                                                                       (const CW*)coefS, hscale, st.ahead)
     BI_DISPATCH_NF(nf_max, BI_VU)
 #undef BI_VU
 }

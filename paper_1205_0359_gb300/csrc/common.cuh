@@ -81,11 +81,13 @@ __device__ __forceinline__ void step_begin() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-// A word of the control block, from L2: the kernel before may have read the
-// block on this SM before its last CTA wrote it.
+// A word of the control block, in a kernel launched ahead from L2: the kernel
+// before may have read the block on this SM before its last CTA wrote it.  (An
+// L2 read in every one of V = W S's short CTAs cost 12% of the update class at
+// 24^3 x 48, so kernels of many CTAs pass whether they were launched ahead.)
 template <class T>
-__device__ __forceinline__ T cget(const T& v) {
-    return __ldcg(&v);
+__device__ __forceinline__ T cget(const T& v, bool ahead = true) {
+    return ahead ? __ldcg(&v) : v;
 }
 
 constexpr int M_MAX = 32;      // largest block width (right-hand sides in a block)

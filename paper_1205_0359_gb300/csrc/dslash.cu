@@ -223,8 +223,8 @@ __global__ void __launch_bounds__(32, (P == PDD || P == P64) ? 12 : 24) dslash_k
     using R = typename Tr<P>::R;
     int nf = nf_static;
     if (ctl) {
-        if (cget(ctl->done)) return;
-        nf = cget(ctl->mk);
+        if (ctl->done) return;
+        nf = ctl->mk;
     }
     // 1D work index: block b covers field b % nfg of site tile b / nfg
     // (fields fastest); a grid smaller than the work strides over it
@@ -422,8 +422,8 @@ __global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kern
     const int grp = (int)(blockIdx.x % (unsigned)ngrp);
     auto idle = [&]() {                      // CTA-uniform
         if (ctl) {
-            if (cget(ctl->done)) return true;
-            nf = cget(ctl->mk);
+            if (cget(ctl->done, ahead)) return true;
+            nf = cget(ctl->mk, ahead);
         }
         return grp * CTA_FIELDS >= nf;
     };
@@ -563,8 +563,8 @@ __global__ void __launch_bounds__(32, (P == PDD || P == P64) ? 12 : 24) dslash_h
     using R = typename Tr<P>::R;
     int nf = nf_static;
     if (ctl) {
-        if (cget(ctl->done)) return;
-        nf = cget(ctl->mk);
+        if (ctl->done) return;
+        nf = ctl->mk;
     }
     const int f = (int)(blockIdx.x % (unsigned)nfg);
     if (f >= nf) return;

@@ -52,12 +52,12 @@ __device__ __forceinline__ size_t fx_at(int y) { return (size_t)(y >> 5) * FX_TI
 __global__ void __launch_bounds__(128) fx_convert_kernel(int4* __restrict__ out, int* __restrict__ eo,
                                                          const double2* __restrict__ in, size_t ld, int V,
                                                          const Ctl* ctl, int nf_static,
-                                                         int* __restrict__ flag) {
+                                                         int* __restrict__ flag, int ahead) {
     step_begin();
     int nf = nf_static;
     if (ctl) {
-        if (cget(ctl->done)) return;
-        nf = cget(ctl->mk);
+        if (cget(ctl->done, ahead)) return;
+        nf = cget(ctl->mk, ahead);
     }
     const int x = (int)(blockIdx.x * 128u + threadIdx.x), f = (int)blockIdx.y;
     if (f >= nf || x >= V) return;
@@ -238,8 +238,8 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
     const int grp = (int)(blockIdx.x % (unsigned)ngrp);
     auto idle = [&]() {                                        // CTA-uniform
         if (ctl) {
-            if (cget(ctl->done)) return true;
-            nf = cget(ctl->mk);
+            if (cget(ctl->done, ahead)) return true;
+            nf = cget(ctl->mk, ahead);
         }
         return grp * nfc >= nf;
     };
@@ -415,7 +415,7 @@ void launch_fx_convert(void* out, int* eo, const void* in, size_t ld, size_t Vf,
                        int nf_max, int* flag, Stream st) {
     const int nfg = ctl ? nf_max : nf_static;
     const dim3 grid((unsigned)((Vf + 127) / 128), (unsigned)nfg);
-    launch_step(fx_convert_kernel, grid, 128, 0, st, (int4*)out, eo, (const double2*)in, ld, (int)Vf, ctl, nf_static, flag);
+    launch_step(fx_convert_kernel, grid, 128, 0, st, (int4*)out, eo, (const double2*)in, ld, (int)Vf, ctl, nf_static, flag, st.ahead);
 }
 
 void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const void* src, const int* es, size_t ld,
