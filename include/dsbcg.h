@@ -98,8 +98,8 @@ typedef struct {
                                accumulated solutions and the m x m coefficient work in
                                IEEE FP64, as with FP64 storage; 0 (opt-in): all of them
                                in double-float arithmetic (DSBCG_PREC_DF32) on the FP32
-                               pipes, about 1.2x faster on GB300, where FP64 runs at
-                               1/64 of the FP32 rate */
+                               pipes (faster where the links are not in SU(3), so that
+                               FP64 applications run at 1/64 of the FP32 rate) */
     int x0;                 /* 1: X's input is an initial guess X_0 for every system (a
                                resumed solve): the joint block solve is skipped and
                                each shift is restarted from its own true residual
