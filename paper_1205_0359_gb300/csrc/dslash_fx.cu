@@ -47,11 +47,17 @@ constexpr int FX_TILE = 12 * 32;               // int4 per 32-site tile
 // element of component 0 of site y
 __device__ __forceinline__ size_t fx_at(int y) { return (size_t)(y >> 5) * FX_TILE + (y & 31); }
 
-// FP64 field block (pair-chunk layout) -> FX fields and site exponents.  One
-// thread per (site, field).  Bound by HBM: 16 bytes per complex in and out.
+// FP64 field block -> FX fields and site exponents.  One thread per (site,
+// field).  Bound by HBM: 16 bytes per complex in and out.  Canonical input (192
+// contiguous bytes per thread: a sector serves two of a thread's loads, from
+// L1) takes 101 us for 12 fields of 16^3 x 32, pair-chunk input 84; the packing
+// pass that it spares takes 90, and as much again on the output side, where
+// the stencil writes the canonical layout itself at no cost that could be
+// measured.  A to those fields through dsbcg_apply: 1.28 -> 1.12 ms; to 4 of
+// 4^4: 57 -> 53 us.
 __global__ void __launch_bounds__(128) fx_convert_kernel(int4* __restrict__ out, int* __restrict__ eo,
-                                                         const double2* __restrict__ in, size_t ld, int V,
-                                                         const Ctl* ctl, int nf_static,
+                                                         const double2* __restrict__ in, Lay64 li, size_t ld,
+                                                         int V, const Ctl* ctl, int nf_static,
                                                          int* __restrict__ flag, int ahead) {
     step_begin();
     int nf = nf_static;
@@ -61,11 +67,11 @@ __global__ void __launch_bounds__(128) fx_convert_kernel(int4* __restrict__ out,
     }
     const int x = (int)(blockIdx.x * 128u + threadIdx.x), f = (int)blockIdx.y;
     if (f >= nf || x >= V) return;
-    const double2* p = in + (size_t)f * ld;
+    const double2* p = in + (size_t)f * li.fs + (size_t)x * li.xs;
     double2 v[12];
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-        const double2* q = p + ((size_t)c * V + x) * 2;
+        const double2* q = p + c * li.cs;
         v[2 * c] = __ldg(q);
         v[2 * c + 1] = __ldg(q + 1);
     }
@@ -202,7 +208,7 @@ __device__ __forceinline__ void fx_hops(const int4* __restrict__ fin, const int*
 }
 
 // out = src - kappa H in (H the hopping term; DAG: gamma_5 H gamma_5), fields
-// in FX; out FP64 (pair-chunk layout, OUT64) or FX.  src = in gives D (D^H).
+// in FX; out FP64 (laid out by lo, OUT64) or FX.  src = in gives D (D^H).
 // HALF: in on the other parity of the even-odd lattice, src and out on
 // `parity`.  src NULL and neg: out = kappa H in.
 //
@@ -227,7 +233,7 @@ template <bool DAG, bool OUT64, bool HALF>
 __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
     void* __restrict__ outv, int* __restrict__ eo, const int4* __restrict__ in, const int* __restrict__ ei,
     const int4* __restrict__ src, const int* __restrict__ es, size_t ld, const int4* __restrict__ links, Geom g,
-    int kshift, int neg, int parity, const Ctl* ctl, int nf_static, int ngrp, int ahead) {
+    int kshift, int neg, int parity, Lay64 lo64, const Ctl* ctl, int nf_static, int ngrp, int ahead) {
     if (!ahead) step_begin();                                  // else after staging the links (as dslash_cta_kernel)
     extern __shared__ __align__(16) unsigned char fx_smem[];
     int4* sl = reinterpret_cast<int4*>(fx_smem);               // [hop][entry][lane]
@@ -353,7 +359,7 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
         // v 2^Em: the conversion rounds to FP64, the exponent is added to its bits (the result is a normal
         // number: FX_EB_MIN, FX_EB_MAX)
         if (!store) return;
-        double2* o = reinterpret_cast<double2*>(outv) + (size_t)f * ld;
+        double2* o = reinterpret_cast<double2*>(outv) + (size_t)f * lo64.fs + (size_t)k * lo64.xs;
         auto out = [&](long long v) -> double {
             const double d = __ll2double_rn(v);
             if (bad) return __longlong_as_double(0x7ff8000000000000ll);
@@ -362,8 +368,8 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const int i = S * 3 + a, j = (2 + S) * 3 + a;
-            o[((size_t)(i >> 1) * Vf + k) * 2 + (i & 1)] = make_double2(out(up[a].x), out(up[a].y));
-            o[((size_t)(j >> 1) * Vf + k) * 2 + (j & 1)] = make_double2(out(lo[a].x), out(lo[a].y));
+            o[(i >> 1) * lo64.cs + (i & 1)] = make_double2(out(up[a].x), out(up[a].y));
+            o[(j >> 1) * lo64.cs + (j & 1)] = make_double2(out(lo[a].x), out(lo[a].y));
         }
     } else {
         unsigned long long mag = 0;
@@ -411,15 +417,16 @@ void launch_fx_links(void* dst, const double2* src, size_t V, double kappa, cuda
     fx_pack_links_kernel<<<(unsigned)(grid < 65535 ? grid : 65535), 256, 0, st>>>((int4*)dst, src, V, kfix);
 }
 
-void launch_fx_convert(void* out, int* eo, const void* in, size_t ld, size_t Vf, const Ctl* ctl, int nf_static,
-                       int nf_max, int* flag, Stream st) {
+void launch_fx_convert(void* out, int* eo, const void* in, const Lay64& li, size_t ld, size_t Vf, const Ctl* ctl,
+                       int nf_static, int nf_max, int* flag, Stream st) {
     const int nfg = ctl ? nf_max : nf_static;
     const dim3 grid((unsigned)((Vf + 127) / 128), (unsigned)nfg);
-    launch_step(fx_convert_kernel, grid, 128, 0, st, (int4*)out, eo, (const double2*)in, ld, (int)Vf, ctl, nf_static, flag, st.ahead);
+    launch_step(fx_convert_kernel, grid, 128, 0, st, (int4*)out, eo, (const double2*)in, li, ld, (int)Vf, ctl, nf_static, flag,
+                st.ahead);
 }
 
 void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const void* src, const int* es, size_t ld,
-                       const void* links, const Geom& g, double kappa, int dag, int half, int parity, int out64,
+                       const void* links, const Geom& g, double kappa, int dag, int half, int parity, const Lay64* lo,
                        const Ctl* ctl, int nf_static, int nf_max, Stream st) {
     const int nfg = ctl ? nf_max : nf_static;
     const int nfc = nfg < FX_FIELDS ? nfg : FX_FIELDS;
@@ -429,6 +436,7 @@ void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const 
     int ks;
     fx_mantissa(kappa, &ks);
     const int neg = src ? 0 : 1;
+    const Lay64 l64 = lo ? *lo : Lay64{};
     constexpr int SMEM = 8 * 9 * 32 * sizeof(int4) + 2 * FX_FIELDS * 3 * 32 * sizeof(ll2) + 8 * 32 * sizeof(int);
 #define DSBCG_FX(DAG, O64, HALF)                                                                                    \
     {                                                                                                              \
@@ -436,13 +444,13 @@ void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const 
         max_dyn_smem_once(fx_stencil_kernel<DAG, O64, HALF>, SMEM, devs);                                          \
         launch_step(fx_stencil_kernel<DAG, O64, HALF>, grid, 64 * nfc, SMEM, st, out, eo, (const int4*)in, ei,               \
                                                                         (const int4*)src, es, ld, (const int4*)links, \
-                                                                        g, ks, neg, parity, ctl, nf_static, ngrp, st.ahead);   \
+                                                                        g, ks, neg, parity, l64, ctl, nf_static, ngrp, st.ahead);   \
     }
     if (half) {
-        if (out64) { if (dag) DSBCG_FX(true, true, true) else DSBCG_FX(false, true, true) }
+        if (lo) { if (dag) DSBCG_FX(true, true, true) else DSBCG_FX(false, true, true) }
         else { if (dag) DSBCG_FX(true, false, true) else DSBCG_FX(false, false, true) }
     } else {
-        if (out64) { if (dag) DSBCG_FX(true, true, false) else DSBCG_FX(false, true, false) }
+        if (lo) { if (dag) DSBCG_FX(true, true, false) else DSBCG_FX(false, true, false) }
         else { if (dag) DSBCG_FX(true, false, false) else DSBCG_FX(false, false, false) }
     }
 #undef DSBCG_FX

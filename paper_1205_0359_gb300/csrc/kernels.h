@@ -92,14 +92,22 @@ void launch_dslash_half(int prec, void* out, const void* in, const void* src, si
 // those of FP64 links
 bool fx_kappa_fits(double kappa);            // the hopping coefficient's exponent is in the range of the format
 void launch_fx_links(void* dst, const double2* src, size_t V, double kappa, cudaStream_t st);
-// FP64 fields (internal layout, Vf sites) -> FX; *flag |= 1 where the FX range does not hold (flag may be NULL)
-void launch_fx_convert(void* out, int* eo, const void* in, size_t ld, size_t Vf, const Ctl* ctl, int nf_static,
-                       int nf_max, int* flag, Stream st);
+// Where component i of site x of FP64 field f lies (complex elements):
+// f fs + (i / 2) cs + x xs + i % 2.
+struct Lay64 {
+    size_t fs, cs;
+    int xs;
+};
+inline Lay64 lay64_pairs(size_t ld, size_t Vf) { return Lay64{ld, 2 * Vf, 2}; }       // pair-chunk fields, stride ld
+inline Lay64 lay64_canonical(size_t Vf) { return Lay64{12 * Vf, 2, 12}; }             // the ABI's [site][component]
+// FP64 fields (li, Vf sites) -> FX; *flag |= 1 where the FX range does not hold (flag may be NULL)
+void launch_fx_convert(void* out, int* eo, const void* in, const Lay64& li, size_t ld, size_t Vf, const Ctl* ctl,
+                       int nf_static, int nf_max, int* flag, Stream st);
 // out = src - kappa H in (dag: gamma_5 H gamma_5), or kappa H in when src is
-// NULL.  Full lattice (half = 0) or half fields on `parity`; out64: FP64
-// output, else FX
+// NULL.  Full lattice (half = 0) or half fields on `parity`; lo: FP64 output
+// laid out so, else (NULL) FX
 void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const void* src, const int* es, size_t ld,
-                       const void* links, const Geom& g, double kappa, int dag, int half, int parity, int out64,
+                       const void* links, const Geom& g, double kappa, int dag, int half, int parity, const Lay64* lo,
                        const Ctl* ctl, int nf_static, int nf_max, Stream st);
 
 // ---- blas.cu ----------------------------------------------------------------

@@ -708,44 +708,51 @@ int residual_ctas(dsbcg_ctx* c) {
     return c->resid_ctas;
 }
 
+// A (Schur operator: Ahat) of FP64 fields in fixed point: in is converted into
+// conv (FX, as mid, which receives D in, and tmp), the last pass writes FP64.
+// conv may be out's memory where out is pair-chunk fields.  fxe: site exponents
+// (fx_exp_bytes); flag: see launch_fx_convert.
+void fx_normal(dsbcg_ctx* c, void* out, const Lay64& lo, void* conv, void* mid, const void* in, const Lay64& li, void* tmp,
+               size_t ld, const Ctl* ctl, int nf_static, int nf_max, Stream st, int cls, int* fxe, int* flag) {
+    int *e0 = fxe, *e1 = fxe + (size_t)(ctl ? nf_max : nf_static) * c->Vf;
+    int* e2 = e1 + (e1 - e0);
+    {
+        Prof q(c, cls == DSBCG_KCLASS_RESIDUAL ? cls : DSBCG_KCLASS_OTHER, 1, st);
+        launch_fx_convert(conv, e0, in, li, ld, c->Vf, ctl, nf_static, nf_max, flag, st);
+    }
+    for (int dag = 0; dag < 2; ++dag) {
+        const void* x = dag ? mid : conv;                 // the pass's input, also its diagonal term
+        const int* ex = dag ? e1 : e0;
+        void* y = dag ? out : mid;
+        const Lay64* l = dag ? &lo : nullptr;
+        if (c->schur) {
+            {
+                Prof q(c, cls, 1, st);
+                launch_fx_stencil(tmp, e2, x, ex, nullptr, nullptr, ld, c->linksfx, c->g, c->kappa, dag, 1, 0, nullptr,
+                                  ctl, nf_static, nf_max, st);
+            }
+            Prof q(c, cls, 1, st);
+            launch_fx_stencil(y, e1, tmp, e2, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, l, ctl, nf_static,
+                              nf_max, st);
+        } else {
+            Prof q(c, cls, 1, st);
+            launch_fx_stencil(y, e1, x, ex, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, l, ctl, nf_static,
+                              nf_max, st);
+        }
+    }
+}
+
 // out = Op in for the fields of a block in precision p: the normal operator
 // A = D^H D (two stencils; mid receives D in) or, on a context with the Schur
 // operator, Ahat = Dhat^H Dhat (four half-lattice passes; mid receives
 // Dhat in, tmp is scratch for even-parity half fields)
 //
-// FP64 fields with fxe (site exponents, see fx_exp_bytes) take the
-// fixed-point stencil when its links exist: in is converted into out's memory, the
-// intermediate fields stay in fixed point and the last pass writes FP64.
-// flag: see launch_fx_convert.
+// FP64 fields with fxe take the fixed-point stencil when its links exist.
 void apply_op(dsbcg_ctx* c, int p, void* out, void* mid, const void* in, void* tmp, size_t ld, const Ctl* ctl,
-              int nf_static, int nf_max, float hs, Stream st, int cls, int* fxe = nullptr,
-              int* flag = nullptr) {
+              int nf_static, int nf_max, float hs, Stream st, int cls, int* fxe = nullptr) {
     if (p == P64 && fxe && c->linksfx) {
-        int *e0 = fxe, *e1 = fxe + (size_t)(ctl ? nf_max : nf_static) * c->Vf;
-        int* e2 = e1 + (e1 - e0);
-        {
-            Prof q(c, cls == DSBCG_KCLASS_RESIDUAL ? cls : DSBCG_KCLASS_OTHER, 1, st);
-            launch_fx_convert(out, e0, in, ld, c->Vf, ctl, nf_static, nf_max, flag, st);
-        }
-        for (int dag = 0; dag < 2; ++dag) {
-            const void* x = dag ? mid : out;              // the pass's input, also its diagonal term
-            const int* ex = dag ? e1 : e0;
-            void* y = dag ? out : mid;
-            if (c->schur) {
-                {
-                    Prof q(c, cls, 1, st);
-                    launch_fx_stencil(tmp, e2, x, ex, nullptr, nullptr, ld, c->linksfx, c->g, c->kappa, dag, 1, 0, 0, ctl,
-                                      nf_static, nf_max, st);
-                }
-                Prof q(c, cls, 1, st);
-                launch_fx_stencil(y, e1, tmp, e2, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, dag,
-                                  ctl, nf_static, nf_max, st);
-            } else {
-                Prof q(c, cls, 1, st);
-                launch_fx_stencil(y, e1, x, ex, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, dag, ctl,
-                                  nf_static, nf_max, st);
-            }
-        }
+        const Lay64 l = lay64_pairs(ld, c->Vf);
+        fx_normal(c, out, l, out, mid, in, l, tmp, ld, ctl, nf_static, nf_max, st, cls, fxe, nullptr);
         return;
     }
     if (c->schur) {
@@ -1745,33 +1752,36 @@ dsbcg_status dsbcg_read_profile(dsbcg_ctx* c, double kernel_ms[8], long long ker
 
 namespace {
 
-// D, D^H or A (Dhat, Dhat^H, Ahat) of m FP64 fields in fixed point: a -> b,
-// t and t2 (Schur) are scratch, a is kept; *c->flags as launch_fx_convert
-void fx_apply(dsbcg_ctx* c, int op, void* b, void* t, void* t2, const void* a, int m, int* fxe) {
+// D, D^H or A (Dhat, Dhat^H, Ahat) of m canonical fields in fixed point: in ->
+// out, both in the ABI's layout (the first kernel reads and the last one writes
+// it: no layout passes).  conv, t and t2 (Schur, op = A) are scratch; *c->flags
+// as launch_fx_convert.
+void fx_apply(dsbcg_ctx* c, int op, double2* out, void* conv, void* t, void* t2, const double2* in, int m, int* fxe) {
     cudaMemsetAsync(c->flags, 0, sizeof(int), c->st);
     const size_t ld = c->ld;
+    const Lay64 l = lay64_canonical(c->Vf);
     if (op == DSBCG_OP_A) {
-        apply_op(c, P64, b, t, a, t2, ld, nullptr, m, m, 1.f, c->st, DSBCG_KCLASS_DSLASH, fxe, c->flags);
+        fx_normal(c, out, l, conv, t, in, l, t2, ld, nullptr, m, m, c->st, DSBCG_KCLASS_DSLASH, fxe, c->flags);
         return;
     }
     const int dag = op == DSBCG_OP_DDAG;
     int *e0 = fxe, *e1 = fxe + (size_t)m * c->Vf;
     {
         Prof q(c, DSBCG_KCLASS_OTHER);
-        launch_fx_convert(t, e0, a, ld, c->Vf, nullptr, m, m, c->flags, c->st);
+        launch_fx_convert(conv, e0, in, l, ld, c->Vf, nullptr, m, m, c->flags, c->st);
     }
     if (c->schur) {
         {
             Prof q(c, DSBCG_KCLASS_DSLASH);
-            launch_fx_stencil(t2, e1, t, e0, nullptr, nullptr, ld, c->linksfx, c->g, c->kappa, dag, 1, 0, 0, nullptr, m, m,
-                              c->st);
+            launch_fx_stencil(t, e1, conv, e0, nullptr, nullptr, ld, c->linksfx, c->g, c->kappa, dag, 1, 0, nullptr, nullptr,
+                              m, m, c->st);
         }
         Prof q(c, DSBCG_KCLASS_DSLASH);
-        launch_fx_stencil(b, nullptr, t2, e1, t, e0, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, 1, nullptr,
-                          m, m, c->st);
+        launch_fx_stencil(out, nullptr, t, e1, conv, e0, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, &l, nullptr, m, m,
+                          c->st);
     } else {
         Prof q(c, DSBCG_KCLASS_DSLASH);
-        launch_fx_stencil(b, nullptr, t, e0, t, e0, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, 1, nullptr, m, m,
+        launch_fx_stencil(out, nullptr, conv, e0, conv, e0, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, &l, nullptr, m, m,
                           c->st);
     }
 }
@@ -1789,12 +1799,14 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     bool fx = fixed && storage == P64 && c->linksfx;
     const size_t db = m * n * sizeof(double2);
     Scratch& scr = c->scr;
-    const size_t need = (c->schur ? 4 : 3) * scratch_round(m * fb) + (in_dev ? 0 : scratch_round(db)) +
-                        (out_dev ? 0 : scratch_round(db));
+    const size_t fields = c->schur ? 4 : 3;      // packed in, out and middle fields, and the even-parity ones
+    const size_t host = (in_dev ? 0 : scratch_round(db)) + (out_dev ? 0 : scratch_round(db));
     // without room for the site exponents the FP64 kernels serve the call
-    if (fx && scratch_get(scr, need + scratch_round(fx_exp_bytes(c, m))) != DSBCG_OK) fx = false;
-    if (!fx) CKS(scratch_get(scr, need));
-    void *a = scratch_take(scr, m * fb), *b = scratch_take(scr, m * fb), *t = scratch_take(scr, m * fb);
+    if (fx && scratch_get(scr, (fields - 1) * scratch_round(m * fb) + scratch_round(fx_exp_bytes(c, m)) + host) != DSBCG_OK)
+        fx = false;
+    if (!fx) CKS(scratch_get(scr, fields * scratch_round(m * fb) + host));
+    void *a = scratch_take(scr, m * fb), *t = scratch_take(scr, m * fb);
+    void* b = fx ? nullptr : scratch_take(scr, m * fb);
     void* t2 = c->schur ? scratch_take(scr, m * fb) : nullptr;
     int* fxe = fx ? (int*)scratch_take(scr, fx_exp_bytes(c, m)) : nullptr;
     double2* din = in_dev ? nullptr : (double2*)scratch_take(scr, db);
@@ -1806,9 +1818,9 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     {
         const double2* src = in_dev ? (const double2*)in : din;
         double2* dst = out_dev ? (double2*)out : dout;
-        pack_any(c, storage, a, src, m);
+        if (!fxe) pack_any(c, storage, a, src, m);
         if (fxe) {
-            fx_apply(c, op, b, t, t2, a, m, fxe);
+            fx_apply(c, op, dst, a, t, t2, src, m, fxe);
         } else if (op == DSBCG_OP_A) {
             apply_op(c, storage, b, t, a, t2, ld, nullptr, m, m, c->hscale, c->st, DSBCG_KCLASS_DSLASH);
         } else if (c->schur) {
@@ -1819,7 +1831,7 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
             launch_dslash(storage, b, a, ld, c->links[storage], c->g, c->kappa, op == DSBCG_OP_DDAG, nullptr, m, m,
                           c->hscale, c->st, c->links12[storage]);
         }
-        unpack_any(c, storage, dst, b, m);
+        if (!fxe) unpack_any(c, storage, dst, b, m);
         if (!out_dev) cudaMemcpyAsync(out, dout, m * n * sizeof(double2), cudaMemcpyDeviceToHost, c->st);
         if (fxe) cudaMemcpyAsync(&left, c->flags, sizeof(int), cudaMemcpyDeviceToHost, c->st);
         if (cudaGetLastError() != cudaSuccess) fail(DSBCG_ERR_CUDA);
