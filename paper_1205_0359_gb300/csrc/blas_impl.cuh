@@ -195,12 +195,12 @@ static __global__ void gram_reduce_kernel(const double* __restrict__ partials, i
 // ---------------------------------------------------------------------------
 template <int P, int NF>
 __global__ void __launch_bounds__(256) block_update_kernel(typename Tr<P>::S2* __restrict__ W,
-                                                           const typename Tr<P>::S2* __restrict__ Y,
-                                                           const typename Tr<P>::S2* __restrict__ Vk,
-                                                           const typename Tr<P>::S2* __restrict__ Vp,
+                                                           const typename Tr<P>::S2* Y,
+                                                           const typename Tr<P>::S2* Vk,
+                                                           const typename Tr<P>::S2* Vp,
                                                            size_t ld, size_t n, const Ctl* ctl,
-                                                           const typename Tr<P>::C* __restrict__ ca,
-                                                           const typename Tr<P>::C* __restrict__ cbh,
+                                                           const typename Tr<P>::C* ca,
+                                                           const typename Tr<P>::C* cbh,
                                                            float hscale, int ahead) {
     step_begin();
     using C = typename Tr<P>::C;
@@ -256,10 +256,10 @@ constexpr int UG_NF_MAX = 12;          // upper tiles (6 at width 12) <= warps (
 
 template <int P, int NF>
 __global__ void __launch_bounds__(UG_ROWS, 2) update_gram_kernel(
-    typename Tr<P>::S2* __restrict__ W, const typename Tr<P>::S2* __restrict__ Y,
-    const typename Tr<P>::S2* __restrict__ Vk, const typename Tr<P>::S2* __restrict__ Vp, size_t ld, size_t n,
-    const Ctl* ctl, int nf_max, const typename Tr<P>::C* __restrict__ ca,
-    const typename Tr<P>::C* __restrict__ cbh, double* __restrict__ partials, float hscale) {
+    typename Tr<P>::S2* __restrict__ W, const typename Tr<P>::S2* Y,
+    const typename Tr<P>::S2* Vk, const typename Tr<P>::S2* Vp, size_t ld, size_t n,
+    const Ctl* ctl, int nf_max, const typename Tr<P>::C* ca,
+    const typename Tr<P>::C* cbh, double* __restrict__ partials, float hscale) {
     step_begin();
     static_assert(NF <= UG_NF_MAX, "fused update and Gram: widths up to 12");
     using C = typename Tr<P>::C;
@@ -522,8 +522,8 @@ __device__ __forceinline__ double warp_transpose_sum(double v[32], int lane) {
 }
 
 template <int P>
-__global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2* __restrict__ X,
-                                                        const typename Tr<P>::S2* __restrict__ Y, size_t ld,
+__global__ void __launch_bounds__(544) gram_tile_kernel(const typename Tr<P>::S2* X,
+                                                        const typename Tr<P>::S2* Y, size_t ld,
                                                         size_t n, Ctl* ctl, int nf_static, int nf_max,
                                                         int herm, int diag_yy, double* __restrict__ partials,
                                                         float hscale, int first_wait) {
@@ -751,9 +751,9 @@ void launch_gram_tile_t(const void* X, const void* Y, size_t ld, size_t n, Ctl* 
 // V_{k+1} = W S (one thread per row; W and V in the storage precision)
 template <int P, int NF>
 __global__ void __launch_bounds__(256) v_update_kernel(typename Tr<P>::S2* __restrict__ Vn,
-                                                       const typename Tr<P>::S2* __restrict__ W, size_t ld,
+                                                       const typename Tr<P>::S2* W, size_t ld,
                                                        size_t n, const Ctl* ctl,
-                                                       const typename Tr<(P == P64 ? P64 : P32)>::C* __restrict__ cS,
+                                                       const typename Tr<(P == P64 ? P64 : P32)>::C* cS,
                                                        float hscale, int ahead) {
     step_begin();
     constexpr int PW = (P == P64) ? P64 : P32;
@@ -810,10 +810,10 @@ __host__ __device__ constexpr size_t sc_smem_bytes() {
 
 template <int P, int PW, int NF, int ROWS>
 __global__ void __launch_bounds__(ROWS, (NF <= 12 && PW == P32) ? 4 : 1) shift_chunk_kernel(
-    const typename Tr<P>::S2* __restrict__ ring, size_t slot_elems, int R, size_t ld,
+    const typename Tr<P>::S2* ring, size_t slot_elems, int R, size_t ld,
     typename Tr<PW>::S2* __restrict__ Pb, typename Tr<PW>::S2* __restrict__ Xb, size_t ldw, size_t n, int s, int m,
-    Ctl* ctl, int k0, int C, const typename Tr<PW>::C* __restrict__ cU,
-    const typename Tr<PW>::C* __restrict__ cL, const int* __restrict__ act, float hscale) {
+    Ctl* ctl, int k0, int C, const typename Tr<PW>::C* cU,
+    const typename Tr<PW>::C* cL, const int* act, float hscale) {
     step_begin();
     using C2 = typename Tr<PW>::C;
     using R2 = typename Tr<PW>::R;
@@ -973,16 +973,16 @@ constexpr int UFX_ROWS = 128;
 
 // tile (NF x NF of M_MAX-strided entries) and its column exponents to shared memory
 template <int NF>
-__device__ __forceinline__ void ufx_stage(int4* st, int* se, const int4* __restrict__ c, const int* __restrict__ ce) {
+__device__ __forceinline__ void ufx_stage(int4* st, int* se, const int4* c, const int* ce) {
     for (int u = threadIdx.x; u < NF * NF; u += blockDim.x) st[u] = c[(u / NF) * M_MAX + u % NF];
     if (threadIdx.x < NF) se[threadIdx.x] = ce[threadIdx.x];
 }
 
 template <int NF>
 __global__ void __launch_bounds__(UFX_ROWS) block_update_fx_kernel(
-    double2* __restrict__ W, const double2* __restrict__ Y, const double2* __restrict__ Vk,
-    const double2* __restrict__ Vp, size_t ld, size_t n, const Ctl* ctl, const int4* __restrict__ ca,
-    const int4* __restrict__ cb, const int* __restrict__ ce, int ahead) {
+    double2* __restrict__ W, const double2* Y, const double2* Vk,
+    const double2* Vp, size_t ld, size_t n, const Ctl* ctl, const int4* ca,
+    const int4* cb, const int* ce, int ahead) {
     step_begin();
     if (cget(ctl->done, ahead)) return;
     const int mk_ = cget(ctl->mk, ahead), mp = (cget(ctl->k, ahead) > 1) ? cget(ctl->mprev, ahead) : 0;
@@ -1027,9 +1027,9 @@ __global__ void __launch_bounds__(UFX_ROWS) block_update_fx_kernel(
 }
 
 template <int NF>
-__global__ void __launch_bounds__(UFX_ROWS) v_update_fx_kernel(double2* __restrict__ Vn, const double2* __restrict__ W,
+__global__ void __launch_bounds__(UFX_ROWS) v_update_fx_kernel(double2* __restrict__ Vn, const double2* W,
                                                                size_t ld, size_t n, const Ctl* ctl,
-                                                               const int4* __restrict__ cS, const int* __restrict__ ce, int ahead) {
+                                                               const int4* cS, const int* ce, int ahead) {
     step_begin();
     if (cget(ctl->done, ahead)) return;
     const int mk_ = cget(ctl->mk, ahead), mn = cget(ctl->mnext, ahead);
@@ -1063,9 +1063,9 @@ __global__ void __launch_bounds__(UFX_ROWS) v_update_fx_kernel(double2* __restri
 
 template <int NF, int ROWS>
 __global__ void __launch_bounds__(ROWS, NF <= 4 ? 4 : NF <= 8 ? 2 : 1) shift_chunk_fx_kernel(
-    const double2* __restrict__ ring, size_t slot_elems, int R, size_t ld, double2* __restrict__ Pb,
+    const double2* ring, size_t slot_elems, int R, size_t ld, double2* __restrict__ Pb,
     double2* __restrict__ Xb, size_t ldw, size_t n, int s, int m, Ctl* ctl, int k0, int C,
-    const int4* __restrict__ cU, const int4* __restrict__ cL, const int* __restrict__ cE, const int* __restrict__ act) {
+    const int4* cU, const int4* cL, const int* cE, const int* act) {
     step_begin();
     const int j = (int)(blockIdx.x % (unsigned)s);
     const int kend = min(k0 + C, cget(ctl->last_step));
@@ -1274,9 +1274,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 template <int P, int NF, int ROWS>
 __global__ void __launch_bounds__(ROWS, NF <= 12 ? 4 : 1) shift_chunk32_kernel(
-    const typename Tr<P>::S2* __restrict__ ring, size_t slot_elems, int R, size_t ld, float2* __restrict__ Pb,
+    const typename Tr<P>::S2* ring, size_t slot_elems, int R, size_t ld, float2* __restrict__ Pb,
     float2* __restrict__ Xb, size_t ldw, size_t n, int s, int m, Ctl* ctl, int k0, int C,
-    const float2* __restrict__ cU, const float2* __restrict__ cL, const int* __restrict__ act, float hscale) {
+    const float2* cU, const float2* cL, const int* act, float hscale) {
     step_begin();
     static_assert(NF % 2 == 0, "column pairs");
     constexpr int NP = NF / 2;

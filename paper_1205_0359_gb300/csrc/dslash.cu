@@ -49,11 +49,12 @@ struct SpinorIO<P64> {
 
 template <>
 struct SpinorIO<P32> {
+    template <bool AHEAD>
     static __device__ __forceinline__ void load(const float2* f, size_t V, size_t x, float2 p[12], float, size_t) {
         const float4* q = reinterpret_cast<const float4*>(f);
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
-            float4 v = __ldg(q + (size_t)c * V + x);
+            const float4 v = ld_prev<AHEAD>(q + (size_t)c * V + x);
             p[2 * c] = make_float2(v.x, v.y);
             p[2 * c + 1] = make_float2(v.z, v.w);
         }
@@ -68,11 +69,12 @@ struct SpinorIO<P32> {
 
 template <class H2, class Cvt>
 struct Spinor16 {
+    template <bool AHEAD>
     static __device__ __forceinline__ void load(const H2* f, size_t V, size_t x, float2 p[12], float inv, size_t) {
         const uint2* q = reinterpret_cast<const uint2*>(f);
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
-            uint2 v = __ldg(q + (size_t)c * V + x);
+            const uint2 v = ld_prev<AHEAD>(q + (size_t)c * V + x);
             const H2* h = reinterpret_cast<const H2*>(&v);
 #pragma unroll
             for (int w = 0; w < 2; ++w) {
@@ -407,14 +409,14 @@ __device__ __forceinline__ void hop_reconstruct(int mu, int dir, const C uh[2][3
 // out = alpha src + beta H in on `parity`, or beta H in without src.
 constexpr int CTA_FIELDS = 4;
 
-template <int P, bool L12, bool DAG, bool HALF>
+template <int P, bool L12, bool DAG, bool HALF, bool AHEAD>
 __global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kernel(
-    typename Tr<P>::S2* __restrict__ out, const typename Tr<P>::S2* __restrict__ in,
-    const typename Tr<P>::S2* __restrict__ src, size_t ld, const typename Tr<P>::S2* __restrict__ links, Geom g,
-    float alpha, float beta, int parity, const Ctl* ctl, int nf_static, int ngrp, int ahead) {
+    typename Tr<P>::S2* __restrict__ out, const typename Tr<P>::S2* in,
+    const typename Tr<P>::S2* src, size_t ld, const typename Tr<P>::S2* __restrict__ links, Geom g,
+    float alpha, float beta, int parity, const Ctl* ctl, int nf_static, int ngrp) {
     // launched ahead: the links, which no kernel of a solve writes, are staged
     // before the wait for the kernel that writes the fields
-    if (!ahead) step_begin();
+    if (!AHEAD) step_begin();
     // [hop][entry][site of the tile]: rows 0 and 1 of SU(3) links (L12), with
     // row 2 rebuilt at each use, else all nine entries
     __shared__ float2 sl[8][L12 ? 6 : 9][32];
@@ -422,12 +424,12 @@ __global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kern
     const int grp = (int)(blockIdx.x % (unsigned)ngrp);
     auto idle = [&]() {                      // CTA-uniform
         if (ctl) {
-            if (cget(ctl->done, ahead)) return true;
-            nf = cget(ctl->mk, ahead);
+            if (cget(ctl->done, AHEAD)) return true;
+            nf = cget(ctl->mk, AHEAD);
         }
         return grp * CTA_FIELDS >= nf;
     };
-    if (!ahead && idle()) return;
+    if (!AHEAD && idle()) return;
     const int tile = (int)(blockIdx.x / (unsigned)ngrp);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const size_t V = (size_t)g.V;
@@ -453,7 +455,7 @@ __global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kern
 #pragma unroll
         for (int e = 0; e < NE; ++e) sl[h][e][lane] = ld_link<P>(u + (size_t)e * V, 0);
     }
-    if (ahead) {
+    if (AHEAD) {
         step_begin();
         if (idle()) return;
     }
@@ -470,7 +472,7 @@ __global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kern
             float sgn;
             const int y = neighbour(g, xs, s, mu, dir == 0 ? 1 : -1, &sgn);
             float2 p[12];
-            SpinorIO<P>::load(fin, (size_t)Vf, (size_t)(HALF ? y >> 1 : y), p, 1.f, 0);
+            SpinorIO<P>::template load<AHEAD>(fin, (size_t)Vf, (size_t)(HALF ? y >> 1 : y), p, 1.f, 0);
             float2 hh[2][3];
             hop_project_signed<DAG>(mu, dir, p, hh);
             if (mu == 3) {                       // the time-boundary sign
@@ -530,7 +532,7 @@ __global__ void __launch_bounds__(32 * CTA_FIELDS, HALF ? 6 : 7) dslash_cta_kern
     float2 p[12];
     const typename Tr<P>::S2* diag = HALF ? src : in;
     if (diag) {
-        SpinorIO<P>::load(diag + (size_t)f * ld, (size_t)Vf, (size_t)k, p, 1.f, 0);
+        SpinorIO<P>::template load<AHEAD>(diag + (size_t)f * ld, (size_t)Vf, (size_t)k, p, 1.f, 0);
 #pragma unroll
         for (int i = 0; i < 12; ++i) {
             const float2 a = acc[i / 3][i % 3];
@@ -692,9 +694,9 @@ void launch_dslash(int prec, void* out, const void* in, size_t ld, const void* l
     dim3 cgrid((unsigned)(ngrp * ((g.V + 31) / 32)));
     dim3 cblock(32 * CTA_FIELDS);
 #define DSBCG_CTA_LAUNCH2(PP, S2T, L12, DAG)                                                                    \
-    launch_step(dslash_cta_kernel<PP, L12, DAG, false>, cgrid, cblock, 0, st,                                             \
-        (S2T*)out, (const S2T*)in, nullptr, ld, (const S2T*)(L12 ? links12 : links), g, 1.f, -(float)kappa, 0,    \
-        ctl, nf_static, ngrp, st.ahead)
+    launch_step(st.ahead ? dslash_cta_kernel<PP, L12, DAG, false, true> : dslash_cta_kernel<PP, L12, DAG, false, false>, \
+                cgrid, cblock, 0, st, (S2T*)out, (const S2T*)in, nullptr, ld, (const S2T*)(L12 ? links12 : links), \
+                g, 1.f, -(float)kappa, 0, ctl, nf_static, ngrp)
 #define DSBCG_CTA_LAUNCH(PP, S2T)                                                                               \
     if (links12) {                                                                                              \
         if (dag) DSBCG_CTA_LAUNCH2(PP, S2T, true, true);                                                        \
@@ -737,9 +739,9 @@ void launch_dslash_half(int prec, void* out, const void* in, const void* src, si
     // FP32 and 16-bit fields: gamma_5 on the input of the first pass and on the
     // output of the second (dag) is gamma_5 H gamma_5 in both
 #define DSBCG_HALF_CTA2(PP, S2T, DAG)                                                                          \
-    launch_step(dslash_cta_kernel<PP, false, DAG, true>, cgrid, cblock, 0, st, (S2T*)out, (const S2T*)in, (const S2T*)src, ld, \
-                                                                      (const S2T*)links, g, (float)alpha,        \
-                                                                      (float)beta, parity, ctl, nf_static, ngrp, st.ahead)
+    launch_step(st.ahead ? dslash_cta_kernel<PP, false, DAG, true, true> : dslash_cta_kernel<PP, false, DAG, true, false>, \
+                cgrid, cblock, 0, st, (S2T*)out, (const S2T*)in, (const S2T*)src, ld, (const S2T*)links, g,        \
+                (float)alpha, (float)beta, parity, ctl, nf_static, ngrp)
 #define DSBCG_HALF_CTA(PP, S2T)                                                                                \
     if (dag) DSBCG_HALF_CTA2(PP, S2T, true);                                                                   \
     else DSBCG_HALF_CTA2(PP, S2T, false)

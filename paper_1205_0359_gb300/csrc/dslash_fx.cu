@@ -56,7 +56,7 @@ __device__ __forceinline__ size_t fx_at(int y) { return (size_t)(y >> 5) * FX_TI
 // measured.  A to those fields through dsbcg_apply: 1.28 -> 1.12 ms; to 4 of
 // 4^4: 57 -> 53 us.
 __global__ void __launch_bounds__(128) fx_convert_kernel(int4* __restrict__ out, int* __restrict__ eo,
-                                                         const double2* __restrict__ in, Lay64 li, size_t ld,
+                                                         const double2* in, Lay64 li, size_t ld,
                                                          int V, const Ctl* ctl, int nf_static,
                                                          int* __restrict__ flag, int ahead) {
     step_begin();
@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(128) fx_convert_kernel(int4* __restrict__ out,
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
         const double2* q = p + c * li.cs;
-        v[2 * c] = __ldg(q);
-        v[2 * c + 1] = __ldg(q + 1);
+        v[2 * c] = q[0];
+        v[2 * c + 1] = q[1];
     }
     int mx = 0;
     unsigned any = 0;
@@ -147,15 +147,15 @@ __device__ __forceinline__ void lacc(ll2& a, ll2 q) {
 // hop's exponent to the accumulators'.  MINUS: projector 1 - gamma_MU, else
 // 1 + gamma_MU.  The result goes to spin S (up) and to the lower spin it
 // rebuilds (lo): the other thread's for mu = x, y, this thread's for z, t.
-template <int MU, bool MINUS, int S>
-__device__ __forceinline__ void fx_hop(const int4* __restrict__ p, const int4* su, int sh, ll2 up[3], ll2 lo[3]) {
+template <int MU, bool MINUS, int S, bool AHEAD>
+__device__ __forceinline__ void fx_hop(const int4* p, const int4* su, int sh, ll2 up[3], ll2 lo[3]) {
     constexpr int T = MU < 2 ? 1 - S : S;                 // lower spin of the projection
     constexpr bool NEG = (MU == 1 || MU == 2) && S == 1 ? !MINUS : MINUS;
     int4 h[3];
     int2 ni[3];                                           // minus the imaginary parts
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const int4 u = __ldg(p + (S * 3 + a) * 32), l = __ldg(p + ((2 + T) * 3 + a) * 32);
+        const int4 u = ld_prev<AHEAD>(p + (S * 3 + a) * 32), l = ld_prev<AHEAD>(p + ((2 + T) * 3 + a) * 32);
         if (MU == 0 || MU == 2) h[a] = NEG ? isubi(u, l) : iaddi(u, l);
         else h[a] = NEG ? isub(u, l) : iadd(u, l);
         ni[a] = make_int2(-h[a].z, -h[a].w);
@@ -195,16 +195,16 @@ __device__ __forceinline__ void fx_hop(const int4* __restrict__ p, const int4* s
 
 // the four hops in x, y (HALFH = 0) or z, t (1); sy: their neighbour sites
 // (stride 32), sh: their shifts, six bits each
-template <bool DAG, int S, int HALFH>
-__device__ __forceinline__ void fx_hops(const int4* __restrict__ fin, const int* sy, const int4* sl, unsigned sh,
+template <bool DAG, int S, int HALFH, bool AHEAD>
+__device__ __forceinline__ void fx_hops(const int4* fin, const int* sy, const int4* sl, unsigned sh,
                                         ll2 up[3], ll2 lo[3]) {
     constexpr int HS = 9 * 32, M = 2 * HALFH;
     sy += 4 * 32 * HALFH;
     sl += 4 * HS * HALFH;
-    fx_hop<M, !DAG, S>(fin + fx_at(sy[0]), sl, (int)sh & 63, up, lo);
-    fx_hop<M, DAG, S>(fin + fx_at(sy[32]), sl + HS, (int)(sh >> 6) & 63, up, lo);
-    fx_hop<M + 1, !DAG, S>(fin + fx_at(sy[64]), sl + 2 * HS, (int)(sh >> 12) & 63, up, lo);
-    fx_hop<M + 1, DAG, S>(fin + fx_at(sy[96]), sl + 3 * HS, (int)(sh >> 18) & 63, up, lo);
+    fx_hop<M, !DAG, S, AHEAD>(fin + fx_at(sy[0]), sl, (int)sh & 63, up, lo);
+    fx_hop<M, DAG, S, AHEAD>(fin + fx_at(sy[32]), sl + HS, (int)(sh >> 6) & 63, up, lo);
+    fx_hop<M + 1, !DAG, S, AHEAD>(fin + fx_at(sy[64]), sl + 2 * HS, (int)(sh >> 12) & 63, up, lo);
+    fx_hop<M + 1, DAG, S, AHEAD>(fin + fx_at(sy[96]), sl + 3 * HS, (int)(sh >> 18) & 63, up, lo);
 }
 
 // out = src - kappa H in (H the hopping term; DAG: gamma_5 H gamma_5), fields
@@ -229,12 +229,12 @@ __device__ __forceinline__ void fx_hops(const int4* __restrict__ fin, const int*
 constexpr int FX_FIELDS = 4;
 static_assert(2 * FX_FIELDS <= 8, "the exchange of leading-zero counts reuses the 8 x 32 words of the sites");
 
-template <bool DAG, bool OUT64, bool HALF>
+template <bool DAG, bool OUT64, bool HALF, bool AHEAD>
 __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
-    void* __restrict__ outv, int* __restrict__ eo, const int4* __restrict__ in, const int* __restrict__ ei,
-    const int4* __restrict__ src, const int* __restrict__ es, size_t ld, const int4* __restrict__ links, Geom g,
-    int kshift, int neg, int parity, Lay64 lo64, const Ctl* ctl, int nf_static, int ngrp, int ahead) {
-    if (!ahead) step_begin();                                  // else after staging the links (as dslash_cta_kernel)
+    void* __restrict__ outv, int* __restrict__ eo, const int4* in, const int* ei,
+    const int4* src, const int* es, size_t ld, const int4* __restrict__ links, Geom g,
+    int kshift, int neg, int parity, Lay64 lo64, const Ctl* ctl, int nf_static, int ngrp) {
+    if (!AHEAD) step_begin();                                  // else after staging the links (as dslash_cta_kernel)
     extern __shared__ __align__(16) unsigned char fx_smem[];
     int4* sl = reinterpret_cast<int4*>(fx_smem);               // [hop][entry][lane]
     ll2* ex = reinterpret_cast<ll2*>(sl + 8 * 9 * 32);         // [warp][colour][lane]
@@ -244,12 +244,12 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
     const int grp = (int)(blockIdx.x % (unsigned)ngrp);
     auto idle = [&]() {                                        // CTA-uniform
         if (ctl) {
-            if (cget(ctl->done, ahead)) return true;
-            nf = cget(ctl->mk, ahead);
+            if (cget(ctl->done, AHEAD)) return true;
+            nf = cget(ctl->mk, AHEAD);
         }
         return grp * nfc >= nf;
     };
-    if (!ahead && idle()) return;
+    if (!AHEAD && idle()) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const size_t V = (size_t)g.V;
     const int Vf = HALF ? g.V / 2 : g.V;
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
             sl[(h * 9 + (fwd ? e : (e % 3) * 3 + e / 3)) * 32 + lane] = make_int4(s * q.x, s * q.y, sz * q.z, sz * q.w);
         }
     }
-    if (ahead) {
+    if (AHEAD) {
         step_begin();
         if (idle()) return;
     }
@@ -312,18 +312,18 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
         for (int a = 0; a < 3; ++a) {
             d[a] = ll2{0, 0};
             if (src) {
-                const int4 u = __ldg(p + a * 32);
+                const int4 u = ld_prev<AHEAD>(p + a * 32);
                 d[a] = ll2{fx_join(u.x, u.y) >> sr << sf, fx_join(u.z, u.w) >> sr << sf};
             }
         }
     };
     if (on) {
         const int* fe = ei + (size_t)f * Vf;
-        if (src) e0 = __ldg(es + (size_t)f * Vf + ks);
+        if (src) e0 = ld_prev<AHEAD>(es + (size_t)f * Vf + ks);
         int eh[8];
 #pragma unroll
         for (int h = 0; h < 8; ++h) {
-            eh[h] = __ldg(fe + sy[h * 32 + lane]) - kshift;
+            eh[h] = ld_prev<AHEAD>(fe + sy[h * 32 + lane]) - kshift;
             Em = max(Em, eh[h]);
         }
         // the diagonal term (at most 2^57) has bits to spare: its unit may be up to 2^4 of the accumulators'
@@ -336,13 +336,13 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
         diag(S, up);
 #pragma unroll
         for (int a = 0; a < 3; ++a) lo[a] = ll2{0, 0};
-        if (S == 0) fx_hops<DAG, 0, 0>(fin, sy + lane, sl + lane, shl, up, lo);
-        else fx_hops<DAG, 1, 0>(fin, sy + lane, sl + lane, shl, up, lo);
+        if (S == 0) fx_hops<DAG, 0, 0, AHEAD>(fin, sy + lane, sl + lane, shl, up, lo);
+        else fx_hops<DAG, 1, 0, AHEAD>(fin, sy + lane, sl + lane, shl, up, lo);
 #pragma unroll
         for (int a = 0; a < 3; ++a) ex[(w * 3 + a) * 32 + lane] = lo[a];
         diag(2 + S, lo);
-        if (S == 0) fx_hops<DAG, 0, 1>(fin, sy + lane, sl + lane, shh, up, lo);
-        else fx_hops<DAG, 1, 1>(fin, sy + lane, sl + lane, shh, up, lo);
+        if (S == 0) fx_hops<DAG, 0, 1, AHEAD>(fin, sy + lane, sl + lane, shh, up, lo);
+        else fx_hops<DAG, 1, 1, AHEAD>(fin, sy + lane, sl + lane, shh, up, lo);
     }
     __syncthreads();
     if (on) {
@@ -438,22 +438,25 @@ void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const 
     const int neg = src ? 0 : 1;
     const Lay64 l64 = lo ? *lo : Lay64{};
     constexpr int SMEM = 8 * 9 * 32 * sizeof(int4) + 2 * FX_FIELDS * 3 * 32 * sizeof(ll2) + 8 * 32 * sizeof(int);
-#define DSBCG_FX(DAG, O64, HALF)                                                                                    \
+#define DSBCG_FX2(DAG, O64, HALF, AHEAD)                                                                            \
     {                                                                                                              \
         static std::atomic<unsigned long long> devs{0};                                                            \
-        max_dyn_smem_once(fx_stencil_kernel<DAG, O64, HALF>, SMEM, devs);                                          \
-        launch_step(fx_stencil_kernel<DAG, O64, HALF>, grid, 64 * nfc, SMEM, st, out, eo, (const int4*)in, ei,               \
-                                                                        (const int4*)src, es, ld, (const int4*)links, \
-                                                                        g, ks, neg, parity, l64, ctl, nf_static, ngrp, st.ahead);   \
+        max_dyn_smem_once(fx_stencil_kernel<DAG, O64, HALF, AHEAD>, SMEM, devs);                                   \
+        launch_step(fx_stencil_kernel<DAG, O64, HALF, AHEAD>, grid, 64 * nfc, SMEM, st, out, eo, (const int4*)in, ei, \
+                    (const int4*)src, es, ld, (const int4*)links, g, ks, neg, parity, l64, ctl, nf_static, ngrp);  \
     }
+#define DSBCG_FX(DAG, O64, HALF) \
+    if (st.ahead) DSBCG_FX2(DAG, O64, HALF, true) else DSBCG_FX2(DAG, O64, HALF, false)
+#define DSBCG_FX1(O64, HALF) \
+    if (dag) { DSBCG_FX(true, O64, HALF) } else { DSBCG_FX(false, O64, HALF) }
     if (half) {
-        if (lo) { if (dag) DSBCG_FX(true, true, true) else DSBCG_FX(false, true, true) }
-        else { if (dag) DSBCG_FX(true, false, true) else DSBCG_FX(false, false, true) }
+        if (lo) { DSBCG_FX1(true, true) } else { DSBCG_FX1(false, true) }
     } else {
-        if (lo) { if (dag) DSBCG_FX(true, true, false) else DSBCG_FX(false, true, false) }
-        else { if (dag) DSBCG_FX(true, false, false) else DSBCG_FX(false, false, false) }
+        if (lo) { DSBCG_FX1(true, false) } else { DSBCG_FX1(false, false) }
     }
+#undef DSBCG_FX1
 #undef DSBCG_FX
+#undef DSBCG_FX2
 }
 
 }  // namespace dsbcg

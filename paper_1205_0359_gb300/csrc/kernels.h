@@ -178,10 +178,10 @@ void launch_small_alpha(SmallState* ss, const Ctl* ctl, const double* partials, 
 // W^H W from the Gram partials, pivoted QR with deflation: S, beta_{k+1}, m_{k+1}
 void launch_small_qr(SmallState* ss, Ctl* ctl, const double* partials, int nblk, int m, double dtol, int wprec,
                      int sfp64, void* coefS_w, int* ce, Stream st);
-// per-shift recurrences (a CTA per shift) and the close of the block step
+// per-shift recurrences (a CTA per shift) and the close of block step `step`
 void launch_small_recur(SmallState* ss, Ctl* ctl, int s, int m, const double* sigma_dev, const double* target_dev,
                         int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* ce, int* active,
-                        int* conv_step, double* res_out, Stream st);
+                        int* conv_step, double* res_out, int step, Stream st);
 const double2* small_state_S(const SmallState* ss);
 
 // ---- force.cu ---------------------------------------------------------------

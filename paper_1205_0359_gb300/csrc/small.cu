@@ -56,7 +56,8 @@ struct SmallSharedT {
     T S[M_MAX * M_MAX];              // V_{k+1} = W S (m_k x m_{k+1})
     T yy[M_MAX / 2];                 // ||A v_i||^2 (real scalars, two per entry)
     double red[RED_SLOTS];           // group sums of the Gram partials (reduce_partials)
-    unsigned ticket[4];              // arrival counters of the multi-CTA kernels (zero between launches)
+    unsigned ticket[3];              // arrival counters of the multi-CTA kernels (zero between launches)
+    unsigned qr_step;                // the block step whose QR is published (released by small_qr_kernel)
 };
 template <class T>
 struct SmallShiftT {
@@ -529,7 +530,7 @@ __host__ __device__ inline int red_groups(int ntiles) {
 }
 
 template <class T>
-__device__ bool reduce_partials(const double* __restrict__ part, int nblk, int nf_max, typename Sc<T>::R* red,
+__device__ bool reduce_partials(const double* part, int nblk, int nf_max, typename Sc<T>::R* red,
                                 unsigned* ticket, bool fp64_part) {
     using S = Sc<T>;
     using R = typename S::R;
@@ -641,7 +642,8 @@ __global__ void small_init_kernel(SmallStateT<T>* ss, Ctl* ctl, const double2* _
     }
     for (int t = threadIdx.x; t < s * M_MAX; t += blockDim.x) ss->sf[t / M_MAX].conv[t % M_MAX] = 0;
     for (int q = threadIdx.x; q < s; q += blockDim.x) ss->sf[q].alive = 1;
-    if (threadIdx.x < 4) ss->sh.ticket[threadIdx.x] = 0;
+    if (threadIdx.x < 3) ss->sh.ticket[threadIdx.x] = 0;
+    if (threadIdx.x == 3) ss->sh.qr_step = 0;
     if (threadIdx.x == 0) {
         ctl->k = 1;
         ctl->mk = r;
@@ -664,7 +666,7 @@ __global__ void small_init_kernel(SmallStateT<T>* ss, Ctl* ctl, const double2* _
 // CTAs reduce, the last one to arrive forms the result.
 template <class T>
 __global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, const Ctl* ctl,
-                                                         const double* __restrict__ part, int nblk, int nf_max,
+                                                         const double* part, int nblk, int nf_max,
                                                          int wprec, void* coef_a, void* coef_bh, int* ce) {
     step_begin();
     using S = Sc<T>;
@@ -712,7 +714,7 @@ __global__ void __launch_bounds__(NT) small_alpha_kernel(SmallStateT<T>* ss, con
 // deflation in the CTA that arrives last, which publishes S, beta_{k+1} and
 // m_{k+1}.
 template <class T>
-__global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* __restrict__ part,
+__global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* ctl, const double* part,
                                                       int nblk, int m, double dtol, int wprec, void* coefS_w, int* ce, int MM) {
     step_begin();
     using S = Sc<T>;
@@ -748,16 +750,20 @@ __global__ void __launch_bounds__(NT) small_qr_kernel(SmallStateT<T>* ss, Ctl* c
         ss->sh.S[t] = (a < mk_ && b < mn) ? Sm[a * MM + b] : cz<T>();
         ss->sh.betan[t] = (a < mn && b < mk_) ? Bn[a * MM + b] : cz<T>();
     }
+    if (threadIdx.x == 0) {
+        ctl->mnext = mn;
+        ctl->deflations = cget(ctl->deflations) + mk_ - mn;
+    }
+    // everything that the recurrences take from here, published for those that
+    // run beside V = W S
+    bsync();
+    if (threadIdx.x == 0) st_release(&ss->sh.qr_step, (unsigned)cget(ctl->k));
     bool fx = false;
     if constexpr (is_fp64<T>()) {
         fx = ce != nullptr;
         if (fx) st_mat_fx((int4*)coefS_w, ce + 2 * M_MAX, mk_, mn, [&](int i, int j) { return Sm[i * MM + j]; });
     }
     if (!fx) st_mat_work<T>(wprec, coefS_w, Sm, MM, mk_, mn);
-    if (threadIdx.x == 0) {
-        ctl->mnext = mn;
-        ctl->deflations = cget(ctl->deflations) + mk_ - mn;
-    }
 }
 
 // One shift's recurrences of block step k (a CTA per shift).
@@ -880,18 +886,23 @@ __global__ void __launch_bounds__(NT) small_recur_kernel(SmallStateT<T>* ss, Ctl
                                                          const double* __restrict__ sigma,
                                                          const double* __restrict__ target, int freeze, int wprec,
                                                          void* coefU_w, void* coefL_w, int* ce, int* active,
-                                                         int* conv_step, double* res_out, int MM, int ahead) {
-    // Launched ahead of v_update's end: the recurrences read nothing that
-    // v_update writes, and it let this kernel in after its own wait, that is
-    // with the QR complete; the last CTA waits for v_update before it closes
-    // the step (whose widths v_update reads), so this kernel ends after it.
-    if (!ahead) step_begin();
+                                                         int* conv_step, double* res_out, int MM, int step, int ahead) {
+    // Launched ahead of v_update's end: the recurrences of this step need the
+    // QR, not V = W S.  The QR releases the step's number after it has written
+    // what they take (all earlier kernels were complete for it); a CTA that
+    // acquires that number runs beside v_update, any other waits for v_update's
+    // end.  (It let this kernel in after its own wait, so the number is normally
+    // there.)  The last CTA waits for v_update before it closes the step, whose
+    // widths v_update reads, so this kernel ends after it.  The release and the
+    // acquire take 0.1-0.2 of the 7.3 ms of a 4^4 FP64 solve with m = 4.
+    const bool beside = ahead && __syncthreads_or(threadIdx.x == 0 && ld_acquire(&ss->sh.qr_step) == (unsigned)step);
+    if (!beside) step_begin();
     if (cget(ctl->done)) return;
     extern __shared__ __align__(16) unsigned char sm[];
     shift_recurrence<T>(ss, ctl, (int)blockIdx.x, m, sigma, target, freeze, wprec, coefU_w, coefL_w, ce, active,
                         conv_step, res_out, MM, sm);
     if (!last_arrival(&ss->sh.ticket[2])) return;
-    if (ahead) step_begin();
+    if (beside) step_begin();
     const int j = threadIdx.x;                     // s <= S_MAX shifts
     const int nalive = __syncthreads_count(j < s && __ldcg(&ss->sf[j < s ? j : 0].alive));
     const int nkd = __syncthreads_count(j < s && __ldcg(&active[j < s ? j : 0]));
@@ -971,18 +982,18 @@ void launch_small_qr(SmallState* ss, Ctl* ctl, const double* partials, int nblk,
 
 void launch_small_recur(SmallState* ss, Ctl* ctl, int s, int m, const double* sigma_dev, const double* target_dev,
                         int freeze, int wprec, int sfp64, void* coefU_w, void* coefL_w, int* ce, int* active,
-                        int* conv_step, double* res_out, Stream st) {
+                        int* conv_step, double* res_out, int step, Stream st) {
     static std::atomic<unsigned long long> devs64{0}, devsdd{0};
     max_dyn_smem_once(small_recur_kernel<double2>, (int)recur_smem(M_MAX), devs64);
     max_dyn_smem_once(small_recur_kernel<ddc>, (int)recur_smem(M_MAX), devsdd);
     if (sfp64)
         launch_step(small_recur_kernel<double2>, s, NT, recur_smem(m), st, as_state<double2>(ss), ctl, s, m, sigma_dev,
                                                                   target_dev, freeze, wprec, coefU_w, coefL_w, ce, active,
-                                                                  conv_step, res_out, m, st.ahead);
+                                                                  conv_step, res_out, m, step, st.ahead);
     else
         launch_step(small_recur_kernel<ddc>, s, NT, recur_smem(m), st, as_state<ddc>(ss), ctl, s, m, sigma_dev, target_dev,
                                                               freeze, wprec, coefU_w, coefL_w, ce, active, conv_step,
-                                                              res_out, m, st.ahead);
+                                                              res_out, m, step, st.ahead);
 }
 
 }  // namespace dsbcg

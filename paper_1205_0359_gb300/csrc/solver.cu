@@ -973,7 +973,8 @@ dsbcg_status lane_enqueue(dsbcg_ctx* c, Lane& L) {
             Prof p(c, DSBCG_KCLASS_SMALL, 1, st);
             launch_small_recur(L.ss, L.ctl, s_in, m_in, L.sigma, L.target, L.freeze, wp, L.sfp64,
                                (char*)L.coefU + (size_t)hs * s_in * cb, (char*)L.coefL + (size_t)hs * s_in * cb,
-                               ceUL ? ceUL + (size_t)hs * s_in * 2 * M_MAX : nullptr, L.active + (size_t)hs * s_in, L.conv_step, L.res, st);
+                               ceUL ? ceUL + (size_t)hs * s_in * 2 * M_MAX : nullptr, L.active + (size_t)hs * s_in, L.conv_step, L.res,
+                               step, st);
         }
         if (L.step - L.k0 == C) flush();
     }
