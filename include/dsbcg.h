@@ -269,7 +269,14 @@ dsbcg_status dsbcg_set_operator(dsbcg_ctx* ctx, int op);
 /* Apply D, D^H or A to m fields: out_i = op(in_i).  The fields are converted
  * to `storage` precision (any dsbcg_prec, including DSBCG_PREC_DF32), the
  * stencil runs in that precision (FP32 arithmetic for FP32/BF16/FP16,
- * double-float for DF32), and the result is converted back.
+ * double-float for DF32), and the result is converted back.  FP64 with links
+ * in SU(3) may run on the integer pipe, in block fixed point (57 bits and one
+ * exponent per site): every complex component of D, D^H and of each pass of A is
+ * then within 32 x 2^-53 of the sum of the magnitudes of its terms, |in| +
+ * |kappa| sum |U| |half spinor|, in the worst case (16 x 2^-53 for the FP64
+ * kernels); inputs for which the format cannot give that (components far below
+ * the rest of their site that nothing larger reaches, NaN, Inf, magnitudes near
+ * the ends of the FP64 range) are answered by the FP64 kernels.
  *   in, out: device or host complex128 [m][n]; they may not overlap. */
 dsbcg_status dsbcg_apply(dsbcg_ctx* ctx, int op, int storage, int m, const void* in, void* out);
 

@@ -16,11 +16,29 @@
 // |k'| < 1, [mu][entry][site]; links in SU(3) only (|u| <= 1).  The factor
 // 2^-ks is an exponent offset of the hopping term.
 //
-// Error.  A hop's result is exact to about one unit 2^E of its neighbour site
-// (the dropped l l products, the rounding of the h l sums and of k' u), and
-// the sum over eight hops adds up to one unit of the largest exponent per
-// hop, a unit being at most 2^-57 of the largest component of the nine sites
-// and typically 2^-60: below the 2^-53 per operation of an FP64 chain.
+// Error.  A unit is 2^Em, Em the largest exponent of the terms of a site.  A
+// hop is exact to 10 units at most: 2.5 from components rounded in the
+// conversion, 3.8 from the rounding of k' u, 1.5 from the dropped l l products
+// and 2 from shifts that round down (all of one sign); the diagonal term to 9
+// and a result kept in the format to 32.  Together 120 units in the worst case
+// and about 8 typically, a unit being at most 2^-57 of the largest component of
+// the nine sites times kappa.  That is an error bound per SITE: relative to the
+// largest component around it, below that of an FP64 chain.
+//
+// Components.  An FP64 chain of 16 operations has every single complex component
+// to 16 x 2^-53 of T, the sum of the magnitudes of its terms, also where all of
+// them are far below the site's largest component (a colour or spin that the
+// links do not mix with a larger one, a single site between zeros).  The format
+// does not.  An application that a caller sees (flag given, CHECK) therefore adds
+// up T, as |re| + |im| of the diagonal term and of each hop's share, and sets
+// *flag where T is below FX_LOW = 2^55 units and the nine sites are not all zero:
+// then the error can exceed 120 / 2^55 = 30 x 2^-53 of T, and dsbcg_apply repeats
+// the call with the FP64 kernels.  Dense fields do not come near: the smallest T
+// of 1.6 million components of Gaussian fields was 2^56.3 to 2^57.4 units (kappa
+// 0.11 to 0.13; half lattice 2^56.0), and the tail falls with the 16th power.
+// Sparse sources and fields that fall by decades from site to site do.  The check
+// takes 1% of an application (A to 12 fields of 16^3 x 32: 1.121 -> 1.133 ms).
+// A solve's applications do not check: its contract is the norm of the residual.
 //
 // Overflow.  The limbs of a projected half spinor are at most 2^29 (sums of
 // two), those of a link at most 2^29 and 2^28.  A link row has norm <= 1, so
@@ -28,7 +46,8 @@
 // sums below 2^61, a hop's result below 2^59.3 and the sum over eight hops and
 // the diagonal term below 2^62.4.
 //
-// A site that is all zero has exponent FX_ZERO.  A site with a NaN, an
+// A site that is all zero has exponent FX_ZERO.  A component that the
+// conversion holds as zero beside larger ones sets *flag.  A site with a NaN, an
 // infinity or a largest exponent outside the range in which every result is
 // a normal FP64 number sets *flag and turns its neighbourhood into NaN
 // (FX_NAN) or, when tiny, counts as zero; dsbcg_apply then repeats the
@@ -97,12 +116,15 @@ __global__ void __launch_bounds__(128) fx_convert_kernel(int4* __restrict__ out,
     const bool live = E != FX_ZERO && E != FX_NAN;
     eo[(size_t)f * V + x] = E;
     int4* o = out + (size_t)f * ld + fx_at(x);
+    bool lost = false;                         // a component that the format holds as zero
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
         const int2 re = fx_split(live ? fx_of_double(v[c].x, eb) : 0ll);
         const int2 im = fx_split(live ? fx_of_double(v[c].y, eb) : 0ll);
         o[c * 32] = make_int4(re.x, re.y, im.x, im.y);
+        lost |= !(re.x | re.y | im.x | im.y) && (v[c].x != 0.0 || v[c].y != 0.0);
     }
+    if (flag && lost && live) atomicOr(flag, 1);
 }
 
 // canonical links -> FX links [mu][entry][site]; kfix = -k' 2^63.  The product
@@ -133,6 +155,8 @@ __device__ __forceinline__ int4 isubi(int4 a, int4 b) { return make_int4(a.x + b
 struct ll2 {
     long long x, y;
 };
+// |v| 2^-32, to one unit
+__device__ __forceinline__ unsigned fx_high(long long v) { return (unsigned)abs((int)(v >> 32)); }
 // a += s q, s = +1 (PLUS) or -1, or s i q (ROT)
 template <bool PLUS, bool ROT>
 __device__ __forceinline__ void lacc(ll2& a, ll2 q) {
@@ -147,8 +171,9 @@ __device__ __forceinline__ void lacc(ll2& a, ll2 q) {
 // hop's exponent to the accumulators'.  MINUS: projector 1 - gamma_MU, else
 // 1 + gamma_MU.  The result goes to spin S (up) and to the lower spin it
 // rebuilds (lo): the other thread's for mu = x, y, this thread's for z, t.
-template <int MU, bool MINUS, int S, bool AHEAD>
-__device__ __forceinline__ void fx_hop(const int4* p, const int4* su, int sh, ll2 up[3], ll2 lo[3]) {
+// CHECK: mg[a] += |re| + |im| of the component's share (high words).
+template <int MU, bool MINUS, int S, bool AHEAD, bool CHECK>
+__device__ __forceinline__ void fx_hop(const int4* p, const int4* su, int sh, ll2 up[3], ll2 lo[3], unsigned mg[3]) {
     constexpr int T = MU < 2 ? 1 - S : S;                 // lower spin of the projection
     constexpr bool NEG = (MU == 1 || MU == 2) && S == 1 ? !MINUS : MINUS;
     int4 h[3];
@@ -183,6 +208,7 @@ __device__ __forceinline__ void fx_hop(const int4* p, const int4* su, int sh, ll
         ll2 q;
         q.x = (hr + (mr >> FX_BASE)) >> sh;
         q.y = (hi + (mi >> FX_BASE)) >> sh;
+        if (CHECK) mg[a] += fx_high(q.x) + fx_high(q.y);
         lacc<true, false>(up[a], q);
         // lower spins of 1 - gamma_mu: i q for x, (q1, -q0) for y, (i q0, -i q1)
         // for z and -q for t; the opposite for 1 + gamma_mu
@@ -195,16 +221,16 @@ __device__ __forceinline__ void fx_hop(const int4* p, const int4* su, int sh, ll
 
 // the four hops in x, y (HALFH = 0) or z, t (1); sy: their neighbour sites
 // (stride 32), sh: their shifts, six bits each
-template <bool DAG, int S, int HALFH, bool AHEAD>
+template <bool DAG, int S, int HALFH, bool AHEAD, bool CHECK>
 __device__ __forceinline__ void fx_hops(const int4* fin, const int* sy, const int4* sl, unsigned sh,
-                                        ll2 up[3], ll2 lo[3]) {
+                                        ll2 up[3], ll2 lo[3], unsigned mg[3]) {
     constexpr int HS = 9 * 32, M = 2 * HALFH;
     sy += 4 * 32 * HALFH;
     sl += 4 * HS * HALFH;
-    fx_hop<M, !DAG, S, AHEAD>(fin + fx_at(sy[0]), sl, (int)sh & 63, up, lo);
-    fx_hop<M, DAG, S, AHEAD>(fin + fx_at(sy[32]), sl + HS, (int)(sh >> 6) & 63, up, lo);
-    fx_hop<M + 1, !DAG, S, AHEAD>(fin + fx_at(sy[64]), sl + 2 * HS, (int)(sh >> 12) & 63, up, lo);
-    fx_hop<M + 1, DAG, S, AHEAD>(fin + fx_at(sy[96]), sl + 3 * HS, (int)(sh >> 18) & 63, up, lo);
+    fx_hop<M, !DAG, S, AHEAD, CHECK>(fin + fx_at(sy[0]), sl, (int)sh & 63, up, lo, mg);
+    fx_hop<M, DAG, S, AHEAD, CHECK>(fin + fx_at(sy[32]), sl + HS, (int)(sh >> 6) & 63, up, lo, mg);
+    fx_hop<M + 1, !DAG, S, AHEAD, CHECK>(fin + fx_at(sy[64]), sl + 2 * HS, (int)(sh >> 12) & 63, up, lo, mg);
+    fx_hop<M + 1, DAG, S, AHEAD, CHECK>(fin + fx_at(sy[96]), sl + 3 * HS, (int)(sh >> 18) & 63, up, lo, mg);
 }
 
 // out = src - kappa H in (H the hopping term; DAG: gamma_5 H gamma_5), fields
@@ -227,18 +253,20 @@ __device__ __forceinline__ void fx_hops(const int4* fin, const int* sy, const in
 // shapes: one thread per site and field 0.60 ms; 80 registers and 24 warps
 // 0.50 (spills); 2 or 3 fields per CTA 0.57-0.60 (links staged more often).
 constexpr int FX_FIELDS = 4;
+constexpr unsigned FX_LOW = 1u << 23;                          // 2^55 units
 static_assert(2 * FX_FIELDS <= 8, "the exchange of leading-zero counts reuses the 8 x 32 words of the sites");
 
-template <bool DAG, bool OUT64, bool HALF, bool AHEAD>
+template <bool DAG, bool OUT64, bool HALF, bool AHEAD, bool CHECK>
 __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
     void* __restrict__ outv, int* __restrict__ eo, const int4* in, const int* ei,
     const int4* src, const int* es, size_t ld, const int4* __restrict__ links, Geom g,
-    int kshift, int neg, int parity, Lay64 lo64, const Ctl* ctl, int nf_static, int ngrp) {
+    int kshift, int neg, int parity, Lay64 lo64, int* flag, const Ctl* ctl, int nf_static, int ngrp) {
     if (!AHEAD) step_begin();                                  // else after staging the links (as dslash_cta_kernel)
     extern __shared__ __align__(16) unsigned char fx_smem[];
     int4* sl = reinterpret_cast<int4*>(fx_smem);               // [hop][entry][lane]
     ll2* ex = reinterpret_cast<ll2*>(sl + 8 * 9 * 32);         // [warp][colour][lane]
     int* sy = reinterpret_cast<int*>(ex + 2 * FX_FIELDS * 3 * 32);     // [hop][lane]
+    unsigned* sg = reinterpret_cast<unsigned*>(sy + 8 * 32);           // CHECK: [warp][colour][lane], twice
     int nf = nf_static;
     const int nw = (int)(blockDim.x >> 5), nfc = nw >> 1;      // warps, fields of the CTA
     const int grp = (int)(blockIdx.x % (unsigned)ngrp);
@@ -304,16 +332,19 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
     int Em = FX_ZERO, e0 = FX_ZERO;
     const int4* fin = in + (size_t)f * ld;
     unsigned shl = 0, shh = 0;
-    // the diagonal term of spin s in the accumulators' unit (zero without src)
-    auto diag = [&](int s, ll2 d[3]) {
+    bool low = false;                                          // CHECK: a component whose terms are too small
+    // the diagonal term of spin s in the accumulators' unit (zero without src); CHECK: its magnitudes in dg
+    auto diag = [&](int s, ll2 d[3], unsigned dg[3]) {
         const int4* p = src + (size_t)f * ld + fx_at(ks) + s * 96;
         const int sr = max(0, min(Em - e0, 63)), sf = max(0, e0 - Em);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             d[a] = ll2{0, 0};
+            if (CHECK) dg[a] = 0;
             if (src) {
                 const int4 u = ld_prev<AHEAD>(p + a * 32);
                 d[a] = ll2{fx_join(u.x, u.y) >> sr << sf, fx_join(u.z, u.w) >> sr << sf};
+                if (CHECK) dg[a] = fx_high(d[a].x) + fx_high(d[a].y);
             }
         }
     };
@@ -333,16 +364,39 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
             shl |= (unsigned)min(Em - eh[h], 63) << (6 * h);
             shh |= (unsigned)min(Em - eh[4 + h], 63) << (6 * h);
         }
-        diag(S, up);
+        // CHECK: mg[a] sums the magnitudes of upper component a; the shares of the
+        // x, y hops also belong to the other warp's lower component (at), and
+        // own turns the sum into that of this thread's lower component
+        unsigned mg[3], dg[3];
+        unsigned *at = sg + (w * 3) * 32 + lane, *own = at + 2 * FX_FIELDS * 3 * 32;
+        diag(S, up, mg);
+        if (CHECK) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) own[a * 32] = mg[a];
+        }
 #pragma unroll
         for (int a = 0; a < 3; ++a) lo[a] = ll2{0, 0};
-        if (S == 0) fx_hops<DAG, 0, 0, AHEAD>(fin, sy + lane, sl + lane, shl, up, lo);
-        else fx_hops<DAG, 1, 0, AHEAD>(fin, sy + lane, sl + lane, shl, up, lo);
+        if (S == 0) fx_hops<DAG, 0, 0, AHEAD, CHECK>(fin, sy + lane, sl + lane, shl, up, lo, mg);
+        else fx_hops<DAG, 1, 0, AHEAD, CHECK>(fin, sy + lane, sl + lane, shl, up, lo, mg);
 #pragma unroll
         for (int a = 0; a < 3; ++a) ex[(w * 3 + a) * 32 + lane] = lo[a];
-        diag(2 + S, lo);
-        if (S == 0) fx_hops<DAG, 0, 1, AHEAD>(fin, sy + lane, sl + lane, shh, up, lo);
-        else fx_hops<DAG, 1, 1, AHEAD>(fin, sy + lane, sl + lane, shh, up, lo);
+        diag(2 + S, lo, dg);
+        if (CHECK) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                at[a * 32] = mg[a] - own[a * 32];
+                own[a * 32] = dg[a] - mg[a];
+            }
+        }
+        if (S == 0) fx_hops<DAG, 0, 1, AHEAD, CHECK>(fin, sy + lane, sl + lane, shh, up, lo, mg);
+        else fx_hops<DAG, 1, 1, AHEAD, CHECK>(fin, sy + lane, sl + lane, shh, up, lo, mg);
+        if (CHECK) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                own[a * 32] += mg[a];                          // without the x, y hops of the other warp
+                low |= mg[a] < FX_LOW;
+            }
+        }
     }
     __syncthreads();
     if (on) {
@@ -351,10 +405,15 @@ __global__ void __launch_bounds__(64 * FX_FIELDS, 2) fx_stencil_kernel(
             const ll2 q = ex[((w ^ 1) * 3 + a) * 32 + lane];
             lo[a].x += q.x;
             lo[a].y += q.y;
+            if (CHECK) {
+                low |= sg[((w ^ 1) * 3 + a) * 32 + lane] + sg[((w + 2 * FX_FIELDS) * 3 + a) * 32 + lane] < FX_LOW;
+            }
         }
     }
     const bool bad = Em > FX_NAN / 2;
     const bool store = on && k < Vf;
+    // (all nine sites zero: so is the result)
+    if (CHECK && store && low && Em > FX_ZERO / 2 && __ldcg(flag) == 0) atomicOr(flag, 1);
     if (OUT64) {
         // v 2^Em: the conversion rounds to FP64, the exponent is added to its bits (the result is a normal
         // number: FX_EB_MIN, FX_EB_MAX)
@@ -427,7 +486,7 @@ void launch_fx_convert(void* out, int* eo, const void* in, const Lay64& li, size
 
 void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const void* src, const int* es, size_t ld,
                        const void* links, const Geom& g, double kappa, int dag, int half, int parity, const Lay64* lo,
-                       const Ctl* ctl, int nf_static, int nf_max, Stream st) {
+                       int* flag, const Ctl* ctl, int nf_static, int nf_max, Stream st) {
     const int nfg = ctl ? nf_max : nf_static;
     const int nfc = nfg < FX_FIELDS ? nfg : FX_FIELDS;
     const int ngrp = (nfg + nfc - 1) / nfc;
@@ -437,16 +496,22 @@ void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const 
     fx_mantissa(kappa, &ks);
     const int neg = src ? 0 : 1;
     const Lay64 l64 = lo ? *lo : Lay64{};
-    constexpr int SMEM = 8 * 9 * 32 * sizeof(int4) + 2 * FX_FIELDS * 3 * 32 * sizeof(ll2) + 8 * 32 * sizeof(int);
-#define DSBCG_FX2(DAG, O64, HALF, AHEAD)                                                                            \
+    constexpr int SMEM0 = 8 * 9 * 32 * sizeof(int4) + 2 * FX_FIELDS * 3 * 32 * sizeof(ll2) + 8 * 32 * sizeof(int);
+    constexpr int SMEMC = SMEM0 + 2 * 2 * FX_FIELDS * 3 * 32 * sizeof(unsigned);
+#define DSBCG_FX2(DAG, O64, HALF, AHEAD, CHECK)                                                                     \
     {                                                                                                              \
+        constexpr int SMEM = CHECK ? SMEMC : SMEM0;                                                                \
         static std::atomic<unsigned long long> devs{0};                                                            \
-        max_dyn_smem_once(fx_stencil_kernel<DAG, O64, HALF, AHEAD>, SMEM, devs);                                   \
-        launch_step(fx_stencil_kernel<DAG, O64, HALF, AHEAD>, grid, 64 * nfc, SMEM, st, out, eo, (const int4*)in, ei, \
-                    (const int4*)src, es, ld, (const int4*)links, g, ks, neg, parity, l64, ctl, nf_static, ngrp);  \
+        max_dyn_smem_once(fx_stencil_kernel<DAG, O64, HALF, AHEAD, CHECK>, SMEM, devs);                            \
+        launch_step(fx_stencil_kernel<DAG, O64, HALF, AHEAD, CHECK>, grid, 64 * nfc, SMEM, st, out, eo,            \
+                    (const int4*)in, ei, (const int4*)src, es, ld, (const int4*)links, g, ks, neg, parity, l64,    \
+                    flag, ctl, nf_static, ngrp);                                                                   \
     }
-#define DSBCG_FX(DAG, O64, HALF) \
-    if (st.ahead) DSBCG_FX2(DAG, O64, HALF, true) else DSBCG_FX2(DAG, O64, HALF, false)
+    // (an application that checks its components is never launched ahead)
+#define DSBCG_FX(DAG, O64, HALF)                          \
+    if (flag) DSBCG_FX2(DAG, O64, HALF, false, true)      \
+    else if (st.ahead) DSBCG_FX2(DAG, O64, HALF, true, false) \
+    else DSBCG_FX2(DAG, O64, HALF, false, false)
 #define DSBCG_FX1(O64, HALF) \
     if (dag) { DSBCG_FX(true, O64, HALF) } else { DSBCG_FX(false, O64, HALF) }
     if (half) {

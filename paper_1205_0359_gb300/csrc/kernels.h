@@ -100,15 +100,18 @@ struct Lay64 {
 };
 inline Lay64 lay64_pairs(size_t ld, size_t Vf) { return Lay64{ld, 2 * Vf, 2}; }       // pair-chunk fields, stride ld
 inline Lay64 lay64_canonical(size_t Vf) { return Lay64{12 * Vf, 2, 12}; }             // the ABI's [site][component]
-// FP64 fields (li, Vf sites) -> FX; *flag |= 1 where the FX range does not hold (flag may be NULL)
+// FP64 fields (li, Vf sites) -> FX; flag (or NULL): *flag |= 1 where the FX
+// range does not hold or a component of a site is lost under the others
 void launch_fx_convert(void* out, int* eo, const void* in, const Lay64& li, size_t ld, size_t Vf, const Ctl* ctl,
                        int nf_static, int nf_max, int* flag, Stream st);
 // out = src - kappa H in (dag: gamma_5 H gamma_5), or kappa H in when src is
 // NULL.  Full lattice (half = 0) or half fields on `parity`; lo: FP64 output
-// laid out so, else (NULL) FX
+// laid out so, else (NULL) FX.  flag (or NULL): *flag |= 1 where a component is
+// not to 32 x 2^-53 of the magnitudes of its terms (FX_LOW); never with a Stream
+// that launches ahead
 void launch_fx_stencil(void* out, int* eo, const void* in, const int* ei, const void* src, const int* es, size_t ld,
                        const void* links, const Geom& g, double kappa, int dag, int half, int parity, const Lay64* lo,
-                       const Ctl* ctl, int nf_static, int nf_max, Stream st);
+                       int* flag, const Ctl* ctl, int nf_static, int nf_max, Stream st);
 
 // ---- blas.cu ----------------------------------------------------------------
 int gram_blocks(size_t n, int nf_max);

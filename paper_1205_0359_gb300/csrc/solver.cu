@@ -355,6 +355,12 @@ dsbcg_status ensure_fx_links(dsbcg_ctx* c) {
     return DSBCG_OK;
 }
 
+// Applications that a caller sees check every component (dslash_fx.cu), and
+// below |kappa| = 2^-6 the hops are so small that dense fields, whose diagonal
+// term is all that is left of them, have components that fail.  Those
+// applications take the FP64 kernels at once.
+bool fx_component_kappa(double kappa) { return fabs(kappa) >= 1.0 / 64; }
+
 // True residuals of m columns in fixed point: always for FP64 storage, and for
 // the reduced storages from FX_RESID_MIN sites x columns of the full lattice.
 // Below it the FP64 residuals run beside latency-bound restarts and cost
@@ -729,14 +735,14 @@ void fx_normal(dsbcg_ctx* c, void* out, const Lay64& lo, void* conv, void* mid, 
             {
                 Prof q(c, cls, 1, st);
                 launch_fx_stencil(tmp, e2, x, ex, nullptr, nullptr, ld, c->linksfx, c->g, c->kappa, dag, 1, 0, nullptr,
-                                  ctl, nf_static, nf_max, st);
+                                  flag, ctl, nf_static, nf_max, st);
             }
             Prof q(c, cls, 1, st);
-            launch_fx_stencil(y, e1, tmp, e2, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, l, ctl, nf_static,
+            launch_fx_stencil(y, e1, tmp, e2, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, l, flag, ctl, nf_static,
                               nf_max, st);
         } else {
             Prof q(c, cls, 1, st);
-            launch_fx_stencil(y, e1, x, ex, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, l, ctl, nf_static,
+            launch_fx_stencil(y, e1, x, ex, x, ex, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, l, flag, ctl, nf_static,
                               nf_max, st);
         }
     }
@@ -1774,16 +1780,16 @@ void fx_apply(dsbcg_ctx* c, int op, double2* out, void* conv, void* t, void* t2,
     if (c->schur) {
         {
             Prof q(c, DSBCG_KCLASS_DSLASH);
-            launch_fx_stencil(t, e1, conv, e0, nullptr, nullptr, ld, c->linksfx, c->g, c->kappa, dag, 1, 0, nullptr, nullptr,
-                              m, m, c->st);
+            launch_fx_stencil(t, e1, conv, e0, nullptr, nullptr, ld, c->linksfx, c->g, c->kappa, dag, 1, 0, nullptr,
+                              c->flags, nullptr, m, m, c->st);
         }
         Prof q(c, DSBCG_KCLASS_DSLASH);
-        launch_fx_stencil(out, nullptr, t, e1, conv, e0, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, &l, nullptr, m, m,
-                          c->st);
+        launch_fx_stencil(out, nullptr, t, e1, conv, e0, ld, c->linksfx, c->g, c->kappa, dag, 1, 1, &l, c->flags, nullptr, m,
+                          m, c->st);
     } else {
         Prof q(c, DSBCG_KCLASS_DSLASH);
-        launch_fx_stencil(out, nullptr, conv, e0, conv, e0, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, &l, nullptr, m, m,
-                          c->st);
+        launch_fx_stencil(out, nullptr, conv, e0, conv, e0, ld, c->linksfx, c->g, c->kappa, dag, 0, 0, &l, c->flags, nullptr,
+                          m, m, c->st);
     }
 }
 
@@ -1796,8 +1802,8 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     const size_t n = c->n, ld = hp_ld(c, storage);
     const size_t fb = prec_elem_bytes(storage) * c->ld;
     const bool in_dev = is_device_ptr(in), out_dev = is_device_ptr(out);
-    if (fixed && storage == P64) CKS(ensure_fx_links(c));
-    bool fx = fixed && storage == P64 && c->linksfx;
+    if (fixed && storage == P64 && fx_component_kappa(c->kappa)) CKS(ensure_fx_links(c));
+    bool fx = fixed && storage == P64 && c->linksfx && fx_component_kappa(c->kappa);
     const size_t db = m * n * sizeof(double2);
     Scratch& scr = c->scr;
     const size_t fields = c->schur ? 4 : 3;      // packed in, out and middle fields, and the even-parity ones
@@ -1813,7 +1819,7 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     double2* din = in_dev ? nullptr : (double2*)scratch_take(scr, db);
     double2* dout = out_dev ? nullptr : (double2*)scratch_take(scr, db);
     dsbcg_status rs = DSBCG_OK;
-    int left = 0;                        // a site was outside the fixed-point range
+    int left = 0;                        // a component was outside what fixed point holds
     auto fail = [&](dsbcg_status s) { rs = s; };
     if (!in_dev) cudaMemcpyAsync(din, in, db, cudaMemcpyHostToDevice, c->st);
     {
@@ -1839,8 +1845,8 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
         if (cudaStreamSynchronize(c->st) != cudaSuccess) fail(DSBCG_ERR_CUDA);
         prof_collect(c);
     }
-    // a site outside the fixed-point range (NaN, Inf, extreme magnitudes):
-    // the FP64 kernels' result replaces this one
+    // a site outside the fixed-point range (NaN, Inf, extreme magnitudes) or a
+    // component too small for it: the FP64 kernels' result replaces this one
     const bool again = rs == DSBCG_OK && left;
     scratch_trim(scr);
     return again ? apply_fields(c, op, storage, m, in, out, false) : rs;
