@@ -1808,23 +1808,29 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     Scratch& scr = c->scr;
     const size_t fields = c->schur ? 4 : 3;      // packed in, out and middle fields, and the even-parity ones
     const size_t host = (in_dev ? 0 : scratch_round(db)) + (out_dev ? 0 : scratch_round(db));
+    // in and out may share memory: the result of an application that may be
+    // repeated from `in` is then held back until it stands
+    const bool overlap = (const char*)in < (const char*)out + db && (const char*)out < (const char*)in + db;
+    const size_t held = overlap && out_dev ? scratch_round(db) : 0;
     // without room for the site exponents the FP64 kernels serve the call
-    if (fx && scratch_get(scr, (fields - 1) * scratch_round(m * fb) + scratch_round(fx_exp_bytes(c, m)) + host) != DSBCG_OK)
+    if (fx && scratch_get(scr, (fields - 1) * scratch_round(m * fb) + scratch_round(fx_exp_bytes(c, m)) + host + held) !=
+                  DSBCG_OK)
         fx = false;
     if (!fx) CKS(scratch_get(scr, fields * scratch_round(m * fb) + host));
+    const bool hold = fx && overlap, direct = out_dev && !hold;
     void *a = scratch_take(scr, m * fb), *t = scratch_take(scr, m * fb);
     void* b = fx ? nullptr : scratch_take(scr, m * fb);
     void* t2 = c->schur ? scratch_take(scr, m * fb) : nullptr;
     int* fxe = fx ? (int*)scratch_take(scr, fx_exp_bytes(c, m)) : nullptr;
     double2* din = in_dev ? nullptr : (double2*)scratch_take(scr, db);
-    double2* dout = out_dev ? nullptr : (double2*)scratch_take(scr, db);
+    double2* dout = direct ? nullptr : (double2*)scratch_take(scr, db);
     dsbcg_status rs = DSBCG_OK;
     int left = 0;                        // a component was outside what fixed point holds
     auto fail = [&](dsbcg_status s) { rs = s; };
     if (!in_dev) cudaMemcpyAsync(din, in, db, cudaMemcpyHostToDevice, c->st);
     {
         const double2* src = in_dev ? (const double2*)in : din;
-        double2* dst = out_dev ? (double2*)out : dout;
+        double2* dst = direct ? (double2*)out : dout;
         if (!fxe) pack_any(c, storage, a, src, m);
         if (fxe) {
             fx_apply(c, op, dst, a, t, t2, src, m, fxe);
@@ -1839,10 +1845,14 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
                           c->hscale, c->st, c->links12[storage]);
         }
         if (!fxe) unpack_any(c, storage, dst, b, m);
-        if (!out_dev) cudaMemcpyAsync(out, dout, m * n * sizeof(double2), cudaMemcpyDeviceToHost, c->st);
+        if (!out_dev && !hold) cudaMemcpyAsync(out, dout, db, cudaMemcpyDeviceToHost, c->st);
         if (fxe) cudaMemcpyAsync(&left, c->flags, sizeof(int), cudaMemcpyDeviceToHost, c->st);
         if (cudaGetLastError() != cudaSuccess) fail(DSBCG_ERR_CUDA);
         if (cudaStreamSynchronize(c->st) != cudaSuccess) fail(DSBCG_ERR_CUDA);
+        if (hold && rs == DSBCG_OK && !left) {
+            cudaMemcpyAsync(out, dout, db, out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->st);
+            if (cudaStreamSynchronize(c->st) != cudaSuccess) fail(DSBCG_ERR_CUDA);
+        }
         prof_collect(c);
     }
     // a site outside the fixed-point range (NaN, Inf, extreme magnitudes) or a
