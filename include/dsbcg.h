@@ -347,6 +347,11 @@ dsbcg_status dsbcg_debug_first_wait(dsbcg_ctx* ctx, int polls);
  * DSBCG_ERR_ARG. */
 dsbcg_status dsbcg_debug_shift_chunk(dsbcg_ctx* ctx, int steps);
 
+/* Test hook for the out-of-memory paths; not for production use.  A device
+ * allocation that would take the context's device memory beyond `bytes` fails as
+ * one that cudaMalloc refuses; bytes < 0 removes the limit (the default). */
+dsbcg_status dsbcg_debug_memory_limit(dsbcg_ctx* ctx, long long bytes);
+
 /* Per-kernel CUDA-event timing inside dsbcg_solve (off by default). */
 dsbcg_status dsbcg_set_profiling(dsbcg_ctx* ctx, int on);
 

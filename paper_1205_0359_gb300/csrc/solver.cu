@@ -34,6 +34,7 @@
 #include <functional>
 #include <mutex>
 #include <thread>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/dsbcg.h"
@@ -60,6 +61,33 @@ struct DevBuf {
 struct Scratch {
     char* p = nullptr;
     size_t bytes = 0, used = 0;
+};
+
+// The device memory a context holds, with a limit that a test can set
+// (dsbcg_debug_memory_limit): an allocation beyond it fails as cudaMalloc does.
+struct DevMem {
+    size_t limit = (size_t)-1, held = 0;
+    std::unordered_map<void*, size_t> sizes;
+    cudaError_t get(void** p, size_t bytes) {
+        *p = nullptr;
+        if (bytes > limit || held > limit - bytes) return cudaErrorMemoryAllocation;
+        const cudaError_t e = cudaMalloc(p, bytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            *p = nullptr;
+            return e;
+        }
+        sizes[*p] = bytes;
+        held += bytes;
+        return e;
+    }
+    void give(void* p) {
+        const auto it = sizes.find(p);
+        if (it == sizes.end()) return;
+        held -= it->second;
+        sizes.erase(it);
+        cudaFree(p);
+    }
 };
 
 struct KEvent {
@@ -128,6 +156,7 @@ struct dsbcg_ctx {
     void *links12_mem[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     void* linksfx_mem = nullptr;
     int* flags = nullptr;                // device words: [0] fixed-point range left, [1, 2] gauge checks
+    DevMem mem;                          // every device block below
     Scratch scr;                         // working fields of apply and force
     float hscale = 1.f;
     bool gauge_ok = false;               // gauge64 holds a checked field and links[] were packed from it
@@ -159,6 +188,7 @@ struct dsbcg_ctx {
         int* fxe = nullptr;                                       // site exponents of the true residuals' fields
         bool fx = false;                                          // sized with the exponents (where there was room)
         bool fx_resid = false;                                    // true residuals take the fixed-point stencil
+        bool no_fx = false;                                       // fits only without the fixed-point buffers
         void *P = nullptr, *Xin = nullptr;                        // work precision
         double2 *B64 = nullptr, *X64 = nullptr, *R64 = nullptr, *T64a = nullptr, *T64b = nullptr, *rhs = nullptr;
         double2 *Xg = nullptr, *Bg = nullptr;
@@ -243,9 +273,8 @@ void* mapped_host_ptr(const void* p) {
 
 dsbcg_status dmalloc(dsbcg_ctx* c, void** p, size_t bytes) {
     if (bytes == 0) bytes = 16;
-    cudaError_t e = cudaMalloc(p, bytes);
+    cudaError_t e = c->mem.get(p, bytes);
     if (e != cudaSuccess) {
-        cudaGetLastError();
         size_t fr = 0, tot = 0;
         cudaMemGetInfo(&fr, &tot);
         cudaGetLastError();
@@ -267,7 +296,7 @@ void free_ws(dsbcg_ctx* c) {
         if (L.ready) cudaEventDestroy(L.ready);
     }
     for (void* p : c->ws.pinned) cudaFreeHost(p);
-    for (void* p : c->ws.mem) cudaFree(p);
+    for (void* p : c->ws.mem) c->mem.give(p);
     c->ws.mem.clear();
     if (c->ws.h_ctl) cudaFreeHost(c->ws.h_ctl);
     if (c->ws.h_norms) cudaFreeHost(c->ws.h_norms);
@@ -279,19 +308,27 @@ void free_ws(dsbcg_ctx* c) {
 size_t prec_elem_bytes(int p) { return (size_t)prec_bytes(p); }
 
 void scratch_free(dsbcg_ctx* c) {
-    if (c->scr.p) cudaFree(c->scr.p);
+    if (c->scr.p) c->mem.give(c->scr.p);
     c->scr = Scratch();
+}
+// Give back the links of the fixed-point stencil, an option that must not cost
+// a call the memory it needs: the FP64 stencil then runs on the FP64 pipe.
+// True if there was something to give back.
+bool fx_links_free(dsbcg_ctx* c) {
+    if (!c->linksfx_mem) return false;
+    c->mem.give(c->linksfx_mem);         // (cudaFree waits for the kernels that read it)
+    c->linksfx = c->linksfx_mem = nullptr;
+    return true;
 }
 // Make at least `bytes` of scratch available and start handing it out anew
 // (scratch_take).  The calls that use it run on the context's stream alone and
 // wait for it before they return, so a later call may write it.
-dsbcg_status scratch_get(Scratch& s, size_t bytes) {
+dsbcg_status scratch_get(dsbcg_ctx* c, size_t bytes) {
+    Scratch& s = c->scr;
     s.used = 0;
     if (s.bytes >= bytes) return DSBCG_OK;
-    if (s.p) cudaFree(s.p);
-    s = Scratch();
-    if (cudaMalloc((void**)&s.p, bytes) != cudaSuccess) {
-        cudaGetLastError();
+    scratch_free(c);
+    if (c->mem.get((void**)&s.p, bytes) != cudaSuccess) {
         s.p = nullptr;
         return DSBCG_ERR_OOM;
     }
@@ -308,24 +345,21 @@ void* scratch_take(Scratch& s, size_t bytes) {
 // Kept blocks are at most 1/32 of the device memory; cudaMalloc and cudaFree
 // cost 0.65 ms of a 1.0 ms application of A to 12 FP32 fields of 16^3 x 32, and
 // 3.2 of 7.1 ms of a force call.
-void scratch_trim(Scratch& s) {
+void scratch_trim(dsbcg_ctx* c) {
+    const Scratch& s = c->scr;
     size_t fr = 0, tot = 0;
     if (s.bytes <= (64u << 20)) return;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) cudaGetLastError();
-    if (s.bytes > tot / 32) {
-        cudaFree(s.p);
-        s = Scratch();
-    }
+    if (s.bytes > tot / 32) scratch_free(c);
 }
 
 // a buffer of packed links, kept for the context's life
 dsbcg_status link_alloc(dsbcg_ctx* c, void** p, size_t bytes_per_site) {
-    if (*p || cudaMalloc(p, c->V * bytes_per_site) == cudaSuccess) return DSBCG_OK;
-    cudaGetLastError();
+    const size_t bytes = c->V * bytes_per_site;
+    if (*p || c->mem.get(p, bytes) == cudaSuccess) return DSBCG_OK;
     scratch_free(c);
-    if (cudaMalloc(p, c->V * bytes_per_site) == cudaSuccess) return DSBCG_OK;
-    cudaGetLastError();
-    *p = nullptr;
+    if (c->mem.get(p, bytes) == cudaSuccess) return DSBCG_OK;
+    if (fx_links_free(c) && c->mem.get(p, bytes) == cudaSuccess) return DSBCG_OK;
     return DSBCG_ERR_OOM;
 }
 
@@ -344,10 +378,16 @@ dsbcg_status ensure_links(dsbcg_ctx* c, int prec) {
     return DSBCG_OK;
 }
 
+// scratch_get for what a call cannot do without
+dsbcg_status scratch_must(dsbcg_ctx* c, size_t bytes) {
+    const dsbcg_status rs = scratch_get(c, bytes);
+    return rs != DSBCG_OK && fx_links_free(c) ? scratch_get(c, bytes) : rs;
+}
+
 // The links of the fixed-point stencil, on first use.  They are an option:
 // without memory for them the FP64 stencil runs on the FP64 pipe.
 dsbcg_status ensure_fx_links(dsbcg_ctx* c) {
-    if (!c->su3 || c->linksfx || !fx_kappa_fits(c->kappa)) return DSBCG_OK;
+    if (!c->su3 || c->linksfx || c->ws.no_fx || !fx_kappa_fits(c->kappa)) return DSBCG_OK;
     if (link_alloc(c, &c->linksfx_mem, 36 * sizeof(double2)) != DSBCG_OK) return DSBCG_OK;
     launch_fx_links(c->linksfx_mem, c->gauge64, c->V, c->kappa, c->st);
     CK(cudaGetLastError());
@@ -406,10 +446,15 @@ int stream_prio(bool refinement) {
 // exponents of a lane's coefficient tiles: a, bh, S, and U, L per chunk slot and shift
 size_t ce_bytes(int chunk, int s) { return (3 + 2 * (size_t)chunk * s) * M_MAX * sizeof(int); }
 
+bool ws_serves(const dsbcg_ctx* c, int m, int s, int prec, int nbb) {
+    const auto& w = c->ws;
+    return w.prec == prec && w.m == m && w.s >= s && w.nbb >= nbb;
+}
+
 dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
     auto& w = c->ws;
     const bool fx = c->linksfx && fx_residuals(c, prec, m);
-    if (w.prec == prec && w.m == m && w.s >= s && w.nbb >= nbb && (!fx || w.fx)) return DSBCG_OK;
+    if (ws_serves(c, m, s, prec, nbb) && (!fx || w.fx)) return DSBCG_OK;
     free_ws(c);
     scratch_free(c);                     // the workspace sizes itself by the memory that is free
     const size_t ld = c->ld, n = c->n;
@@ -468,10 +513,10 @@ dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
     int chunk0 = chunk_steps((size_t)m * fb, 16, 16);
     for (;; chunk0 /= 2) {
         void *ring = nullptr, *cu = nullptr, *cl = nullptr, *act = nullptr;
-        if (cudaMalloc(&ring, (size_t)(chunk0 + 1) * m * fb) == cudaSuccess &&
-            cudaMalloc(&cu, (size_t)chunk0 * s * tb) == cudaSuccess &&
-            cudaMalloc(&cl, (size_t)chunk0 * s * tb) == cudaSuccess &&
-            cudaMalloc(&act, (size_t)chunk0 * s * sizeof(int)) == cudaSuccess) {
+        if (c->mem.get(&ring, (size_t)(chunk0 + 1) * m * fb) == cudaSuccess &&
+            c->mem.get(&cu, (size_t)chunk0 * s * tb) == cudaSuccess &&
+            c->mem.get(&cl, (size_t)chunk0 * s * tb) == cudaSuccess &&
+            c->mem.get(&act, (size_t)chunk0 * s * sizeof(int)) == cudaSuccess) {
             w.vring = ring;
             w.coefU = cu;
             w.coefL = cl;
@@ -479,9 +524,7 @@ dsbcg_status ensure_ws(dsbcg_ctx* c, int m, int s, int prec, int nbb) {
             for (void* q : {ring, cu, cl, act}) w.mem.push_back(q);
             break;
         }
-        cudaGetLastError();
-        for (void* q : {ring, cu, cl, act})
-            if (q) cudaFree(q);
+        for (void* q : {ring, cu, cl, act}) c->mem.give(q);
         if (chunk0 == 1) {
             fprintf(stderr, "dsbcg: device allocation of the two-block basis ring (%zu bytes) failed\n",
                     (size_t)2 * m * fb);
@@ -1108,11 +1151,19 @@ dsbcg_status solve_core(dsbcg_ctx* c, int m, const void* B, int nbb, int s, cons
     // significands) for the reduced storages; the m x m work likewise
     const int sfp64 = (!mixed || prm.fp64_residuals) ? 1 : 0;
     const int hp = sfp64 ? P64 : PDD;
+    if (!ws_serves(c, m, s, prec, nbb)) free_ws(c);
     CKS(ensure_links(c, prec));
     CKS(ensure_links(c, hp));
     if (hp == P64 && fx_residuals(c, prec, m)) CKS(ensure_fx_links(c));
-    CKS(ensure_ws(c, m, s, prec, nbb));
     auto& w = c->ws;
+    // the fixed-point links and exponents are an option: a workspace that does
+    // not fit beside them is sized without, and keeps them off while it lasts
+    dsbcg_status ws = ensure_ws(c, m, s, prec, nbb);
+    if (ws == DSBCG_ERR_OOM && fx_links_free(c)) {
+        ws = ensure_ws(c, m, s, prec, nbb);
+        w.no_fx = ws == DSBCG_OK;
+    }
+    CKS(ws);
     w.fx_resid = fx_residuals(c, prec, m);
     const size_t n = c->n, ld = c->ld;
     const size_t db = ld * sizeof(double2);
@@ -1667,8 +1718,8 @@ dsbcg_status dsbcg_update_gauge(dsbcg_ctx* c, const void* gauge) {
     for (int p = 0; p < 5; ++p) c->links[p] = c->links12[p] = nullptr;
     c->linksfx = nullptr;
     const size_t bytes = c->V * 36 * sizeof(double2);
-    if (!c->gauge64) CK(cudaMalloc((void**)&c->gauge64, bytes));
-    if (!c->flags) CK(cudaMalloc((void**)&c->flags, 4 * sizeof(int)));
+    if (!c->gauge64) CK(c->mem.get((void**)&c->gauge64, bytes));
+    if (!c->flags) CK(c->mem.get((void**)&c->flags, 4 * sizeof(int)));
     CK(cudaMemcpyAsync(c->gauge64, gauge, bytes, is_device_ptr(gauge) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                        c->st));
     CK(cudaMemsetAsync(c->flags + 1, 0, 2 * sizeof(int), c->st));
@@ -1704,13 +1755,13 @@ void dsbcg_destroy(dsbcg_ctx* c) {
     if (!c) return;
     free_ws(c);
     scratch_free(c);
+    fx_links_free(c);
     for (int p = 0; p < 5; ++p) {
-        if (c->links_mem[p]) cudaFree(c->links_mem[p]);
-        if (c->links12_mem[p]) cudaFree(c->links12_mem[p]);
+        c->mem.give(c->links_mem[p]);
+        c->mem.give(c->links12_mem[p]);
     }
-    if (c->linksfx_mem) cudaFree(c->linksfx_mem);
-    if (c->flags) cudaFree(c->flags);
-    if (c->gauge64) cudaFree(c->gauge64);
+    c->mem.give(c->flags);
+    c->mem.give(c->gauge64);
     if (c->rst) cudaStreamDestroy(c->rst);
     if (c->ev_joint) cudaEventDestroy(c->ev_joint);
     if (c->ev_ref) cudaEventDestroy(c->ev_ref);
@@ -1725,6 +1776,12 @@ void dsbcg_destroy(dsbcg_ctx* c) {
 dsbcg_status dsbcg_debug_shift_chunk(dsbcg_ctx* c, int steps) {
     if (!c || steps < 0 || steps > CTL_HIST) return DSBCG_ERR_ARG;
     c->force_chunk = steps;
+    return DSBCG_OK;
+}
+
+dsbcg_status dsbcg_debug_memory_limit(dsbcg_ctx* c, long long bytes) {
+    if (!c) return DSBCG_ERR_ARG;
+    c->mem.limit = bytes < 0 ? (size_t)-1 : (size_t)bytes;
     return DSBCG_OK;
 }
 
@@ -1812,11 +1869,11 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     // repeated from `in` is then held back until it stands
     const bool overlap = (const char*)in < (const char*)out + db && (const char*)out < (const char*)in + db;
     const size_t held = overlap && out_dev ? scratch_round(db) : 0;
-    // without room for the site exponents the FP64 kernels serve the call
-    if (fx && scratch_get(scr, (fields - 1) * scratch_round(m * fb) + scratch_round(fx_exp_bytes(c, m)) + host + held) !=
+    // without room beside the fixed-point links the FP64 kernels serve the call
+    if (fx && scratch_get(c, (fields - 1) * scratch_round(m * fb) + scratch_round(fx_exp_bytes(c, m)) + host + held) !=
                   DSBCG_OK)
         fx = false;
-    if (!fx) CKS(scratch_get(scr, fields * scratch_round(m * fb) + host));
+    if (!fx) CKS(scratch_must(c, fields * scratch_round(m * fb) + host));
     const bool hold = fx && overlap, direct = out_dev && !hold;
     void *a = scratch_take(scr, m * fb), *t = scratch_take(scr, m * fb);
     void* b = fx ? nullptr : scratch_take(scr, m * fb);
@@ -1858,7 +1915,7 @@ dsbcg_status apply_fields(dsbcg_ctx* c, int op, int storage, int m, const void* 
     // a site outside the fixed-point range (NaN, Inf, extreme magnitudes) or a
     // component too small for it: the FP64 kernels' result replaces this one
     const bool again = rs == DSBCG_OK && left;
-    scratch_trim(scr);
+    scratch_trim(c);
     return again ? apply_fields(c, op, storage, m, in, out, false) : rs;
 }
 
@@ -1902,8 +1959,8 @@ dsbcg_status dsbcg_force(dsbcg_ctx* c, int m, int s, const void* X, const void* 
     // the kernel writes 16-byte elements: straight into the caller's device buffer when it is aligned to them
     const bool direct = ud && (size_t)dU % sizeof(double2) == 0;
     Scratch& scr = c->scr;
-    CKS(scratch_get(scr, 4 * scratch_round(nf * fb) + (direct ? 0 : scratch_round(ub)) + scratch_round(nf * sizeof(double)) +
-                                (xd && ldv ? 0 : scratch_round(cb))));
+    CKS(scratch_must(c, 4 * scratch_round(nf * fb) + (direct ? 0 : scratch_round(ub)) + scratch_round(nf * sizeof(double)) +
+                            (xd && ldv ? 0 : scratch_round(cb))));
     void *xf = scratch_take(scr, nf * fb), *lf = scratch_take(scr, nf * fb), *ex = scratch_take(scr, nf * fb),
          *el = scratch_take(scr, nf * fb);
     double2* du = direct ? (double2*)dU : (double2*)scratch_take(scr, ub);
@@ -1939,7 +1996,7 @@ dsbcg_status dsbcg_force(dsbcg_ctx* c, int m, int s, const void* X, const void* 
         if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(c->st) != cudaSuccess) rs = DSBCG_ERR_CUDA;
         prof_collect(c);
     }
-    scratch_trim(scr);
+    scratch_trim(c);
     return rs;
 }
 
@@ -1967,9 +2024,11 @@ dsbcg_status dsbcg_backward(dsbcg_ctx* c, int m, const void* B, int s, const dou
     const bool need_x = gsigma || gU;
     std::vector<void*> owned;
     auto dalloc = [&](void** p, size_t bytes) -> dsbcg_status {
-        if (cudaMalloc(p, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            return DSBCG_ERR_OOM;
+        if (c->mem.get(p, bytes) != cudaSuccess) {
+            // what the context could do without goes first
+            scratch_free(c);
+            fx_links_free(c);
+            if (c->mem.get(p, bytes) != cudaSuccess) return DSBCG_ERR_OOM;
         }
         owned.push_back(*p);
         return DSBCG_OK;
@@ -2068,7 +2127,7 @@ dsbcg_status dsbcg_backward(dsbcg_ctx* c, int m, const void* B, int s, const dou
     };
     rs = run();
     cudaStreamSynchronize(c->st);
-    for (void* p : owned) cudaFree(p);
+    for (void* p : owned) c->mem.give(p);
     if (stats) {
         stats->block_steps = steps;
         stats->mvms = mvms;

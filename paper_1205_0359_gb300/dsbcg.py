@@ -97,6 +97,8 @@ def lib():
     L.dsbcg_debug_first_wait.restype = ip
     L.dsbcg_debug_shift_chunk.argtypes = [vp, ip]
     L.dsbcg_debug_shift_chunk.restype = ip
+    L.dsbcg_debug_memory_limit.argtypes = [vp, ctypes.c_longlong]
+    L.dsbcg_debug_memory_limit.restype = ip
     L.dsbcg_set_operator.argtypes = [vp, ip]
     L.dsbcg_set_operator.restype = ip
     L.dsbcg_set_profiling.argtypes = [vp, ip]
@@ -189,6 +191,11 @@ class Context:
         """dsbcg_debug_shift_chunk (test hook): caps the shift-update chunk
         at `steps` block steps (1..16); 0 restores the automatic length."""
         _check(lib().dsbcg_debug_shift_chunk(self._ctx, int(steps)), "dsbcg_debug_shift_chunk")
+
+    def debug_memory_limit(self, nbytes):
+        """dsbcg_debug_memory_limit (test hook): device allocations beyond
+        nbytes in all fail; -1 removes the limit."""
+        _check(lib().dsbcg_debug_memory_limit(self._ctx, int(nbytes)), "dsbcg_debug_memory_limit")
 
     def set_profiling(self, on=True):
         _check(lib().dsbcg_set_profiling(self._ctx, int(bool(on))), "dsbcg_set_profiling")
