@@ -24,8 +24,10 @@
  * by the library's kernels; other host memory is staged through device
  * buffers on the context's stream.  The caller owns every buffer it passes;
  * the library never frees them.  A context owns its workspace (including
- * the streams of its concurrent restarts) and its packed copies of the gauge
- * field.
+ * the streams of its concurrent restarts), its packed copies of the gauge
+ * field (one per precision used) and one block of working fields for dsbcg_apply
+ * and dsbcg_force, kept from call to call up to 1/32 of the device memory, so
+ * the first such call on a context also pays for its allocation.
  *
  * Errors: every call returns a dsbcg_status; nothing is thrown across the
  * ABI.  After DSBCG_ERR_CUDA the context should be destroyed.
@@ -153,7 +155,9 @@ dsbcg_status dsbcg_create(dsbcg_ctx** out, const int dims[4], const void* gauge,
 
 /* Replace the gauge field of an existing context (same dims).  The new field
  * is checked for NaN/Inf (DSBCG_ERR_NONFINITE) and packed again for every
- * precision on first use.  After any failed update the context holds no
+ * precision on first use; the buffers of the old field's copies are kept for
+ * it, but those that only links in SU(3) have are given back when the new field
+ * is not.  After any failed update the context holds no
  * gauge field: dsbcg_solve, dsbcg_apply, dsbcg_apply_static and dsbcg_force
  * return DSBCG_ERR_ARG until an update succeeds. */
 dsbcg_status dsbcg_update_gauge(dsbcg_ctx* ctx, const void* gauge);

@@ -1732,6 +1732,13 @@ dsbcg_status dsbcg_update_gauge(dsbcg_ctx* c, const void* gauge) {
     const int h = hf[0], hs = hf[1];
     if (h) return DSBCG_ERR_NONFINITE;
     c->su3 = (hs == 0);
+    if (!c->su3) {                       // nothing fills the copies that only SU(3) links have
+        fx_links_free(c);
+        for (void*& p : c->links12_mem) {
+            c->mem.give(p);
+            p = nullptr;
+        }
+    }
     CKS(ensure_links(c, P64));
     c->gauge_ok = true;
     return DSBCG_OK;

@@ -111,3 +111,27 @@ def test_in_place_application_at_the_limit():
     assert _apply(ctx, F, out=F) == 0
     ctx.close()
     assert (F - want).abs().max() <= 4 * 64 * 2.0 ** -53 * B.abs().max()
+
+
+def test_gauge_update_off_su3_gives_the_su3_copies_back():
+    """FP64 and FP32 applications on SU(3) links hold fixed-point links (576 bytes
+    per site) and 12-real ones (192); after an update to a field off SU(3) the
+    device has that memory free again, to the 2 MB granularity of two blocks."""
+    dims = (16, 16, 16, 16)
+    V = synth.volume(dims)
+    U = synth.su3_links(dims, 0.4, np.random.Generator(np.random.PCG64(5)))
+    F = torch.ones((1, 12 * V), dtype=torch.complex128, device=DEV)
+    off = torch.from_numpy(U * 1.01).to(DEV)
+    ctx = dsbcg.Context(dims, torch.from_numpy(U).to(DEV), 0.12)
+    try:
+        for storage in ("fp64", "fp32"):
+            ctx.apply("D", F, storage=storage)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ctx.update_gauge(off)
+        assert torch.cuda.mem_get_info()[0] - before >= 768 * V - (4 << 20)
+        ctx.update_gauge(torch.from_numpy(U).to(DEV))       # and back: both copies are made anew
+        for storage in ("fp64", "fp32"):
+            ctx.apply("D", F, storage=storage)
+    finally:
+        ctx.close()
