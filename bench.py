@@ -65,6 +65,52 @@ def imad_peak_tops(sm_mhz):
     return 152 * 64 * float(sm_mhz) * 1e6 / 1e12
 
 
+def residual_roofline(launches, nbytes, ms, V, m, sm_mhz):
+    """Roofline entry of the true-residual class r = b - sigma x - A x of m
+    columns per call, from the class's launches, algorithmic bytes (two links
+    passes and 8 m fields a call) and event time.  A call is two stencils, the
+    residual and its column norms (4 launches), and in block fixed point one
+    conversion more (5): the launches say which stencil ran.  Its work goes
+    against the integer multiply-add peak (1728 a site, field and D) or, for
+    the FP64 kernels, the FP64 peak, at the sampled SM clock."""
+    calls = nbytes / (16.0 * V * (72.0 + 96.0 * m))
+    fixed = launches > 4.5 * calls
+    nd = 2.0 * V * m * calls                          # sites x fields x D
+    flop = WILSON_FLOP_PER_SITE * nd
+    out = {"kernel": f"residual ({'fixed-point' if fixed else 'FP64'} stencil D, D^H + r = b - sigma x - A x)",
+           "bound": "alu", "traffic": None, "flop_per_solve": flop, "fields_per_solve": round(m * calls, 1),
+           "ms_per_solve": round(ms, 3)}
+    if fixed:
+        ach, pk = FX_MAD_PER_SITE * nd / (ms / 1e3) / 1e12, imad_peak_tops(sm_mhz)
+        out.update(unit="Tmad/s", mads_per_solve=FX_MAD_PER_SITE * nd,
+                   peak_source=f"derived: 152 SMs x 64 mad.wide/clock x {sm_mhz:.0f} MHz (sampled)")
+    else:
+        ach, pk = flop / (ms / 1e3) / 1e12, fp64_alu_peak_tflops(sm_mhz)
+        out.update(unit="TFLOP/s", peak_source=f"derived: 152 SMs x 2 FP64 FMA/clock x 2 flop x {sm_mhz:.0f} MHz (sampled)")
+    out.update(achieved=round(ach, 4), peak=round(pk, 4), frac=round(ach / pk, 4))
+    return out
+
+
+def fp64_stencil_roofline(launches, calls, per_call, ms, V, m, sm_mhz):
+    """The FP64 stencil of `calls` applications with per_call D each, from the
+    launches per class and the event time of the stencil class: in block fixed
+    point an application has one conversion beside its D launches; without one,
+    or where it was repeated, the FP64 kernels answered."""
+    fixed = launches["other"] == calls and launches["dslash"] == per_call * calls
+    t = ms / launches["dslash"] / 1e3
+    flop = WILSON_FLOP_PER_SITE * V * m
+    if fixed:
+        ach, pk, unit = FX_MAD_PER_SITE * V * m / t / 1e12, imad_peak_tops(sm_mhz), "Tmad/s"
+        src = f"derived: 152 SMs x 64 mad.wide/clock x {sm_mhz:.0f} MHz"
+    else:
+        ach, pk, unit = flop / t / 1e12, fp64_alu_peak_tflops(sm_mhz), "TFLOP/s"
+        src = f"derived: 152 SMs x 2 FP64 FMA/clock x 2 flop x {sm_mhz:.0f} MHz"
+    return {"kernel": "fx_stencil (FP64 in block fixed point)" if fixed else "dslash (FP64)", "bound": "alu",
+            "achieved": round(ach, 4), "peak": round(pk, 4), "unit": unit, "frac": round(ach / pk, 4),
+            "ms_per_launch": round(t * 1e3, 4), "flop_per_launch": flop, "TFLOPs": round(flop / t / 1e12, 4),
+            "peak_source": src}
+
+
 def fp32_alu_peak_tflops(sm_mhz):
     """FP32 FMA peak of a GB300 from unit counts and the SM clock: 152 SMs x
     128 FP32 lanes, one FMA (2 flop) per lane per clock.  The packed FMA
@@ -298,7 +344,7 @@ def run_ours(args):
             if kfl[q] > 0:
                 kernels[q]["TFLOPs"] = kfl[q] / (kms[q] / 1e3) / 1e12
     # HBM-bound classes in the reduced-precision storage; the true-residual
-    # class runs the fixed-point FP64 stencil, bound by the integer pipes, and the
+    # class runs the FP64 stencil, bound by the integer or FP64 pipes, and the
     # shift update (P_j, X_j on chip over a chunk of steps) by the FP32 FMA pipe
     hbm_bound = [q for q in ("dslash", "gram", "update") if q in kernels]
     dom = max(hbm_bound, key=lambda q: kms[q])
@@ -316,22 +362,7 @@ def run_ours(args):
                 "peak_source": f"{peak_kind} HBM copy bandwidth"}
 
     def residual_roof():
-        """FP64 true residuals r = b - sigma x - A x: each call converts its
-        fields to block fixed point, applies D and D^H to them (1728 integer
-        multiply-adds per site and field each) and forms the residual and its
-        norms; the class's multiply-adds over its event time against the
-        integer multiply-add peak at the sampled SM clock."""
-        calls = kla["residual"] / 5.0                 # conversion + 2 stencils + residual + column reduction
-        V = wl["B"].shape[1] // 12
-        nfields = (kby["residual"] / 16.0 - 72.0 * V * calls) / (8.0 * wl["B"].shape[1])
-        mads = 2.0 * FX_MAD_PER_SITE * V * nfields
-        ach = mads / (kms["residual"] / 1e3) / 1e12
-        pk = imad_peak_tops(clk_mhz)
-        return {"kernel": "residual (fixed-point FP64 stencil D, D^H + r = b - sigma x - A x)", "bound": "alu",
-                "achieved": round(ach, 4), "peak": round(pk, 4), "unit": "Tmad/s", "frac": round(ach / pk, 4),
-                "traffic": None, "mads_per_solve": mads, "flop_per_solve": 2.0 * WILSON_FLOP_PER_SITE * V * nfields,
-                "fields_per_solve": round(nfields, 1), "ms_per_solve": round(kms["residual"], 3),
-                "peak_source": f"derived: 152 SMs x 64 mad.wide/clock x {clk_mhz:.0f} MHz (sampled)"}
+        return residual_roofline(kla["residual"], kby["residual"], kms["residual"], n // 12, m, clk_mhz)
 
     def shift_roof():
         """Shift update over chunks of block steps: X_j += P_j Ut_j and
@@ -487,7 +518,7 @@ def run_ours(args):
                               "mixed_error_vs_fp64": {"max": float(err.max()),
                                                       "per_pair": [[float(f"{v:.3e}") for v in r] for r in err]}}
         del X64
-        # the FP64 stencil is bound by the integer pipes, not by HBM: time its D
+        # the FP64 stencil is bound by its pipe, not by HBM: time its D
         # launches (library CUDA events) on the workload's m fields
         try:
             ctx.set_profiling(True)
@@ -497,20 +528,12 @@ def run_ours(args):
             for _ in range(reps):
                 ctx.apply("A", B, storage="fp64")
             kms64, kl64 = ctx.read_profile()
-            ms_launch = kms64["dslash"] / kl64["dslash"]
             V = n // 12
-            flop = WILSON_FLOP_PER_SITE * V * m
             sm_mhz = (clk or {}).get("sm_mhz") or 2070.0
-            mads = FX_MAD_PER_SITE * V * m
-            pk = imad_peak_tops(sm_mhz)
-            ach = mads / (ms_launch / 1e3) / 1e12
+            sr = fp64_stencil_roofline(kl64, reps, 2, kms64["dslash"], V, m, sm_mhz)
             gb = (2.0 * m * n * 16 + 36.0 * V * 16) / 1e9
-            line["fp64_plain"]["stencil_roofline"] = {
-                "kernel": "fx_stencil (FP64 in block fixed point)", "bound": "alu", "achieved": round(ach, 4),
-                "peak": round(pk, 4), "unit": "Tmad/s", "frac": round(ach / pk, 4), "ms_per_launch": round(ms_launch, 4),
-                "flop_per_launch": flop, "TFLOPs": round(flop / (ms_launch / 1e3) / 1e12, 4),
-                "hbm_GBps": round(gb / (ms_launch / 1e3), 1),
-                "peak_source": f"derived: 152 SMs x 64 mad.wide/clock x {sm_mhz:.0f} MHz"}
+            sr["hbm_GBps"] = round(gb / (kms64["dslash"] / kl64["dslash"] / 1e3), 1)
+            line["fp64_plain"]["stencil_roofline"] = sr
         except Exception as e:           # the FP64 stencil figure must not cost the bench line
             line["fp64_plain"]["stencil_roofline"] = {"error": repr(e)[:300]}
         finally:
@@ -620,9 +643,10 @@ def _stencil_rate(ctx, B, storage, m, n, peak, clk_mhz):
            "frac_of_hbm": round(gb / (ms / 1e3) / peak, 4),
            "TFLOPs": round(WILSON_FLOP_PER_SITE * V * m / (ms / 1e3) / 1e12, 3)}
     if storage == "fp64":
-        mads = FX_MAD_PER_SITE * V * m / (ms / 1e3) / 1e12
+        sr = fp64_stencil_roofline(kl, reps, 1, kms["dslash"], V, m, clk_mhz)
         out["bound"] = "alu"
-        out["frac_of_imad_peak"] = round(mads / imad_peak_tops(clk_mhz), 4)
+        if sr["unit"] == "Tmad/s":
+            out["frac_of_imad_peak"] = sr["frac"]
         out["ratio_to_fp64_pipe_peak"] = round(out["TFLOPs"] / fp64_alu_peak_tflops(clk_mhz), 4)
     else:
         out["bound"] = "hbm"
