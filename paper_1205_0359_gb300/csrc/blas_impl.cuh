@@ -919,8 +919,8 @@ __global__ void __launch_bounds__(ROWS, (NF <= 12 && PW == P32) ? 4 : 1) shift_c
     }
 }
 
-// The same chunk for FP64 fields in block fixed point (fx.cuh), block widths up
-// to SHIFT_FX_NF_MAX.  P_j's row is held as limbs with one exponent per row, X_j's
+// The same chunk for FP64 fields in block fixed point (fx.cuh), for the block
+// widths of coef_fx.  P_j's row is held as limbs with one exponent per row, X_j's
 // in FP64; the coefficient tiles arrive as limbs with one exponent per column
 // (written by the m x m kernel), so right-hand sides of any scale keep their
 // own.  Per step
@@ -931,8 +931,11 @@ __global__ void __launch_bounds__(ROWS, (NF <= 12 && PW == P32) ? 4 : 1) shift_c
 //                       result does not depend on the chunk length) and split.
 // Limbs of P_j hold 56 bits and those of the coefficients 57, so the middle
 // sums stay below 2^62 at width 12.  A product sum is exact to about one unit of
-// 2^-56 of the row's largest entry times the column's, below the 2^-53 of every
-// step of an FP64 chain.  Bound: 24 NF^2 mad.wide per row and step at 64 per SM
+// 2^-56 of the row's largest entry times the column's.  That is a bound per row,
+// not per product: where an entry of the row is far below the largest one its
+// share is known to fewer bits than in an FP64 chain.  Over a field it is below
+// the 2^-53 of every step of such a chain relative to the norm of the block
+// (columns of V have norm 1), which is what X's residual is measured by.  Bound: 24 NF^2 mad.wide per row and step at 64 per SM
 // and clock beside 6 NF conversions and additions on the FP64 pipe, where the
 // FP64 form takes 8 NF^2 FMA at 2 per SM and clock.
 // A row with a NaN or an infinity, or a bad coefficient column, ends as NaN.

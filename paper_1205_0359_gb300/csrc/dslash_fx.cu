@@ -43,8 +43,10 @@
 // Overflow.  The limbs of a projected half spinor are at most 2^29 (sums of
 // two), those of a link at most 2^29 and 2^28.  A link row has norm <= 1, so
 // the h h sums of a component stay below 2^29 2^29 sqrt(6) < 2^60, the mixed
-// sums below 2^61, a hop's result below 2^59.3 and the sum over eight hops and
-// the diagonal term below 2^62.4.
+// sums below 2^61, a hop's result below 2^59.3 (sqrt(6) 2^58).  The diagonal term
+// may lie 2^4 above the accumulators' unit, so that it reaches 2^61: the sum over
+// eight hops (2^62.3) and the diagonal term stays below 2^62.8, and no term may
+// take another bit.
 //
 // A site that is all zero has exponent FX_ZERO.  A component that the
 // conversion holds as zero beside larger ones sets *flag.  A site with a NaN, an

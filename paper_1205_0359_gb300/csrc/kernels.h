@@ -131,7 +131,10 @@ void launch_gram_reduce(const double* partials, int nblk, int nf_max, int herm, 
                         cudaStream_t st);
 // FP64 blocks of widths up to 12 run their products with the m x m coefficients
 // in block fixed point (fx.cuh): the coefficient tiles then hold limbs, and ce
-// (else NULL) their column exponents, M_MAX words per tile
+// (else NULL) their column exponents, M_MAX words per tile.  Wider blocks stay
+// on the FP64 pipe: at 16 the limb sums still fit (2^61.6) but the shift update
+// spills (728 bytes; 255 registers).  16^4, s = 4, m = 13 and 16 take 1084 and 1148 ms
+// there, with a 16-wide fixed-point form 827 and 923, which is not built.
 inline bool coef_fx(int prec, int m) { return prec == P64 && m <= 12; }
 // W = Y - V a - Vp b^H, coefficients from the device (work precision copies;
 // ce: exponents of a, then of b^H)

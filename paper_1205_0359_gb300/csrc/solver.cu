@@ -403,12 +403,15 @@ bool fx_component_kappa(double kappa) { return fabs(kappa) >= 1.0 / 64; }
 
 // True residuals of m columns in fixed point: always for FP64 storage, and for
 // the reduced storages from FX_RESID_MIN sites x columns of the full lattice.
-// Below it the FP64 residuals run beside latency-bound restarts and cost
-// little, and the solutions stay bitwise those of the FP64 chain, which an
-// FP32 link gradient that rounds them to 24 bits shows.  Solves (m of them,
-// s = 8, FP32 storage) on the FP64 pipe / in fixed point, ms: 8^3 x 16, 8:
-// 24.4 / 22.2; 8^3 x 16, 12: 35.5 / 32.3; 8^2 x 16^2, 8 (at the line): 34.7 /
-// 28.6; 12^3 x 24, 6: 53.6 / 44.2; 12^3 x 24, 12: 99.4 / 80.3.
+// The line is a choice of arithmetic, not of time: below it the FP64 residuals
+// run beside latency-bound restarts, and the solutions stay bitwise those of the
+// FP64 chain.  What that keeps is small: link gradients in FP32 storage (m = 2,
+// 5, 8 on 8^3 x 16 and 7 x 9 x 10 x 13) are as far from FP64 ones either way (2.4
+// to 4.4e-7, the two differing by 1e-5 of that).  Solves (m of them, s = 8, FP32
+// storage, tol 1e-8) on the FP64 pipe / in fixed point, ms: 4^3 x 8, 4: 8.4 / 8.3;
+// 8^3 x 16, 2: 10.8 / 10.1; 8^3 x 16, 5: 15.8 / 14.7; 8^3 x 16, 8: 20.1 / 17.9;
+// 8^2 x 16^2, 7: 27.4 / 23.1; at the line and above (other shifts) 8^2 x 16^2, 8:
+// 34.7 / 28.6; 12^3 x 24, 6: 53.6 / 44.2; 12^3 x 24, 12: 99.4 / 80.3.
 constexpr size_t FX_RESID_MIN = (size_t)1 << 17;
 bool fx_residuals(const dsbcg_ctx* c, int prec, int m) { return prec == P64 || c->V * m >= FX_RESID_MIN; }
 // site exponents of the fields of one fixed-point operator application of m
@@ -950,10 +953,16 @@ dsbcg_status lane_start(dsbcg_ctx* c, Lane& L, const void* rhs, int rhs_prec, si
 // Block steps of fewer than AHEAD_MAX sites x columns (of the full lattice) are
 // bound by launch and m x m latency: their kernels are launched ahead (Stream).
 // Above it the waiting CTAs hold slots that the running kernels of this and the
-// other lanes would use.  ms per call, plain / ahead: fp64 4^4 m=4 (1 k) 9.1 /
-// 7.2, rational step 8^3 x 16 m=2 (16 k) 26.6 / 23.8, gradient 7x9x10x13 m=5
-// (41 k) 25.4 / 22.7; Schur 12^3 x 24 m=6 (249 k) 19.6 / 20.2, fp64 16^4 m=4 (262
-// k) 119 / 133, fp32 16^3 x 32 m=12 (1.6 M) 244 / 250.
+// other lanes would use.  Where that begins depends on the width: on narrow
+// blocks, whose steps are short beside their stencils, at the line; wide ones
+// gain to about twice it, a few percent that a second constant would be for.
+// ms per call, plain / ahead (thousands of site-columns), s = 4: FP64 8^3 x 16,
+// m = 4 (33) 17.5 / 17.8, m = 8 (66) 43.2 / 39.8; 8^2 x 16^2, m = 6 (98) 64.1 / 61.5,
+// m = 8 (131) 77.2 / 74.3, m = 12 (197) 152.3 / 148.1; 16^4, m = 2 (131) 52.3 / 64.9;
+// 12^3 x 24, m = 4 (166) 51.4 / 58.7.  FP32, the same: 11.1 / 9.1, 15.8 / 13.9, 17.7 /
+// 16.3, 17.9 / 16.7, 27.8 / 27.2, 17.8 / 19.4, 17.7 / 17.0.  Schur, FP32: 12^3 x 24, m = 3
+// (124) 10.8 / 9.8, m = 6 (249) 19.6 / 20.2.  FP64 16^4, m = 4 (262) 119 / 133; FP32
+// 16^3 x 32, m = 12 (1573) 244 / 250.
 constexpr size_t AHEAD_MAX = (size_t)1 << 17;
 bool steps_ahead(const dsbcg_ctx* c, int m) { return !c->profiling && c->V * m < AHEAD_MAX; }
 
