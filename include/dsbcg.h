@@ -59,6 +59,20 @@ typedef enum {
  * accumulated solutions are IEEE FP64 by default (dsbcg_params.fp64_residuals
  * = 1); for the reduced storages dsbcg_params.fp64_residuals = 0 selects
  * double-float arithmetic for them instead.
+ * "FP64" fields, coefficients, residuals and solutions are held as FP64
+ * numbers. Where the links are in SU(3) (to 1e-10), the operator inside
+ * FP64-storage solves and inside the true residuals of wider reduced-storage
+ * solves runs on the integer pipe in block fixed point: 57 bits under one
+ * exponent per site, for the links 2^-58 of one.  So do, in FP64 storage with
+ * m <= 12 and on any links, the updates of the blocks and of the shifted
+ * solutions: 56 bits under one exponent per row (the numbers of one site and
+ * component in all vectors of a block) and 57 under one per coefficient
+ * column.  Their errors are no larger than those of FP64 arithmetic relative
+ * to the norm of a vector, which is what tol and the reported residuals are
+ * relative to; a number far below the others under its exponent is known to
+ * fewer than 53 bits.  The operator on links off SU(3), or without device
+ * memory for the fixed-point links, wider blocks and the m x m work run in
+ * IEEE FP64 arithmetic.
  * DSBCG_PREC_DF32 ("double-float"): each real number is an unevaluated sum
  * hi + lo of two FP32 words (48-bit significand, FP32 exponent range,
  * arithmetic on the FP32 pipes through error-free transformations).  It is
@@ -136,7 +150,7 @@ typedef struct {
 #define DSBCG_KCLASS_GRAM 1         /* tall-skinny Gram products */
 #define DSBCG_KCLASS_UPDATE 2       /* block update W = Y - V a - V' b^H and V' = W S */
 #define DSBCG_KCLASS_SHIFT 3        /* shift update of P_j, X_j over a chunk of steps */
-#define DSBCG_KCLASS_SMALL 4        /* FP64 m x m kernels */
+#define DSBCG_KCLASS_SMALL 4        /* m x m kernels */
 #define DSBCG_KCLASS_RESIDUAL 5     /* true residuals (FP64 or double-float) */
 #define DSBCG_KCLASS_OTHER 6
 
@@ -291,8 +305,11 @@ dsbcg_status dsbcg_apply(dsbcg_ctx* ctx, int op, int storage, int m, const void*
  * this entry point exists for callers that cannot call cudaMalloc at the time
  * of the call, e.g. code whose memory pool has already reserved the whole GPU,
  * or latency-critical loops where cudaMalloc's implicit device
- * synchronisation is not acceptable.  Same operation, arguments and result as
- * dsbcg_apply, with these differences:
+ * synchronisation is not acceptable.  Same operation and arguments as
+ * dsbcg_apply, and the same result to the rounding of the stencil, with these
+ * differences:
+ *   - FP64 always runs in the FP64 kernels (dsbcg_apply: in block fixed point on
+ *     links in SU(3));
  *   - in and out must be device pointers (host buffers would need staging);
  *   - the packed working fields live in one static device array of
  *     DSBCG_STATIC_SCRATCH_BYTES (32 MiB) that every GPU which loads the library
