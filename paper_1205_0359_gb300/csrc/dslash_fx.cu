@@ -37,7 +37,9 @@
 // of 1.6 million components of Gaussian fields was 2^56.3 to 2^57.4 units (kappa
 // 0.11 to 0.13; half lattice 2^56.0), and the tail falls with the 16th power.
 // Sparse sources and fields that fall by decades from site to site do.  The check
-// takes 1% of an application (A to 12 fields of 16^3 x 32: 1.121 -> 1.133 ms).
+// takes 2% of an application (A to 12 fields of 16^3 x 32: 1.12 -> 1.14 ms), and
+// a call that fails it 0.05 to 1.1 ms more than the FP64 kernels (4^4: 0.095 ->
+// 0.144 ms, 16^3 x 32: 5.26 -> 6.35).
 // A solve's applications do not check: its contract is the norm of the residual.
 //
 // Overflow.  The limbs of a projected half spinor are at most 2^29 (sums of
